@@ -193,14 +193,14 @@ int alloc(relu_qp_t h, T** p, size_t count) {
 }
 
 // FP64 building blocks of the offline stage (setup_fp64.cu), on h->stream:
-// C = alpha op(A) op(B) + beta C (row-major); in-place blocked Cholesky K = L L^T
-// (Linv: ceil(n / kCholNB) diagonal-block inverses of kCholNB^2, T: n x kCholNB
-// scratch, *flag set on a pivot <= 0); Rhs (n x NR) <- K^{-1} Rhs (T2: kCholNB x NR).
-constexpr int kCholNB = 64;
+// C = alpha op(A) op(B) + beta C (row-major); D (ldd) <- K^{-1} for nb symmetric positive
+// definite n x n matrices s doubles apart (lower triangles read, Km overwritten; Lm and Li:
+// n x n scratch each, same spacing; D sD doubles apart; flag[b] set on a pivot <= 0).
+constexpr int kCholNB = 32;
 int dgemm(relu_qp_t h, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, int lda,
           const double* B, int ldb, double beta, double* C, int ldc);
-int cholesky(relu_qp_t h, double* Km, int n, double* Linv, double* T, int* flag);
-int chol_solve(relu_qp_t h, const double* L, int n, const double* Linv, double* Rhs, int NR, double* T2);
+int spd_inverse(relu_qp_t h, int nb, int n, double* Km, double* Lm, double* Li, long long s, double* D, int ldd,
+                long long sD, int* flag);
 // Condensing of a linear MPC problem (condense.cu); error text in *err.
 int condense_mpc(int nx, int nu, int N, const double* A, const double* B, const double* Q, const double* R,
                  const double* QN, bool state_rows, const double* K, int precondition, void* stream, double* P,
@@ -237,7 +237,7 @@ int batch_update_x0(relu_qp_t h, int B, const float* X0);
 int batch_solve(relu_qp_t h, int B, const float* Xw, const float* Lw, const int* rw, double eps_abs,
                 double eps_rel, int max_iter, float* Xo, float* Zo, float* Lo, relu_qp_info* infos);
 // BF16 hi/mid/lo parts of the FP64 layer for the tcgen05 backend (setup_fp64.cu).
-int pack_bf16_layer(relu_qp_t h, int r, const double* X, const double* AX);
+int pack_bf16_layer(relu_qp_t h, int r, const double* X, const double* V);
 int pack_bf16_check(relu_qp_t h, const double* dP, const double* dA);
 int batch_finish_setup(relu_qp_t h);
 // Continuous batching (batch.cu).

@@ -115,21 +115,20 @@ struct Ctx {
 
 // K (nu x nx) = (R + B^T X B)^{-1} B^T X A for the current X.
 int gain(Ctx& c, int nx, int nu, const double* A, const double* B, const double* R, const double* X, double* BtX,
-         double* G, double* K, double* Linv, double* T, double* T2, int* flag) {
+         double* G, double* K0, double* K, double* S, int* flag) {
     relu_qp_t h = &c.h;
     RQ_TRY(dgemm(h, true, false, nu, nx, nx, 1.0, B, nu, X, nx, 0.0, BtX, nx));        // B^T X
     RQ_CUDA(h, cudaMemcpyAsync(G, R, sizeof(double) * nu * nu, cudaMemcpyDeviceToDevice, h->stream));
     RQ_TRY(dgemm(h, false, false, nu, nu, nx, 1.0, BtX, nx, B, nu, 1.0, G, nu));        // R + B^T X B
-    RQ_TRY(dgemm(h, false, false, nu, nx, nx, 1.0, BtX, nx, A, nx, 0.0, K, nx));        // B^T X A
-    RQ_TRY(cholesky(h, G, nu, Linv, T, flag));
-    RQ_TRY(chol_solve(h, G, nu, Linv, K, nx, T2));
-    return RELU_QP_OK;
+    RQ_TRY(dgemm(h, false, false, nu, nx, nx, 1.0, BtX, nx, A, nx, 0.0, K0, nx));       // B^T X A
+    const size_t uu = (size_t)nu * nu;
+    RQ_TRY(spd_inverse(h, 1, nu, G, S, S + uu, (long long)uu, S + 2 * uu, nu, (long long)uu, flag));
+    return dgemm(h, false, false, nu, nx, nu, 1.0, S + 2 * uu, nu, K0, nx, 0.0, K, nx);
 }
 
 int lqr_gain(Ctx& c, int nx, int nu, const double* A, const double* B, const double* Q, const double* R, double* K) {
     relu_qp_t h = &c.h;
-    const int nblk = ceil_div(nu, kCholNB);
-    double *X, *Xn, *BtX, *G, *AmBK, *XA, *Linv, *T, *T2;
+    double *X, *Xn, *BtX, *G, *AmBK, *XA, *K0, *S;
     unsigned long long* red;
     int* flag;
     RQ_TRY(c.buf(&X, (size_t)nx * nx));
@@ -138,9 +137,8 @@ int lqr_gain(Ctx& c, int nx, int nu, const double* A, const double* B, const dou
     RQ_TRY(c.buf(&G, (size_t)nu * nu));
     RQ_TRY(c.buf(&AmBK, (size_t)nx * nx));
     RQ_TRY(c.buf(&XA, (size_t)nx * nx));
-    RQ_TRY(c.buf(&Linv, (size_t)nblk * kCholNB * kCholNB));
-    RQ_TRY(c.buf(&T, (size_t)nu * kCholNB));
-    RQ_TRY(c.buf(&T2, (size_t)kCholNB * nx));
+    RQ_TRY(c.buf(&K0, (size_t)nu * nx));
+    RQ_TRY(c.buf(&S, 3 * (size_t)nu * nu));
     RQ_TRY(c.buf(&red, 2 * kRiccatiCheckEvery));
     RQ_TRY(c.buf(&flag, 1));
     RQ_CUDA(h, cudaMemcpyAsync(X, Q, sizeof(double) * nx * nx, cudaMemcpyDeviceToDevice, h->stream));
@@ -148,7 +146,7 @@ int lqr_gain(Ctx& c, int nx, int nu, const double* A, const double* B, const dou
     for (int it = 0; it < kRiccatiMaxIter && !converged; it += kRiccatiCheckEvery) {
         RQ_CUDA(h, cudaMemsetAsync(red, 0, sizeof(unsigned long long) * 2 * kRiccatiCheckEvery, h->stream));
         for (int s = 0; s < kRiccatiCheckEvery; ++s) {
-            RQ_TRY(gain(c, nx, nu, A, B, R, X, BtX, G, K, Linv, T, T2, flag));
+            RQ_TRY(gain(c, nx, nu, A, B, R, X, BtX, G, K0, K, S, flag));
             RQ_CUDA(h, cudaMemcpyAsync(AmBK, A, sizeof(double) * nx * nx, cudaMemcpyDeviceToDevice, h->stream));
             RQ_TRY(dgemm(h, false, false, nx, nx, nu, -1.0, B, nu, K, nx, 1.0, AmBK, nx));    // A - B K
             RQ_TRY(dgemm(h, false, false, nx, nx, nx, 1.0, X, nx, AmBK, nx, 0.0, XA, nx));     // X (A - B K)
@@ -177,7 +175,7 @@ int lqr_gain(Ctx& c, int nx, int nu, const double* A, const double* B, const dou
     }
     if (!converged)
         return fail(h, RELU_QP_ERR_INVALID, "condense: the Riccati iteration did not converge");
-    return gain(c, nx, nu, A, B, R, X, BtX, G, K, Linv, T, T2, flag);
+    return gain(c, nx, nu, A, B, R, X, BtX, G, K0, K, S, flag);
 }
 
 int condense(Ctx& c, int nx, int nu, int N, const double* hA, const double* hB, const double* hQ, const double* hR,
@@ -267,6 +265,8 @@ int condense_mpc(int nx, int nu, int N, const double* A, const double* B, const 
                  double* Acon, double* F, double* E, double* K_out, std::string* err) {
     Ctx c;
     c.h.stream = (cudaStream_t)stream;
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&c.h.num_sms, cudaDevAttrMultiProcessorCount, dev);
     const int rc = condense(c, nx, nu, N, A, B, Q, R, QN, state_rows, K, precondition, P, Acon, F, E, K_out);
     if (rc != RELU_QP_OK) *err = c.h.err;
     return rc;
