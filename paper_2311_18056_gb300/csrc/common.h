@@ -199,6 +199,9 @@ int alloc(relu_qp_t h, T** p, size_t count) {
 constexpr int kCholNB = 32;
 int dgemm(relu_qp_t h, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, int lda,
           const double* B, int ldb, double beta, double* C, int ldc);
+// (dgemm_strided: nb products with beta = 0, operands tA, tB, tC doubles apart)
+int dgemm_strided(relu_qp_t h, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, int lda,
+                  long long tA, const double* B, int ldb, long long tB, double* C, int ldc, long long tC, int nb);
 int spd_inverse(relu_qp_t h, int nb, int n, double* Km, double* Lm, double* Li, long long s, double* D, int ldd,
                 long long sD, int* flag);
 // Condensing of a linear MPC problem (condense.cu); error text in *err.

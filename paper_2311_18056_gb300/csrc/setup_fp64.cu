@@ -417,6 +417,16 @@ int dgemm(relu_qp_t h, bool ta, bool tb, int M, int N, int K, double alpha, cons
     return dgemm_batch(h, gemm(ta, tb, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc), 1);
 }
 
+int dgemm_strided(relu_qp_t h, bool ta, bool tb, int M, int N, int K, double alpha, const double* A, int lda,
+                  long long tA, const double* B, int ldb, long long tB, double* C, int ldc, long long tC, int nb) {
+    Gemm g = gemm(ta, tb, M, N, K, alpha, A, lda, B, ldb, 0.0, C, ldc);
+    g.nb2 = nb;
+    g.tA = tA;
+    g.tB = tB;
+    g.tC = g.tD = tC;
+    return dgemm_batch(h, g, 1);
+}
+
 int spd_inverse(relu_qp_t h, int nb, int n, double* Km, double* Lm, double* Li, long long s, double* D, int ldd,
                 long long sD, int* flag) {
     for (int b = 0; b < nb; ++b) RQ_CUDA(h, cudaMemsetAsync(Li + b * s, 0, sizeof(double) * n * n, h->stream));

@@ -112,3 +112,36 @@ def test_condense_smallest_shapes(rq):
             o = C.condense_mpc(A, B, Q, R, N, umin=-np.ones(nu), umax=np.ones(nu))
             for k in ("P", "A", "F", "E", "K"):
                 assert close(g[k], o[k], 1e-9), (nx, N, k)
+
+
+@pytest.mark.parametrize("nx,nu,N", [(15, 17, 3), (33, 5, 17), (65, 31, 2), (160, 3, 4), (161, 3, 4)])
+def test_condense_at_tile_and_doubling_edges(rq, nx, nu, N):
+    """Sizes around the product tiles, ragged doublings of the powers, and both sides of the
+    largest plant whose Riccati iterates are doubled (160 states); full weight matrices."""
+    A, B, _, _ = plant(nx * 100 + nu, nx, nu)
+    rng = np.random.default_rng(nx)
+    M = rng.standard_normal((nx, nx)) / np.sqrt(nx)
+    Q, R, QN = M @ M.T + 0.1 * np.eye(nx), 0.1 * np.eye(nu) + 0.01, 2.0 * np.eye(nx)
+    Q = 0.5 * (Q + Q.T)
+    g = rq.condense_mpc(A, B, Q, R, N, QN=QN, umin=-np.ones(nu), umax=np.ones(nu), xmin=-np.ones(nx))
+    o = C.condense_mpc(A, B, Q, R, N, QN=QN, umin=-np.ones(nu), umax=np.ones(nu), xmin=-np.ones(nx))
+    for k in ("K", "P", "A", "F", "E"):
+        assert close(g[k], o[k], 1e-9), k
+
+
+def test_condense_weights_outside_the_doubling(rq):
+    """Weights that the doubling does not take: R semidefinite (B'XB makes the step's matrix
+    definite), and an indefinite Q, go through the plain iteration as before; R + B'XB that is not
+    positive definite is still refused."""
+    A, B, Q, _ = plant(21, 6, 2)
+    R = np.zeros((2, 2))
+    g = rq.condense_mpc(A, B, Q, R, 5, umin=-np.ones(2), umax=np.ones(2))
+    X = Q.copy()
+    for _ in range(2000):
+        K = np.linalg.solve(R + B.T @ X @ B, B.T @ X @ A)
+        X = Q + A.T @ X @ (A - B @ K)
+        X = 0.5 * (X + X.T)
+    assert close(g["K"], np.linalg.solve(R + B.T @ X @ B, B.T @ X @ A), 1e-9)
+    with pytest.raises(rq.ReluQPError) as e:
+        rq.condense_mpc(A, B, -Q, 1e-3 * np.eye(2), 5, umin=-np.ones(2), umax=np.ones(2))
+    assert e.value.kind in ("NOT_PD", "INVALID")
