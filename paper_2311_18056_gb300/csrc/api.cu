@@ -93,7 +93,7 @@ int upload_scaling(relu_qp_t h) {
     const int n = h->n, m = h->m, mm = m > 0 ? m : 1;
     std::vector<float> f(n > mm ? n : mm);
     auto put = [&](float** dst, int len, auto fn) -> int {
-        RQ_TRY(rq::alloc(h, dst, (size_t)len));
+        RQ_TRY(rq::alloc(h, dst, rq::round_up(len, 16)));   // (the split backend reads padded rows)
         for (int k = 0; k < len; ++k) f[k] = (float)fn(k);
         RQ_CUDA(h, cudaMemcpy(*dst, f.data(), sizeof(float) * len, cudaMemcpyHostToDevice));
         return RELU_QP_OK;
@@ -159,7 +159,7 @@ int setup_impl(relu_qp_t h, const double* P, const double* q, const double* A, c
     h->h_u.assign(u, u + m);
     h->eq.resize(m);
     std::vector<double> row_scale(m);
-    std::vector<float> rs(m > 0 ? m : 1, 1.0f);
+    std::vector<float> rs(rq::round_up(m > 0 ? m : 1, 16), 1.0f);
     for (int i = 0; i < m; ++i) {
         h->eq[i] = (l[i] == u[i]) ? 1 : 0;
         row_scale[i] = h->eq[i] ? h->opts.eq_scale : 1.0;
@@ -183,7 +183,7 @@ int setup_impl(relu_qp_t h, const double* P, const double* q, const double* A, c
     RQ_TRY(rq::alloc(h, &h->q32, (size_t)n));
     RQ_TRY(rq::alloc(h, &h->l32, (size_t)(m > 0 ? m : 1)));
     RQ_TRY(rq::alloc(h, &h->u32, (size_t)(m > 0 ? m : 1)));
-    RQ_TRY(rq::alloc(h, &h->rs32, (size_t)(m > 0 ? m : 1)));
+    RQ_TRY(rq::alloc(h, &h->rs32, rs.size()));
     RQ_CUDA(h, cudaMemcpy(h->rs32, rs.data(), sizeof(float) * rs.size(), cudaMemcpyHostToDevice));
     rq::SingleWork& w = h->sw;
     RQ_TRY(rq::alloc(h, &w.y, (size_t)h->ldw));

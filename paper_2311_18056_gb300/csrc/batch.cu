@@ -40,12 +40,13 @@ struct W32Ptrs {
     const float* w[RQ_MAX_RHO];
 };
 
-// C[i][j] = alpha * sum_k X[i][k] W[j][k] + (off ? off[j] : 0), bounds-checked
-// (problem updates; not on the per-layer path).
+// C[i][j'] = alpha * sum_k X[i][k] W[j][k] + (off ? off[j] : 0), bounds-checked
+// (problem updates; not on the per-layer path); j' = j, or j + shift from j = split on
+// (rows of a layer into its padded layout).
 __global__ void __launch_bounds__(256) sgemm_nt_kernel(int M, int N, int K, const float* __restrict__ X, int ldx,
                                                        const float* __restrict__ W, int ldw, float alpha,
                                                        const float* __restrict__ off, float* __restrict__ C,
-                                                       int ldc) {
+                                                       int ldc, int split, int shift) {
     __shared__ float Xs[16][64 + 4];
     __shared__ float Ws[16][64 + 4];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -86,7 +87,7 @@ __global__ void __launch_bounds__(256) sgemm_nt_kernel(int M, int N, int K, cons
         for (int v = 0; v < 4; ++v) {
             const int j = j0 + tx + 16 * v;
             if (j >= N) continue;
-            C[(size_t)i * ldc + j] = alpha * acc[u][v] + (off ? off[j] : 0.f);
+            C[(size_t)i * ldc + j + (j >= split ? shift : 0)] = alpha * acc[u][v] + (off ? off[j] : 0.f);
         }
     }
 }
@@ -204,8 +205,7 @@ __device__ __forceinline__ bool fp32_slots(const BatchParams& p, int& tile, int&
     return TS == kSlotTile || p.perm[slot0] >= 0;
 }
 
-// One layer for every active slot tile (FP32 backend, and the accurate first
-// layer of a chunk in the BF16 split form).
+// One layer for every active slot tile (FP32 backend).
 template <int TS, int TR>
 __global__ void __launch_bounds__(256) batch_layer_fp32_kernel(BatchParams p, W32Ptrs wp) {
     int tile, slot0;
@@ -468,15 +468,15 @@ __global__ void batch_init_kernel(BatchParams p, int B, int warm, int lam_given,
     }
     if (lane < RW_WORDS) p.RED[(size_t)qp * RW_WORDS + lane] = 0u;
     if (qp >= B) return;
-    for (int i = lane; i < p.m; i += 32) {
+    // (the padding is zeroed too: a QP of NaN data leaves NaN there)
+    for (int i = lane; i < p.ldm; i += 32) {
         const size_t o = (size_t)qp * p.ldm + i;
-        const float ax = warm ? p.AY[o] : 0.f;
+        const float ax = warm && i < p.m ? p.AY[o] : 0.f;
         p.AY[o] = ax;
         p.Z[o] = ax;
-        p.LAM[o] = lam_given ? p.LSTD[o] : 0.f;
+        p.LAM[o] = lam_given && i < p.m ? p.LSTD[o] : 0.f;
     }
-    if (!warm)
-        for (int k = lane; k < p.n; k += 32) p.Y[(size_t)qp * p.ldn + k] = 0.f;
+    for (int k = (warm ? p.n : 0) + lane; k < p.ldn; k += 32) p.Y[(size_t)qp * p.ldn + k] = 0.f;
 }
 
 // out[r] = max_k |X[r][k] f[k]| (f = nullptr: 1).
@@ -522,10 +522,10 @@ __global__ void build_wc32_kernel(const float* __restrict__ P32, const float* __
 }
 
 int sgemm_nt(relu_qp_t h, int M, int N, int K, const float* X, int ldx, const float* W, int ldw, float alpha,
-             const float* off, float* C, int ldc) {
+             const float* off, float* C, int ldc, int split = 0, int shift = 0) {
     if (M <= 0 || N <= 0) return RELU_QP_OK;
     dim3 grid(ceil_div(N, 64), ceil_div(M, 64));
-    sgemm_nt_kernel<<<grid, 256, 0, h->stream>>>(M, N, K, X, ldx, W, ldw, alpha, off, C, ldc);
+    sgemm_nt_kernel<<<grid, 256, 0, h->stream>>>(M, N, K, X, ldx, W, ldw, alpha, off, C, ldc, split, shift);
     RQ_CUDA(h, cudaGetLastError());
     ++h->launches;
     return RELU_QP_OK;
@@ -546,6 +546,7 @@ BatchParams base_params(relu_qp_t h) {
     p.cap = w.cap;
     p.slots = w.slots;
     p.nr = h->nr;
+    p.bsh = w.nP - h->n;
     for (int r = 0; r < h->nr; ++r) {
         p.rho[r] = (float)h->be[r].rho;
         p.rhod[r] = h->be[r].rho;
@@ -558,6 +559,17 @@ BatchParams base_params(relu_qp_t h) {
     p.L = w.L; p.U = w.U; p.Q = w.Q; p.BIAS = w.BIAS; p.QN = w.QN;
     p.perm = w.perm; p.tile_rho = w.tile_rho; p.counters = w.counters; p.RED = w.RED;
     return p;
+}
+
+// p in the backend's row layout (the padded one of the split form), for the kernels that
+// run the layers and the residual products and fill their operand
+BatchParams layer_params(relu_qp_t h, const BatchParams& p) {
+    BatchParams q = p;
+    q.n = h->bw.nP;
+    q.m = h->bw.RP - h->bw.nP;
+    q.R = h->bw.RP;
+    q.bsh = 0;
+    return q;
 }
 
 int scale_rows(relu_qp_t h, float* X, int rows, int cols, int ld, const float* f) {
@@ -593,7 +605,6 @@ size_t batch_slot_bytes(relu_qp_t h) {
     b += sizeof(int);                                   // perm
     if (w.prec == RELU_QP_PREC_BF16X3) {
         b += 2 * w.ldR * f;                             // C, SREF
-        b += w.ldk * f + w.ldkc * f;                    // S32, CK32
         b += 2 * (7 * (size_t)w.ldk + 3 * (size_t)w.ldkc);   // BF16 operand parts and check operand
     } else {
         b += 2 * w.ldk * f + w.ldkc * f;                // S32 pair, CK32
@@ -608,15 +619,18 @@ int batch_alloc(relu_qp_t h) {
     w.cap = h->opts.max_batch;
     w.prec = h->opts.batch_precision;
     w.slots = (int)round_up(w.cap, kSlotTile) + nr * kSlotTile;
-    w.ldn = (int)round_up(n, 4);
-    w.ldm = (int)round_up(mm, 4);
-    w.ldR = (int)round_up(R, 4);
-    w.ldk = h->ldw;
+    const bool bf16 = w.prec == RELU_QP_PREC_BF16X3;
+    w.nP = bf16 ? (int)round_up(n, 16) : n;
+    w.RP = bf16 ? w.nP + (int)round_up(m, 16) : R;
+    w.ldn = (int)round_up(n, bf16 ? 16 : 4);
+    w.ldm = (int)round_up(mm, bf16 ? 16 : 4);
+    w.ldR = (int)round_up(w.RP, 4);
+    w.ldk = (int)round_up(w.RP, 64);
     w.n64 = (int)round_up(n, 64);
     w.m64 = (int)round_up(mm, 64);
     w.ldkc = w.n64 + w.m64;
-    w.Rpad = (int)round_up(R, 256);
-    w.npad = (int)round_up(n + m, 256);
+    w.Rpad = (int)round_up(w.RP, 256);
+    w.npad = w.Rpad;
     const size_t cap = w.cap;
     RQ_TRY(alloc(h, &w.Y, cap * w.ldn));
     RQ_TRY(alloc(h, &w.Q, cap * w.ldn));
@@ -643,11 +657,9 @@ int batch_alloc(relu_qp_t h) {
     RQ_TRY(alloc(h, &w.perm, (size_t)w.slots));
     RQ_TRY(alloc(h, &w.tile_rho, (size_t)w.slots / kSlotTile));
     RQ_TRY(alloc(h, &w.counters, CNT_WORDS));
-    if (w.prec == RELU_QP_PREC_BF16X3) {
+    if (bf16) {
         RQ_TRY(alloc(h, &w.C, cap * w.ldR));
         RQ_TRY(alloc(h, &w.SREF, cap * w.ldR));
-        RQ_TRY(alloc(h, &w.S32, (size_t)w.slots * w.ldk));   // FP32 operand of the accurate layer
-        RQ_TRY(alloc(h, &w.CK32, (size_t)w.slots * w.ldkc));  // FP32 check operand
         RQ_TRY(alloc(h, &w.Wc32, (size_t)(n + m) * w.ldkc));
         RQ_TRY(dev_alloc(h, &w.OPND, sizeof(uint16_t) * 7 * (size_t)w.slots * w.ldk + 1024));
         RQ_TRY(dev_alloc(h, &w.CK, sizeof(uint16_t) * 3 * (size_t)w.slots * w.ldkc + 1024));
@@ -690,7 +702,7 @@ __global__ void tune_perm_kernel(int slots, int cap, int active_tiles, int per_t
 // the next solve.  RELU_QP_TUNE_LOG=1 prints the measurements to stderr.
 int tc_tune(relu_qp_t h) {
     BatchWork& w = h->bw;
-    BatchParams p = base_params(h);
+    BatchParams p = layer_params(h, base_params(h));
     const size_t opart = (size_t)w.slots * w.ldk;
     __nv_bfloat16* OP = static_cast<__nv_bfloat16*>(w.OPND);
     p.flags = EPI_REFINE;
@@ -839,7 +851,7 @@ int batch_update(relu_qp_t h, int B, const float* Q, const float* L, const float
     if (Q) {
         for (int r = 0; r < h->nr; ++r)
             RQ_TRY(sgemm_nt(h, B, R, n, w.Q, w.ldn, h->be[r].Bop, n, 1.f, nullptr,
-                            w.BIAS + (size_t)r * w.cap * w.ldR, w.ldR));
+                            w.BIAS + (size_t)r * w.cap * w.ldR, w.ldR, n, w.nP - n));
         row_absmax_kernel<<<ceil_div(B * 32, 256), 256, 0, h->stream>>>(w.Q, B, n, w.ldn, h->sc_rx, w.QN);
         RQ_CUDA(h, cudaGetLastError());
         ++h->launches;
@@ -905,7 +917,7 @@ int batch_update_x0(relu_qp_t h, int B, const float* X0) {
     }
     for (int r = 0; r < h->nr; ++r)
         RQ_TRY(sgemm_nt(h, B, R, nx, w.X0, w.ldx, w.G[r], w.ldx, 1.f, nullptr, w.BIAS + (size_t)r * w.cap * w.ldR,
-                        w.ldR));
+                        w.ldR, n, w.nP - n));
     row_absmax_kernel<<<ceil_div(B * 32, 256), 256, 0, h->stream>>>(w.Q, B, n, w.ldn, h->sc_rx, w.QN);
     RQ_CUDA(h, cudaGetLastError());
     ++h->launches;
@@ -914,7 +926,7 @@ int batch_update_x0(relu_qp_t h, int B, const float* X0) {
 }
 
 // Regroup the active QPs among the first nqp QP indices into slots (assign)
-// and write the FP32 operand of the next chunk's first layer (fill).
+// and write the operand of the next chunk's first layer (fill).
 int regroup_slots(relu_qp_t h, const BatchParams& p, int nqp, bool assign) {
     BatchWork& w = h->bw;
     const bool bf16 = w.prec == RELU_QP_PREC_BF16X3;
@@ -926,9 +938,8 @@ int regroup_slots(relu_qp_t h, const BatchParams& p, int nqp, bool assign) {
         RQ_CUDA(h, cudaGetLastError());
         ++h->launches;
     }
-    const bool split_operand = bf16 && w.rebase_tc;
     batch_fill_kernel<<<(int)((size_t)w.slots * (w.ldk / 4) / 256 + 1), 256, 0, h->stream>>>(
-        p, w.rho_idx, split_operand ? nullptr : w.S32, split_operand ? OP + 4 * opart : nullptr, opart);
+        layer_params(h, p), w.rho_idx, bf16 ? nullptr : w.S32, bf16 ? OP + 4 * opart : nullptr, opart);
     RQ_CUDA(h, cudaGetLastError());
     ++h->launches;
     return RELU_QP_OK;
@@ -954,15 +965,14 @@ int run_layers(relu_qp_t h, const BatchParams& p, int len, bool check, int activ
     if (bf16 && w.chunk_sync && len > 1 && j_end > 1)
         RQ_CUDA(h, cudaMemsetAsync(w.chunk_sync, 0, sizeof(unsigned) * 2 * tiles_max, h->stream));
     for (int j = j_begin; j < std::min(len, j_end); ++j) {
-        BatchParams q = p;
+        BatchParams q = layer_params(h, p);
         q.flags = 0;
         if (j == len - 1) q.flags |= EPI_LAST | (check ? EPI_CHECK : 0u);
         if (bf16) {
             q.flags |= EPI_REFINE | (j == 0 ? EPI_REBASE : 0u);
             q.Dhi = OP + (size_t)(2 * (j & 1)) * opart;
             q.Dlo = q.Dhi + opart;
-            if (w.check_tc) q.CK = static_cast<__nv_bfloat16*>(w.CK);
-            else q.CK32 = w.CK32;
+            q.CK = static_cast<__nv_bfloat16*>(w.CK);
             if (j == 1 && w.chunk_sync) {
                 // layers 1 .. len-1 in one persistent launch when the tile's CTAs fit in one wave:
                 // the resident-weight kernel for one tile of few QPs (when the tuner chose it),
@@ -991,29 +1001,20 @@ int run_layers(relu_qp_t h, const BatchParams& p, int len, bool check, int activ
                 if (rc != RELU_QP_ERR_UNSUPPORTED) return rc;
                 // refused: one launch per layer below (which records the span's start again)
             }
-            if (j == 0 && !w.rebase_tc) {
-                // accurate layer c = Wt s_ref + b in FP32 on the CUDA cores (round to
-                // nearest); the tensor core's truncating accumulation of the full
-                // operand would set the fixed point's accuracy instead
-                q.Sin = w.S32;
-                RQ_TRY(layer32(h, q, wp, tiles_max, active));
-                ++h->launches;
-            } else {
-                // operand set read by this layer: 4..6 = s (3-way), else pair ((j-1)&1)
-                if (timed && j == 1) RQ_CUDA(h, cudaEventRecord(h->prof_ev[prof_used], h->stream));
-                RQ_TRY(tc_layer(h, q, j == 0 ? -1 : ((j - 1) & 1), tiles_max,
-                                tiles_now > 0 ? tiles_now : ceil_div(active, kSlotTile) + h->nr - 1, j > 0));
-                ++h->launches;
-                if (j > 0) {
-                    ++h->layer_launches;
-                    // three BF16 products of the (n+m) x (n+m) factored layer per active QP
-                    h->layer_flops += 2.0 * 3.0 * (double)R * (double)R * (double)active;
-                }
-                if (timed && j == len - 1) {
-                    RQ_CUDA(h, cudaEventRecord(h->prof_ev[prof_used + 1], h->stream));
-                    h->prof_span_launches.push_back(len - 1);
-                    prof_used += 2;
-                }
+            // operand set read by this layer: 4..6 = s (3-way), else pair ((j-1)&1)
+            if (timed && j == 1) RQ_CUDA(h, cudaEventRecord(h->prof_ev[prof_used], h->stream));
+            RQ_TRY(tc_layer(h, q, j == 0 ? -1 : ((j - 1) & 1), tiles_max,
+                            tiles_now > 0 ? tiles_now : ceil_div(active, kSlotTile) + h->nr - 1, j > 0));
+            ++h->launches;
+            if (j > 0) {
+                ++h->layer_launches;
+                // three BF16 products of the (n+m) x (n+m) factored layer per active QP
+                h->layer_flops += 2.0 * 3.0 * (double)R * (double)R * (double)active;
+            }
+            if (timed && j == len - 1) {
+                RQ_CUDA(h, cudaEventRecord(h->prof_ev[prof_used + 1], h->stream));
+                h->prof_span_launches.push_back(len - 1);
+                prof_used += 2;
             }
         } else {
             q.Sin = w.S32 + (size_t)(j & 1) * opart;
@@ -1041,8 +1042,8 @@ int run_layers(relu_qp_t h, const BatchParams& p, int len, bool check, int activ
 int run_check(relu_qp_t h, const BatchParams& p, int active, int tiles_now) {
     BatchWork& w = h->bw;
     const int tiles_max = w.slots / kSlotTile;
-    BatchParams q = p;
-    if (w.prec == RELU_QP_PREC_BF16X3 && w.check_tc) {
+    BatchParams q = layer_params(h, p);
+    if (w.prec == RELU_QP_PREC_BF16X3) {
         q.CK = static_cast<__nv_bfloat16*>(w.CK);
         const int active_tiles =
             tiles_now > 0 ? tiles_now : std::min(tiles_max, ceil_div(active, kSlotTile) + h->nr - 1);
@@ -1265,7 +1266,9 @@ __global__ void serve_admit_kernel(BatchParams p, int k, const int* __restrict__
         p.Y[(size_t)qp * p.ldn + t] = v;
         Xc[(size_t)j * p.ldn + t] = v;
     }
-    for (int i = lane; i < p.m; i += 32) p.LAM[(size_t)qp * p.ldm + i] = warm ? Wl[(size_t)c * p.ldm + i] : 0.f;
+    for (int i = lane; i < p.ldm; i += 32)
+        p.LAM[(size_t)qp * p.ldm + i] = warm && i < p.m ? Wl[(size_t)c * p.ldm + i] : 0.f;
+    for (int t = p.n + lane; t < p.ldn; t += 32) p.Y[(size_t)qp * p.ldn + t] = 0.f;   // padding
     if (lane == 0) {
         status[qp] = QP_ACTIVE;
         rho_idx[qp] = warm ? Wr[c] : rho0;
@@ -1302,8 +1305,12 @@ __global__ void serve_scatter_kernel(BatchParams p, int k, const int* __restrict
         p.AY[o] = AYc[oc];
         p.Z[o] = AYc[oc];
     }
+    for (int i = p.m + lane; i < p.ldm; i += 32) {   // padding
+        p.AY[(size_t)qp * p.ldm + i] = 0.f;
+        p.Z[(size_t)qp * p.ldm + i] = 0.f;
+    }
     for (int r = 0; r < p.nr; ++r)
-        for (int t = lane; t < p.R; t += 32)
+        for (int t = lane; t < p.ldR; t += 32)
             BIAS[((size_t)r * p.cap + qp) * p.ldR + t] = Bc[((size_t)r * p.cap + j) * p.ldR + t];
 }
 
@@ -1501,7 +1508,7 @@ int family_launch(relu_qp_server_t s, ServeFamily& f) {
         }
         for (int r = 0; r < h->nr; ++r)
             RQ_TRY(sgemm_nt(h, k, R, nx, f.d.x0c, w.ldx, w.G[r], w.ldx, 1.f, nullptr,
-                            f.d.Bc + (size_t)r * w.cap * w.ldR, w.ldR));
+                            f.d.Bc + (size_t)r * w.cap * w.ldR, w.ldR, n, w.nP - n));
         serve_scatter_kernel<<<ceil_div(k * 32, 256), 256, 0, f.stream>>>(p, k, f.d.idx, f.d.Qc, f.d.Lc, f.d.Uc,
                                                                          f.d.Bc, f.d.AYc, w.Q, w.L, w.U, w.BIAS,
                                                                          w.QN);

@@ -35,6 +35,7 @@ enum { CNT_TILES = 0, CNT_ACTIVE = 1, CNT_ERR = 2, CNT_WORDS = 4 };
 
 struct BatchParams {
     int n, m, R, ldn, ldm, ldR, ldk, n64, ldkc, cap, slots, nr;
+    int bsh;                                 // BIAS columns of A x rows: r + bsh (nP - n; the padded layout's n: 0)
     float rho[RQ_MAX_RHO];
     double rhod[RQ_MAX_RHO];
     double logrho[RQ_MAX_RHO];              // log of each bank entry (the penalty rule's distance)
@@ -87,8 +88,8 @@ __device__ __forceinline__ void put_check(const BatchParams& p, int slot, int co
     }
 }
 
-// The element-wise part of one layer for output row r of the QP in `slot`
-// (Eq. gpu_update in the factored form; see setup_fp64.cu):
+// The element-wise part of one layer (Eq. gpu_update in the factored form; see
+// setup_fp64.cu):
 //   t = acc + b (or + c in the refined form), x rows: x+ = t;
 //   Ax rows i:  r_i = (Ax)_i - z_i + lam'_i/rho_i,  z+ = clamp(t + r_i, l_i, u_i),
 //               lam'+ = rho_i r_i,  (Ax)+ = t,  operand entry 2 rho_i z+ - lam'+.
@@ -123,62 +124,27 @@ __device__ __forceinline__ float ax_row_carry(float ay, float zi, float li, floa
     return ay - zi + li / rho_i;
 }
 
+// One row of an FP32 layer (FP32 backend; the split form's is chunk4_apply).
 __device__ __forceinline__ void layer_elem(const BatchParams& p, int slot, int qp, int ri, int r, float acc) {
     const unsigned f = p.flags;
-    const bool refine_only = (f & EPI_REFINE) && !(f & EPI_REBASE);
-    // the split form writes x, Ax, z, lam' only at a chunk's last layer (its other layers,
-    // the accurate first one included, keep chunk-local data: c, s_ref, r and the operand)
-    const bool store_state = !(f & EPI_REFINE) || (f & EPI_LAST);
-    const size_t oR = (size_t)qp * p.ldR + r;
-    const float* bias = p.BIAS + (size_t)ri * p.cap * p.ldR;
-    float t;
-    if (f & EPI_REBASE) {
-        t = acc + bias[oR];
-        p.C[oR] = t;
-    } else if (f & EPI_REFINE) {
-        t = acc + p.C[oR];
-    } else {
-        t = acc + bias[oR];
-    }
+    const float t = acc + p.BIAS[((size_t)ri * p.cap + qp) * p.ldR + r + (r >= p.n ? p.bsh : 0)];
     float s_new;
     if (r < p.n) {
-        const size_t o = (size_t)qp * p.ldn + r;
-        if (f & EPI_REBASE) p.SREF[oR] = p.Y[o];
-        if (store_state) p.Y[o] = t;
+        p.Y[(size_t)qp * p.ldn + r] = t;
         s_new = t;
         if (f & EPI_CHECK) put_check(p, slot, r, t);
     } else {
         const int i = r - p.n;
         const size_t o = (size_t)qp * p.ldm + i;
         const float rho_i = p.rho[ri] * p.rs[i];
-        float rr;
-        if (refine_only) {
-            rr = p.RR[o];
-        } else {
-            const float ay = p.AY[o], zi = p.Z[o], li = p.LAM[o];
-            if (f & EPI_REBASE) p.SREF[oR] = next_operand(rho_i, zi, li);
-            rr = ax_row_carry(ay, zi, li, rho_i);
-        }
+        const float rr = ax_row_carry(p.AY[o], p.Z[o], p.LAM[o], rho_i);
         float zn, ln;
         ax_row_update(t, rr, p.L[o], p.U[o], rho_i, zn, ln, s_new);
-        if (f & EPI_REFINE) p.RR[o] = t - zn + rr;
-        if (store_state) {
-            p.AY[o] = t;
-            p.Z[o] = zn;
-            p.LAM[o] = ln;
-        }
+        p.AY[o] = t;
+        p.Z[o] = zn;
+        p.LAM[o] = ln;
     }
-    if (!(f & EPI_LAST)) {
-        const size_t so = (size_t)slot * p.ldk + r;
-        if (f & EPI_REFINE) {
-            __nv_bfloat16 hi, lo;
-            split2(s_new - p.SREF[oR], hi, lo);
-            p.Dhi[so] = hi;
-            p.Dlo[so] = lo;
-        } else {
-            p.Sout[so] = s_new;
-        }
-    }
+    if (!(f & EPI_LAST)) p.Sout[(size_t)slot * p.ldk + r] = s_new;
 }
 
 __device__ __forceinline__ void ld4(const float* __restrict__ src, float (&v)[4]) {
@@ -193,8 +159,8 @@ __device__ __forceinline__ void st4(float* __restrict__ dst, const float (&v)[4]
     *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
 }
 
-// layer_elem for 4 consecutive rows r0..r0+3 of one QP, all x rows or all Ax
-// rows, 16-byte aligned, in two halves: chunk4_load reads every input the
+// The split form's layer for 4 consecutive rows r0..r0+3 of one QP, all x rows or all Ax
+// rows (both parts are padded to multiples of 16), in two halves: chunk4_load reads every input the
 // layer needs (none of it depends on the product) and chunk4_apply combines it
 // with the product and writes the new state.  The tensor-core epilogue issues
 // the loads of all its 4-row pieces before the first apply, so one memory
@@ -227,7 +193,9 @@ __device__ __forceinline__ void chunk4_apply(const BatchParams& p, int slot, int
                                              const float (&acc)[4], Chunk4& c, const float (&rs)[4]) {
     const unsigned f = p.flags;
     const size_t oR = (size_t)qp * p.ldR + r0;
-    const bool store_state = !(f & EPI_REFINE) || (f & EPI_LAST);   // as layer_elem
+    // x, Ax, z and lam' are written only at a chunk's last layer (its other layers, the
+    // accurate first one included, keep chunk-local data: c, s_ref, r and the operand)
+    const bool store_state = !(f & EPI_REFINE) || (f & EPI_LAST);
     float s_new[4];
     if (r0 < p.n) {
 #pragma unroll

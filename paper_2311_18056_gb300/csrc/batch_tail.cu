@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) batch_tail_kernel(TailArgs a)
         const int o_qp = own ? a.qlist[oj] : 0, o_ri = own ? s_ri[oj] : 0, o_r = row_beg + orl;
         float rb = 0.f, ray = 0.f, rz = 0.f, rlam = 0.f, rlo = 0.f, rup = 0.f, rrho = 0.f;
         if (own) {
-            rb = p.BIAS[((size_t)o_ri * p.cap + o_qp) * p.ldR + o_r];
+            rb = p.BIAS[((size_t)o_ri * p.cap + o_qp) * p.ldR + o_r + (o_r >= p.n ? p.bsh : 0)];
             if (o_r >= p.n) {
                 const size_t o = (size_t)o_qp * p.ldm + (o_r - p.n);
                 ray = p.AY[o];
@@ -618,17 +618,17 @@ __global__ void tail_list_kernel(int B, const int* __restrict__ status, int* lis
 
 // floats of the scratch region: the step partials of `pass_rows` rows of the layer
 // product [kTailMax][pass_rows][ps], or the checks' per-warp round partials
-size_t tail_scratch(const BatchWork& w, int pass_rows) {
-    const size_t ps = (size_t)((w.ldk / kStep) | 1);
+size_t tail_scratch(relu_qp_t h, int pass_rows) {
+    const size_t ps = (size_t)((h->ldw / kStep) | 1);
     return std::max((size_t)kTailWarps * kRB * kTailMax * kPbs, (size_t)pass_rows * kTailMax * ps);
 }
 
 // staged operands [kTailMax][steps][kStepPad] + scratch (+ the cached Wt rows
 // [rows][ldk steps][kStepPad])
-size_t tail_smem(const BatchWork& w, int pass_rows, int cached_rows) {
-    const size_t steps = (size_t)std::max(w.ldk, w.ldkc) / kStep;
-    return ((size_t)kTailMax * steps * kStepPad + tail_scratch(w, pass_rows) +
-            (size_t)cached_rows * (w.ldk / kStep) * kStepPad) *
+size_t tail_smem(relu_qp_t h, int pass_rows, int cached_rows) {
+    const size_t steps = (size_t)std::max(h->ldw, h->bw.ldkc) / kStep;
+    return ((size_t)kTailMax * steps * kStepPad + tail_scratch(h, pass_rows) +
+            (size_t)cached_rows * (h->ldw / kStep) * kStepPad) *
            sizeof(float);
 }
 
@@ -636,7 +636,7 @@ size_t tail_smem(const BatchWork& w, int pass_rows, int cached_rows) {
 
 int batch_tail_alloc(relu_qp_t h) {
     BatchWork& w = h->bw;
-    RQ_TRY(alloc(h, &w.TS, 2 * (size_t)kTailMax * w.ldk));
+    RQ_TRY(alloc(h, &w.TS, 2 * (size_t)kTailMax * h->ldw));
     RQ_TRY(alloc(h, &w.TCK, (size_t)kTailMax * w.ldkc));
     RQ_TRY(alloc(h, &w.TRED, 3 * (size_t)kTailMax * RW_WORDS));
     RQ_TRY(alloc(h, &w.TBAR, 4));
@@ -651,7 +651,7 @@ int batch_tail_alloc(relu_qp_t h) {
     const int rpc = ceil_div(h->R, grid);
     for (int cache = 1; cache >= 0; --cache) {
         for (int pr = rpc;; pr = std::max(kRG, pr / 2)) {
-            const size_t smem = tail_smem(w, pr, cache ? rpc : 0);
+            const size_t smem = tail_smem(h, pr, cache ? rpc : 0);
             if (smem + 1024 <= (size_t)smem_max) {
                 RQ_CUDA(h, cudaFuncSetAttribute(batch_tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 (int)smem));
@@ -681,7 +681,8 @@ int batch_tail(relu_qp_t h, const BatchParams& p, const DecideArgs& d, int nq, i
     RQ_CUDA(h, cudaMemsetAsync(w.TRED, 0, sizeof(unsigned) * 3 * kTailMax * RW_WORDS, h->stream));
     RQ_CUDA(h, cudaMemsetAsync(w.TBAR, 0, sizeof(unsigned) * 4, h->stream));
     TailArgs a{};
-    a.p = p;
+    a.p = p;               // rows [x; Ax] without the split form's padding, as the FP32 bank has them
+    a.p.ldk = h->ldw;
     a.p.CK32 = w.TCK;
     a.p.CK = nullptr;
     a.d = d;
@@ -699,7 +700,7 @@ int batch_tail(relu_qp_t h, const BatchParams& p, const DecideArgs& d, int nq, i
     a.ci = h->opts.check_interval;
     a.rpc = w.tail_rpc;
     a.pr = w.tail_pr;
-    a.scratch = (int)tail_scratch(w, w.tail_pr);
+    a.scratch = (int)tail_scratch(h, w.tail_pr);
     a.wcache = w.tail_cache;
     a.regs = w.tail_pr >= w.tail_rpc && w.tail_rpc * kTailMax <= kTailThreads ? 1 : 0;
     a.timeout_ns = 2000000000LL;

@@ -571,19 +571,10 @@ __device__ __forceinline__ bool tile_epilogue(const BatchParams& p, const TcArgs
     // the columns this warp finalises (none for a split warp that only sends)
     const int cbeg = DSPLIT ? own0 : own0 + half * PER;
     const int cend = holds_own ? cbeg + (DSPLIT ? OWN : PER) : cbeg;
-    const bool n_aligned = (p.n & 3) == 0;
-    auto whole_at = [&](int c0) {
-        const int r0 = row0 + c0;
-        return MODE <= MODE_LAYER_ACCURATE && r0 + 16 <= g.rows && (r0 + 16 <= p.n || (r0 >= p.n && n_aligned));
-    };
-    // residual products: 16-row pieces of rows of x only or of A x only take the
-    // transposed path as well (the drained sums of every slot of the warp are in
-    // shared memory, so the transposition needs no extra buffer)
+    // a 16-row piece holds rows of x only or of A x only, all of them in range (both parts are
+    // padded to multiples of 16), or lies beyond the last row
     constexpr bool CHECK = MODE == MODE_CHECK1 || MODE == MODE_CHECK2;
-    auto check_whole_at = [&](int c0) {
-        const int r0 = row0 + c0;
-        return CHECK && r0 + 16 <= g.rows && (r0 + 16 <= p.n || (r0 >= p.n && n_aligned));
-    };
+    auto in_range = [&](int c0) { return row0 + c0 < g.rows; };
     float mx[4][4];   // per pass (QP): the residual maxima of the transposed pieces
 #pragma unroll
     for (int a = 0; a < 4; ++a)
@@ -602,7 +593,7 @@ __device__ __forceinline__ bool tile_epilogue(const BatchParams& p, const TcArgs
         if (r0 >= p.n) ld4(p.rs + (r0 - p.n), dst);
     };
     // the inputs of the first chunk load while the MMAs run
-    if (cend > cbeg && whole_at(cbeg)) {
+    if (!CHECK && cend > cbeg && in_range(cbeg)) {
         load_rs(cbeg, rs);
 #pragma unroll
         for (int pass = 0; pass < 4; ++pass) load_pass(cbeg, pass);
@@ -735,16 +726,14 @@ __device__ __forceinline__ bool tile_epilogue(const BatchParams& p, const TcArgs
     if (!ready) {
         if (lane == 0) { wait_failed(g.err, DRAIN ? WS_DRAIN_READY : WS_EPI_ACC); *s_fail = 1; }
     } else {
-        float ra = 0.f, rb = 0.f, rc = 0.f, rd = 0.f;
-        // inputs of the next whole chunk load pass by pass as this chunk's
-        // passes finish, so that a memory round trip overlaps a chunk of work
-        for (int c0 = cbeg; c0 < cend; c0 += 16) {
+        // inputs of the next piece load pass by pass as this piece's passes finish, so that a
+        // memory round trip overlaps a piece of work
+        for (int c0 = cbeg; c0 < cend && in_range(c0); c0 += 16) {
             const int r0 = row0 + c0;
-            const bool whole = whole_at(c0);
             const int cn = c0 + 16;
-            const bool next_whole = cn < cend && whole_at(cn);
-            if (next_whole) load_rs(cn, rs_next);
-            if (CHECK && check_whole_at(c0)) {
+            const bool next = !CHECK && cn < cend && in_range(cn);
+            if (next) load_rs(cn, rs_next);
+            if (CHECK) {
                 // lane = 4 * (slot % 8) + row group: rows r0 + cg .. + 3 of the slot
                 // pass * 8 + lane / 4, read from that slot's drained sums
                 __syncwarp();
@@ -800,67 +789,37 @@ __device__ __forceinline__ bool tile_epilogue(const BatchParams& p, const TcArgs
 #pragma unroll
                 for (int t = 0; t < 16; ++t) v[t] = tot[t];
             }
-            if (whole) {
-                // the source rows: this warp's transpose buffer (refined), or the
-                // drained sums, which already hold every slot of the warp
-                const float* base;
-                int stride, off;
-                if (DRAIN) {
-                    base = drain + (warp - 2) * 32 * (DW + 1);
-                    stride = DW + 1;
-                    off = c0 - dbeg;
-                } else {
-                    float* xb = xpose + (warp - 2) * 32 * 17;       // [32 slots][16 rows]
+            // the source rows: this warp's transpose buffer (refined), or the
+            // drained sums, which already hold every slot of the warp
+            const float* base;
+            int stride, off;
+            if (DRAIN) {
+                base = drain + (warp - 2) * 32 * (DW + 1);
+                stride = DW + 1;
+                off = c0 - dbeg;
+            } else {
+                float* xb = xpose + (warp - 2) * 32 * 17;       // [32 slots][16 rows]
 #pragma unroll
-                    for (int t = 0; t < 16; ++t) xb[lane * 17 + t] = v[t];
-                    base = xb;
-                    stride = 17;
-                    off = 0;
+                for (int t = 0; t < 16; ++t) xb[lane * 17 + t] = v[t];
+                base = xb;
+                stride = 17;
+                off = 0;
+            }
+            __syncwarp();
+#pragma unroll
+            for (int pass = 0; pass < 4; ++pass) {
+                const int sl = pass * 8 + (lane >> 2);          // slot within the warp's 32
+                if (qq[pass] >= 0) {
+                    float a4[4];
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) a4[t] = base[sl * stride + off + cg + t];
+                    chunk4_apply(p, slot0 + q * 32 + sl, qq[pass], ri, r0 + cg, a4, in[pass], rs);
                 }
-                __syncwarp();
-#pragma unroll
-                for (int pass = 0; pass < 4; ++pass) {
-                    const int sl = pass * 8 + (lane >> 2);          // slot within the warp's 32
-                    if (qq[pass] >= 0) {
-                        float a4[4];
-#pragma unroll
-                        for (int t = 0; t < 4; ++t) a4[t] = base[sl * stride + off + cg + t];
-                        chunk4_apply(p, slot0 + q * 32 + sl, qq[pass], ri, r0 + cg, a4, in[pass], rs);
-                    }
-                    if (next_whole) load_pass(cn, pass);
-                }
-#pragma unroll
-                for (int k = 0; k < 4; ++k) rs[k] = rs_next[k];
-                __syncwarp();
-                continue;
+                if (next) load_pass(cn, pass);
             }
-            if (qp >= 0) {
-#pragma unroll 4
-                for (int t = 0; t < 16; ++t) {
-                    const int r = r0 + t;
-                    if (r >= g.rows) continue;
-                    if (MODE == MODE_CHECK1) check1_elem(p, slot, qp, ri, r, v[t], ra, rb, rc, rd);
-                    else if (MODE == MODE_CHECK2) check2_elem(p, qp, r, v[t], ra, rb);
-                    else layer_elem(p, slot, qp, ri, r, v[t]);
-                }
-            }
-            if (next_whole) {
 #pragma unroll
-                for (int pass = 0; pass < 4; ++pass) load_pass(cn, pass);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) rs[k] = rs_next[k];
-            }
-        }
-        if (qp >= 0) {
-            if (MODE == MODE_CHECK1) {
-                red_slot(p.RED, qp, RW_RP, ra);
-                red_slot(p.RED, qp, RW_AX, rb);
-                red_slot(p.RED, qp, RW_Z, rc);
-                red_slot(p.RED, qp, RW_PX, rd);
-            } else if (MODE == MODE_CHECK2) {
-                red_slot(p.RED, qp, RW_RD, ra);
-                red_slot(p.RED, qp, RW_ATL, rb);
-            }
+            for (int k = 0; k < 4; ++k) rs[k] = rs_next[k];
+            __syncwarp();
         }
         if (CHECK) {
             // the transposed pieces: the 4 lanes of a slot (lane & 3 = row group)
@@ -1454,8 +1413,6 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
         const int fr0 = row0 + fr;
         const bool mine = es < c.ncols;
         const int eqp = mine ? p.perm[slot0 + es] : -1;
-        const bool n_aligned = (p.n & 3) == 0;
-        auto whole4 = [&](int r0) { return r0 + 4 <= g.rows && (r0 + 4 <= p.n || (r0 >= p.n && n_aligned)); };
         // sender side: lane = row 32 q + lane of the block; rows 16 o .. 16 o + 15 go to rank o
         const int srow = q * 32 + lane;
         const int owner = srow / kSmallOwn;
@@ -1470,7 +1427,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
             if (eqp >= 0) {
 #pragma unroll
                 for (int h2 = 0; h2 < 2; ++h2)
-                    if (whole4(fr0 + 4 * h2)) chunk4_load(pj, eqp, ri, fr0 + 4 * h2, in[h2]);
+                    if (fr0 + 4 * h2 < g.rows) chunk4_load(pj, eqp, ri, fr0 + 4 * h2, in[h2]);
             }
             // the accumulators of layer j
             bool ready = true;
@@ -1527,14 +1484,11 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
 #pragma unroll
                 for (int h2 = 0; h2 < 2; ++h2) {
                     const int r0 = fr0 + 4 * h2;
-                    if (whole4(r0)) {
+                    if (r0 < g.rows) {
                         float rs4[4] = {1.f, 1.f, 1.f, 1.f};
                         if (r0 >= p.n) ld4(p.rs + (r0 - p.n), rs4);
                         const float a4[4] = {acc[4 * h2], acc[4 * h2 + 1], acc[4 * h2 + 2], acc[4 * h2 + 3]};
                         chunk4_apply(pj, slot0 + es, eqp, ri, r0, a4, in[h2], rs4);
-                    } else {
-                        for (int t = 0; t < 4; ++t)
-                            if (r0 + t < g.rows) layer_elem(pj, slot0 + es, eqp, ri, r0 + t, acc[4 * h2 + t]);
                     }
                 }
             }
@@ -1906,7 +1860,7 @@ int tc_layer(relu_qp_t h, const BatchParams& p, int operand_set, int tiles, int 
     TcState* st = static_cast<TcState*>(w.tc);
     TcArgs g{};
     g.num_kb = w.ldk / kBK;
-    g.rows = h->R;
+    g.rows = w.RP;
     g.err = st->err;
     g.b_rho_stride = 3 * w.Rpad;
     for (int b = 0; b < 3; ++b) g.b_row[b] = b * w.Rpad;
@@ -1931,10 +1885,10 @@ int tc_chunk(relu_qp_t h, const BatchParams& p, int nl, unsigned last_flags, int
     if (!chunk_has(lc.ks, bn)) return RELU_QP_ERR_UNSUPPORTED;
     const int tiles_y = std::min(active_tiles, w.slots / kSlotTile);
     // all CTAs of the active tiles co-resident, one per SM
-    if ((long long)lc.ks * ceil_div(h->R, bn) * tiles_y > h->num_sms) return RELU_QP_ERR_UNSUPPORTED;
+    if ((long long)lc.ks * ceil_div(w.RP, bn) * tiles_y > h->num_sms) return RELU_QP_ERR_UNSUPPORTED;
     TcArgs g{};
     g.num_kb = w.ldk / kBK;
-    g.rows = h->R;
+    g.rows = w.RP;
     g.err = st->err;
     g.b_rho_stride = 3 * w.Rpad;
     for (int b = 0; b < 3; ++b) g.b_row[b] = b * w.Rpad;
@@ -1964,7 +1918,7 @@ int small_clusters_fit(relu_qp_t h) {
         return 0;
     }
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(kSmallKS * ceil_div(h->R, kSmallRows), 1);
+    cfg.gridDim = dim3(kSmallKS * ceil_div(h->bw.RP, kSmallRows), 1);
     cfg.blockDim = dim3(kSmallThreads);
     cfg.dynamicSmemBytes = SmallSmem<64>::kBytes;
     cfg.stream = h->stream;
@@ -1989,9 +1943,9 @@ bool tc_small_eligible(relu_qp_t h, int active, int active_tiles) {
     if (!st || !st->small_ok || !w.chunk_sync || active_tiles != 1 || active < 1 || active > 64) return false;
     const int nkb = w.ldk / kBK;
     if (ceil_div(nkb, kSmallKS) > kSmallMaxKb || nkb < kSmallKS) return false;
-    if ((long long)kSmallKS * ceil_div(h->R, kSmallRows) > h->num_sms) return false;
+    if ((long long)kSmallKS * ceil_div(h->bw.RP, kSmallRows) > h->num_sms) return false;
     if (st->small_clusters < 0) st->small_clusters = small_clusters_fit(h);
-    return st->small_clusters >= ceil_div(h->R, kSmallRows);
+    return st->small_clusters >= ceil_div(h->bw.RP, kSmallRows);
 }
 
 void tc_small_set(relu_qp_t h, bool use) { static_cast<TcState*>(h->bw.tc)->small_use = use; }
@@ -2003,7 +1957,7 @@ int tc_small(relu_qp_t h, const BatchParams& p, int nl, unsigned last_flags, int
     if (nl < 1 || !tc_small_eligible(h, active, active_tiles)) return RELU_QP_ERR_UNSUPPORTED;
     TcArgs g{};
     g.num_kb = w.ldk / kBK;
-    g.rows = h->R;
+    g.rows = w.RP;
     g.err = st->err;
     g.b_rho_stride = 3 * w.Rpad;
     for (int b = 0; b < 3; ++b) g.b_row[b] = b * w.Rpad;
@@ -2028,7 +1982,7 @@ int tc_check(relu_qp_t h, const BatchParams& p, int phase, int tiles, int active
     TcArgs g{};
     g.num_kb = (phase == 1 ? w.n64 : w.m64) / kBK;
     g.k_off = phase == 1 ? 0 : w.n64;
-    g.rows = phase == 1 ? h->n + h->m : h->n;
+    g.rows = phase == 1 ? w.RP : w.nP;
     g.err = st->err;
     g.b_rho_stride = 0;
     for (int a = 0; a < 3; ++a) {

@@ -93,11 +93,9 @@ struct SingleWork64 {
 // Workspace of batched solves (allocated when opts.max_batch > 0).
 struct BatchWork {
     int cap = 0, slots = 0, prec = 0, B = 0;
-    int rebase_tc = 1;   // BF16 form: 1 = accurate layer on the tensor cores (3-way split, every
-                         // k-block's products drained into FP32 sums; default), 0 = on the CUDA
-                         // cores in FP32
-    int check_tc = 1;    // BF16 form: 1 = residual products on the tensor cores (3-way split,
-                         // drained like the accurate layer; default), 0 = on the CUDA cores in FP32
+    // rows of the layer: x in [0, nP), A x in [nP, RP).  FP32 form: nP = n, RP = n + m.  BF16
+    // form: both parts padded with zero rows to multiples of 16, the epilogues' piece
+    int nP = 0, RP = 0;
     int ldn = 0, ldm = 0, ldR = 0, ldk = 0, n64 = 0, m64 = 0, ldkc = 0, Rpad = 0, npad = 0;
     // check matrix [[P, A^T], [A, 0]]: (n + m) rows (padded to npad), ldkc = n64 + m64 columns
     // per-QP state (QP-indexed rows)

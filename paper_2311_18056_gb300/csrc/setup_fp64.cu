@@ -322,26 +322,28 @@ __device__ __forceinline__ void split3_f64(double v, __nv_bfloat16& a, __nv_bflo
     c = __double2bfloat16(r1 - (double)__bfloat162float(b));
 }
 
-// The three BF16 parts of the factored layer [X V] (rows [x; Ax], K-major rows of ldk).
-__global__ void pack_bf16_layer_kernel(const double* __restrict__ X, const double* __restrict__ V, int n, int m,
+// The three BF16 parts of the factored layer [X V] (rows [x; Ax], K-major rows of ldk);
+// rows and columns of A x start at nP.
+__global__ void pack_bf16_layer_kernel(const double* __restrict__ X, const double* __restrict__ V, int n, int m, int nP,
                                        int ldk, size_t part, __nv_bfloat16* __restrict__ out) {
     const int R = n + m;
     const size_t total = (size_t)R * ldk;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
          e += (size_t)gridDim.x * blockDim.x) {
         const int r = (int)(e / ldk), k = (int)(e % ldk);
-        const double v = k < n ? X[(size_t)r * n + k] : k < R ? V[(size_t)r * m + k - n] : 0.0;
+        const double v = k < n ? X[(size_t)r * n + k] : k >= nP && k < nP + m ? V[(size_t)r * m + k - nP] : 0.0;
         __nv_bfloat16 a, b, c;
         split3_f64(v, a, b, c);
-        out[e] = a;
-        out[e + part] = b;
-        out[e + 2 * part] = c;
+        const size_t o = (size_t)(r < n ? r : r - n + nP) * ldk + k;
+        out[o] = a;
+        out[o + part] = b;
+        out[o + 2 * part] = c;
     }
 }
 
 // The three BF16 parts of the check matrix [[P, A^T], [A, 0]] (x columns
-// [0, n64), multiplier columns [n64, n64 + m); rows [0, n) and [n, n + m)).
-__global__ void pack_bf16_check_kernel(const double* __restrict__ P, const double* __restrict__ A, int n, int m,
+// [0, n64), multiplier columns [n64, n64 + m); rows [0, n) and [nP, nP + m)).
+__global__ void pack_bf16_check_kernel(const double* __restrict__ P, const double* __restrict__ A, int n, int m, int nP,
                                        int n64, int ldkc, size_t part, __nv_bfloat16* __restrict__ out) {
     const size_t total = (size_t)(n + m) * ldkc;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
@@ -356,9 +358,10 @@ __global__ void pack_bf16_check_kernel(const double* __restrict__ P, const doubl
         }
         __nv_bfloat16 a, b, c;
         split3_f64(v, a, b, c);
-        out[e] = a;
-        out[e + part] = b;
-        out[e + 2 * part] = c;
+        const size_t o = (size_t)(j < n ? j : j - n + nP) * ldkc + k;
+        out[o] = a;
+        out[o + part] = b;
+        out[o + 2 * part] = c;
     }
 }
 
@@ -513,7 +516,8 @@ int pack_bf16_layer(relu_qp_t h, int r, const double* X, const double* V) {
     BatchWork& w = h->bw;
     const size_t part = (size_t)w.Rpad * w.ldk;
     __nv_bfloat16* out = static_cast<__nv_bfloat16*>(w.WB) + (size_t)r * 3 * part;
-    pack_bf16_layer_kernel<<<grid1d((size_t)h->R * w.ldk), 256, 0, h->stream>>>(X, V, h->n, h->m, w.ldk, part, out);
+    pack_bf16_layer_kernel<<<grid1d((size_t)h->R * w.ldk), 256, 0, h->stream>>>(X, V, h->n, h->m, w.nP,
+                                                                                       w.ldk, part, out);
     RQ_CUDA(h, cudaGetLastError());
     return RELU_QP_OK;
 }
@@ -522,7 +526,7 @@ int pack_bf16_check(relu_qp_t h, const double* dP, const double* dA) {
     BatchWork& w = h->bw;
     const size_t part = (size_t)w.npad * w.ldkc;
     pack_bf16_check_kernel<<<grid1d((size_t)(h->n + h->m) * w.ldkc), 256, 0, h->stream>>>(
-        dP, dA, h->n, h->m, w.n64, w.ldkc, part, static_cast<__nv_bfloat16*>(w.WCB));
+        dP, dA, h->n, h->m, w.nP, w.n64, w.ldkc, part, static_cast<__nv_bfloat16*>(w.WCB));
     RQ_CUDA(h, cudaGetLastError());
     return RELU_QP_OK;
 }

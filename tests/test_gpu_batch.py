@@ -357,3 +357,33 @@ def test_tail_kernel_iterates(rq, prec, case, B):
             worst[name] = max(worst[name], rel(got, ref))
     print(f"{case} prec={prec} B={B}: error vs oracle {worst}")
     assert worst["tail"] <= tol and worst["tiled"] <= tol, worst
+
+
+@pytest.mark.parametrize("n,m", [(16, 16), (17, 15), (31, 33), (33, 1), (48, 0), (65, 130), (210, 77)])
+def test_padded_row_layout(rq, n, m):
+    """Split backend: x and A x rows padded to multiples of 16 (ragged n, m, and m = 0), iterates
+    within the form's 1e-4; a QP of non-finite data leaves nothing behind in the padding."""
+    rng = np.random.default_rng([3, n, m])
+    M = rng.standard_normal((n, n))
+    P = M @ M.T / n + 0.5 * np.eye(n)
+    A = rng.standard_normal((m, n)) / np.sqrt(n)
+    B = 21
+    Q = 2.0 * rng.standard_normal((B, n))
+    L = -rng.uniform(0.1, 1.0, (B, m))
+    U = rng.uniform(0.1, 1.0, (B, m))
+    s = rq.ReluQP(P, A if m else None, L[0], U[0], q=Q[0], sigma=SIGMA, rho_bank=BANK, check_interval=0, max_batch=B,
+                  precision=1)
+    try:
+        bad = Q.copy()
+        bad[3] = np.nan
+        for data in (Q, bad, Q):
+            s.update_batch(data, L, U)
+            out = s.solve_batch(max_iter=30)
+            for b in range(B):
+                if np.isnan(data[b]).any():
+                    continue
+                v = O.layer_iterates(P, Q[b], A, L[b], U[b], SIGMA, BANK[0], 30)[-1]
+                got = np.concatenate([out["x"][b], out["z"][b]]).astype(np.float64)
+                assert rel(got, v[:n + m]) <= TOL_ITER[1], b
+    finally:
+        s.close()
