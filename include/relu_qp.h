@@ -185,8 +185,8 @@ int relu_qp_solve(relu_qp_t h, const double* x_warm, const double* lam_warm, int
  * unbounded time) or an application whose own allocator owns device memory.
  * The paper has no counterpart; it is a deployment variant of the same solve.
  *
- * It allocates nothing: the solve's scratch (iterate, layer operands,
- * residual vectors, grid-barrier and reduction words) lives in one fixed
+ * It allocates nothing: the solve's scratch in device memory (the words that
+ * hand operands and residuals from CTA to CTA) lives in one fixed
  * 192 KiB device array inside the library, which every GPU that loads the
  * library holds until the process exits.  The layer bank and problem data
  * come from relu_qp_setup / relu_qp_update on h as usual.
@@ -199,7 +199,7 @@ int relu_qp_solve(relu_qp_t h, const double* x_warm, const double* lam_warm, int
  * Limits and rules: n + m <= 4096 (larger problems return RELU_QP_ERR_INVALID
  * before any GPU work).  All calls share the one array, so calls whose GPU
  * work overlaps (other streams or threads) race; order them.  The array keeps
- * the last call's contents; each call clears what must start at zero.  The
+ * the last call's contents; each call clears what it uses.  The
  * call is synchronous: it returns once the outputs and info are written.  The
  * first call for each device looks the array's device address up
  * (cudaGetSymbolAddress) with the handle's device current; make that first
@@ -438,10 +438,10 @@ long long relu_qp_device_bytes(relu_qp_t h);
  * ---- launch shape of the single-QP FP32 solve --------------------------------
  * relu_qp_setup times candidate launch shapes of the solve kernel behind
  * relu_qp_solve (the online stage of Algorithm 1, Sec. III-B) and keeps the
- * fastest: a cooperative grid of `ctas` CTAs with a grid barrier between
- * layers, or one thread-block cluster of `ctas` CTAs (cluster = ctas) that keep
- * the layer's operand in distributed shared memory and synchronise through
- * cluster-scope mbarriers.  Each row's dot product and update is the same
+ * fastest: a cooperative grid of `ctas` CTAs that exchange the layer's operand
+ * through global memory (one CTA alone: its shared memory), or one thread-block
+ * cluster of `ctas` CTAs (cluster = ctas) that write it into each other's shared
+ * memory.  Each row's dot product and update is the same
  * arithmetic in every shape, so the results do not depend on the choice; these
  * calls exist for tests and tuning.
  *
@@ -470,10 +470,9 @@ int relu_qp_single_set_config(relu_qp_t h, int ctas, int cluster);
  *   CTA waits until timeout_ns); kind 1: the same barrier with the right
  *   arrival count (passes; the control case); kind 2: an mbarrier wait that
  *   nothing completes; kind 3: a layer-counter wait that nothing increments;
- *   kind 4: a cluster of 2 CTAs whose cluster barrier (the one the
- *   single-QP solve uses in its cluster form) expects one arrival more than
- *   there are CTAs; kind 5: the same barrier with the right count, three
- *   rounds (passes).  timeout_ns in [1e3, 1e9].  *status receives the
+ *   kind 4: a cluster of 2 CTAs whose exchange (the one the single-QP solve
+ *   uses in its cluster form) expects one word more than is sent;
+ *   kind 5: the same exchange with the right count, three rounds (passes).  timeout_ns in [1e3, 1e9].  *status receives the
  *   kernel's error word (RELU_QP_ERR_TIMEOUT, or 0 when the wait completed),
  *   *ms (may be NULL) the device time of the launch.  Returns INVALID, OOM,
  *   CUDA, UNSUPPORTED (no cooperative or cluster launch) or OK.

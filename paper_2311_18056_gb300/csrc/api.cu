@@ -114,19 +114,13 @@ int upload_scaling(relu_qp_t h) {
 
 int upload_problem(relu_qp_t h) {
     const int n = h->n, m = h->m;
-    std::vector<float> q(n);
+    // (the staging and the device copies of the last call are free: every call ends synchronised)
+    float *q = h->sw.pin, *l = q + n, *u = l + m;
     for (int j = 0; j < n; ++j) q[j] = (float)(h->scaled ? h->sC * h->sD[j] * h->h_q[j] : h->h_q[j]);
-    RQ_CUDA(h, cudaMemcpyAsync(h->q32, q.data(), sizeof(float) * n, cudaMemcpyHostToDevice, h->stream));
-    if (m > 0) {
-        std::vector<float> l(m), u(m);
-        for (int i = 0; i < m; ++i) {
-            const double e = h->scaled ? h->sE[i] : 1.0;
-            l[i] = (float)(e * h->h_l[i]);
-            u[i] = (float)(e * h->h_u[i]);
-        }
-        RQ_CUDA(h, cudaMemcpyAsync(h->l32, l.data(), sizeof(float) * m, cudaMemcpyHostToDevice, h->stream));
-        RQ_CUDA(h, cudaMemcpyAsync(h->u32, u.data(), sizeof(float) * m, cudaMemcpyHostToDevice, h->stream));
-        RQ_CUDA(h, cudaStreamSynchronize(h->stream));
+    for (int i = 0; i < m; ++i) {
+        const double e = h->scaled ? h->sE[i] : 1.0;
+        l[i] = (float)(e * h->h_l[i]);
+        u[i] = (float)(e * h->h_u[i]);
     }
     double qn = 0.0;
     for (int i = 0; i < n; ++i) qn = std::fmax(qn, std::fabs(h->h_q[i]));
@@ -141,7 +135,7 @@ int upload_problem(relu_qp_t h) {
         }
         RQ_TRY(rq::single64_upload(h, q64.data(), l64.data(), u64.data()));
     }
-    RQ_TRY(rq::compute_bias(h));
+    RQ_TRY(rq::single_update(h));
     RQ_CUDA(h, cudaStreamSynchronize(h->stream));
     return RELU_QP_OK;
 }
@@ -180,27 +174,12 @@ int setup_impl(relu_qp_t h, const double* P, const double* q, const double* A, c
     RQ_TRY(rq::alloc(h, &h->P32, (size_t)n * ldp));
     RQ_TRY(rq::alloc(h, &h->A32, (size_t)(m > 0 ? m : 1) * ldp));
     RQ_TRY(rq::alloc(h, &h->At32, (size_t)n * ldt));
-    RQ_TRY(rq::alloc(h, &h->q32, (size_t)n));
-    RQ_TRY(rq::alloc(h, &h->l32, (size_t)(m > 0 ? m : 1)));
-    RQ_TRY(rq::alloc(h, &h->u32, (size_t)(m > 0 ? m : 1)));
+    RQ_TRY(rq::alloc(h, &h->q32, (size_t)n + 2 * (size_t)m));   // q, l, u
+    h->l32 = h->q32 + n;
+    h->u32 = h->l32 + m;
     RQ_TRY(rq::alloc(h, &h->rs32, rs.size()));
     RQ_CUDA(h, cudaMemcpy(h->rs32, rs.data(), sizeof(float) * rs.size(), cudaMemcpyHostToDevice));
-    rq::SingleWork& w = h->sw;
-    RQ_TRY(rq::alloc(h, &w.y, (size_t)h->ldw));
-    RQ_TRY(rq::alloc(h, &w.z, (size_t)ldt));
-    RQ_TRY(rq::alloc(h, &w.lam, (size_t)ldt));
-    RQ_TRY(rq::alloc(h, &w.Ay, (size_t)ldt));
-    RQ_TRY(rq::alloc(h, &w.s0, (size_t)h->ldw));
-    RQ_TRY(rq::alloc(h, &w.s1, (size_t)h->ldw));
-    RQ_TRY(rq::alloc(h, &w.Py, (size_t)ldp));
-    RQ_TRY(rq::alloc(h, &w.Axf, (size_t)ldt));
-    RQ_TRY(rq::alloc(h, &w.lstd, (size_t)ldt));
-    RQ_TRY(rq::alloc(h, &w.xin, (size_t)ldp));
-    RQ_TRY(rq::alloc(h, &w.lin, (size_t)ldt));
-    RQ_TRY(rq::alloc(h, &w.red, 3 * 8));
-    RQ_TRY(rq::alloc(h, &w.bar, 2));
-    RQ_TRY(rq::alloc(h, &w.out_i, 8));
-    RQ_TRY(rq::alloc(h, &w.out_f, 8));
+    RQ_TRY(rq::single_alloc(h));
     if (h->opts.max_batch > 0) RQ_TRY(rq::batch_alloc(h));
     // problem scaling: the offline stage below sees the scaled P and A
     std::vector<double> Ps, As;
@@ -424,36 +403,25 @@ int relu_qp_solve(relu_qp_t h, const double* x_warm, const double* lam_warm, int
         if (info) *info = inf;
         return RELU_QP_OK;
     }
-    const float* xin = nullptr;
-    const float* lin = nullptr;
+    std::vector<float> xf, lf;
     if (x_warm) {
         // scaled handles: xb = x / D, lamb = c lam / E
-        std::vector<float> xf(n);
-        for (int j = 0; j < n; ++j) xf[j] = (float)(h->scaled ? x_warm[j] / h->sD[j] : x_warm[j]);
-        RQ_CUDA(h, cudaMemcpyAsync(h->sw.xin, xf.data(), sizeof(float) * n, cudaMemcpyHostToDevice, h->stream));
-        xin = h->sw.xin;
+        xf.resize(n);
+        for (int j = 0; j < n; ++j) xf[j] = (float)(sc ? x_warm[j] / h->sD[j] : x_warm[j]);
         if (lam_warm && m > 0) {
-            std::vector<float> lf(m);
-            for (int i = 0; i < m; ++i) lf[i] = (float)(h->scaled ? h->sC * lam_warm[i] / h->sE[i] : lam_warm[i]);
-            RQ_CUDA(h, cudaMemcpyAsync(h->sw.lin, lf.data(), sizeof(float) * m, cudaMemcpyHostToDevice,
-                                       h->stream));
-            lin = h->sw.lin;
+            lf.resize(m);
+            for (int i = 0; i < m; ++i) lf[i] = (float)(sc ? h->sC * lam_warm[i] / h->sE[i] : lam_warm[i]);
         }
-        RQ_CUDA(h, cudaStreamSynchronize(h->stream));
     }
     relu_qp_info inf{};
-    RQ_TRY(rq::single_solve(h, xin, lin, ri, eps_abs, eps_rel, max_iter, &inf));
+    RQ_TRY(rq::single_solve(h, x_warm ? xf.data() : nullptr, lf.empty() ? nullptr : lf.data(), ri, eps_abs, eps_rel,
+                            max_iter, &inf));
     // scaled handles: x = D xb, z = zb / E, lam = E lamb / c
-    std::vector<float> buf((size_t)(n > m ? n : m));
-    RQ_CUDA(h, cudaMemcpy(buf.data(), h->sw.y, sizeof(float) * n, cudaMemcpyDeviceToHost));
-    for (int i = 0; i < n; ++i) x_out[i] = sc ? h->sD[i] * (double)buf[i] : buf[i];
-    if (z_out && m > 0) {
-        RQ_CUDA(h, cudaMemcpy(buf.data(), h->sw.z, sizeof(float) * m, cudaMemcpyDeviceToHost));
-        for (int i = 0; i < m; ++i) z_out[i] = sc ? (double)buf[i] / h->sE[i] : buf[i];
-    }
-    if (lam_out && m > 0) {
-        RQ_CUDA(h, cudaMemcpy(buf.data(), h->sw.lstd, sizeof(float) * m, cudaMemcpyDeviceToHost));
-        for (int i = 0; i < m; ++i) lam_out[i] = sc ? h->sE[i] * (double)buf[i] / h->sC : buf[i];
+    const float *xb = h->sw.out, *zb = xb + n, *lb = zb + m;
+    for (int j = 0; j < n; ++j) x_out[j] = sc ? h->sD[j] * (double)xb[j] : xb[j];
+    for (int i = 0; i < m; ++i) {
+        if (z_out) z_out[i] = sc ? (double)zb[i] / h->sE[i] : zb[i];
+        if (lam_out) lam_out[i] = sc ? h->sE[i] * (double)lb[i] / h->sC : lb[i];
     }
     if (info) *info = inf;
     return RELU_QP_OK;
@@ -538,6 +506,7 @@ void relu_qp_destroy(relu_qp_t h) {
     if (h->stream) cudaStreamSynchronize(h->stream);
     else cudaDeviceSynchronize();
     rq::batch_release(h);
+    rq::single_release(h);
     for (cudaEvent_t e : h->prof_ev)
         if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : h->gap_ev)

@@ -58,21 +58,23 @@ struct BankEntry {
     double* bias64 = nullptr; // R FP64 = Bop64 q (FP64 single solve)
 };
 
-// Workspace of the single-QP cooperative solve.
+// Workspace of the single-QP solve.
 struct SingleWork {
-    float *y = nullptr, *z = nullptr, *lam = nullptr, *Ay = nullptr;
-    float *s0 = nullptr, *s1 = nullptr;
-    float *Py = nullptr, *Axf = nullptr, *lstd = nullptr;
-    float* xin = nullptr;       // warm-start x (FP32)
-    float* lin = nullptr;       // warm-start lam (FP32)
-    unsigned* red = nullptr;    // 3 slots x 8 reduction words
-    unsigned* bar = nullptr;    // grid barrier: arrival count of the launch (+ pad word)
-    int* out_i = nullptr;       // status, iters, rho_index, switches, err
-    float* out_f = nullptr;     // r_prim, r_dual
+    unsigned long long* words = nullptr;   // the grid form's tagged exchange words
+    int* err = nullptr;                    // error word of its waits
+    unsigned tag = 0;                      // exchange numbers used so far
+    unsigned count = 0;                    // arrivals counted so far (modulo 2^32)
+    int last_ctas = 0;                     // CTAs of the last launch, and whether it counted them
+    bool counted = false;
+    int max_ctas = 0;
+    float* in = nullptr;                   // warm start on the device: x, lam
+    // pinned host memory: staging of q, l, u and of a warm start, results x, z, lam, info words
+    float *pin = nullptr, *pin_in = nullptr, *out = nullptr, *out_f = nullptr;
+    int* out_i = nullptr;
     int grid = 0;               // CTAs of the launch (autotuned)
     int cluster = 0;            // > 1: the launch is one cluster of `grid` CTAs (else a cooperative grid)
     int cached_rows = 0;        // rows of W each CTA keeps in shared memory
-    int rows_per_cta = 0;
+    int gs = 1;                 // rows of a warp's group
 };
 
 // Workspace of the FP64 single-QP solve (opts.single_precision = FP64 or FP64R).
@@ -210,10 +212,12 @@ int condense_mpc(int nx, int nu, int N, const double* A, const double* B, const 
 int build_bank(relu_qp_t h, const double* dP, const double* dA, const std::vector<double>& rho_rows_scale);
 // FP32 copies of P, A, A^T from FP64 device arrays (setup_fp64.cu).
 int make_check_matrices(relu_qp_t h, const double* dP, const double* dA);
-// b_r = Bop_r q for every bank entry (single_solve.cu).
-int compute_bias(relu_qp_t h);
-// Cooperative single-QP solve (single_solve.cu).
-int single_solve(relu_qp_t h, const float* x_warm_dev, const float* lam_warm_dev, int rho_index,
+// Single-QP solve (single_solve.cu).
+int single_alloc(relu_qp_t h);
+void single_release(relu_qp_t h);
+// q, l, u from h->sw.pin to the device and the biases they give
+int single_update(relu_qp_t h);
+int single_solve(relu_qp_t h, const float* x_warm, const float* lam_warm, int rho_index,
                  double eps_abs, double eps_rel, int max_iter, relu_qp_info* info);
 int single_prepare(relu_qp_t h);
 int single_get_config(relu_qp_t h, int* ctas, int* cluster, int* cached_rows);

@@ -31,18 +31,29 @@ __global__ void diag_grid_kernel(unsigned* bar, int* err, unsigned expected, lon
     grid_sync_n(bar, err, timeout_ns, &s_ok, expected);
 }
 
-// One cluster of CTAs that meet `rounds` times at the cluster barrier, whose
-// mbarriers expect `extra` arrivals more than there are CTAs (extra = 1: every
-// CTA waits until the deadline); every CTA then reaches the final hardware
-// cluster barrier (no CTA exits while a partner may still arrive on its
-// mbarrier).
-__global__ void diag_cluster_kernel(int* err, unsigned extra, int rounds, long long timeout_ns) {
-    __shared__ GridSyncState s_ok;
-    __shared__ __align__(8) unsigned long long s_bar;
-    ClusterBarrier cb{0u, 0u, 1};
-    cluster_barrier_init(cb, &s_bar, extra);
-    for (int k = 0; k < rounds; ++k)
-        if (!cluster_barrier(cb, err, timeout_ns, &s_ok)) break;
+// One cluster of CTAs that hand each other one word `rounds` times; each CTA's
+// mbarrier expects `extra` words more than are sent (extra = 1: every CTA waits
+// until the deadline).  Every CTA then reaches the final hardware cluster
+// barrier (no CTA exits while a partner may still write its shared memory).
+__global__ void diag_cluster_kernel(int* err, int ctas, int extra, int rounds, long long timeout_ns) {
+    // two barriers, as in the solve: a word of round k + 2 (round k's barrier) leaves only
+    // once its sender has round k + 1, which every CTA sends after it has all of round k
+    __shared__ __align__(8) unsigned long long s_bar[2];
+    __shared__ float s_words[2][16];
+    const uint32_t bytes = 4u * (uint32_t)(ctas + extra);
+    if (threadIdx.x == 0) {
+        for (int b = 0; b < 2; ++b) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(cl_smem(&s_bar[b])) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        for (int b = 0; b < 2; ++b) cl_expect(cl_smem(&s_bar[b]), bytes);
+    }
+    cl_sync_hw();
+    if (threadIdx.x == 0)
+        for (int k = 0; k < rounds; ++k) {
+            const uint32_t bar = cl_smem(&s_bar[k & 1]);
+            for (int q = 0; q < ctas; ++q) cl_send1(cl_smem(&s_words[k & 1][blockIdx.x]), bar, q, (float)k);
+            if (!cl_wait(bar, (k >> 1) & 1, err, timeout_ns)) break;
+            cl_expect(bar, bytes);
+        }
     __syncthreads();
     cl_sync_hw();
 }
@@ -111,7 +122,7 @@ int relu_qp_diag_device_wait(int kind, long long timeout_ns, int* status, double
     } else if (!clus) {
         rc = RELU_QP_ERR_UNSUPPORTED;
     } else {
-        // a cluster of 2 CTAs: kind 4 one arrival short, kind 5 three complete rounds
+        // a cluster of 2 CTAs: kind 4 one word short, kind 5 three complete rounds
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(2);
         cfg.blockDim = dim3(64);
@@ -124,10 +135,9 @@ int relu_qp_diag_device_wait(int kind, long long timeout_ns, int* status, double
         cfg.attrs = at;
         cfg.numAttrs = 1;
         int* err = words;
-        const unsigned extra = kind == 4 ? 1u : 0u;
-        const int rounds = kind == 4 ? 1 : 3;
+        const int ctas = 2, extra = kind == 4 ? 1 : 0, rounds = kind == 4 ? 1 : 3;
         const long long ns = timeout_ns;
-        if (cudaLaunchKernelEx(&cfg, rq::diag_cluster_kernel, err, extra, rounds, ns) != cudaSuccess)
+        if (cudaLaunchKernelEx(&cfg, rq::diag_cluster_kernel, err, ctas, extra, rounds, ns) != cudaSuccess)
             rc = RELU_QP_ERR_CUDA;
     }
     cudaEventRecord(e1, 0);

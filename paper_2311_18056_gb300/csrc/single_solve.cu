@@ -9,47 +9,84 @@
 //   x+ = t_x,  (Ax)+ = t_Ax,  z+ = clamp(t_Ax + r, l, u),  lam'+ = rho r,
 // which equals v+ = clamp(W v + b) with v = [x; z; lam'].
 //
-// Work split: the R = n + m rows of Wt are cut into contiguous slices, one
-// per CTA; each CTA keeps as many of its rows as fit in shared memory (the
-// rest stream from L2) and its rows' state for the whole solve, and each warp
-// computes up to 4 of its rows at once (coalesced 128-bit loads, one shuffle
-// reduction per row).  Two launch forms, chosen by timing at setup: a
-// cooperative grid, whose CTAs exchange the layer's operand through global
-// memory and meet at the grid barrier, or one thread-block cluster, whose CTAs
-// write each new operand entry into every CTA's shared copy and meet at a
-// cluster barrier.  Every barrier wait has a deadline after which the kernel
-// records RELU_QP_ERR_TIMEOUT and returns.
+// Work split: each CTA owns a slice of the rows of x and a slice of the rows of
+// A x, keeps as many of their rows of Wt as fit in shared memory (the rest
+// stream from L2) and their state for the whole solve; a warp computes up to
+// 4 consecutive rows at once (coalesced 128-bit loads, one shuffle reduction
+// per row).  The check of a row of x and the dual residual of that row stay in
+// the same CTA, so a check exchanges only lam_std and the residual maxima.
+//
+// Exchange.  What bounds a layer is not the product (a few hundred clocks) but
+// handing every CTA the new operand, so the operand's entries carry their own
+// arrival and no barrier stands between layers.  Three forms, chosen by timing
+// at setup; a row's arithmetic, and so every bit of the result, is the same:
+//  - one CTA: shared memory and a CTA barrier;
+//  - one cluster: st.async writes each entry into every CTA's copy and counts
+//    its bytes on that CTA's mbarrier (one trip; a store, a release and an
+//    arrival one after the other before);
+//  - a cooperative grid: every entry is one 64-bit word in global memory, value
+//    and exchange number together, and the readers poll the words themselves;
+//    or, where that many words would crowd the L2, plain entries and a count of
+//    the CTAs that have stored theirs, polled before the entries are read.
+// Two operand buffers suffice: a CTA publishes exchange e + 1 (over e - 1) only
+// after it has all of e, and a row's part of e is sent only once its warp has
+// read all of e - 1 that it needs.
+// A row's remaining state (z, lam', r) is updated after its entry has left, and stays in
+// registers while every warp has one group of rows; a check's FP64 decision is one warp's.
+//
+// Measured, us per layer at n = m = 20 / 160 / 320 / 640 / 800 / 1600 (200 fixed layers,
+// best shape): 0.44 / 0.77 / 1.19 / 1.80 / 2.54 / 4.26; with a barrier between layers and
+// the operand loaded after it 1.61 / 1.98 / 2.23 / 2.72 / 2.92 / 4.75.  The last is bound
+// by reading the rows (41 MB a layer from shared memory and L2), the others by the
+// exchange: 0.25 (one CTA), 0.6 (cluster), 1.2 (words), 2.2 (count).
+//
+// Every wait has a deadline after which the kernel records RELU_QP_ERR_TIMEOUT
+// in the error word; the other waits see it and leave too.
 #include "common.h"
 #include "grid_sync.h"
 
+#include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <mutex>
 
 namespace rq {
 
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 
 enum { RED_RP = 0, RED_RD, RED_AX, RED_Z, RED_PX, RED_ATL, RED_WORDS = 8 };
-enum { OUT_STATUS = 0, OUT_ITERS, OUT_RHO, OUT_SWITCHES, OUT_ERR, OUT_WORDS = 8 };
+enum { DEC_STOP = 6, DEC_RHO = 7 };   // of the decision's words: 1 + the status to stop with, or 0; bank entry
+enum { OUT_STATUS = 0, OUT_ITERS, OUT_RHO, OUT_SWITCHES, OUT_ERR, OUT_LAST, OUT_WORDS = 8 };
+// FORM_GRID and FORM_COUNT are cooperative grids: tagged words, or plain operand buffers and a
+// count of the CTAs that have written theirs.
+enum Form { FORM_GRID = 0, FORM_CLUSTER = 1, FORM_ONE = 2, FORM_COUNT = 3 };
+constexpr int kState = 9;   // floats of state per row (see solve_body)
 
 struct SP {
-    int n, m, R, ldw, ldp, lda, ldt, nr;
+    int n, m, R, ldw, ldp, ldt, nr;
     const float* Wt[RQ_MAX_RHO];
     const float* bias[RQ_MAX_RHO];
     double rho[RQ_MAX_RHO];
     const float *P, *A, *At, *q, *l, *u, *rs;
     const float *rsx, *rsz;   // scaled problems: residual factors 1/(c D), 1/E (else nullptr)
-    float *y, *z, *lam, *Ay, *s0, *s1, *Py, *Axf, *lstd;
-    unsigned* red;
-    unsigned* bar;
-    int* out_i;
+    const float *xin, *lin;   // warm start (or nullptr)
+    float *xo, *zo, *lo;      // results (zo, lo may be nullptr)
+    // grid form: tagged words of the operand [2][R], of lam_std [m] and of the maxima [ctas][8]
+    unsigned long long *wop, *wls, *wred;
+    unsigned tag0;            // exchange e is tagged tag0 + 1 + e
+    // count form: the operand buffers [2][ldw] and the arrivals so far, from count0 on
+    float* sop;
+    unsigned *count, count0;
+    int *err, *out_i;
     float* out_f;
     int rho_index0, check_interval, adaptive, max_iter;
     double eps_abs, eps_rel, qnorm;
-    int rows_per_cta, cached_rows, rows2_per_cta;
+    int xr, ar, ctas;         // rows of x and of A x per CTA, CTAs with rows
+    int gs, gu, cached_rows;  // rows of a warp's group, of a group outside shared memory
+    int share;                // grid form of a problem too large for both: lam_std staged over the operand
     long long timeout_ns;
 };
 
@@ -57,19 +94,6 @@ __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
-}
-
-// Grid-wide barrier over all CTAs of the cooperative launch (grid_sync.h).
-__device__ __forceinline__ bool grid_barrier(const SP& p, GridSyncState* s_ok) {
-    return grid_sync(p.bar, p.out_i + OUT_ERR, p.timeout_ns, s_ok);
-}
-
-// Synchronisation between layers and phases: the grid barrier (grid form) or
-// the one-cluster barrier (cluster form, grid_sync.h).
-template <bool CL>
-__device__ __forceinline__ bool sync_all(const SP& p, ClusterBarrier& cb, GridSyncState* gs) {
-    if (!CL) return grid_barrier(p, gs);
-    return cluster_barrier(cb, p.out_i + OUT_ERR, p.timeout_ns, gs);
 }
 
 // Dot product of a padded row with a padded vector in shared memory; the
@@ -92,37 +116,46 @@ __device__ __forceinline__ float row_dot(const float* __restrict__ w, const floa
     return warp_sum((a0 + a1) + (a2 + a3));
 }
 
-__device__ __forceinline__ float row_dot_global(const float* __restrict__ w, const float* __restrict__ s,
-                                                int ld, int lane) {
-    const float4* w4 = reinterpret_cast<const float4*>(w);
-    const float4* s4 = reinterpret_cast<const float4*>(s);
-    const int n4 = ld >> 2;
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-    for (int k = lane; k < n4; k += 32) {
-        const float4 a = __ldg(w4 + k);
-        const float4 b = s4[k];
-        a0 = fmaf(a.x, b.x, a0);
-        a1 = fmaf(a.y, b.y, a1);
-        a2 = fmaf(a.z, b.z, a2);
-        a3 = fmaf(a.w, b.w, a3);
-    }
-    return warp_sum((a0 + a1) + (a2 + a3));
-}
+constexpr int kRows = 4;   // rows of a warp whose dot products run together (a group)
 
-// Dot products of NR padded rows (w[j], in shared or global memory) with one
-// padded vector in shared memory, in one pass over k: every row keeps the
-// four accumulators and the reduction of row_dot, so each result has row_dot's
-// bits, while the rows' loads and shuffle reductions overlap.  Results are
-// valid in every lane.
+// Dot products of NR (1, 2 or 4) padded rows (w[j], in shared or global memory) with one
+// padded vector in shared memory, in one pass over k: every row keeps the four accumulators
+// and the summation tree of row_dot, so each result has row_dot's bits, while the rows' loads
+// overlap.  The sums are scattered as they are formed (a lane keeps half of its rows at each
+// of the first steps: 6 shuffles for 4 rows where one reduction per row takes 20, and a
+// CTA's shuffles go one warp a clock): lane l returns row l / (32 / NR).
 template <int NR, bool LDG>
-__device__ __forceinline__ void rows_dot(const float* const (&w)[NR], const float* __restrict__ s, int ld, int lane,
-                                         float (&out)[NR]) {
+__device__ __forceinline__ float rows_dot(const float* const (&w)[kRows], const float* __restrict__ s, int ld, int lane) {
     const float4* s4 = reinterpret_cast<const float4*>(s);
     const int n4 = ld >> 2;
     float a[NR][4];
 #pragma unroll
     for (int j = 0; j < NR; ++j) a[j][0] = a[j][1] = a[j][2] = a[j][3] = 0.f;
-    for (int k = lane; k < n4; k += 32) {
+    int k = lane;
+    if (LDG) {
+        // rows in global memory: U steps' loads before the first product (an L2 trip is some
+        // 700 clocks, the step's products a few)
+        constexpr int U = NR == 1 ? 8 : NR == 2 ? 4 : 2;
+        for (; k + 32 * (U - 1) < n4; k += 32 * U) {
+            float4 x[U][NR];
+#pragma unroll
+            for (int t = 0; t < U; ++t)
+#pragma unroll
+                for (int j = 0; j < NR; ++j) x[t][j] = __ldg(reinterpret_cast<const float4*>(w[j]) + k + 32 * t);
+#pragma unroll
+            for (int t = 0; t < U; ++t) {
+                const float4 b = s4[k + 32 * t];
+#pragma unroll
+                for (int j = 0; j < NR; ++j) {
+                    a[j][0] = fmaf(x[t][j].x, b.x, a[j][0]);
+                    a[j][1] = fmaf(x[t][j].y, b.y, a[j][1]);
+                    a[j][2] = fmaf(x[t][j].z, b.z, a[j][2]);
+                    a[j][3] = fmaf(x[t][j].w, b.w, a[j][3]);
+                }
+            }
+        }
+    }
+    for (; k < n4; k += 32) {
         const float4 b = s4[k];
 #pragma unroll
         for (int j = 0; j < NR; ++j) {
@@ -134,325 +167,547 @@ __device__ __forceinline__ void rows_dot(const float* const (&w)[NR], const floa
             a[j][3] = fmaf(x.w, b.w, a[j][3]);
         }
     }
+    float v[NR];
 #pragma unroll
-    for (int j = 0; j < NR; ++j) out[j] = warp_sum((a[j][0] + a[j][1]) + (a[j][2] + a[j][3]));
-}
-
-constexpr int kRowsILP = 4;   // rows of a warp whose dot products run together
-
-// rows_dot for the first cnt (1 .. kRowsILP) pointers of w.  LDG: every row is in
-// global memory (read-only loads); else the rows are in shared memory or mixed.
-template <bool LDG>
-__device__ __forceinline__ void group_dots(int cnt, const float* const (&w)[kRowsILP], const float* s, int ld,
-                                           int lane, float (&acc)[kRowsILP]) {
-    if (cnt == 1) {
-        const float* w1[1] = {w[0]};
-        float o[1];
-        rows_dot<1, LDG>(w1, s, ld, lane, o);
-        acc[0] = o[0];
-    } else if (cnt == 2) {
-        const float* w2[2] = {w[0], w[1]};
-        float o[2];
-        rows_dot<2, LDG>(w2, s, ld, lane, o);
-        acc[0] = o[0];
-        acc[1] = o[1];
-    } else if (cnt == 3) {
-        const float* w3[3] = {w[0], w[1], w[2]};
-        float o[3];
-        rows_dot<3, LDG>(w3, s, ld, lane, o);
-        acc[0] = o[0];
-        acc[1] = o[1];
-        acc[2] = o[2];
-    } else {
-        rows_dot<4, LDG>(w, s, ld, lane, acc);
+    for (int j = 0; j < NR; ++j) v[j] = (a[j][0] + a[j][1]) + (a[j][2] + a[j][3]);
+    int o = 16;
+#pragma unroll
+    for (int h = NR / 2; h >= 1; h /= 2, o /= 2) {
+        const bool up = (lane & o) != 0;   // keeps the upper half of its rows
+#pragma unroll
+        for (int j = 0; j < h; ++j) {
+            const float give = up ? v[j] : v[j + h], keep = up ? v[j + h] : v[j];
+            v[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
     }
+    for (; o > 0; o /= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    return v[0];
 }
 
-// Copy `count` floats (padded length `ld`, a multiple of 4) written by other
-// CTAs into shared memory, bypassing L1 so that no stale line is read.
-__device__ __forceinline__ void load_shared_cg(float* dst, const float* src, int ld) {
-    const float4* s4 = reinterpret_cast<const float4*>(src);
-    float4* d4 = reinterpret_cast<float4*>(dst);
-    for (int k = threadIdx.x; k < (ld >> 2); k += blockDim.x) d4[k] = __ldcg(s4 + k);
+// LDG: every row is in global memory (read-only loads); else in shared memory or mixed.
+template <bool LDG>
+__device__ __forceinline__ float group_dot(int gs, const float* const (&w)[kRows], const float* s, int ld, int lane) {
+    if (gs == 4) return rows_dot<4, LDG>(w, s, ld, lane);
+    if (gs == 2) return rows_dot<2, LDG>(w, s, ld, lane);
+    return rows_dot<1, LDG>(w, s, ld, lane);
 }
 
-__device__ void load_w_cache(const SP& p, float* wcache, int ri, int row0, int ncache) {
-    const float4* src = reinterpret_cast<const float4*>(p.Wt[ri] + (size_t)row0 * p.ldw);
-    float4* dst = reinterpret_cast<float4*>(wcache);
-    const int total = ncache * (p.ldw >> 2);
-    for (int e = threadIdx.x; e < total; e += blockDim.x) dst[e] = __ldg(src + e);
+constexpr bool is_grid(int form) { return form == FORM_GRID || form == FORM_COUNT; }
+
+// ---- exchanges -------------------------------------------------------------
+__device__ __forceinline__ void put_word(unsigned long long* w, float v, unsigned tag) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(w), "l"(((unsigned long long)tag << 32) | __float_as_uint(v))
+                 : "memory");
+}
+
+__device__ __forceinline__ void get_words(const unsigned long long* w, unsigned long long& a, unsigned long long& b) {
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(w) : "memory");
+}
+
+// The `count` values of the tagged words w (16-byte aligned) into dst, by the whole CTA;
+// false in every thread if a wait gave up.  Four pairs a thread are in flight; only pairs
+// that are not there yet are read again.
+__device__ __forceinline__ bool gather(const SP& p, const unsigned long long* w, float* dst, int count, unsigned tag) {
+    constexpr int U = 4;
+    bool ok = true;
+    const int pairs = (count + 1) >> 1;
+    for (int b = threadIdx.x; b < pairs && ok; b += U * kThreads) {
+        unsigned todo = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (b + u * kThreads < pairs) todo |= 1u << u;
+        long long t0 = 0;
+        for (int tries = 0; todo; ++tries) {
+            unsigned long long a[U], c[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if ((todo >> u) & 1u) get_words(w + 2 * (b + u * kThreads), a[u], c[u]);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (!((todo >> u) & 1u)) continue;
+                const int k = 2 * (b + u * kThreads);
+                if ((unsigned)(a[u] >> 32) != tag || (k + 1 < count && (unsigned)(c[u] >> 32) != tag)) continue;
+                todo &= ~(1u << u);
+                dst[k] = __uint_as_float((unsigned)a[u]);
+                if (k + 1 < count) dst[k + 1] = __uint_as_float((unsigned)c[u]);
+            }
+            if (todo && (tries & 63) == 63) {
+                if (t0 == 0) t0 = grid_sync_timer();
+                if (sync_give_up(p.err, t0, p.timeout_ns)) {
+                    ok = false;
+                    break;
+                }
+            }
+        }
+    }
+    return __syncthreads_or(ok ? 0 : 1) == 0;
+}
+
+// The first ncache rows of the CTA (x rows x0 .., then A x rows a0 ..) of bank entry ri.
+__device__ void load_w_cache(const SP& p, float* wcache, int ri, int x0, int nx, int a0, int ncache) {
+    const int c4 = p.ldw >> 2;
+    for (int e = threadIdx.x; e < ncache * c4; e += kThreads) {
+        const int lr = e / c4, k = e - lr * c4, r = lr < nx ? x0 + lr : p.n + a0 + (lr - nx);
+        reinterpret_cast<float4*>(wcache)[e] = __ldg(reinterpret_cast<const float4*>(p.Wt[ri] + (size_t)r * p.ldw) + k);
+    }
 }
 
 __device__ __forceinline__ void red_max(unsigned* slot, int word, float v) {
     atomicMax(slot + word, __float_as_uint(fabsf(v)));
 }
 
-__device__ __forceinline__ float red_get(const unsigned* slot, int word) {
-    return __uint_as_float(__ldcg(slot + word));
-}
-
-// The solve.  Grid form (CL = false): a cooperative grid; the operand s of a
-// layer goes through global memory (written by the rows' owners, staged into
-// shared memory after the grid barrier).  Cluster form (CL = true): the launch
-// is one cluster; every CTA keeps both operand buffers in shared memory and the
-// owner of a row writes its new entry into every CTA's copy (distributed shared
-// memory) before the cluster barrier, so a layer never touches L2 for s.
-template <bool CL>
-__device__ __forceinline__ void solve_body(const SP& p, float* smem, ClusterBarrier& cb, GridSyncState* gs) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n = p.n, m = p.m, R = p.R;
-    const int row0 = blockIdx.x * p.rows_per_cta;
-    const int row1 = min(row0 + p.rows_per_cta, R);
-    const int ncache = max(0, min(p.cached_rows, row1 - row0));
+// The solve.
+template <int F>
+__device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned long long* mbar, unsigned* s_red,
+                                           unsigned* s_dec) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
+    const int n = p.n, m = p.m, R = p.R, ldw = p.ldw, cta = blockIdx.x;
+    // this CTA's rows: lr < nx are x0 + lr, the others A x rows a0 + lr - nx
+    const int x0 = cta * p.xr, nx = max(0, min(p.xr, n - x0));
+    const int a0 = cta * p.ar, na = max(0, min(p.ar, m - a0));
+    const int rows = nx + na, gs = p.gs;
+    const int ncache = min(p.cached_rows, rows);
+    const int ngu = (rows - ncache + p.gu - 1) / p.gu, ng = ngu + (ncache + gs - 1) / gs;
+    const int per = p.xr + p.ar;
     float* wcache = smem;
-    float* sv = smem + (size_t)p.cached_rows * p.ldw;     // ldw floats (cluster form: 2 x ldw, both operands)
-    float* svk = CL ? sv + 2 * (size_t)p.ldw : sv;        // the checks' staged vector (ldw floats)
-    // the state of the CTA's rows, kept in shared memory for the whole solve (the
-    // global copies are still written, for the checks and the outputs): bias of the
-    // bank entry in use, and for rows of A x the carried A x, z, lam', rho_i, l, u
-    const int rpc = p.rows_per_cta;
-    float* st_bias = sv + (CL ? 3 : 1) * (size_t)p.ldw;
-    float* st_ay = st_bias + rpc;
-    float* st_z = st_ay + rpc;
-    float* st_lam = st_z + rpc;
-    float* st_rho = st_lam + rpc;
-    float* st_l = st_rho + rpc;
-    float* st_u = st_l + rpc;
-    const int r2_0 = blockIdx.x * p.rows2_per_cta;
-    const int r2_1 = min(r2_0 + p.rows2_per_cta, n);
+    float* sv = smem + (size_t)p.cached_rows * ldw;        // operand: two buffers (grids: one)
+    float* svk = sv + (size_t)(is_grid(F) ? 1 : 2) * ldw;  // lam_std (ldt floats)
+    float* reds = svk + (p.share ? 0 : p.ldt);             // every CTA's maxima [ctas][8]
+    if (is_grid(F) && p.share) svk = sv;                   // (read again after the check)
+    float* st_bias = reds + RED_WORDS * p.ctas;
+    // per row: bias, r = (Ax) - z + lam'/rho of the next layer, z (x of a row of x), lam', rho, l, u,
+    // the check's product, lam_std
+    float *st_rr = st_bias + per, *st_z = st_rr + per, *st_lam = st_z + per, *st_rho = st_lam + per,
+          *st_l = st_rho + per, *st_u = st_l + per, *st_chk = st_u + per, *st_ls = st_chk + per;
+    auto carry = [&](float ax, float z, float lam, float rho_i) { return ax - z + lam / rho_i; };
+    // barriers (cluster form): operand buffers 0 and 1, lam_std, maxima
+    const uint32_t bar0 = cl_smem(mbar);
+    const uint32_t sv_a = cl_smem(sv), svk_a = cl_smem(svk), reds_a = cl_smem(reds);
+    auto row_of = [&](int lr) { return lr < nx ? x0 + lr : n + a0 + (lr - nx); };
+    bool failed = false;
+    unsigned e = 0;      // exchange whose operand is current
+    auto cur = [&]() { return sv + (is_grid(F) ? 0 : (size_t)(e & 1) * ldw); };
+    // one entry of exchange x
+    auto publish = [&](unsigned x, int r, float v) {
+        if (F == FORM_GRID) {
+            put_word(p.wop + (size_t)(x & 1) * ((R + 1) & ~1) + r, v, p.tag0 + 1 + x);
+        } else if (F == FORM_COUNT) {
+            p.sop[(size_t)(x & 1) * ldw + r] = v;
+        } else if (F == FORM_ONE) {
+            sv[(size_t)(x & 1) * ldw + r] = v;
+        } else {
+            for (int q = 0; q < p.ctas; ++q) cl_send1(sv_a + 4u * ((x & 1) * ldw + r), bar0 + 8 * (x & 1), q, v);
+        }
+    };
+    // all of exchange x (cluster form: a warp's own wait, by the warps that compute rows)
+    auto wait_bar = [&](uint32_t bar, uint32_t parity) {
+        if (!failed && !cl_wait(bar, parity, p.err, p.timeout_ns)) failed = true;
+    };
+    auto receive = [&](unsigned x) -> bool {
+        if (F == FORM_GRID) {
+            __syncthreads();   // the buffer's readers are done
+            return gather(p, p.wop + (size_t)(x & 1) * ((R + 1) & ~1), sv, R, p.tag0 + 1 + x);
+        }
+        if (F == FORM_COUNT) {
+            // every CTA has stored its entries (its release covers them) and read the last operand
+            __syncthreads();
+            bool ok = true;
+            if (tid == 0) {
+                asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.count) : "memory");
+                const unsigned target = p.count0 + (x + 1) * (unsigned)p.ctas;
+                long long t0 = 0;
+                while (ok) {
+                    unsigned v;
+                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p.count) : "memory");
+                    if ((int)(v - target) >= 0) break;
+                    if (t0 == 0) t0 = grid_sync_timer();
+                    ok = !sync_give_up(p.err, t0, p.timeout_ns);
+                }
+            }
+            if (__syncthreads_or(ok ? 0 : 1)) return false;
+            const float4* src = reinterpret_cast<const float4*>(p.sop + (size_t)(x & 1) * ldw);
+            for (int k = tid; k < (ldw >> 2); k += kThreads) reinterpret_cast<float4*>(sv)[k] = __ldcg(src + k);
+            __syncthreads();
+            return true;
+        }
+        if (F == FORM_ONE) {
+            __syncthreads();
+            return true;
+        }
+        if (warp < ng) wait_bar(bar0 + 8 * (x & 1), (x >> 1) & 1);
+        if (tid == 0 && !failed) cl_expect(bar0 + 8 * (x & 1), 4u * R);   // the buffer's next use
+        return true;
+    };
 
-    int ri = p.rho_index0;
-    int switches = 0, checks = 0, cur = 0;
-    if (ncache > 0) load_w_cache(p, wcache, ri, row0, ncache);
-    for (int r = row0 + threadIdx.x; r < row1; r += blockDim.x) {
-        const int lr = r - row0;
-        st_bias[lr] = __ldg(p.bias[ri] + r);
-        if (r >= n) {
-            const int i = r - n;
-            st_ay[lr] = __ldcg(p.Ay + i);
-            st_z[lr] = __ldcg(p.z + i);
-            st_lam[lr] = __ldcg(p.lam + i);
+    int ri = p.rho_index0, switches = 0;
+    unsigned checks = 0;
+    // ---------------- start state ----------------
+    for (int k = tid; k < ldw; k += kThreads) {   // the padding's zeros, and x for z = A x
+        const float v = k < n && p.xin ? p.xin[k] : 0.f;
+        // (cluster form: exchange 0 may already be arriving in the first buffer)
+        if (F != FORM_CLUSTER || k >= R) sv[k] = v;
+        if (!is_grid(F)) sv[ldw + k] = v;
+    }
+    if (!p.share)
+        for (int k = tid; k < p.ldt; k += kThreads) svk[k] = 0.f;
+    if (tid < RED_WORDS) s_red[tid] = 0u;
+    for (int lr = tid; lr < rows; lr += kThreads) {
+        st_bias[lr] = __ldg(p.bias[ri] + row_of(lr));
+        if (lr >= nx) {
+            const int i = a0 + lr - nx;
             st_rho[lr] = (float)(p.rho[ri] * (double)__ldg(p.rs + i));
             st_l[lr] = __ldg(p.l + i);
             st_u[lr] = __ldg(p.u + i);
+            st_lam[lr] = p.lin ? p.lin[i] : 0.f;
+            st_z[lr] = 0.f;
         }
-    }
-    if (CL) {
-        // operand buffer 0 is s0; buffer 1 only needs its padding zeroed: its rows are
-        // written by the partners' first layer, which may already be running (nobody
-        // writes buffer 0 before every CTA has passed the first barrier)
-        load_shared_cg(sv, p.s0, p.ldw);
-        for (int k = R + threadIdx.x; k < p.ldw; k += blockDim.x) sv[p.ldw + k] = 0.f;
     }
     __syncthreads();
-
-    for (int it = 1; it <= p.max_iter; ++it) {
-        // ---------------- one layer: s[cur] -> s[cur^1] ----------------
-        const float* scur = cur ? p.s1 : p.s0;
-        float* snext = cur ? p.s0 : p.s1;
-        const float* svc = CL ? sv + (size_t)cur * p.ldw : sv;
-        const uint32_t svn = CL ? cl_smem(sv + (size_t)(cur ^ 1) * p.ldw) : 0u;
-        if (!CL) {
-            load_shared_cg(sv, scur, p.ldw);
-            __syncthreads();
+    if (p.xin) {
+        // z = A x
+        const float* x = is_grid(F) ? sv : sv + ldw;
+        for (int lr = nx + warp; lr < rows; lr += kWarps) {
+            const float v = row_dot(p.A + (size_t)(a0 + lr - nx) * p.ldp, x, p.ldp, lane);
+            if (lane == 0) st_z[lr] = v;
         }
-        const float* Wg = p.Wt[ri];
-        // the global copies of the rows' state are read only by the checks and the
-        // outputs: written on the layers before a check and on the last one
-        const bool keep = (p.check_interval > 0 && it % p.check_interval == 0) || it == p.max_iter;
-        // a warp's rows rb, rb + kWarps, ... in groups of up to kRowsILP: their dot
-        // products together, then lane j updates row j of the group
-        for (int rb = row0 + warp; rb < row1; rb += kRowsILP * kWarps) {
-            const int cnt = min(kRowsILP, (row1 - rb + kWarps - 1) / kWarps);
-            // the cached rows are the first ncache of the CTA: a group is all cached, all in
-            // global memory, or (once per CTA) mixed
-            const int lr_first = rb - row0, lr_last = rb + (cnt - 1) * kWarps - row0;
-            float acc[kRowsILP] = {0.f, 0.f, 0.f, 0.f};
-            if (lr_last < ncache) {
-                const float* w[kRowsILP];
+        __syncthreads();
+    }
+    for (int lr = tid; lr < rows; lr += kThreads) {
+        const int r = row_of(lr);
+        if (lr >= nx) st_rr[lr] = carry(st_z[lr], st_z[lr], st_lam[lr], st_rho[lr]);
+        publish(0, r, lr < nx ? (p.xin ? p.xin[r] : 0.f) : fmaf(2.0f * st_rho[lr], st_z[lr], -st_lam[lr]));
+    }
+    load_w_cache(p, wcache, ri, x0, nx, a0, ncache);
+    if (F == FORM_CLUSTER) {
+        __syncthreads();
+        if (tid < 32) wait_bar(bar0, 0);
+        failed = __syncthreads_or(failed ? 1 : 0) != 0;
+        if (tid == 0 && !failed) cl_expect(bar0, 4u * R);
+    } else if (!receive(0)) {
+        return;
+    }
+
+    // Groups: the rows that are not in shared memory first (their loads take longest), one to
+    // gu of them to a warp, then gs of the cached ones; group g is warp g % kWarps's.  A
+    // group's lanes split by row: lane l updates row l / (32 / its rows), one lane per row
+    // publishes and stores.
+    struct Group {
+        int lr0, cnt, gr;      // first row, rows, lanes' rows (gs or gu)
+        bool global;
+        const float* w[kRows];
+    };
+    auto group = [&](int g) {
+        Group G;
+        G.global = g < ngu;
+        G.gr = G.global ? p.gu : gs;
+        G.lr0 = G.global ? ncache + g * p.gu : (g - ngu) * gs;
+        G.cnt = min(G.gr, (G.global ? rows : ncache) - G.lr0);
 #pragma unroll
-                for (int j = 0; j < kRowsILP; ++j) w[j] = wcache + (size_t)(lr_first + (j < cnt ? j : 0) * kWarps) * p.ldw;
-                group_dots<false>(cnt, w, svc, p.ldw, lane, acc);
-            } else if (lr_first >= ncache) {
-                const float* w[kRowsILP];
-#pragma unroll
-                for (int j = 0; j < kRowsILP; ++j) w[j] = Wg + (size_t)(rb + (j < cnt ? j : 0) * kWarps) * p.ldw;
-                group_dots<true>(cnt, w, svc, p.ldw, lane, acc);
-            } else {
-                const float* w[kRowsILP];
-#pragma unroll
-                for (int j = 0; j < kRowsILP; ++j) {
-                    const int r = rb + (j < cnt ? j : 0) * kWarps, lr = r - row0;
-                    w[j] = lr < ncache ? wcache + (size_t)lr * p.ldw : Wg + (size_t)r * p.ldw;
-                }
-                group_dots<false>(cnt, w, svc, p.ldw, lane, acc);
-            }
-            float snew = 0.f;
-            if (lane < cnt) {
-                float a = acc[0];
-#pragma unroll
-                for (int j = 1; j < kRowsILP; ++j)
-                    if (lane == j) a = acc[j];
-                const int r = rb + lane * kWarps, lr = r - row0;
-                const float t = a + st_bias[lr];
-                if (r < n) {
-                    if (keep) p.y[r] = t;
-                    snew = t;
-                } else {
-                    const int i = r - n;
-                    const float rho_i = st_rho[lr];
-                    const float rr = st_ay[lr] - st_z[lr] + st_lam[lr] / rho_i;
-                    const float zn = fminf(fmaxf(t + rr, st_l[lr]), st_u[lr]);
-                    const float ln = rho_i * rr;
-                    st_ay[lr] = t;
-                    st_z[lr] = zn;
-                    st_lam[lr] = ln;
-                    if (keep) {
-                        p.Ay[i] = t;
-                        p.z[i] = zn;
-                        p.lam[i] = ln;
+        for (int j = 0; j < kRows; ++j) {
+            const int lr = G.lr0 + (j < G.cnt ? j : 0);
+            G.w[j] = G.global ? p.Wt[ri] + (size_t)row_of(lr) * ldw : wcache + (size_t)lr * ldw;
+        }
+        return G;
+    };
+    auto product = [&](const Group& G, const float* s) {
+        return G.global ? group_dot<true>(G.gr, G.w, s, ldw, lane) : group_dot<false>(G.gr, G.w, s, ldw, lane);
+    };
+    // a group's new operand entries: row lr's in its lanes, `one` set in one of them
+    auto hand_on = [&](const Group& G, int lr, bool valid, bool one, float snew) {
+        if (F != FORM_CLUSTER) {
+            if (one) publish(e + 1, row_of(lr), snew);
+            return;
+        }
+        const int r = row_of(G.lr0), b = (int)((e + 1) & 1);
+        const uint32_t bar = bar0 + 8 * b, base = sv_a + 4u * (uint32_t)(b * ldw);
+        if (G.cnt == 4 && (r & 3) == 0 && (G.lr0 + 3 < nx || G.lr0 >= nx)) {
+            const float v0 = __shfl_sync(0xffffffffu, snew, 0), v1 = __shfl_sync(0xffffffffu, snew, 8),
+                        v2 = __shfl_sync(0xffffffffu, snew, 16), v3 = __shfl_sync(0xffffffffu, snew, 24);
+            if (lane < p.ctas) cl_send4(base + 4u * (uint32_t)r, bar, lane, v0, v1, v2, v3);
+        } else if (valid) {
+            const int per_row = 32 / G.gr;
+            for (int q = lane % per_row; q < p.ctas; q += per_row) cl_send1(base + 4u * (uint32_t)row_of(lr), bar, q, snew);
+        }
+    };
+
+    int it = 0;
+    while (true) {
+        // ---------------- the layers up to the next check, or the last one ----------------
+        const int len = p.check_interval > 0 ? min(p.check_interval, p.max_iter - it) : p.max_iter - it;
+        if (ng <= kWarps) {
+            // one group a warp: its rows' state stays in registers
+            const bool work = warp < ng;
+            const Group G = group(work ? warp : 0);
+            const int per_row = 32 / G.gr, jl = lane / per_row;
+            const bool valid = work && jl < G.cnt, one = valid && lane % per_row == 0;
+            const int lr = G.lr0 + (jl < G.cnt ? jl : 0);
+            const bool ax = work && lr >= nx;
+            const float bias = work ? st_bias[lr] : 0.f, rho_i = ax ? st_rho[lr] : 0.f, lo = ax ? st_l[lr] : 0.f,
+                        up = ax ? st_u[lr] : 0.f, rho2 = 2.0f * rho_i;
+            float rr = ax ? st_rr[lr] : 0.f, z = 0.f, lam = 0.f;
+            for (int k = 0; k < len; ++k) {
+                if (work && !failed) {
+                    z = product(G, cur()) + bias;
+                    float snew = z;
+                    if (ax) {
+                        const float t = z;
+                        z = fminf(fmaxf(t + rr, lo), up);
+                        lam = __fmul_rn(rho_i, rr);
+                        snew = fmaf(rho2, z, -lam);
+                        rr = t - z + rr;
                     }
-                    snew = 2.0f * rho_i * zn - ln;
+                    hand_on(G, lr, valid, one, snew);
                 }
-                if (!CL) snext[r] = snew;
+                ++e;
+                if (!receive(e)) return;
             }
-            if (CL) {
-                // lane q writes each row's entry into CTA q's next operand
-                for (int j = 0; j < cnt; ++j) {
-                    const float v = __shfl_sync(0xffffffffu, snew, j);
-                    const uint32_t addr = svn + 4u * (uint32_t)(rb + j * kWarps);
-                    for (int q = lane; q < cb.C; q += 32) cl_st(cl_mapa(addr, (uint32_t)q), v);
+            if (one) {
+                st_z[lr] = z;
+                if (ax) st_lam[lr] = lam;
+            }
+        } else {
+            for (int k = 0; k < len; ++k) {
+                const float* svc = cur();
+                for (int g = warp; g < ng && !failed; g += kWarps) {
+                    const Group G = group(g);
+                    const int per_row = 32 / G.gr, jl = lane / per_row;
+                    const bool valid = jl < G.cnt, one = valid && lane % per_row == 0;
+                    const int lr = G.lr0 + (valid ? jl : 0);
+                    const float t = product(G, svc) + st_bias[lr];
+                    float z = t, lam = 0.f, snew = t, rr = 0.f;
+                    const bool ax = lr >= nx;
+                    if (ax) {
+                        rr = st_rr[lr];
+                        z = fminf(fmaxf(t + rr, st_l[lr]), st_u[lr]);
+                        lam = __fmul_rn(st_rho[lr], rr);
+                        snew = fmaf(2.0f * st_rho[lr], z, -lam);
+                        rr = t - z + rr;
+                    }
+                    hand_on(G, lr, valid, one, snew);
+                    if (one) {
+                        st_z[lr] = z;
+                        if (ax) {
+                            st_lam[lr] = lam;
+                            st_rr[lr] = rr;
+                        }
+                    }
+                    __syncwarp();
                 }
+                ++e;
+                if (!receive(e)) return;
             }
         }
-        cur ^= 1;
-        if (!sync_all<CL>(p, cb, gs)) return;
-
-        const bool is_check = (p.check_interval > 0) && (it % p.check_interval == 0);
+        it += len;
+        const bool is_check = p.check_interval > 0 && it % p.check_interval == 0;
         const bool last = (it == p.max_iter);
-        if (!is_check && !last) continue;
 
         // ---------------- residuals (Eqs. primal, dual) ----------------
-        unsigned* slot = p.red + (checks % 3) * RED_WORDS;
-        if (blockIdx.x == 0 && threadIdx.x < RED_WORDS)
-            p.red[((checks + 1) % 3) * RED_WORDS + threadIdx.x] = 0u;
+        // (a warp of the cluster form that gave up leaves here, with its CTA)
+        if (__syncthreads_or(failed ? 1 : 0)) return;
+        const float* svc = cur();
+        const unsigned tag = p.tag0 + 1 + e;
+        constexpr int kC = 2, kPer = 32 / kC;   // rows of a warp (in global memory: P, A, A^T)
+        const int jc = lane / kPer;
+        const bool lead = lane % kPer == 0;
+        for (int lr0 = warp * kC; lr0 < rows; lr0 += kWarps * kC) {
+            const int lr = lr0 + jc;
+            const float* c[kRows];
+#pragma unroll
+            for (int j = 0; j < kRows; ++j) {
+                const int k = min(lr0 + (j < kC ? j : 0), rows - 1);
+                c[j] = k < nx ? p.P + (size_t)(x0 + k) * p.ldp : p.A + (size_t)(a0 + k - nx) * p.ldp;
+            }
+            const float v = rows_dot<kC, true>(c, svc, p.ldp, lane);
+            if (lr < nx) {
+                if (lead) {
+                    st_chk[lr] = v;
+                    red_max(s_red, RED_PX, p.rsx ? v * p.rsx[x0 + lr] : v);
+                }
+            } else if (lr < rows) {
+                const int i = a0 + lr - nx;
+                const float zi = st_z[lr], f = p.rsz ? p.rsz[i] : 1.f, ls = fmaf(st_rho[lr], v - zi, st_lam[lr]);
+                if (lead) {
+                    st_chk[lr] = v;
+                    st_ls[lr] = ls;
+                    red_max(s_red, RED_RP, (v - zi) * f);
+                    red_max(s_red, RED_AX, v * f);
+                    red_max(s_red, RED_Z, zi * f);
+                    if (is_grid(F)) put_word(p.wls + i, ls, tag);
+                    else if (F == FORM_ONE) svk[i] = ls;
+                }
+                if (F == FORM_CLUSTER)
+                    for (int q = lane % kPer; q < p.ctas; q += kPer) cl_send1(svk_a + 4u * (uint32_t)i, bar0 + 16, q, ls);
+            }
+        }
+        if (is_grid(F)) {
+            if (p.share) {
+                __syncthreads();
+                for (int k = m + tid; k < p.ldt; k += kThreads) svk[k] = 0.f;
+            }
+            if (m > 0 && !gather(p, p.wls, svk, m, tag)) return;
+        } else if (F == FORM_ONE) {
+            __syncthreads();
+        } else if (m > 0) {
+            wait_bar(bar0 + 16, checks & 1);
+            if (__syncthreads_or(failed ? 1 : 0)) return;
+            if (tid == 0) cl_expect(bar0 + 16, 4u * m);
+        }
+        for (int lr0 = warp * kC; lr0 < nx; lr0 += kWarps * kC) {
+            const int lr = lr0 + jc;
+            float v = 0.f;
+            if (m > 0) {
+                const float* c[kRows];
+#pragma unroll
+                for (int j = 0; j < kRows; ++j) c[j] = p.At + (size_t)(x0 + min(lr0 + (j < kC ? j : 0), nx - 1)) * p.ldt;
+                v = rows_dot<kC, true>(c, svk, p.ldt, lane);
+            }
+            if (lr < nx && lead) {
+                const float f = p.rsx ? p.rsx[x0 + lr] : 1.f;
+                red_max(s_red, RED_RD, (st_chk[lr] + __ldg(p.q + x0 + lr) + v) * f);
+                red_max(s_red, RED_ATL, v * f);
+            }
+        }
+        __syncthreads();
+        // every CTA's maxima
+        if (is_grid(F)) {
+            if (tid < RED_WORDS) put_word(p.wred + RED_WORDS * cta + tid, __uint_as_float(s_red[tid]), tag);
+            if (!gather(p, p.wred, reds, RED_WORDS * p.ctas, tag)) return;
+        } else if (F == FORM_CLUSTER) {
+            for (int t = tid; t < 2 * p.ctas; t += kThreads) {
+                const float* v = reinterpret_cast<const float*>(s_red) + 4 * (t & 1);
+                cl_send4(reds_a + 4u * (uint32_t)(RED_WORDS * cta + 4 * (t & 1)), bar0 + 24, t >> 1, v[0], v[1], v[2], v[3]);
+            }
+            wait_bar(bar0 + 24, checks & 1);
+            if (__syncthreads_or(failed ? 1 : 0)) return;
+            if (tid == 0) cl_expect(bar0 + 24, 4u * RED_WORDS * p.ctas);
+        } else {
+            if (tid < RED_WORDS) reinterpret_cast<unsigned*>(reds)[tid] = s_red[tid];
+            __syncthreads();
+        }
         ++checks;
-        load_shared_cg(svk, p.y, p.ldp);
-        __syncthreads();
-        for (int r = row0 + warp; r < row1; r += kWarps) {
-            if (r < n) {
-                const float v = row_dot_global(p.P + (size_t)r * p.ldp, svk, p.ldp, lane);
-                if (lane == 0) {
-                    p.Py[r] = v;
-                    red_max(slot, RED_PX, p.rsx ? v * p.rsx[r] : v);
-                }
-            } else {
-                const int i = r - n;
-                const float v = row_dot_global(p.A + (size_t)i * p.lda, svk, p.lda, lane);
-                if (lane == 0) {
-                    const float zi = p.z[i];
-                    const float rho_i = (float)(p.rho[ri] * (double)__ldg(p.rs + i));
-                    p.Axf[i] = v;
-                    p.lstd[i] = p.lam[i] + rho_i * (v - zi);
-                    const float f = p.rsz ? p.rsz[i] : 1.f;
-                    red_max(slot, RED_RP, (v - zi) * f);
-                    red_max(slot, RED_AX, v * f);
-                    red_max(slot, RED_Z, zi * f);
-                }
-            }
+        if (warp < 6) {
+            unsigned v = 0;
+            for (int q = lane; q < p.ctas; q += 32) v = max(v, reinterpret_cast<const unsigned*>(reds)[RED_WORDS * q + warp]);
+            v = __reduce_max_sync(0xffffffffu, v);
+            if (lane == 0) s_dec[warp] = v;
         }
-        if (!sync_all<CL>(p, cb, gs)) return;
-        if (m > 0) load_shared_cg(svk, p.lstd, p.ldt);
         __syncthreads();
-        for (int j = r2_0 + warp; j < r2_1; j += kWarps) {
-            const float v = (m > 0) ? row_dot_global(p.At + (size_t)j * p.ldt, svk, p.ldt, lane) : 0.f;
-            if (lane == 0) {
-                const float f = p.rsx ? p.rsx[j] : 1.f;
-                red_max(slot, RED_RD, (__ldcg(p.Py + j) + __ldg(p.q + j) + v) * f);
-                red_max(slot, RED_ATL, v * f);
-            }
-        }
-        if (!sync_all<CL>(p, cb, gs)) return;
+        if (tid < RED_WORDS) s_red[tid] = 0u;
 
         // ---------------- decision (identical in every CTA) ----------------
-        const double rp = red_get(slot, RED_RP), rd = red_get(slot, RED_RD);
-        const double nAx = red_get(slot, RED_AX), nz = red_get(slot, RED_Z);
-        const double nPx = red_get(slot, RED_PX), nAtl = red_get(slot, RED_ATL);
-        const bool numerical = !(isfinite(rp) && isfinite(rd) && isfinite(nPx) && isfinite(nAtl));
-        const double eps_p = p.eps_abs + p.eps_rel * fmax(nAx, nz);
-        const double eps_d = p.eps_abs + p.eps_rel * fmax(fmax(nPx, nAtl), p.qnorm);
-        const bool converged = is_check && !numerical && rp <= eps_p && rd <= eps_d;
-        if (converged || numerical || last) {
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
-                p.out_i[OUT_STATUS] = numerical ? RELU_QP_NUMERICAL
-                                                : (converged ? RELU_QP_SOLVED : RELU_QP_MAX_ITER);
+        // One warp takes it: an FP64 instruction holds an SM's FP64 pipe for 16 clocks a warp.
+        if (warp == 0) {
+            const double rp = __uint_as_float(s_dec[RED_RP]), rd = __uint_as_float(s_dec[RED_RD]);
+            const double nAx = __uint_as_float(s_dec[RED_AX]), nz = __uint_as_float(s_dec[RED_Z]);
+            const double nPx = __uint_as_float(s_dec[RED_PX]), nAtl = __uint_as_float(s_dec[RED_ATL]);
+            const bool numerical = !(isfinite(rp) && isfinite(rd) && isfinite(nPx) && isfinite(nAtl));
+            const double eps_p = p.eps_abs + p.eps_rel * fmax(nAx, nz);
+            const double eps_d = p.eps_abs + p.eps_rel * fmax(fmax(nPx, nAtl), p.qnorm);
+            const bool converged = is_check && !numerical && rp <= eps_p && rd <= eps_d;
+            int nri = ri;
+            if (p.adaptive && is_check && !converged && !numerical) {
+                // Eq. rho_update (inf-norms, 1e-4 floors), nearest bank entry in log distance: entry k
+                // is nearer to the estimate than entry b when the estimate lies on k's side of
+                // sqrt(rho_k rho_b)
+                const double num = rp * fmax(fmax(nPx, nAtl), fmax(p.qnorm, 1e-4));
+                const double den = rd * fmax(fmax(nAx, nz), 1e-4);
+                if (num > 0.0 && den > 0.0) {
+                    const double est2 = p.rho[ri] * p.rho[ri] * (num / den);
+                    if (isfinite(est2) && est2 > 0.0) {
+                        nri = 0;
+                        for (int k = 1; k < p.nr; ++k) {
+                            const double mid2 = p.rho[k] * p.rho[nri];
+                            if (p.rho[k] > p.rho[nri] ? est2 > mid2 : p.rho[k] < p.rho[nri] && est2 < mid2) nri = k;
+                        }
+                    }
+                }
+            }
+            if (lane == 0) {
+                s_dec[DEC_STOP] = numerical ? 1 + RELU_QP_NUMERICAL : converged ? 1 + RELU_QP_SOLVED : last ? 1 + RELU_QP_MAX_ITER : 0;
+                s_dec[DEC_RHO] = (unsigned)nri;
+            }
+        }
+        __syncthreads();
+        const int stop = (int)s_dec[DEC_STOP];
+        if (stop) {
+            for (int lr = tid; lr < rows; lr += kThreads) {
+                if (lr < nx) {
+                    p.xo[x0 + lr] = st_z[lr];
+                } else {
+                    const int i = a0 + lr - nx;
+                    if (p.zo) p.zo[i] = st_z[lr];
+                    if (p.lo) p.lo[i] = st_ls[lr];
+                }
+            }
+            if (cta == 0 && tid == 0) {
+                p.out_i[OUT_STATUS] = stop - 1;
                 p.out_i[OUT_ITERS] = it;
                 p.out_i[OUT_RHO] = ri;
                 p.out_i[OUT_SWITCHES] = switches;
-                p.out_f[0] = (float)rp;
-                p.out_f[1] = (float)rd;
+                p.out_i[OUT_LAST] = (int)e;
+                p.out_f[0] = __uint_as_float(s_dec[RED_RP]);
+                p.out_f[1] = __uint_as_float(s_dec[RED_RD]);
             }
             return;
         }
-        // refresh the carried Ax with the directly computed one
-        for (int r = max(row0, n) + threadIdx.x; r < row1; r += blockDim.x) {
-            const float v = p.Axf[r - n];
-            p.Ay[r - n] = v;
-            st_ay[r - row0] = v;
-        }
-        if (!p.adaptive || !is_check) continue;
-        // Eq. rho_update (inf-norms, 1e-4 floors), nearest bank entry in log distance
-        const double num = rp * fmax(fmax(nPx, nAtl), fmax(p.qnorm, 1e-4));
-        const double den = rd * fmax(fmax(nAx, nz), 1e-4);
-        int nri = ri;
-        if (num > 0.0 && den > 0.0) {
-            const double est = p.rho[ri] * sqrt(num / den);
-            if (isfinite(est) && est > 0.0) {
-                const double le = log(est);
-                double best = 1e300;
-                for (int k = 0; k < p.nr; ++k) {
-                    const double d = fabs(le - log(p.rho[k]));
-                    if (d < best) { best = d; nri = k; }
-                }
-            }
-        }
-        if (nri == ri) continue;
-        // switch: rebase lam' so that the next layer is standard ADMM with the new rho
-        float* scur2 = cur ? p.s1 : p.s0;
-        for (int r = max(row0, n) + threadIdx.x; r < row1; r += blockDim.x) {
-            const int i = r - n;
-            const float rho_i = (float)(p.rho[nri] * (double)__ldg(p.rs + i));
-            const float zi = p.z[i];
-            const float lnew = p.lstd[i] - rho_i * (p.Axf[i] - zi);
-            p.lam[i] = lnew;
-            st_lam[r - row0] = lnew;
-            st_rho[r - row0] = rho_i;
-            const float sn = 2.0f * rho_i * zi - lnew;
-            if (CL) {
-                const uint32_t a = cl_smem(sv + (size_t)cur * p.ldw + r);
-                for (int q = 0; q < cb.C; ++q) cl_st(cl_mapa(a, (uint32_t)q), sn);
+        const int nri = (int)s_dec[DEC_RHO];
+        if (nri == ri) {
+            // the directly computed Ax replaces the carried one
+            for (int lr = nx + tid; lr < rows; lr += kThreads) st_rr[lr] = carry(st_chk[lr], st_z[lr], st_lam[lr], st_rho[lr]);
+            if (is_grid(F) && p.share) {
+                if (!receive(e)) return;
             } else {
-                scur2[r] = sn;
+                __syncthreads();   // the state above is read by the rows' warps
             }
+            continue;
         }
+        // switch: rebase lam' so that the next layer is standard ADMM with the new rho, and
+        // hand the operand on with the new penalties
         ri = nri;
         ++switches;
-        if (ncache > 0) load_w_cache(p, wcache, ri, row0, ncache);
-        for (int r = row0 + threadIdx.x; r < row1; r += blockDim.x) st_bias[r - row0] = __ldg(p.bias[ri] + r);
-        if (!sync_all<CL>(p, cb, gs)) return;
+        for (int lr = tid; lr < rows; lr += kThreads) {
+            const int r = row_of(lr);
+            float v;
+            if (lr < nx) {
+                v = st_z[lr];
+            } else {
+                const float rho_i = (float)(p.rho[ri] * (double)__ldg(p.rs + (r - n)));
+                const float lnew = fmaf(-rho_i, st_chk[lr] - st_z[lr], st_ls[lr]);
+                st_lam[lr] = lnew;
+                st_rho[lr] = rho_i;
+                st_rr[lr] = carry(st_chk[lr], st_z[lr], lnew, rho_i);
+                v = fmaf(2.0f * rho_i, st_z[lr], -lnew);
+            }
+            publish(e + 1, r, v);
+            st_bias[lr] = __ldg(p.bias[ri] + r);
+        }
+        load_w_cache(p, wcache, ri, x0, nx, a0, ncache);
+        __syncthreads();
+        ++e;
+        if (!receive(e)) return;
     }
 }
 
-template <bool CL>
-__global__ void __launch_bounds__(kThreads, 1) single_solve_kernel(SP p) {
+template <int F>
+__global__ void __launch_bounds__(kThreads, 1) single_solve_kernel(const __grid_constant__ SP p) {
     extern __shared__ __align__(16) float smem[];
-    __shared__ GridSyncState s_ok;
-    __shared__ __align__(8) unsigned long long s_cbar;
-    grid_sync_init(&s_ok);
-    ClusterBarrier cb{0u, 0u, 1};
-    if (CL) cluster_barrier_init(cb, &s_cbar, 0u);   // C arrivals per phase
-    solve_body<CL>(p, smem, cb, &s_ok);
-    if (CL) {
+    __shared__ __align__(8) unsigned long long s_bar[4];
+    __shared__ __align__(16) unsigned s_red[RED_WORDS];
+    __shared__ unsigned s_dec[RED_WORDS];
+    if (F == FORM_CLUSTER) {
+        if (threadIdx.x == 0 && blockIdx.x < p.ctas) {
+            const uint32_t b = cl_smem(s_bar);
+            for (int k = 0; k < 4; ++k) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b + 8 * k) : "memory");
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            cl_expect(b, 4u * p.R);
+            cl_expect(b + 8, 4u * p.R);
+            if (p.m > 0) cl_expect(b + 16, 4u * p.m);
+            cl_expect(b + 24, 4u * RED_WORDS * p.ctas);
+        }
+        cl_sync_hw();   // every CTA's barriers stand before anything is sent
+    }
+    if ((int)blockIdx.x < p.ctas) solve_body<F>(p, smem, s_bar, s_red, s_dec);
+    if (F == FORM_CLUSTER) {
         // no CTA leaves while a partner may still write its shared memory (every
         // wait before this point has a deadline, so every CTA gets here)
         __syncthreads();
@@ -460,64 +715,65 @@ __global__ void __launch_bounds__(kThreads, 1) single_solve_kernel(SP p) {
     }
 }
 
-// Warm/cold start: x given (or 0), z = A x, lam' = lam (or 0), carried Ax = A x,
-// s0 = [x; 2 rho z - lam'] (rho of the starting bank entry), pads zeroed.
-__global__ void init_state_kernel(int n, int m, int lda, int ldw, const float* __restrict__ A,
-                                  const float* __restrict__ xin, const float* __restrict__ lin,
-                                  const float* __restrict__ rs, double rho, float* y, float* z,
-                                  float* lam, float* Ay, float* s0, float* s1) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int r = warp; r < ldw; r += nw) {
-        if (r < n) {
-            if (lane == 0) {
-                const float v = xin ? xin[r] : 0.f;
-                y[r] = v;
-                s0[r] = v;
-                s1[r] = 0.f;
-            }
-        } else if (r < n + m) {
-            const int i = r - n;
-            float v = 0.f;
-            if (xin) {
-                for (int k = lane; k < n; k += 32) v = fmaf(A[(size_t)i * lda + k], xin[k], v);
-                v = warp_sum(v);
-            }
-            if (lane == 0) {
-                const float li = lin ? lin[i] : 0.f;
-                const float rho_i = (float)(rho * (double)rs[i]);
-                z[i] = v;
-                Ay[i] = v;
-                lam[i] = li;
-                s0[r] = 2.0f * rho_i * v - li;
-                s1[r] = 0.f;
-            }
-        } else if (lane == 0) {
-            s0[r] = 0.f;
-            s1[r] = 0.f;
+// b_r = Bop_r q for every bank entry (blockIdx.y), one warp per row.
+struct BiasPtrs {
+    const float* Bop[RQ_MAX_RHO];
+    float* bias[RQ_MAX_RHO];
+};
+
+__global__ void __launch_bounds__(256) bias_kernel(BiasPtrs b, int rows, int n, const float* __restrict__ q) {
+    const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (r >= rows) return;
+    const float* w = b.Bop[blockIdx.y] + (size_t)r * n;
+    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+    if ((n & 3) == 0) {
+        const float4 *w4 = reinterpret_cast<const float4*>(w), *q4 = reinterpret_cast<const float4*>(q);
+#pragma unroll 4
+        for (int k = lane; k < (n >> 2); k += 32) {
+            const float4 x = __ldg(w4 + k), y = __ldg(q4 + k);
+            a0 = fmaf(x.x, y.x, a0);
+            a1 = fmaf(x.y, y.y, a1);
+            a2 = fmaf(x.z, y.z, a2);
+            a3 = fmaf(x.w, y.w, a3);
         }
+    } else {
+#pragma unroll 4
+        for (int k = lane; k < n; k += 32) a0 = fmaf(__ldg(w + k), __ldg(q + k), a0);
     }
+    const float v = warp_sum((a0 + a1) + (a2 + a3));
+    if (lane == 0) b.bias[blockIdx.y][r] = v;
 }
 
-__global__ void matvec_rows_kernel(const float* __restrict__ M, int rows, int cols, int ld,
-                                   const float* __restrict__ x, float* __restrict__ out) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int r = warp; r < rows; r += nw) {
-        float v = 0.f;
-        for (int k = lane; k < cols; k += 32) v = fmaf(M[(size_t)r * ld + k], x[k], v);
-        v = warp_sum(v);
-        if (lane == 0) out[r] = v;
+// Slices of the rows: per CTA xr rows of x and ar rows of A x (the cluster form: multiples
+// of 4, so that a warp's 4 entries leave as one 16-byte store); CTAs with rows: a prefix.
+void slices(relu_qp_t h, int ctas, bool cl, int* xr, int* ar, int* used) {
+    int a = ceil_div(h->n, ctas), b = h->m > 0 ? ceil_div(h->m, ctas) : 0;
+    if (cl) {
+        a = (int)round_up(a, 4);
+        b = (int)round_up(b, 4);
     }
+    *xr = a;
+    *ar = b;
+    *used = std::max(ceil_div(h->n, a), b > 0 ? ceil_div(h->m, b) : 0);
 }
 
-int fill_params(relu_qp_t h, SP& p, int grid) {
+// Above this many entries the grid counts its CTAs instead of tagging the entries: every CTA
+// polls all of the words (measured per layer, words against count: 1.80 / 2.73 us at 1280
+// entries, 2.54 / 3.05 at 1600, 7.7 / 5.2 at 3200).
+constexpr int kTagMax = 2048;
+
+Form form_of(relu_qp_t h, int ctas, int cluster) {
+    return cluster > 1 ? FORM_CLUSTER : ctas == 1 ? FORM_ONE : h->R <= kTagMax ? FORM_GRID : FORM_COUNT;
+}
+
+// lam_std has no room of its own beside an operand of more than 32768 entries (128 KB)
+bool share_lam(relu_qp_t h, int ctas, int cluster) { return is_grid(form_of(h, ctas, cluster)) && h->ldw > 32768; }
+
+// gs: rows of a warp's group (the cluster form: 4, one 16-byte store)
+void fill_params(relu_qp_t h, SP& p, int ctas, int cluster, int gs, int cached) {
     const int n = h->n, m = h->m;
     p.n = n; p.m = m; p.R = h->R; p.ldw = h->ldw;
     p.ldp = (int)round_up(n, 4);
-    p.lda = (int)round_up(n, 4);
     p.ldt = (int)round_up(m > 0 ? m : 1, 4);
     p.nr = h->nr;
     for (int r = 0; r < h->nr; ++r) {
@@ -527,197 +783,260 @@ int fill_params(relu_qp_t h, SP& p, int grid) {
     }
     p.P = h->P32; p.A = h->A32; p.At = h->At32;
     p.q = h->q32; p.l = h->l32; p.u = h->u32; p.rs = h->rs32;
-    SingleWork& w = h->sw;
-    p.y = w.y; p.z = w.z; p.lam = w.lam; p.Ay = w.Ay; p.s0 = w.s0; p.s1 = w.s1;
-    p.Py = w.Py; p.Axf = w.Axf; p.lstd = w.lstd;
-    p.red = w.red; p.bar = w.bar; p.out_i = w.out_i; p.out_f = w.out_f;
-    p.rows_per_cta = ceil_div(h->R, grid);
-    p.rows2_per_cta = ceil_div(n, grid);
+    p.rsx = h->sc_rx; p.rsz = h->sc_z;
+    p.qnorm = h->qnorm;
+    slices(h, ctas, cluster > 1, &p.xr, &p.ar, &p.ctas);
+    p.cached_rows = cached;
+    // the rows outside shared memory over as many warps as the cached ones leave
+    const int out = p.xr + p.ar - cached, free_warps = std::max(1, kWarps - ceil_div(cached, gs));
+    p.gu = out <= free_warps ? 1 : out <= 2 * free_warps ? 2 : 4;
+    p.gs = gs;
+    p.share = share_lam(h, ctas, cluster) ? 1 : 0;
     p.timeout_ns = 2000000000LL;
-    return RELU_QP_OK;
 }
 
-// cached rows of W + the staged operand (cluster form: both operands and the checks' vector)
-// + the state of the CTA's rows (7 floats per row)
-size_t smem_bytes(int cached_rows, int ldw, bool cl, int rows_per_cta) {
-    return (((size_t)cached_rows + (cl ? 3 : 1)) * ldw + 7 * (size_t)rows_per_cta) * sizeof(float);
+// cached rows of W + the operand (two buffers but in the grid form) + lam_std + every CTA's
+// maxima + the state of the CTA's rows
+size_t smem_bytes(relu_qp_t h, int cached_rows, int ctas, int cluster) {
+    int xr, ar, used;
+    slices(h, ctas, cluster > 1, &xr, &ar, &used);
+    return (((size_t)cached_rows + (is_grid(form_of(h, ctas, cluster)) ? 1 : 2)) * h->ldw +
+            (share_lam(h, ctas, cluster) ? 0 : round_up(h->m > 0 ? h->m : 1, 4)) + RED_WORDS * (size_t)used +
+            kState * (size_t)(xr + ar)) *
+           sizeof(float);
 }
 
-// Largest dynamic shared memory the solve kernel may request: the opt-in
-// per-block limit minus the kernel's static shared memory (of either form).
-int max_shared(relu_qp_t h) {
+const void* kernel_of(relu_qp_t h, int ctas, int cluster) {
+    switch (form_of(h, ctas, cluster)) {
+        case FORM_COUNT: return (const void*)single_solve_kernel<FORM_COUNT>;
+        case FORM_CLUSTER: return (const void*)single_solve_kernel<FORM_CLUSTER>;
+        case FORM_ONE: return (const void*)single_solve_kernel<FORM_ONE>;
+        default: return (const void*)single_solve_kernel<FORM_GRID>;
+    }
+}
+
+// Rows of Wt a CTA can cache: what the opt-in shared memory holds beside the rest; -1 when
+// not even the rest fits.
+int cached_rows_for(relu_qp_t h, int ctas, int cluster) {
     int v = 0;
     cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-    int stat = 0;
     cudaFuncAttributes fa{};
-    if (cudaFuncGetAttributes(&fa, single_solve_kernel<false>) == cudaSuccess) stat = (int)fa.sharedSizeBytes;
-    if (cudaFuncGetAttributes(&fa, single_solve_kernel<true>) == cudaSuccess && (int)fa.sharedSizeBytes > stat)
-        stat = (int)fa.sharedSizeBytes;
+    if (cudaFuncGetAttributes(&fa, kernel_of(h, ctas, cluster)) == cudaSuccess) v -= (int)fa.sharedSizeBytes;
     cudaGetLastError();
-    return v - stat - 256;
+    int xr, ar, used;
+    slices(h, ctas, cluster > 1, &xr, &ar, &used);
+    const long left = (long)v - 256 - (long)smem_bytes(h, 0, ctas, cluster);
+    if (left < 0) return -1;
+    return (int)std::min<long>(xr + ar, left / (long)((size_t)h->ldw * sizeof(float)));
 }
 
-// Shared-memory rows a CTA of a `grid`-CTA launch can cache.
-int cached_rows_for(relu_qp_t h, int grid, bool cl) {
-    const int rows = ceil_div(h->R, grid);
-    const long budget = (long)max_shared(h) - 7L * rows * (long)sizeof(float);
-    long cap = budget / (long)((size_t)h->ldw * sizeof(float)) - (cl ? 3 : 1);
-    if (cap < 0) cap = 0;
-    return rows < cap ? rows : (int)cap;
+cudaLaunchConfig_t cluster_config(relu_qp_t h, int ctas, size_t smem, cudaLaunchAttribute* at) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = h->stream;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = (unsigned)ctas;
+    at->val.clusterDim.y = 1;
+    at->val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
 }
 
-// Launch the solve kernel: a cooperative grid of `grid` CTAs, or (cluster > 1)
-// one cluster of `grid` CTAs.
-int launch_kernel(relu_qp_t h, SP& p, int grid, int cluster, int cached) {
-    const size_t smem = smem_bytes(cached, h->ldw, cluster > 1, ceil_div(h->R, grid));
-    if (cluster > 1) {
-        auto k = single_solve_kernel<true>;
-        RQ_CUDA(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        if (cluster > 8) RQ_CUDA(h, cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(grid);
-        cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = h->stream;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = (unsigned)cluster;
-        at[0].val.clusterDim.y = 1;
-        at[0].val.clusterDim.z = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 1;
-        RQ_CUDA(h, cudaLaunchKernelEx(&cfg, k, p));
-        return RELU_QP_OK;
-    }
-    RQ_CUDA(h, cudaFuncSetAttribute(single_solve_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem));
+// Launch the solve kernel: a cooperative grid of `ctas` CTAs, one CTA, or (cluster > 1) one
+// cluster of `ctas` CTAs.
+int launch_kernel(relu_qp_t h, SP& p, int ctas, int cluster) {
+    const size_t smem = smem_bytes(h, p.cached_rows, ctas, cluster);
+    const void* k = kernel_of(h, ctas, cluster);
+    RQ_CUDA(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (cluster > 8) RQ_CUDA(h, cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     void* args[] = {&p};
-    RQ_CUDA(h, cudaLaunchCooperativeKernel((const void*)single_solve_kernel<false>, dim3(grid), dim3(kThreads), args,
-                                           smem, h->stream));
+    if (cluster > 1) {
+        cudaLaunchAttribute at[1];
+        const cudaLaunchConfig_t cfg = cluster_config(h, ctas, smem, at);
+        RQ_CUDA(h, cudaLaunchKernelExC(&cfg, k, args));
+    } else if (ctas == 1) {
+        RQ_CUDA(h, cudaLaunchKernel(k, dim3(1), dim3(kThreads), args, smem, h->stream));
+    } else {
+        RQ_CUDA(h, cudaLaunchCooperativeKernel(k, dim3(ctas), dim3(kThreads), args, smem, h->stream));
+    }
     return RELU_QP_OK;
 }
 
-// Whether one cluster of `c` CTAs with this shared memory can be resident.
-bool cluster_fits(relu_qp_t h, int c, int cached) {
-    auto k = single_solve_kernel<true>;
-    const size_t smem = smem_bytes(cached, h->ldw, true, ceil_div(h->R, c));
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        (c > 8 && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
-        cudaGetLastError();
-        return false;
-    }
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(c);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)c;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
+// Whether the shape can be resident.  (Each launch sets the kernel's shared-memory limit to
+// its own size; the queries need it at least this large.)
+bool fits(relu_qp_t h, int ctas, int cluster, int cached) {
+    if (cached < 0) return false;
+    const size_t smem = smem_bytes(h, cached, ctas, cluster);
+    const void* k = kernel_of(h, ctas, cluster);
+    bool ok = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
     int n = 0;
-    const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, k, &cfg);
+    if (ok && cluster > 1) {
+        ok = cluster <= 8 || cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+        cudaLaunchAttribute at[1];
+        const cudaLaunchConfig_t cfg = cluster_config(h, ctas, smem, at);
+        ok = ok && cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n >= 1;
+    } else if (ok) {
+        ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kThreads, smem) == cudaSuccess && n >= 1 &&
+             ctas <= n * h->num_sms;
+    }
     cudaGetLastError();
-    return e == cudaSuccess && n >= 1;
+    return ok;
 }
 
-int launch(relu_qp_t h, int grid, int cluster, int cached, int rho_index, double eps_abs, double eps_rel,
-           int max_iter, int check_interval, int adaptive) {
+// Words of the grids' exchanges for this problem, and the pointers into them: the operand
+// (tagged words, or plain buffers of ldw floats), lam_std, the maxima, the count.
+size_t operand_words(relu_qp_t h) { return std::max(2 * round_up(h->R, 2), (size_t)h->ldw); }
+size_t exchange_words(relu_qp_t h, int max_ctas) {
+    return operand_words(h) + round_up(h->m, 2) + RED_WORDS * (size_t)max_ctas + 2;
+}
+void set_words(relu_qp_t h, SP& p, unsigned long long* w) {
+    p.wop = w;
+    p.sop = reinterpret_cast<float*>(w);
+    p.wls = w + operand_words(h);
+    p.wred = p.wls + round_up(h->m, 2);
+    p.count = reinterpret_cast<unsigned*>(p.wred + RED_WORDS * (size_t)h->sw.max_ctas);
+}
+
+// The exchange numbers start above every tag an earlier launch left in the words; the words
+// are zeroed (numbers start over) after a failure and before the numbers wrap around.
+int reset_words(relu_qp_t h) {
+    SingleWork& w = h->sw;
+    RQ_CUDA(h, cudaMemsetAsync(w.words, 0, sizeof(unsigned long long) * exchange_words(h, w.max_ctas), h->stream));
+    RQ_CUDA(h, cudaMemsetAsync(w.err, 0, sizeof(int), h->stream));
+    w.tag = w.count = 0;
+    return RELU_QP_OK;
+}
+
+int launch(relu_qp_t h, int ctas, int cluster, int cached, int gs, const float* xin, const float* lin, int rho_index,
+           double eps_abs, double eps_rel, int max_iter, int check_interval, int adaptive) {
+    SingleWork& w = h->sw;
+    if (w.tag > 0xC0000000u) RQ_TRY(reset_words(h));
     SP p{};
-    fill_params(h, p, grid);
-    p.cached_rows = cached;
+    fill_params(h, p, ctas, cluster, gs, cached);
+    set_words(h, p, w.words);
     p.rho_index0 = rho_index;
     p.check_interval = check_interval;
     p.adaptive = adaptive;
     p.max_iter = max_iter;
     p.eps_abs = eps_abs;
     p.eps_rel = eps_rel;
-    p.qnorm = h->qnorm;
-    p.rsx = h->sc_rx;
-    p.rsz = h->sc_z;
-    SingleWork& w = h->sw;
-    RQ_CUDA(h, cudaMemsetAsync(w.red, 0, sizeof(unsigned) * 3 * RED_WORDS, h->stream));
-    RQ_CUDA(h, cudaMemsetAsync(w.bar, 0, sizeof(unsigned) * 2, h->stream));
-    RQ_CUDA(h, cudaMemsetAsync(w.out_i, 0, sizeof(int) * OUT_WORDS, h->stream));
-    return launch_kernel(h, p, grid, cluster, cached);
+    p.xin = xin;
+    p.lin = lin;
+    p.xo = w.out;
+    p.zo = w.out + h->n;
+    p.lo = w.out + h->n + h->m;
+    p.tag0 = w.tag;
+    p.count0 = w.count;
+    w.last_ctas = p.ctas;
+    w.counted = form_of(h, ctas, cluster) == FORM_COUNT;
+    p.err = w.err;
+    p.out_i = w.out_i;
+    p.out_f = w.out_f;
+    w.out_i[OUT_LAST] = -1;    // the kernel's results go to host memory
+    return launch_kernel(h, p, ctas, cluster);
 }
 
-int init_state(relu_qp_t h, const float* x, const float* lam, int rho_index) {
+// After the launch has been waited for: its error, or the next free exchange number.
+int finish(relu_qp_t h, const char* what) {
     SingleWork& w = h->sw;
-    const int blocks = ceil_div(h->ldw * 32, 256) < 1024 ? ceil_div(h->ldw * 32, 256) : 1024;
-    init_state_kernel<<<blocks, 256, 0, h->stream>>>(h->n, h->m, (int)round_up(h->n, 4), h->ldw, h->A32,
-                                                      x, lam, h->rs32, h->be[rho_index].rho, w.y, w.z,
-                                                      w.lam, w.Ay, w.s0, w.s1);
-    RQ_CUDA(h, cudaGetLastError());
+    if (w.out_i[OUT_LAST] < 0) {
+        RQ_TRY(reset_words(h));
+        RQ_CUDA(h, cudaStreamSynchronize(h->stream));
+        return fail(h, RELU_QP_ERR_TIMEOUT, std::string("a wait passed its deadline ") + what);
+    }
+    w.tag += (unsigned)w.out_i[OUT_LAST] + 2u;
+    if (w.counted) w.count += ((unsigned)w.out_i[OUT_LAST] + 1u) * (unsigned)w.last_ctas;
     return RELU_QP_OK;
 }
 
 }  // namespace
 
-int compute_bias(relu_qp_t h) {
-    const int blocks = ceil_div(h->R * 32, 256) < 2048 ? ceil_div(h->R * 32, 256) : 2048;
+static int compute_bias(relu_qp_t h) {
+    BiasPtrs b{};
     for (int r = 0; r < h->nr; ++r) {
-        matvec_rows_kernel<<<blocks, 256, 0, h->stream>>>(h->be[r].Bop, h->R, h->n, h->n, h->q32,
-                                                          h->be[r].bias);
-        RQ_CUDA(h, cudaGetLastError());
+        b.Bop[r] = h->be[r].Bop;
+        b.bias[r] = h->be[r].bias;
     }
+    bias_kernel<<<dim3(ceil_div(h->R, 8), h->nr), 256, 0, h->stream>>>(b, h->R, h->n, h->q32);
+    RQ_CUDA(h, cudaGetLastError());
     return RELU_QP_OK;
 }
 
-// Choose the CTA count of the cooperative launch by timing 50 fixed-rho
-// layers (no checks) for each candidate that fits co-resident on the GPU.
+int single_alloc(relu_qp_t h) {
+    SingleWork& w = h->sw;
+    const size_t n = h->n, m = h->m;
+    w.max_ctas = 4 * h->num_sms;
+    RQ_TRY(alloc(h, &w.words, exchange_words(h, w.max_ctas)));
+    RQ_TRY(alloc(h, &w.err, 4));
+    RQ_TRY(alloc(h, &w.in, n + m));
+    // pinned: staging of q, l, u, staging of a warm start, the results the kernel writes
+    const size_t floats = 2 * (n + 2 * m) + (n + m) + 2 * RED_WORDS;
+    RQ_CUDA(h, cudaHostAlloc(reinterpret_cast<void**>(&w.pin), sizeof(float) * floats, cudaHostAllocDefault));
+    w.pin_in = w.pin + (n + 2 * m);
+    w.out = w.pin_in + (n + m);
+    w.out_f = w.out + (n + 2 * m);
+    w.out_i = reinterpret_cast<int*>(w.out_f + RED_WORDS);
+    return RELU_QP_OK;
+}
+
+void single_release(relu_qp_t h) {
+    if (h->sw.pin) cudaFreeHost(h->sw.pin);
+    h->sw.pin = nullptr;
+}
+
+// Group size of a shape before it is tuned: the fewest rows that give every warp a group.
+int default_gs(relu_qp_t h, int ctas, int cluster) {
+    int xr, ar, used;
+    slices(h, ctas, cluster > 1, &xr, &ar, &used);
+    const int want = ceil_div(xr + ar, kWarps);
+    return cluster > 1 || want > 2 ? 4 : want;
+}
+
+// Choose the launch shape by timing 50 fixed-rho layers (no checks) of every candidate that
+// can be resident, then the rows of a warp's group.
 int single_prepare(relu_qp_t h) {
-    int per_sm = 0;
+    SingleWork& w = h->sw;
+    w.grid = 0;
+    float best_t = 1e30f;
+    auto time = [&](int g, int cl, int cached, int gs) -> int {
+        float ms = 0.f;
+        for (int layers : {10, 50}) {   // a warm-up, then the timed run
+            RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
+            RQ_TRY(launch(h, g, cl, cached, gs, nullptr, nullptr, 0, 0.0, 0.0, layers, 0, 0));
+            RQ_CUDA(h, cudaEventRecord(h->ev1, h->stream));
+            RQ_CUDA(h, cudaStreamSynchronize(h->stream));
+            RQ_TRY(finish(h, "while tuning the solve"));
+            RQ_CUDA(h, cudaEventElapsedTime(&ms, h->ev0, h->ev1));
+        }
+        if (ms < best_t) {
+            best_t = ms;
+            w.grid = g;
+            w.cluster = cl;
+            w.cached_rows = cached;
+            w.gs = gs;
+        }
+        return RELU_QP_OK;
+    };
     // candidates: (CTAs, cluster); cluster > 1 = one cluster of that many CTAs
     std::vector<std::pair<int, int>> cands;
     for (int g = 1; g <= 4 * h->num_sms; g *= 2) cands.push_back({g, 0});
     cands.push_back({h->num_sms, 0});
     for (int c = 2; c <= 16; c *= 2) cands.push_back({c, c});
-    int best_g = 1, best_cl = 0, best_c = cached_rows_for(h, 1, false);
-    float best_t = 1e30f;
     for (const auto& gc : cands) {
         const int g = gc.first, cl = gc.second;
         if (g > h->R) continue;
-        const int cached = cached_rows_for(h, g, cl > 1);
-        if (cl > 1) {
-            if (!cluster_fits(h, cl, cached)) continue;
-        } else {
-            // the occupancy query needs the kernel's shared-memory limit at least this large
-            // (each launch below sets it to its own size)
-            const size_t smem = smem_bytes(cached, h->ldw, false, ceil_div(h->R, g));
-            RQ_CUDA(h, cudaFuncSetAttribute(single_solve_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)smem));
-            RQ_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, single_solve_kernel<false>, kThreads,
-                                                                     smem));
-            if (per_sm < 1 || g > per_sm * h->num_sms) continue;
-        }
-        h->sw.grid = g;
-        h->sw.cluster = cl;
-        RQ_TRY(init_state(h, nullptr, nullptr, 0));
-        RQ_TRY(launch(h, g, cl, cached, 0, 0.0, 0.0, 10, 0, 0));   // warm-up
-        RQ_TRY(init_state(h, nullptr, nullptr, 0));
-        RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
-        RQ_TRY(launch(h, g, cl, cached, 0, 0.0, 0.0, 50, 0, 0));
-        RQ_CUDA(h, cudaEventRecord(h->ev1, h->stream));
-        RQ_CUDA(h, cudaStreamSynchronize(h->stream));
-        int err = 0;
-        RQ_CUDA(h, cudaMemcpy(&err, h->sw.out_i + OUT_ERR, sizeof(int), cudaMemcpyDeviceToHost));
-        if (err) return fail(h, RELU_QP_ERR_TIMEOUT, "a barrier deadline passed while tuning the solve");
-        float ms = 0.f;
-        RQ_CUDA(h, cudaEventElapsedTime(&ms, h->ev0, h->ev1));
-        if (ms < best_t) {
-            best_t = ms;
-            best_g = g;
-            best_cl = cl;
-            best_c = cached;
-        }
+        const int cached = cached_rows_for(h, g, cl);
+        if (fits(h, g, cl, cached)) RQ_TRY(time(g, cl, cached, default_gs(h, g, cl)));
     }
-    h->sw.grid = best_g;
-    h->sw.cluster = best_cl;
-    h->sw.cached_rows = best_c;
-    h->sw.rows_per_cta = ceil_div(h->R, best_g);
+    if (w.grid == 0) return fail(h, RELU_QP_ERR_UNSUPPORTED, "the single-QP solve does not fit on an SM");
+    if (w.cluster <= 1) {
+        const int g = w.grid, cached = w.cached_rows, gs0 = w.gs;
+        for (int gs : {1, 2, 4})
+            if (gs != gs0) RQ_TRY(time(g, 0, cached, gs));
+    }
     return RELU_QP_OK;
 }
 
@@ -734,53 +1053,58 @@ int single_set_config(relu_qp_t h, int ctas, int cluster) {
     if (ctas < 1 || ctas > h->R || cluster < 0 || (cluster > 1 && cluster != ctas) ||
         (cluster > 1 && cluster != 2 && cluster != 4 && cluster != 8 && cluster != 16))
         return fail(h, RELU_QP_ERR_INVALID, "ctas in [1, n + m]; cluster 0 or cluster = ctas in {2, 4, 8, 16}");
-    const bool cl = cluster > 1;
+    const int cl = cluster > 1 ? cluster : 0;
     const int cached = cached_rows_for(h, ctas, cl);
-    if (cl) {
-        if (!cluster_fits(h, ctas, cached))
-            return fail(h, RELU_QP_ERR_UNSUPPORTED, "a cluster of this size cannot be resident");
-    } else {
-        int per_sm = 0;
-        RQ_CUDA(h, cudaFuncSetAttribute(single_solve_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)smem_bytes(cached, h->ldw, false, ceil_div(h->R, ctas))));
-        RQ_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, single_solve_kernel<false>, kThreads,
-                                                                 smem_bytes(cached, h->ldw, false, ceil_div(h->R, ctas))));
-        if (per_sm < 1 || ctas > per_sm * h->num_sms)
-            return fail(h, RELU_QP_ERR_UNSUPPORTED, "that many CTAs cannot be co-resident");
-    }
+    if (ctas > h->sw.max_ctas || !fits(h, ctas, cl, cached))
+        return fail(h, RELU_QP_ERR_UNSUPPORTED, cl ? "a cluster of this size cannot be resident"
+                                                   : "that many CTAs cannot be co-resident");
     h->sw.grid = ctas;
-    h->sw.cluster = cl ? cluster : 0;
+    h->sw.cluster = cl;
     h->sw.cached_rows = cached;
-    h->sw.rows_per_cta = ceil_div(h->R, ctas);
+    h->sw.gs = default_gs(h, ctas, cl);
     return RELU_QP_OK;
 }
 
+int single_update(relu_qp_t h) {
+    RQ_CUDA(h, cudaMemcpyAsync(h->q32, h->sw.pin, sizeof(float) * (h->n + 2 * (size_t)h->m), cudaMemcpyHostToDevice,
+                               h->stream));
+    return compute_bias(h);
+}
+
+void fill_info(relu_qp_t h, relu_qp_info* info) {
+    if (!info) return;
+    const SingleWork& w = h->sw;
+    float ms = 0.f;
+    cudaEventElapsedTime(&ms, h->ev0, h->ev1);
+    info->status = w.out_i[OUT_STATUS];
+    info->iters = w.out_i[OUT_ITERS];
+    info->rho_index = w.out_i[OUT_RHO];
+    info->rho_switches = w.out_i[OUT_SWITCHES];
+    info->r_prim = w.out_f[0];
+    info->r_dual = w.out_f[1];
+    info->solve_ms = ms;
+}
+
+// x_warm, lam_warm: the host's FP32 warm start (lam_warm may be nullptr: zeros).  The
+// results are in h->sw.out: x, z, lam.
 int single_solve(relu_qp_t h, const float* x_warm, const float* lam_warm, int rho_index, double eps_abs,
                  double eps_rel, int max_iter, relu_qp_info* info) {
     SingleWork& w = h->sw;
-    RQ_TRY(init_state(h, x_warm, lam_warm, rho_index));
-    RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
-    RQ_TRY(launch(h, w.grid, w.cluster, w.cached_rows, rho_index, eps_abs, eps_rel, max_iter,
-                  h->opts.check_interval, h->opts.adaptive_rho));
-    h->launches += 2;
-    RQ_CUDA(h, cudaEventRecord(h->ev1, h->stream));
-    int oi[OUT_WORDS];
-    float of[2];
-    RQ_CUDA(h, cudaMemcpyAsync(oi, w.out_i, sizeof(oi), cudaMemcpyDeviceToHost, h->stream));
-    RQ_CUDA(h, cudaMemcpyAsync(of, w.out_f, sizeof(of), cudaMemcpyDeviceToHost, h->stream));
-    RQ_CUDA(h, cudaStreamSynchronize(h->stream));
-    if (oi[OUT_ERR]) return fail(h, RELU_QP_ERR_TIMEOUT, "a barrier deadline passed in relu_qp_solve");
-    if (info) {
-        float ms = 0.f;
-        cudaEventElapsedTime(&ms, h->ev0, h->ev1);
-        info->status = oi[OUT_STATUS];
-        info->iters = oi[OUT_ITERS];
-        info->rho_index = oi[OUT_RHO];
-        info->rho_switches = oi[OUT_SWITCHES];
-        info->r_prim = of[0];
-        info->r_dual = of[1];
-        info->solve_ms = ms;
+    const size_t n = h->n, m = h->m;
+    const bool lam = x_warm && lam_warm && m > 0;
+    if (x_warm) {
+        std::memcpy(w.pin_in, x_warm, sizeof(float) * n);
+        if (lam) std::memcpy(w.pin_in + n, lam_warm, sizeof(float) * m);
+        RQ_CUDA(h, cudaMemcpyAsync(w.in, w.pin_in, sizeof(float) * (n + (lam ? m : 0)), cudaMemcpyHostToDevice, h->stream));
     }
+    RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
+    RQ_TRY(launch(h, w.grid, w.cluster, w.cached_rows, w.gs, x_warm ? w.in : nullptr, lam ? w.in + n : nullptr, rho_index, eps_abs,
+                  eps_rel, max_iter, h->opts.check_interval, h->opts.adaptive_rho));
+    h->launches += 1;
+    RQ_CUDA(h, cudaEventRecord(h->ev1, h->stream));
+    RQ_CUDA(h, cudaStreamSynchronize(h->stream));
+    RQ_TRY(finish(h, "in relu_qp_solve"));
+    fill_info(h, info);
     return RELU_QP_OK;
 }
 
@@ -804,8 +1128,8 @@ int single_solve(relu_qp_t h, const float* x_warm, const float* lam_warm, int rh
 // ---------------------------------------------------------------------------
 namespace {
 
-// 3 * ldw + ldp + 6 * ldt + 64 words for n + m <= kNoAllocMaxRows (see
-// noalloc_words); 49152 floats = 192 KiB.
+// the grid form's exchange words for n + m <= kNoAllocMaxRows and the error word; 49152
+// floats = 192 KiB.
 constexpr int kNoAllocMaxRows = 4096;
 constexpr size_t kNoAllocWords = 49152;
 static __device__ __align__(256) float g_noalloc_scratch[kNoAllocWords];
@@ -813,8 +1137,6 @@ static __device__ __align__(256) float g_noalloc_scratch[kNoAllocWords];
 constexpr int kMaxDevices = 64;
 float* g_noalloc_ptr[kMaxDevices] = {};
 std::mutex g_noalloc_mutex;
-
-size_t noalloc_words(int ldw, int ldp, int ldt) { return 3 * (size_t)ldw + ldp + 6 * (size_t)ldt + 64; }
 
 // Device address of the array on the handle's device, looked up once per
 // device (a host-side use of the symbol itself would not be a device address).
@@ -866,9 +1188,8 @@ int noalloc_check_ptr(relu_qp_t h, const void* ptr, const char* name) {
 int single_solve_noalloc(relu_qp_t h, const float* x_warm, const float* lam_warm, int rho_index, double eps_abs,
                          double eps_rel, int max_iter, float* x_out, float* z_out, float* lam_out,
                          relu_qp_info* info) {
-    const int n = h->n, m = h->m;
-    const int ldp = (int)round_up(n, 4), ldt = (int)round_up(m > 0 ? m : 1, 4), ldw = h->ldw;
-    if (h->R > kNoAllocMaxRows || noalloc_words(ldw, ldp, ldt) > kNoAllocWords)
+    const size_t words = exchange_words(h, h->sw.max_ctas);
+    if (h->R > kNoAllocMaxRows || 2 * words + 4 > kNoAllocWords)
         return fail(h, RELU_QP_ERR_INVALID, "relu_qp_solve_noalloc supports n + m <= " +
                                                 std::to_string(kNoAllocMaxRows) + " (fixed scratch of " +
                                                 std::to_string(kNoAllocWords * 4 / 1024) + " KiB)");
@@ -879,70 +1200,33 @@ int single_solve_noalloc(relu_qp_t h, const float* x_warm, const float* lam_warm
     RQ_TRY(noalloc_check_ptr(h, lam_out, "lam_out"));
     float* base = nullptr;
     RQ_TRY(noalloc_scratch(h, &base));
-    // carve the scratch: vectors first (16-byte aligned offsets), then the words
-    float* y = base;
-    float* s0 = y + ldw;
-    float* s1 = s0 + ldw;
-    float* Py = s1 + ldw;
-    float* z = Py + ldp;
-    float* lam = z + ldt;
-    float* Ay = lam + ldt;
-    float* Axf = Ay + ldt;
-    float* lstd = Axf + ldt;
-    float* spare = lstd + ldt;            // ldt floats, unused
-    unsigned* red = reinterpret_cast<unsigned*>(spare + ldt);   // 3 x 8 words
-    unsigned* bar = red + 3 * RED_WORDS;                        // 2 words (+6 pad)
-    int* out_i = reinterpret_cast<int*>(bar + 8);               // OUT_WORDS
-    float* out_f = reinterpret_cast<float*>(out_i + OUT_WORDS); // 8 words
+    SingleWork& w = h->sw;
     SP p{};
-    fill_params(h, p, h->sw.grid);
-    p.y = y; p.z = z; p.lam = lam; p.Ay = Ay; p.s0 = s0; p.s1 = s1;
-    p.Py = Py; p.Axf = Axf; p.lstd = lstd;
-    p.red = red; p.bar = bar; p.out_i = out_i; p.out_f = out_f;
-    p.cached_rows = h->sw.cached_rows;
+    fill_params(h, p, w.grid, w.cluster, w.gs, w.cached_rows);
+    set_words(h, p, reinterpret_cast<unsigned long long*>(base));
+    p.err = reinterpret_cast<int*>(base + 2 * words);
     p.rho_index0 = rho_index;
     p.check_interval = h->opts.check_interval;
     p.adaptive = h->opts.adaptive_rho;
     p.max_iter = max_iter;
     p.eps_abs = eps_abs;
     p.eps_rel = eps_rel;
-    p.qnorm = h->qnorm;
-    p.rsx = h->sc_rx;
-    p.rsz = h->sc_z;
-    // parts that must start at zero: x and lam_std padding (read as whole
-    // padded vectors by the check), reduction slots, barrier and result words
-    RQ_CUDA(h, cudaMemsetAsync(y, 0, sizeof(float) * ldw, h->stream));
-    RQ_CUDA(h, cudaMemsetAsync(lstd, 0, sizeof(float) * ldt, h->stream));
-    RQ_CUDA(h, cudaMemsetAsync(red, 0, sizeof(unsigned) * (3 * RED_WORDS + 8) + sizeof(int) * OUT_WORDS +
-                                           sizeof(float) * 8, h->stream));
-    const int blocks = ceil_div(ldw * 32, 256) < 1024 ? ceil_div(ldw * 32, 256) : 1024;
-    init_state_kernel<<<blocks, 256, 0, h->stream>>>(n, m, ldp, ldw, h->A32, x_warm, lam_warm, h->rs32,
-                                                      h->be[rho_index].rho, y, z, lam, Ay, s0, s1);
-    RQ_CUDA(h, cudaGetLastError());
+    p.xin = x_warm;
+    p.lin = lam_warm;
+    p.xo = x_out;
+    p.zo = h->m > 0 ? z_out : nullptr;
+    p.lo = h->m > 0 ? lam_out : nullptr;
+    p.tag0 = 0;                    // the words start at zero: other handles leave theirs in the array
+    p.out_i = w.out_i;
+    p.out_f = w.out_f;
+    w.out_i[OUT_LAST] = -1;
+    RQ_CUDA(h, cudaMemsetAsync(base, 0, sizeof(float) * (2 * words + 4), h->stream));
     RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
-    RQ_TRY(launch_kernel(h, p, h->sw.grid, h->sw.cluster, p.cached_rows));
+    RQ_TRY(launch_kernel(h, p, w.grid, w.cluster));
     RQ_CUDA(h, cudaEventRecord(h->ev1, h->stream));
-    RQ_CUDA(h, cudaMemcpyAsync(x_out, y, sizeof(float) * n, cudaMemcpyDeviceToDevice, h->stream));
-    if (z_out && m > 0) RQ_CUDA(h, cudaMemcpyAsync(z_out, z, sizeof(float) * m, cudaMemcpyDeviceToDevice, h->stream));
-    if (lam_out && m > 0)
-        RQ_CUDA(h, cudaMemcpyAsync(lam_out, lstd, sizeof(float) * m, cudaMemcpyDeviceToDevice, h->stream));
-    int oi[OUT_WORDS];
-    float of[2];
-    RQ_CUDA(h, cudaMemcpyAsync(oi, out_i, sizeof(oi), cudaMemcpyDeviceToHost, h->stream));
-    RQ_CUDA(h, cudaMemcpyAsync(of, out_f, sizeof(of), cudaMemcpyDeviceToHost, h->stream));
     RQ_CUDA(h, cudaStreamSynchronize(h->stream));
-    if (oi[OUT_ERR]) return fail(h, RELU_QP_ERR_TIMEOUT, "a barrier deadline passed in relu_qp_solve_noalloc");
-    if (info) {
-        float ms = 0.f;
-        cudaEventElapsedTime(&ms, h->ev0, h->ev1);
-        info->status = oi[OUT_STATUS];
-        info->iters = oi[OUT_ITERS];
-        info->rho_index = oi[OUT_RHO];
-        info->rho_switches = oi[OUT_SWITCHES];
-        info->r_prim = of[0];
-        info->r_dual = of[1];
-        info->solve_ms = ms;
-    }
+    if (w.out_i[OUT_LAST] < 0) return fail(h, RELU_QP_ERR_TIMEOUT, "a wait passed its deadline in relu_qp_solve_noalloc");
+    fill_info(h, info);
     return RELU_QP_OK;
 }
 

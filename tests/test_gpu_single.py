@@ -280,3 +280,55 @@ def test_update_rejects_changed_equality_pattern(rq):
         s.update(l=l2)
     assert e.value.kind == "INVALID"
     s.close()
+
+
+@pytest.mark.parametrize("dims", [(1, 0, 0, 0), (2, 3, 0, 0), (5, 11, 1, 2), (31, 2, 0, 0), (40, 40, 0, 0), (63, 130, 7, 9),
+                                  (257, 33, 0, 0)])
+def test_every_launch_shape_on_ragged_sizes(rq, dims):
+    """Rows that do not divide over the CTAs, fewer rows of a kind than CTAs, n off a multiple of
+    4, check intervals of 1 and none: every shape gives the bits of one CTA, and fixed layers
+    match the oracle's iterates to 1e-5."""
+    P, q, A, l, u = random_qp(5, *dims)
+    n, m = dims[:2]
+    rng = np.random.default_rng(2)
+    xw, lw = rng.standard_normal(n), rng.standard_normal(m)
+    for ci in (0, 1, 25):
+        s = rq.ReluQP(P, A if m else None, l, u, q=q, sigma=SIGMA, rho_bank=BANK, check_interval=ci)
+        ref = None
+        for ctas, cluster in [(1, 0), (2, 0), (3, 0), (17, 0), (152, 0), (2, 2), (4, 4), (8, 8), (16, 16)]:
+            if ctas > n + m:
+                continue
+            try:
+                s.set_single_config(ctas, cluster)
+            except rq.ReluQPError as e:
+                assert e.code == -6, e
+                continue
+            outs = [s.solve(eps_abs=0.0, max_iter=30), s.solve(x_warm=xw, lam_warm=lw, rho_index=1, eps_abs=1e-4, max_iter=120)]
+            if ref is None:
+                ref = outs
+                if ci == 0:
+                    v = O.layer_iterates(P, q, A, l, u, SIGMA, BANK[0], 30)[-1]
+                    assert rel(np.concatenate([outs[0]["x"], outs[0]["z"]]), v[:n + m]) <= 1e-5
+            for a, b in zip(outs, ref):
+                assert (a["iters"], a["rho_index"], a["status"]) == (b["iters"], b["rho_index"], b["status"]), (ctas, cluster)
+                for k in ("x", "z", "lam"):
+                    assert np.array_equal(a[k], b[k]), (ci, ctas, cluster, k)
+        s.close()
+
+
+def test_operand_larger_than_both_staged_vectors(rq):
+    """n + m above 32768: lam_std is staged over the operand, which is read again after a check."""
+    n, m = 100, 32720
+    rng = np.random.default_rng(8)
+    M = rng.standard_normal((n, n))
+    P = M @ M.T / n + 0.5 * np.eye(n)
+    A = rng.standard_normal((m, n)) / np.sqrt(n)
+    q = 2.0 * rng.standard_normal(n)
+    l, u = -np.ones(m), np.ones(m)
+    s = rq.ReluQP(P, A, l, u, q=q, sigma=SIGMA, rho_bank=(0.01, 0.1))
+    o = s.solve(eps_abs=1e-3, max_iter=4000)
+    s.close()
+    assert o["status"] == rq.SOLVED and o["iters"] > 25
+    assert np.max(np.abs(A @ o["x"] - o["z"])) <= 1e-3 * RES_SLACK
+    assert np.max(np.abs(P @ o["x"] + q + A.T @ o["lam"])) <= 1e-3 * RES_SLACK
+    assert np.all(o["z"] >= l - 1e-6) and np.all(o["z"] <= u + 1e-6)
