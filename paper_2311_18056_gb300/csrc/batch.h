@@ -485,6 +485,10 @@ __device__ __forceinline__ int decide_qp(const BatchParams& p, const DecideArgs&
     return x.act;
 }
 
+// refined-layer configuration: K split over a cluster of ks CTAs, tile width bn
+struct LayerCfg {
+    int ks, bn;
+};
 // --- entry points of the tcgen05 backend (batch_tc.cu) ---------------------
 int tc_prepare(relu_qp_t h);                     // BF16 splits of every W_rho and of [P | A^T]
 // operand_set < 0: accurate (3-way) layer; pdl: programmatic dependent launch on the
@@ -499,6 +503,7 @@ int tc_check(relu_qp_t h, const BatchParams& p, int phase, int tiles, int active
 // layers one by one.
 int tc_chunk(relu_qp_t h, const BatchParams& p, int nl, unsigned last_flags, int active_tiles);
 void tc_disable_chunk(relu_qp_t h);
+bool tc_chunk_fits(relu_qp_t h, LayerCfg c, int active_tiles);   // whether tc_chunk runs this configuration
 // Resident-weight chunk kernel (one slot tile of at most 64 active QPs, the
 // layer's rows of Wt kept in shared memory over a cluster of 8 CTAs that
 // split k): refined layers 1 .. nl of a chunk, as tc_chunk.
@@ -509,10 +514,6 @@ int tc_small(relu_qp_t h, const BatchParams& p, int nl, unsigned last_flags, int
 void tc_small_set(relu_qp_t h, bool use);   // use it where eligible (set by the tuner)
 bool tc_small_chosen(relu_qp_t h);
 void tc_release(relu_qp_t h);
-// refined-layer configuration: K split over a cluster of ks CTAs, tile width bn
-struct LayerCfg {
-    int ks, bn;
-};
 int tc_layer_cfgs(relu_qp_t h, std::vector<LayerCfg>& out);          // every configuration the problem allows
 int tc_set_layer_cfg(relu_qp_t h, LayerCfg c);                        // one for every tile count
 int tc_set_layer_table(relu_qp_t h, const std::vector<LayerCfg>& by_tiles);  // [t] = for t active slot tiles

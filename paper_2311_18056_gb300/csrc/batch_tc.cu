@@ -1876,16 +1876,21 @@ int tc_layer(relu_qp_t h, const BatchParams& p, int operand_set, int tiles, int 
     return dispatch_refined(h, c.bn, c.ks, st->wb_map, p, g, st->opnd_map, tiles, pdl);
 }
 
+bool tc_chunk_fits(relu_qp_t h, LayerCfg c, int active_tiles) {
+    const BatchWork& w = h->bw;
+    // all CTAs of the active tiles co-resident, one per SM
+    return w.chunk_sync && static_cast<const TcState*>(w.tc)->chunk_ok && chunk_has(c.ks, c.bn) &&
+           (long long)c.ks * ceil_div(w.RP, c.bn) * std::min(active_tiles, w.slots / kSlotTile) <= h->num_sms;
+}
+
 int tc_chunk(relu_qp_t h, const BatchParams& p, int nl, unsigned last_flags, int active_tiles) {
     BatchWork& w = h->bw;
     TcState* st = static_cast<TcState*>(w.tc);
     if (!st->chunk_ok || nl < 1 || active_tiles < 1) return RELU_QP_ERR_UNSUPPORTED;
     const LayerCfg lc = cfg_for(st, active_tiles);
     const int bn = lc.bn;
-    if (!chunk_has(lc.ks, bn)) return RELU_QP_ERR_UNSUPPORTED;
+    if (!tc_chunk_fits(h, lc, active_tiles)) return RELU_QP_ERR_UNSUPPORTED;
     const int tiles_y = std::min(active_tiles, w.slots / kSlotTile);
-    // all CTAs of the active tiles co-resident, one per SM
-    if ((long long)lc.ks * ceil_div(w.RP, bn) * tiles_y > h->num_sms) return RELU_QP_ERR_UNSUPPORTED;
     TcArgs g{};
     g.num_kb = w.ldk / kBK;
     g.rows = w.RP;

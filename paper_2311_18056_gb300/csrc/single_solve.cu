@@ -48,6 +48,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <functional>
 #include <mutex>
 
 namespace rq {
@@ -1001,7 +1002,7 @@ int single_prepare(relu_qp_t h) {
     SingleWork& w = h->sw;
     w.grid = 0;
     float best_t = 1e30f;
-    auto time = [&](int g, int cl, int cached, int gs) -> int {
+    auto time = [&](int g, int cl, int cached, int gs, float* out) -> int {
         float ms = 0.f;
         for (int layers : {10, 50}) {   // a warm-up, then the timed run
             RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
@@ -1018,24 +1019,33 @@ int single_prepare(relu_qp_t h) {
             w.cached_rows = cached;
             w.gs = gs;
         }
+        *out = ms;
         return RELU_QP_OK;
     };
-    // candidates: (CTAs, cluster); cluster > 1 = one cluster of that many CTAs
-    std::vector<std::pair<int, int>> cands;
-    for (int g = 1; g <= 4 * h->num_sms; g *= 2) cands.push_back({g, 0});
-    cands.push_back({h->num_sms, 0});
-    for (int c = 2; c <= 16; c *= 2) cands.push_back({c, c});
-    for (const auto& gc : cands) {
-        const int g = gc.first, cl = gc.second;
-        if (g > h->R) continue;
-        const int cached = cached_rows_for(h, g, cl);
-        if (fits(h, g, cl, cached)) RQ_TRY(time(g, cl, cached, default_gs(h, g, cl)));
+    // Grids, then clusters, the largest first.  The time falls, if at all, to one minimum and
+    // then rises with the rows per CTA, so a family ends at the first shape 1.3x slower than its
+    // best (a small grid or cluster of a large problem takes 100 times the best: 25 ms of the
+    // setup at n = m = 800).
+    std::vector<int> grids{h->num_sms}, clusters{16, 8, 4, 2};
+    for (int g = 1; g <= 4 * h->num_sms; g *= 2) grids.push_back(g);
+    std::sort(grids.begin(), grids.end(), std::greater<int>());
+    for (const bool cl : {false, true}) {
+        float family = 1e30f;
+        for (int c : cl ? clusters : grids) {
+            const int cached = c <= h->R ? cached_rows_for(h, c, cl ? c : 0) : -1;
+            if (!fits(h, c, cl ? c : 0, cached)) continue;
+            float ms = 0.f;
+            RQ_TRY(time(c, cl ? c : 0, cached, default_gs(h, c, cl ? c : 0), &ms));
+            if (ms > 1.3f * family || ms > 3.0f * best_t) break;
+            family = std::min(family, ms);
+        }
     }
     if (w.grid == 0) return fail(h, RELU_QP_ERR_UNSUPPORTED, "the single-QP solve does not fit on an SM");
     if (w.cluster <= 1) {
         const int g = w.grid, cached = w.cached_rows, gs0 = w.gs;
+        float ms;
         for (int gs : {1, 2, 4})
-            if (gs != gs0) RQ_TRY(time(g, 0, cached, gs));
+            if (gs != gs0) RQ_TRY(time(g, 0, cached, gs, &ms));
     }
     return RELU_QP_OK;
 }
