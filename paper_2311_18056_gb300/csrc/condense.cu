@@ -123,26 +123,34 @@ __global__ void prefix_kernel(const double* __restrict__ Y, const double* __rest
 }
 
 // Winv = (I + W)^{-1} (n x n, n <= kGaussMax) in one CTA: in-place Gauss-Jordan
-// elimination with row pivoting in shared memory.  Bound by the FP64 pipe of one SM
-// (n^3 FMAs at two a clock: 52 us at n = 60) and the barriers of n steps; a singular
-// matrix leaves infinities or NaN, which the caller's convergence test sees.
+// elimination with row pivoting in shared memory.  A thread keeps its column (j = lane +
+// 32 c) while it walks down the rows, so an element costs two shared reads, an FMA and a
+// store; rows are exchanged by name (piv) and moved once at the end.  Bound by the FP64
+// pipe of one SM (n^3 FMAs at two a clock, 52 us at n = 60) and three barriers a step.
+// (226 us a call at n = 60; 279 with a division per element for its row and column.)  A singular matrix
+// leaves infinities or NaN, which the caller's convergence test sees.
 constexpr int kGaussMax = 160;
 constexpr int kGaussThreads = 512;
 
 __global__ void __launch_bounds__(kGaussThreads) gauss_inverse_kernel(const double* __restrict__ W, int n,
                                                                       double* __restrict__ Winv) {
     extern __shared__ double gsm[];
-    __shared__ double col[kGaussMax];
-    __shared__ int piv[kGaussMax];
-    const int ld = n | 1, tid = threadIdx.x;
-    for (int e = tid; e < n * n; e += kGaussThreads) gsm[(e / n) * ld + e % n] = W[e] + (e / n == e % n ? 1.0 : 0.0);
+    __shared__ double col[kGaussMax], row[kGaussMax];
+    __shared__ int piv[kGaussMax], used[kGaussMax];   // step k's row; whether a row has been one
+    __shared__ double s_inv;
+    const int ld = n | 1, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int kW = kGaussThreads / 32;
+    for (int i = warp; i < n; i += kW)
+        for (int j = lane; j < n; j += 32) gsm[i * ld + j] = W[(size_t)i * n + j] + (i == j ? 1.0 : 0.0);
+    for (int i = tid; i < n; i += kGaussThreads) used[i] = 0;
     __syncthreads();
     for (int k = 0; k < n; ++k) {
-        if (tid < 32) {
+        if (warp == 0) {
+            // the largest element of column k among the rows not used yet (the first of equals)
             double best = -1.0;
-            int at = k;
-            for (int i = k + tid; i < n; i += 32) {
-                const double v = fabs(gsm[i * ld + k]);
+            int at = n;
+            for (int i = lane; i < n; i += 32) {
+                const double v = used[i] ? -1.0 : fabs(gsm[i * ld + k]);
                 if (v > best) {
                     best = v;
                     at = i;
@@ -156,45 +164,38 @@ __global__ void __launch_bounds__(kGaussThreads) gauss_inverse_kernel(const doub
                     at = a;
                 }
             }
-            if (tid == 0) piv[k] = at;
+            if (at >= n) {   // only NaN left: any unused row
+                at = 0;
+                while (at < n - 1 && used[at]) ++at;
+            }
+            if (lane == 0) {
+                piv[k] = at;
+                used[at] = 1;
+                s_inv = 1.0 / gsm[at * ld + k];
+            }
         }
         __syncthreads();
         const int p = piv[k];
-        for (int j = tid; j < n; j += kGaussThreads) {
-            const double v = gsm[p * ld + j];
-            if (p != k) {
-                gsm[p * ld + j] = gsm[k * ld + j];
-                gsm[k * ld + j] = v;
+        const double inv = s_inv;
+        // minus column k, and row p times the inverse pivot
+        if (tid < kGaussThreads / 2) {
+            for (int i = tid; i < n; i += kGaussThreads / 2) col[i] = -gsm[i * ld + k];
+        } else {
+            for (int j = tid - kGaussThreads / 2; j < n; j += kGaussThreads / 2) row[j] = j == k ? inv : gsm[p * ld + j] * inv;
+        }
+        __syncthreads();
+        for (int j = lane; j < n; j += 32) {
+            const double r = row[j];
+            for (int i = warp; i < n; i += kW) {
+                double* w = gsm + i * ld + j;
+                *w = i == p ? r : j == k ? col[i] * inv : fma(col[i], r, *w);
             }
         }
         __syncthreads();
-        const double inv = 1.0 / gsm[k * ld + k];
-        for (int i = tid; i < n; i += kGaussThreads) col[i] = i == k ? 0.0 : gsm[i * ld + k];
-        __syncthreads();
-        for (int j = tid; j < n; j += kGaussThreads) gsm[k * ld + j] = j == k ? inv : gsm[k * ld + j] * inv;
-        __syncthreads();
-        for (int e = tid; e < n * n; e += kGaussThreads) {
-            const int i = e / n, j = e % n;
-            if (i == k) continue;
-            double* w = gsm + i * ld + j;
-            *w = j == k ? -col[i] * inv : fma(-col[i], gsm[k * ld + j], *w);
-        }
-        __syncthreads();
     }
-    // the row exchanges, undone as column exchanges in reverse
-    for (int i = tid; i < n; i += kGaussThreads) {
-        double* w = gsm + i * ld;
-        for (int k = n - 1; k >= 0; --k) {
-            const int p = piv[k];
-            if (p != k) {
-                const double t = w[k];
-                w[k] = w[p];
-                w[p] = t;
-            }
-        }
-    }
-    __syncthreads();
-    for (int e = tid; e < n * n; e += kGaussThreads) Winv[e] = gsm[(e / n) * ld + e % n];
+    // step k worked on row piv[k] and column k: element (piv[i], j) is the inverse's (i, piv[j])
+    for (int i = warp; i < n; i += kW)
+        for (int j = lane; j < n; j += 32) Winv[(size_t)i * n + piv[j]] = gsm[piv[i] * ld + j];
 }
 
 // X <- (X + X^T) / 2 (n x n, rows of ld) and, with red, the convergence measures of a
