@@ -319,12 +319,11 @@ class ReluQP:
                                               xo, zo, lo, inf))
         res = {"x": out[0], "z": out[1], "lam": out[2]}
         if infos:
-            res["status"] = np.array([i.status for i in inf])
-            res["iters"] = np.array([i.iters for i in inf])
-            res["rho_index"] = np.array([i.rho_index for i in inf])
-            res["rho_switches"] = np.array([i.rho_switches for i in inf])
-            res["r_prim"] = np.array([i.r_prim for i in inf])
-            res["r_dual"] = np.array([i.r_dual for i in inf])
+            rec = np.frombuffer(inf, dtype=np.dtype(Info))
+            for k in ("status", "iters", "rho_index", "rho_switches"):
+                res[k] = rec[k].astype(np.int64)
+            for k in ("r_prim", "r_dual"):
+                res[k] = rec[k].copy()
             res["solve_ms"] = inf[0].solve_ms if B else 0.0
         return res
 

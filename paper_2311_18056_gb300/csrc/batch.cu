@@ -40,54 +40,94 @@ struct W32Ptrs {
     const float* w[RQ_MAX_RHO];
 };
 
-// C[i][j'] = alpha * sum_k X[i][k] W[j][k] + (off ? off[j] : 0), bounds-checked
-// (problem updates; not on the per-layer path); j' = j, or j + shift from j = split on
-// (rows of a layer into its padded layout).
-__global__ void __launch_bounds__(256) sgemm_nt_kernel(int M, int N, int K, const float* __restrict__ X, int ldx,
-                                                       const float* __restrict__ W, int ldw, float alpha,
-                                                       const float* __restrict__ off, float* __restrict__ C,
-                                                       int ldc, int split, int shift) {
+// Problem updates: up to kMaps products of one X (M x K) with different W (N x K) in one
+// launch, C[i][j'] = alpha * sum_k X[i][k] W[j][k] + (off ? off[j] : 0), with a second result
+// C2 of the same sums and its own offsets (l and u), and j' = j, or j + shift from
+// j = split on (rows of a layer into its padded layout).  Every sum runs over k in order.
+// One update is 3 + n_rho maps of a few microseconds each (at 250 QPs, nx = 70: seven
+// launches, 173 us, when each was a kernel of 16 to 25 tiles): together they fill the SMs.
+// Rows and columns in 64 x 64 tiles, 4 x 4 outputs a thread; the next 16 columns of k are
+// loaded into registers while the current ones are multiplied.
+constexpr int kMaps = RQ_MAX_RHO + 4;
+
+struct MapTask {
+    const float* W;
+    const float *off, *off2;
+    float *C, *C2;
+    int N, ldw, ldc, split, shift, tile0;   // tile0: first column tile of the launch
+    float alpha;
+};
+
+struct MapTasks {
+    MapTask t[kMaps];
+    int count;
+};
+
+__global__ void __launch_bounds__(256) map_kernel(int M, int K, const float* __restrict__ X, int ldx, const MapTasks ts) {
     __shared__ float Xs[16][64 + 4];
     __shared__ float Ws[16][64 + 4];
+    int a = 0;
+    while (a + 1 < ts.count && (int)blockIdx.x >= ts.t[a + 1].tile0) ++a;
+    const MapTask& T = ts.t[a];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int i0 = blockIdx.y * 64, j0 = blockIdx.x * 64;
+    const int i0 = blockIdx.y * 64, j0 = (blockIdx.x - T.tile0) * 64;
+    const int lr = threadIdx.x >> 2, lk = (threadIdx.x & 3) * 4;   // this thread loads 4 columns of one row of each
+    const int gi = i0 + lr, gj = j0 + lr;
+    const bool vx = (ldx & 3) == 0 && gi < M, vw = (T.ldw & 3) == 0 && gj < T.N;
+    float xr[4], wr[4];
+    auto fetch4 = [&](const float* row, bool vec, bool in, int k, float (&v)[4]) {
+        if (vec && k + 4 <= K) {
+            const float4 q = *reinterpret_cast<const float4*>(row + k);
+            v[0] = q.x;
+            v[1] = q.y;
+            v[2] = q.z;
+            v[3] = q.w;
+        } else {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = in && k + u < K ? row[k + u] : 0.f;
+        }
+    };
+    auto fetch = [&](int k0) {
+        fetch4(X + (size_t)gi * ldx, vx, gi < M, k0 + lk, xr);
+        fetch4(T.W + (size_t)gj * T.ldw, vw, gj < T.N, k0 + lk, wr);
+    };
     float acc[4][4];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
+        for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
+    fetch(0);
     for (int k0 = 0; k0 < K; k0 += 16) {
-        for (int e = threadIdx.x; e < 1024; e += 256) {
-            const int row = e >> 4, k = e & 15;
-            const int gi = i0 + row, gj = j0 + row, gk = k0 + k;
-            Xs[k][row] = (gi < M && gk < K) ? X[(size_t)gi * ldx + gk] : 0.f;
-            Ws[k][row] = (gj < N && gk < K) ? W[(size_t)gj * ldw + gk] : 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            Xs[lk + u][lr] = xr[u];
+            Ws[lk + u][lr] = wr[u];
         }
         __syncthreads();
+        if (k0 + 16 < K) fetch(k0 + 16);
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
-            float a[4], b[4];
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                a[t] = Xs[k][ty + 16 * t];
-                b[t] = Ws[k][tx + 16 * t];
-            }
+            const float4 x = *reinterpret_cast<const float4*>(&Xs[k][ty * 4]);
+            const float4 w = *reinterpret_cast<const float4*>(&Ws[k][tx * 4]);
+            const float xa[4] = {x.x, x.y, x.z, x.w}, wa[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
             for (int u = 0; u < 4; ++u)
 #pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
+                for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(xa[u], wa[v], acc[u][v]);
         }
         __syncthreads();
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        const int i = i0 + ty + 16 * u;
+        const int i = i0 + ty * 4 + u;
         if (i >= M) continue;
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            const int j = j0 + tx + 16 * v;
-            if (j >= N) continue;
-            C[(size_t)i * ldc + j + (j >= split ? shift : 0)] = alpha * acc[u][v] + (off ? off[j] : 0.f);
+            const int j = j0 + tx * 4 + v;
+            if (j >= T.N) continue;
+            const size_t o = (size_t)i * T.ldc + j + (j >= T.split ? T.shift : 0);
+            T.C[o] = T.alpha * acc[u][v] + (T.off ? T.off[j] : 0.f);
+            if (T.C2) T.C2[o] = T.alpha * acc[u][v] + T.off2[j];
         }
     }
 }
@@ -455,28 +495,46 @@ __global__ void batch_fill_kernel(BatchParams p, const int* __restrict__ rho_idx
 
 // Start state per QP: x given (Y) or 0, z = A x (AY holds A x for warm starts),
 // lam' = lam_warm (staged in LSTD) or 0.
-__global__ void batch_init_kernel(BatchParams p, int B, int warm, int lam_given, const int* __restrict__ rw,
-                                  int rho0, int* status, int* rho_idx, int* iters, int* nsw) {
-    const int qp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (qp >= p.cap) return;
-    if (lane == 0) {
+// One block per QP.
+constexpr int kInitThreads = 128;
+__global__ void __launch_bounds__(kInitThreads) batch_init_kernel(BatchParams p, int B, int warm, int lam_given,
+                                                                  const int* __restrict__ rw, int rho0, int* status,
+                                                                  int* rho_idx, int* iters, int* nsw) {
+    const int qp = blockIdx.x, tid = threadIdx.x;
+    if (tid == 0) {
         status[qp] = qp < B ? QP_ACTIVE : QP_UNUSED;
-        rho_idx[qp] = (qp < B && rw) ? rw[qp] : rho0;
+        rho_idx[qp] = (qp < B && rw) ? rw[qp] : rho0;   // (rw may be iters: read first)
         iters[qp] = 0;
         nsw[qp] = 0;
     }
-    if (lane < RW_WORDS) p.RED[(size_t)qp * RW_WORDS + lane] = 0u;
+    if (tid < RW_WORDS) p.RED[(size_t)qp * RW_WORDS + tid] = 0u;
     if (qp >= B) return;
     // (the padding is zeroed too: a QP of NaN data leaves NaN there)
-    for (int i = lane; i < p.ldm; i += 32) {
+    for (int i = tid; i < p.ldm; i += kInitThreads) {
         const size_t o = (size_t)qp * p.ldm + i;
         const float ax = warm && i < p.m ? p.AY[o] : 0.f;
         p.AY[o] = ax;
         p.Z[o] = ax;
         p.LAM[o] = lam_given && i < p.m ? p.LSTD[o] : 0.f;
     }
-    for (int k = (warm ? p.n : 0) + lane; k < p.ldn; k += 32) p.Y[(size_t)qp * p.ldn + k] = 0.f;
+    for (int k = (warm ? p.n : 0) + tid; k < p.ldn; k += kInitThreads) p.Y[(size_t)qp * p.ldn + k] = 0.f;
+}
+
+// The solve's records as the caller's relu_qp_info (solve_ms is the host's).
+__global__ void pack_info_kernel(int B, const int* __restrict__ status, const int* __restrict__ iters,
+                                 const int* __restrict__ rho_idx, const int* __restrict__ nsw,
+                                 const float* __restrict__ rp, const float* __restrict__ rd, relu_qp_info* out) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b >= B) return;
+    relu_qp_info r;
+    r.status = status[b];
+    r.iters = iters[b];
+    r.rho_index = rho_idx[b];
+    r.rho_switches = nsw[b];
+    r.r_prim = rp[b];
+    r.r_dual = rd[b];
+    r.solve_ms = 0.0;
+    out[b] = r;
 }
 
 // out[r] = max_k |X[r][k] f[k]| (f = nullptr: 1).
@@ -521,15 +579,24 @@ __global__ void build_wc32_kernel(const float* __restrict__ P32, const float* __
     }
 }
 
-int sgemm_nt(relu_qp_t h, int M, int N, int K, const float* X, int ldx, const float* W, int ldw, float alpha,
-             const float* off, float* C, int ldc, int split = 0, int shift = 0) {
-    if (M <= 0 || N <= 0) return RELU_QP_OK;
-    dim3 grid(ceil_div(N, 64), ceil_div(M, 64));
-    sgemm_nt_kernel<<<grid, 256, 0, h->stream>>>(M, N, K, X, ldx, W, ldw, alpha, off, C, ldc, split, shift);
-    RQ_CUDA(h, cudaGetLastError());
-    ++h->launches;
-    return RELU_QP_OK;
-}
+// The maps of one X, gathered and launched together.
+struct Maps {
+    MapTasks ts{};
+    int tiles = 0;
+    void add(int N, const float* W, int ldw, float alpha, const float* off, float* C, int ldc, int split = 0, int shift = 0,
+             const float* off2 = nullptr, float* C2 = nullptr) {
+        if (N <= 0) return;
+        ts.t[ts.count++] = MapTask{W, off, off2, C, C2, N, ldw, ldc, split, shift, tiles, alpha};
+        tiles += ceil_div(N, 64);
+    }
+    int run(relu_qp_t h, int M, int K, const float* X, int ldx) const {
+        if (M <= 0 || ts.count == 0) return RELU_QP_OK;
+        map_kernel<<<dim3(tiles, ceil_div(M, 64)), 256, 0, h->stream>>>(M, K, X, ldx, ts);
+        RQ_CUDA(h, cudaGetLastError());
+        ++h->launches;
+        return RELU_QP_OK;
+    }
+};
 
 BatchParams base_params(relu_qp_t h) {
     BatchWork& w = h->bw;
@@ -550,7 +617,6 @@ BatchParams base_params(relu_qp_t h) {
     for (int r = 0; r < h->nr; ++r) {
         p.rho[r] = (float)h->be[r].rho;
         p.rhod[r] = h->be[r].rho;
-        p.logrho[r] = std::log(h->be[r].rho);
     }
     p.rs = h->rs32;
     p.rsx = h->sc_rx;
@@ -674,6 +740,7 @@ int batch_alloc(relu_qp_t h) {
     }
     RQ_TRY(batch_tail_alloc(h));
     RQ_CUDA(h, cudaMallocHost(reinterpret_cast<void**>(&w.cnt_host), sizeof(int) * CNT_WORDS));
+    RQ_CUDA(h, cudaMallocHost(reinterpret_cast<void**>(&w.info_host), sizeof(relu_qp_info) * cap));
     RQ_CUDA(h, cudaEventCreateWithFlags(&w.ev_cnt, cudaEventDisableTiming));
     return RELU_QP_OK;
 }
@@ -826,7 +893,9 @@ void batch_release(relu_qp_t h) {
     if (h->bw.tc) tc_release(h);
     if (h->bw.cnt_host) cudaFreeHost(h->bw.cnt_host);
     if (h->bw.ev_cnt) cudaEventDestroy(h->bw.ev_cnt);
+    if (h->bw.info_host) cudaFreeHost(h->bw.info_host);
     h->bw.cnt_host = nullptr;
+    h->bw.info_host = nullptr;
     h->bw.ev_cnt = nullptr;
 }
 
@@ -858,9 +927,10 @@ int batch_update(relu_qp_t h, int B, const float* Q, const float* L, const float
     if (L && m > 0) RQ_TRY(scale_rows(h, w.L, B, m, w.ldm, h->sc_e));
     if (U && m > 0) RQ_TRY(scale_rows(h, w.U, B, m, w.ldm, h->sc_e));
     if (Q) {
+        Maps maps;
         for (int r = 0; r < h->nr; ++r)
-            RQ_TRY(sgemm_nt(h, B, R, n, w.Q, w.ldn, h->be[r].Bop, n, 1.f, nullptr,
-                            w.BIAS + (size_t)r * w.cap * w.ldR, w.ldR, n, w.nP - n));
+            maps.add(R, h->be[r].Bop, n, 1.f, nullptr, w.BIAS + (size_t)r * w.cap * w.ldR, w.ldR, n, w.nP - n);
+        RQ_TRY(maps.run(h, B, n, w.Q, w.ldn));
         row_absmax_kernel<<<ceil_div(B * 32, 256), 256, 0, h->stream>>>(w.Q, B, n, w.ldn, h->sc_rx, w.QN);
         RQ_CUDA(h, cudaGetLastError());
         ++h->launches;
@@ -909,8 +979,11 @@ int batch_set_parametric(relu_qp_t h, int nx, const double* F, const double* E, 
         RQ_CUDA(h, cudaMemcpy(w.l0, lo.data(), sizeof(float) * m, cudaMemcpyHostToDevice));
         RQ_CUDA(h, cudaMemcpy(w.u0, up.data(), sizeof(float) * m, cudaMemcpyHostToDevice));
     }
-    for (int r = 0; r < h->nr; ++r)   // G_r = Bop_r F
-        RQ_TRY(sgemm_nt(h, R, nx, n, h->be[r].Bop, n, w.Ft32, w.ldn, 1.f, nullptr, w.G[r], w.ldx));
+    for (int r = 0; r < h->nr; ++r) {   // G_r = Bop_r F
+        Maps maps;
+        maps.add(nx, w.Ft32, w.ldn, 1.f, nullptr, w.G[r], w.ldx);
+        RQ_TRY(maps.run(h, R, n, h->be[r].Bop, n));
+    }
     RQ_CUDA(h, cudaStreamSynchronize(h->stream));
     return RELU_QP_OK;
 }
@@ -919,14 +992,12 @@ int batch_update_x0(relu_qp_t h, int B, const float* X0) {
     BatchWork& w = h->bw;
     const int n = h->n, m = h->m, R = h->R, nx = w.nx;
     RQ_TRY(copy_rows_in(h, w.X0, w.ldx, X0, B, nx));
-    RQ_TRY(sgemm_nt(h, B, n, nx, w.X0, w.ldx, w.F32, w.ldx, 1.f, nullptr, w.Q, w.ldn));
-    if (m > 0) {
-        RQ_TRY(sgemm_nt(h, B, m, nx, w.X0, w.ldx, w.E32, w.ldx, -1.f, w.l0, w.L, w.ldm));
-        RQ_TRY(sgemm_nt(h, B, m, nx, w.X0, w.ldx, w.E32, w.ldx, -1.f, w.u0, w.U, w.ldm));
-    }
+    Maps maps;
+    maps.add(n, w.F32, w.ldx, 1.f, nullptr, w.Q, w.ldn);
+    maps.add(m, w.E32, w.ldx, -1.f, w.l0, w.L, w.ldm, 0, 0, w.u0, w.U);
     for (int r = 0; r < h->nr; ++r)
-        RQ_TRY(sgemm_nt(h, B, R, nx, w.X0, w.ldx, w.G[r], w.ldx, 1.f, nullptr, w.BIAS + (size_t)r * w.cap * w.ldR,
-                        w.ldR, n, w.nP - n));
+        maps.add(R, w.G[r], w.ldx, 1.f, nullptr, w.BIAS + (size_t)r * w.cap * w.ldR, w.ldR, n, w.nP - n);
+    RQ_TRY(maps.run(h, B, nx, w.X0, w.ldx));
     row_absmax_kernel<<<ceil_div(B * 32, 256), 256, 0, h->stream>>>(w.Q, B, n, w.ldn, h->sc_rx, w.QN);
     RQ_CUDA(h, cudaGetLastError());
     ++h->launches;
@@ -1096,14 +1167,16 @@ int batch_solve(relu_qp_t h, int B, const float* Xw, const float* Lw, const int*
     if (Xw) {
         RQ_TRY(copy_rows_in(h, w.Y, w.ldn, Xw, B, n));
         RQ_TRY(scale_rows(h, w.Y, B, n, w.ldn, h->sc_xi));
-        if (m > 0) RQ_TRY(sgemm_nt(h, B, m, n, w.Y, w.ldn, h->A32, (int)round_up(n, 4), 1.f, nullptr, w.AY, w.ldm));
+        Maps maps;
+        maps.add(m, h->A32, (int)round_up(n, 4), 1.f, nullptr, w.AY, w.ldm);
+        RQ_TRY(maps.run(h, B, n, w.Y, w.ldn));
     }
     if (Lw && m > 0) {
         RQ_TRY(copy_rows_in(h, w.LSTD, w.ldm, Lw, B, m));
         RQ_TRY(scale_rows(h, w.LSTD, B, m, w.ldm, h->sc_li));
     }
     RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
-    batch_init_kernel<<<ceil_div(w.cap * 32, 256), 256, 0, h->stream>>>(p, B, Xw != nullptr, Lw != nullptr && m > 0,
+    batch_init_kernel<<<w.cap, kInitThreads, 0, h->stream>>>(p, B, Xw != nullptr, Lw != nullptr && m > 0,
                                                                         rw_dev, rho0, w.status, w.rho_idx, w.iters,
                                                                         w.nsw);
     RQ_CUDA(h, cudaGetLastError());
@@ -1210,26 +1283,15 @@ int batch_solve(relu_qp_t h, int B, const float* Xw, const float* Lw, const int*
     if (Zo && m > 0) RQ_CUDA(h, cudaMemcpyAsync(Zo, w.ZO, sizeof(float) * B * m, cudaMemcpyDefault, h->stream));
     if (Lo && m > 0) RQ_CUDA(h, cudaMemcpyAsync(Lo, w.LO, sizeof(float) * B * m, cudaMemcpyDefault, h->stream));
     if (infos) {
-        std::vector<int> st(B), itv(B), ri(B), sw(B);
-        std::vector<float> rp(B), rd(B);
-        RQ_CUDA(h, cudaMemcpyAsync(st.data(), w.status, sizeof(int) * B, cudaMemcpyDeviceToHost, h->stream));
-        RQ_CUDA(h, cudaMemcpyAsync(itv.data(), w.iters, sizeof(int) * B, cudaMemcpyDeviceToHost, h->stream));
-        RQ_CUDA(h, cudaMemcpyAsync(ri.data(), w.rho_idx, sizeof(int) * B, cudaMemcpyDeviceToHost, h->stream));
-        RQ_CUDA(h, cudaMemcpyAsync(sw.data(), w.nsw, sizeof(int) * B, cudaMemcpyDeviceToHost, h->stream));
-        RQ_CUDA(h, cudaMemcpyAsync(rp.data(), w.rp, sizeof(float) * B, cudaMemcpyDeviceToHost, h->stream));
-        RQ_CUDA(h, cudaMemcpyAsync(rd.data(), w.rd, sizeof(float) * B, cudaMemcpyDeviceToHost, h->stream));
+        pack_info_kernel<<<ceil_div(B, 256), 256, 0, h->stream>>>(B, w.status, w.iters, w.rho_idx, w.nsw, w.rp, w.rd,
+                                                                 w.info_host);
+        RQ_CUDA(h, cudaGetLastError());
+        ++h->launches;
         RQ_CUDA(h, cudaStreamSynchronize(h->stream));
         float ms = 0.f;
         cudaEventElapsedTime(&ms, h->ev0, h->ev1);
-        for (int b = 0; b < B; ++b) {
-            infos[b].status = st[b];
-            infos[b].iters = itv[b];
-            infos[b].rho_index = ri[b];
-            infos[b].rho_switches = sw[b];
-            infos[b].r_prim = rp[b];
-            infos[b].r_dual = rd[b];
-            infos[b].solve_ms = ms;
-        }
+        std::memcpy(infos, w.info_host, sizeof(relu_qp_info) * B);
+        for (int b = 0; b < B; ++b) infos[b].solve_ms = ms;
     }
     RQ_CUDA(h, cudaStreamSynchronize(h->stream));
     return RELU_QP_OK;
@@ -1509,15 +1571,14 @@ int family_launch(relu_qp_server_t s, ServeFamily& f) {
                                                                        w.nsw, f.d.client_of, f.d.Xc);
         RQ_SCUDA(s, cudaGetLastError());
         ++h->launches;
-        RQ_TRY(sgemm_nt(h, k, n, nx, f.d.x0c, w.ldx, w.F32, w.ldx, 1.f, nullptr, f.d.Qc, w.ldn));
-        if (m > 0) {
-            RQ_TRY(sgemm_nt(h, k, m, nx, f.d.x0c, w.ldx, w.E32, w.ldx, -1.f, w.l0, f.d.Lc, w.ldm));
-            RQ_TRY(sgemm_nt(h, k, m, nx, f.d.x0c, w.ldx, w.E32, w.ldx, -1.f, w.u0, f.d.Uc, w.ldm));
-            RQ_TRY(sgemm_nt(h, k, m, n, f.d.Xc, w.ldn, h->A32, (int)round_up(n, 4), 1.f, nullptr, f.d.AYc, w.ldm));
-        }
+        Maps maps, warm;
+        maps.add(n, w.F32, w.ldx, 1.f, nullptr, f.d.Qc, w.ldn);
+        maps.add(m, w.E32, w.ldx, -1.f, w.l0, f.d.Lc, w.ldm, 0, 0, w.u0, f.d.Uc);
         for (int r = 0; r < h->nr; ++r)
-            RQ_TRY(sgemm_nt(h, k, R, nx, f.d.x0c, w.ldx, w.G[r], w.ldx, 1.f, nullptr,
-                            f.d.Bc + (size_t)r * w.cap * w.ldR, w.ldR, n, w.nP - n));
+            maps.add(R, w.G[r], w.ldx, 1.f, nullptr, f.d.Bc + (size_t)r * w.cap * w.ldR, w.ldR, n, w.nP - n);
+        RQ_TRY(maps.run(h, k, nx, f.d.x0c, w.ldx));
+        warm.add(m, h->A32, (int)round_up(n, 4), 1.f, nullptr, f.d.AYc, w.ldm);
+        RQ_TRY(warm.run(h, k, n, f.d.Xc, w.ldn));
         serve_scatter_kernel<<<ceil_div(k * 32, 256), 256, 0, f.stream>>>(p, k, f.d.idx, f.d.Qc, f.d.Lc, f.d.Uc,
                                                                          f.d.Bc, f.d.AYc, w.Q, w.L, w.U, w.BIAS,
                                                                          w.QN);
@@ -1647,7 +1708,7 @@ int server_create(relu_qp_server_t* out, relu_qp_t const* families, int nf, cons
         RQ_TRY(shost(s, f, &f.h_cnt, 8));
         RQ_TRY(shost(s, f, &f.h_out, cap * f.ldo));
         // every QP index starts free
-        batch_init_kernel<<<ceil_div(w.cap * 32, 256), 256, 0, f.stream>>>(base_params(h), 0, 0, 0, nullptr, f.rho0,
+        batch_init_kernel<<<w.cap, kInitThreads, 0, f.stream>>>(base_params(h), 0, 0, 0, nullptr, f.rho0,
                                                                            w.status, w.rho_idx, w.iters, w.nsw);
         RQ_SCUDA(s, cudaGetLastError());
         RQ_SCUDA(s, cudaMemsetAsync(w.counters, 0, sizeof(int) * CNT_WORDS, f.stream));

@@ -38,7 +38,6 @@ struct BatchParams {
     int bsh;                                 // BIAS columns of A x rows: r + bsh (nP - n; the padded layout's n: 0)
     float rho[RQ_MAX_RHO];
     double rhod[RQ_MAX_RHO];
-    double logrho[RQ_MAX_RHO];              // log of each bank entry (the penalty rule's distance)
     const float* rs;                         // per-row penalty scale (1 or eq_scale)
     // scaled problems: the residual and norm factors back to the original problem,
     // 1/(c D) for rows of x and 1/E for constraint rows (nullptr without scaling)
@@ -446,17 +445,7 @@ __device__ __forceinline__ Decision decide_eval(const BatchParams& p, const Deci
     if (d.adaptive) {
         const double num = rp * fmax(fmax(npx, natl), fmax(qn, 1e-4));
         const double den = rd * fmax(fmax(nax, nz), 1e-4);
-        if (num > 0.0 && den > 0.0) {
-            const double est = p.rhod[ri] * sqrt(num / den);
-            if (isfinite(est) && est > 0.0) {
-                const double le = log(est);
-                double best = 1e300;
-                for (int k = 0; k < p.nr; ++k) {
-                    const double dd = fabs(le - p.logrho[k]);
-                    if (dd < best) { best = dd; x.nri = k; }
-                }
-            }
-        }
+        if (num > 0.0 && den > 0.0) x.nri = nearest_entry(p.rhod, p.nr, ri, p.rhod[ri] * p.rhod[ri] * (num / den));
         if (x.nri != ri) x.act = 2;
     }
     return x;

@@ -129,6 +129,7 @@ struct BatchWork {
     int tail_pr = 0;                       // rows of the layer product per pass of the tail kernel
     size_t tail_smem = 0;                  // its dynamic shared memory
     unsigned* chunk_sync = nullptr;        // per slot tile: layer counters of the persistent chunk kernel
+    relu_qp_info* info_host = nullptr;     // pinned records of a solve, written by the device
     int* cnt_host = nullptr;               // pinned host copy of the counters read back after a check
     cudaEvent_t ev_cnt = nullptr;          // recorded after that copy
 };
@@ -263,6 +264,20 @@ long long server_bytes_in_use(relu_qp_server_t s);
 // device bytes of one QP slot of a batched handle (every array that scales with max_batch)
 size_t batch_slot_bytes(relu_qp_t h);
 void batch_release(relu_qp_t h);
+
+// Bank entry nearest, in log distance, to the penalty estimate given by its square (ri if
+// that is not a positive number): entry k is nearer than entry b when the estimate lies on
+// k's side of sqrt(rho_k rho_b).  (No logarithms: an SM takes 16 clocks for one FP64
+// instruction of a warp.)
+__device__ __forceinline__ int nearest_entry(const double* rho, int nr, int ri, double est2) {
+    if (!(isfinite(est2) && est2 > 0.0)) return ri;
+    int b = 0;
+    for (int k = 1; k < nr; ++k) {
+        const double mid2 = rho[k] * rho[b];
+        if (rho[k] > rho[b] ? est2 > mid2 : rho[k] < rho[b] && est2 < mid2) b = k;
+    }
+    return b;
+}
 
 inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
 inline size_t round_up(size_t a, size_t b) { return (a + b - 1) / b * b; }

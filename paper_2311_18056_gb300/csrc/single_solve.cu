@@ -607,21 +607,10 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
             const bool converged = is_check && !numerical && rp <= eps_p && rd <= eps_d;
             int nri = ri;
             if (p.adaptive && is_check && !converged && !numerical) {
-                // Eq. rho_update (inf-norms, 1e-4 floors), nearest bank entry in log distance: entry k
-                // is nearer to the estimate than entry b when the estimate lies on k's side of
-                // sqrt(rho_k rho_b)
+                // Eq. rho_update (inf-norms, 1e-4 floors), nearest bank entry in log distance
                 const double num = rp * fmax(fmax(nPx, nAtl), fmax(p.qnorm, 1e-4));
                 const double den = rd * fmax(fmax(nAx, nz), 1e-4);
-                if (num > 0.0 && den > 0.0) {
-                    const double est2 = p.rho[ri] * p.rho[ri] * (num / den);
-                    if (isfinite(est2) && est2 > 0.0) {
-                        nri = 0;
-                        for (int k = 1; k < p.nr; ++k) {
-                            const double mid2 = p.rho[k] * p.rho[nri];
-                            if (p.rho[k] > p.rho[nri] ? est2 > mid2 : p.rho[k] < p.rho[nri] && est2 < mid2) nri = k;
-                        }
-                    }
-                }
+                if (num > 0.0 && den > 0.0) nri = nearest_entry(p.rho, p.nr, ri, p.rho[ri] * p.rho[ri] * (num / den));
             }
             if (lane == 0) {
                 s_dec[DEC_STOP] = numerical ? 1 + RELU_QP_NUMERICAL : converged ? 1 + RELU_QP_SOLVED : last ? 1 + RELU_QP_MAX_ITER : 0;
