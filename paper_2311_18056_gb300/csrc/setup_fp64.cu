@@ -7,7 +7,12 @@
 //   K   = P + sigma I + rho_r C                  (the matrix of Eq. Xbar_update)
 //   K   = L L^T                                  (blocked right-looking Cholesky)
 //   D   = K^{-1} = L^{-T} L^{-1}                 (L^{-1} by recursive doubling)
-//   [D; AD], V = [D A^T; A D A^T], X = [D; AD] (sigma I - rho_r C)
+//   T   = L^{-1} A^T,  V = [D A^T; A D A^T] = [L^{-T} T; T^T T]
+//   X   = sigma [D; AD] - rho_r V diag(s) A      (= [D; AD] (sigma I - rho_r C))
+// (A row with a large penalty has a small column of T, and V and X keep their relative
+// accuracy there.  With A D A^T formed from D, and X as [D; AD] (sigma I - rho_r C), the
+// multipliers of rows with 1000 rho came out 1e-8 off after 75 layers in 64 bits; formed so,
+// 1e-11, as from solving K X = [sigma I - rho_r C, A^T, -I].)
 // X, V and -[D; AD] hold the layer in the factored form used on the hot path:
 //   [x+; (Ax)+] = [X V] [x; 2 rho z - lam'] - [D; AD] q,
 // which is Eq. gpu_update with its z and lam columns merged
@@ -535,8 +540,8 @@ int build_bank(relu_qp_t h, const double* dP, const double* dA, const std::vecto
     const int n = h->n, m = h->m, R = h->R, nr = h->nr;
     const size_t nn = (size_t)n * n;
     Scratch s{h, {}};
-    // scratch of one entry: K, L, L^{-1} (reused for X where it fits), [D; AD], V
-    const bool alias = R <= 3 * n;
+    // scratch of one entry: K, L, L^{-1} (reused for T and X where they fit), [D; AD], V
+    const bool alias = m <= 2 * n;
     const size_t per = 3 * nn + (size_t)R * n + (size_t)R * m + (alias ? 0 : (size_t)R * n);
     // as many entries together as fit 4 GiB of scratch (at least one)
     const int ge = (int)std::max<size_t>(1, std::min<size_t>(nr, ((size_t)4 << 30) / (8 * per)));
@@ -568,19 +573,24 @@ int build_bank(relu_qp_t h, const double* dP, const double* dA, const std::vecto
         RQ_CUDA(h, cudaGetLastError());
         RQ_TRY(spd_inverse(h, nb, n, Km, Lm, Li, st, DS, n, st, flag + r0));
         if (m > 0) {
-            double* AD = DS + nn;
-            Gemm g = gemm(false, false, m, n, n, 1.0, dA, n, DS, n, 0.0, AD, n);
-            g.sB = g.sC = g.sD = st;
-            RQ_TRY(dgemm_batch(h, g, nb));
-            g = gemm(false, true, m, m, n, 1.0, AD, n, dA, n, 0.0, V + (size_t)n * m, m);
+            double *AD = DS + nn, *T = alias ? W : X;   // (K and L, or X, are free now or still)
+            Gemm g = gemm(false, true, n, m, n, 1.0, Li, n, dA, n, 0.0, T, m);
             g.sA = g.sC = g.sD = st;
+            g.flags = G_KEND_M;
+            RQ_TRY(dgemm_batch(h, g, nb));
+            g = gemm(true, false, m, m, n, 1.0, T, m, T, m, 0.0, V + (size_t)n * m, m);
+            g.sA = g.sB = g.sC = g.sD = st;
             g.flags = G_LOWER | G_MIRROR;
             RQ_TRY(dgemm_batch(h, g, nb));
-            transpose_f64_kernel<<<dim3(ceil_div(n, 32), ceil_div(m, 32), nb), dim3(32, 8), 0, h->stream>>>(AD, st, V,
-                                                                                                        st, m, n);
+            g = gemm(true, false, n, m, n, 1.0, Li, n, T, m, 0.0, V, m);
+            g.sA = g.sB = g.sC = g.sD = st;
+            g.flags = G_KBEG_M;
+            RQ_TRY(dgemm_batch(h, g, nb));
+            transpose_f64_kernel<<<dim3(ceil_div(m, 32), ceil_div(n, 32), nb), dim3(32, 8), 0, h->stream>>>(V, st, AD,
+                                                                                                        st, n, m);
             RQ_CUDA(h, cudaGetLastError());
         }
-        Gemm g = gemm(false, false, R, n, m > 0 ? n : 0, 0.0, DS, n, C, n, h->sigma, X, n);
+        Gemm g = gemm(false, false, R, n, m, 0.0, V, m, sA, n, h->sigma, X, n);
         for (int z = 0; z < nb; ++z) g.alpha[z] = -rho.v[z];
         g.D = DS;
         g.sA = g.sC = g.sD = st;
