@@ -5,6 +5,7 @@
 #include <cmath>
 #include <cstring>
 #include <new>
+#include <type_traits>
 
 namespace {
 thread_local std::string g_setup_error;
@@ -115,27 +116,27 @@ int upload_scaling(relu_qp_t h) {
 int upload_problem(relu_qp_t h) {
     const int n = h->n, m = h->m;
     // (the staging and the device copies of the last call are free: every call ends synchronised)
-    float *q = h->sw.pin, *l = q + n, *u = l + m;
-    for (int j = 0; j < n; ++j) q[j] = (float)(h->scaled ? h->sC * h->sD[j] * h->h_q[j] : h->h_q[j]);
-    for (int i = 0; i < m; ++i) {
-        const double e = h->scaled ? h->sE[i] : 1.0;
-        l[i] = (float)(e * h->h_l[i]);
-        u[i] = (float)(e * h->h_u[i]);
-    }
+    auto stage = [&](auto* q, auto* l, auto* u) {
+        using T = std::remove_reference_t<decltype(*q)>;
+        for (int j = 0; j < n; ++j) q[j] = (T)(h->scaled ? h->sC * h->sD[j] * h->h_q[j] : h->h_q[j]);
+        for (int i = 0; i < m; ++i) {
+            const double e = h->scaled ? h->sE[i] : 1.0;
+            l[i] = (T)(e * h->h_l[i]);
+            u[i] = (T)(e * h->h_u[i]);
+        }
+    };
     double qn = 0.0;
     for (int i = 0; i < n; ++i) qn = std::fmax(qn, std::fabs(h->h_q[i]));
     h->qnorm = qn;
     if (h->opts.single_precision != RELU_QP_PREC_FP32) {
-        std::vector<double> q64(n), l64(m), u64(m);
-        for (int j = 0; j < n; ++j) q64[j] = h->scaled ? h->sC * h->sD[j] * h->h_q[j] : h->h_q[j];
-        for (int i = 0; i < m; ++i) {
-            const double e = h->scaled ? h->sE[i] : 1.0;
-            l64[i] = e * h->h_l[i];
-            u64[i] = e * h->h_u[i];
-        }
-        RQ_TRY(rq::single64_upload(h, q64.data(), l64.data(), u64.data()));
+        double* q = h->sw64.pin;
+        stage(q, q + n, q + n + m);
+        RQ_TRY(rq::single64_update(h));
+    } else {
+        float* q = h->sw.pin;
+        stage(q, q + n, q + n + m);
+        RQ_TRY(rq::single_update(h));
     }
-    RQ_TRY(rq::single_update(h));
     RQ_CUDA(h, cudaStreamSynchronize(h->stream));
     return RELU_QP_OK;
 }
@@ -507,6 +508,7 @@ void relu_qp_destroy(relu_qp_t h) {
     else cudaDeviceSynchronize();
     rq::batch_release(h);
     rq::single_release(h);
+    rq::single64_release(h);
     for (cudaEvent_t e : h->prof_ev)
         if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : h->gap_ev)

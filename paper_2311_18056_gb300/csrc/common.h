@@ -79,17 +79,17 @@ struct SingleWork {
 
 // Workspace of the FP64 single-QP solve (opts.single_precision = FP64 or FP64R).
 struct SingleWork64 {
-    double *y = nullptr, *z = nullptr, *lam = nullptr, *Ay = nullptr;
-    double *s0 = nullptr, *s1 = nullptr;
-    double *Py = nullptr, *Axf = nullptr, *lstd = nullptr;
-    double *xin = nullptr, *lin = nullptr;
-    double *c = nullptr, *sref = nullptr;   // refined form: anchor layer product and its operand
-    float* d32 = nullptr;                   // refined form: FP32 increment of the next layer (ldw)
-    unsigned long long* red = nullptr;   // 3 slots x 8 reduction words (bits of non-negative doubles)
-    unsigned* bar = nullptr;             // grid barrier: arrival count of the launch (+ pad word)
-    int* out_i = nullptr;                // status, iters, rho_index, switches, err
-    double* out_f = nullptr;             // r_prim, r_dual
-    int grid = 0;
+    unsigned long long* words = nullptr;   // operand exchange: two buffers of 2 R words
+    double* lstd = nullptr;                // lam_std of a check
+    double* in = nullptr;                  // warm start on the device: x, lam
+    unsigned long long* red = nullptr;     // 3 slots x 8 reduction words (bits of non-negative doubles)
+    unsigned* count = nullptr;             // arrivals (modulo 2^32), pad, error word
+    unsigned tag = 0, counted = 0;         // exchange numbers and arrivals so far
+    int last_ctas = 0, grid = 0;
+    size_t smem_max = 0;
+    // pinned host memory: staging of q, l, u and of a warm start, results x, z, lam, info words
+    double *pin = nullptr, *pin_in = nullptr, *out = nullptr, *out_f = nullptr;
+    int* out_i = nullptr;
 };
 
 // Workspace of batched solves (allocated when opts.max_batch > 0).
@@ -229,7 +229,9 @@ int single_solve_noalloc(relu_qp_t h, const float* x_warm, const float* lam_warm
                          relu_qp_info* info);
 // FP64 single-QP solve (single_solve64.cu).
 int single64_alloc(relu_qp_t h, const double* P, const double* A);
-int single64_upload(relu_qp_t h, const double* q, const double* l, const double* u);
+void single64_release(relu_qp_t h);
+// q, l, u from h->sw64.pin to the device and the biases they give
+int single64_update(relu_qp_t h);
 int single64_prepare(relu_qp_t h);
 int single64_solve(relu_qp_t h, const double* x_warm, const double* lam_warm, int rho_index, double eps_abs,
                    double eps_rel, int max_iter, double* x_out, double* z_out, double* lam_out,

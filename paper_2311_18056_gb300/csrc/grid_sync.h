@@ -1,5 +1,4 @@
-// Grid-wide barrier of the cooperative kernels (single_solve64.cu,
-// batch_tail.cu): every CTA of the launch must be
+// Grid-wide barrier of the cooperative kernels (batch_tail.cu): every CTA of the launch must be
 // co-resident.  bar[0] counts every arrival of the launch (zeroed before the
 // launch, never reset during it); each CTA keeps the number of barriers it has
 // passed (its epoch), so barrier e is complete once the count reaches
@@ -121,6 +120,80 @@ __device__ __forceinline__ bool sync_give_up(int* err, long long t0, long long t
     if (grid_sync_timer() - t0 <= timeout_ns) return false;
     atomicExch(err, RELU_QP_ERR_TIMEOUT);
     return true;
+}
+
+// ---- exchanges of a cooperative grid ----
+// One 64-bit word in global memory: 32 bits of value and the exchange's number, which a
+// reader polls together (a 64-bit access is one access; no ordering between words is needed).
+__device__ __forceinline__ void put_word(unsigned long long* w, unsigned v, unsigned tag) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(w), "l"(((unsigned long long)tag << 32) | v) : "memory");
+}
+__device__ __forceinline__ void put_words2(unsigned long long* w, unsigned a, unsigned b, unsigned tag) {
+    const unsigned long long t = (unsigned long long)tag << 32;
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(w), "l"(t | a), "l"(t | b) : "memory");
+}
+__device__ __forceinline__ void get_words(const unsigned long long* w, unsigned long long& a, unsigned long long& b) {
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(w) : "memory");
+}
+
+// `count` tagged words from w on (16-byte aligned), by a CTA of THREADS threads: store(k, a, b,
+// two) gets words k and (two) k + 1.  False in every thread if a wait gave up.  Four pairs a
+// thread are in flight; only pairs that are not there yet are read again.
+template <int THREADS, class Store>
+__device__ __forceinline__ bool gather_words(const unsigned long long* w, int count, unsigned tag, int* err,
+                                             long long timeout_ns, Store store) {
+    constexpr int U = 4;
+    bool ok = true;
+    const int pairs = (count + 1) >> 1;
+    for (int b = threadIdx.x; b < pairs && ok; b += U * THREADS) {
+        unsigned todo = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (b + u * THREADS < pairs) todo |= 1u << u;
+        long long t0 = 0;
+        for (int tries = 0; todo; ++tries) {
+            unsigned long long a[U], c[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if ((todo >> u) & 1u) get_words(w + 2 * (b + u * THREADS), a[u], c[u]);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (!((todo >> u) & 1u)) continue;
+                const int k = 2 * (b + u * THREADS);
+                const bool two = k + 1 < count;
+                if ((unsigned)(a[u] >> 32) != tag || (two && (unsigned)(c[u] >> 32) != tag)) continue;
+                todo &= ~(1u << u);
+                store(k, (unsigned)a[u], (unsigned)c[u], two);
+            }
+            if (todo && (tries & 63) == 63) {
+                if (t0 == 0) t0 = grid_sync_timer();
+                if (sync_give_up(err, t0, timeout_ns)) {
+                    ok = false;
+                    break;
+                }
+            }
+        }
+    }
+    return __syncthreads_or(ok ? 0 : 1) == 0;
+}
+
+// Arrive (the release covers the CTA's stores) and wait until the count reaches `target`
+// (modulo 2^32); false in every thread if the wait gave up.
+__device__ __forceinline__ bool count_wait(unsigned* count, unsigned target, int* err, long long timeout_ns) {
+    __syncthreads();
+    bool ok = true;
+    if (threadIdx.x == 0) {
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+        long long t0 = 0;
+        while (ok) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
+            if ((int)(v - target) >= 0) break;
+            if (t0 == 0) t0 = grid_sync_timer();
+            ok = !sync_give_up(err, t0, timeout_ns);
+        }
+    }
+    return __syncthreads_or(ok ? 0 : 1) == 0;
 }
 
 // ---- one thread-block cluster instead of a cooperative grid ----

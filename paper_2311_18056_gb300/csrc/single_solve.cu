@@ -196,52 +196,12 @@ __device__ __forceinline__ float group_dot(int gs, const float* const (&w)[kRows
 constexpr bool is_grid(int form) { return form == FORM_GRID || form == FORM_COUNT; }
 
 // ---- exchanges -------------------------------------------------------------
-__device__ __forceinline__ void put_word(unsigned long long* w, float v, unsigned tag) {
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(w), "l"(((unsigned long long)tag << 32) | __float_as_uint(v))
-                 : "memory");
-}
-
-__device__ __forceinline__ void get_words(const unsigned long long* w, unsigned long long& a, unsigned long long& b) {
-    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(w) : "memory");
-}
-
-// The `count` values of the tagged words w (16-byte aligned) into dst, by the whole CTA;
-// false in every thread if a wait gave up.  Four pairs a thread are in flight; only pairs
-// that are not there yet are read again.
+// The `count` values of the tagged words w into dst, by the whole CTA.
 __device__ __forceinline__ bool gather(const SP& p, const unsigned long long* w, float* dst, int count, unsigned tag) {
-    constexpr int U = 4;
-    bool ok = true;
-    const int pairs = (count + 1) >> 1;
-    for (int b = threadIdx.x; b < pairs && ok; b += U * kThreads) {
-        unsigned todo = 0;
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (b + u * kThreads < pairs) todo |= 1u << u;
-        long long t0 = 0;
-        for (int tries = 0; todo; ++tries) {
-            unsigned long long a[U], c[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u)
-                if ((todo >> u) & 1u) get_words(w + 2 * (b + u * kThreads), a[u], c[u]);
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (!((todo >> u) & 1u)) continue;
-                const int k = 2 * (b + u * kThreads);
-                if ((unsigned)(a[u] >> 32) != tag || (k + 1 < count && (unsigned)(c[u] >> 32) != tag)) continue;
-                todo &= ~(1u << u);
-                dst[k] = __uint_as_float((unsigned)a[u]);
-                if (k + 1 < count) dst[k + 1] = __uint_as_float((unsigned)c[u]);
-            }
-            if (todo && (tries & 63) == 63) {
-                if (t0 == 0) t0 = grid_sync_timer();
-                if (sync_give_up(p.err, t0, p.timeout_ns)) {
-                    ok = false;
-                    break;
-                }
-            }
-        }
-    }
-    return __syncthreads_or(ok ? 0 : 1) == 0;
+    return gather_words<kThreads>(w, count, tag, p.err, p.timeout_ns, [&](int k, unsigned a, unsigned b, bool two) {
+        dst[k] = __uint_as_float(a);
+        if (two) dst[k + 1] = __uint_as_float(b);
+    });
 }
 
 // The first ncache rows of the CTA (x rows x0 .., then A x rows a0 ..) of bank entry ri.
@@ -291,7 +251,7 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
     // one entry of exchange x
     auto publish = [&](unsigned x, int r, float v) {
         if (F == FORM_GRID) {
-            put_word(p.wop + (size_t)(x & 1) * ((R + 1) & ~1) + r, v, p.tag0 + 1 + x);
+            put_word(p.wop + (size_t)(x & 1) * ((R + 1) & ~1) + r, __float_as_uint(v), p.tag0 + 1 + x);
         } else if (F == FORM_COUNT) {
             p.sop[(size_t)(x & 1) * ldw + r] = v;
         } else if (F == FORM_ONE) {
@@ -310,22 +270,8 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
             return gather(p, p.wop + (size_t)(x & 1) * ((R + 1) & ~1), sv, R, p.tag0 + 1 + x);
         }
         if (F == FORM_COUNT) {
-            // every CTA has stored its entries (its release covers them) and read the last operand
-            __syncthreads();
-            bool ok = true;
-            if (tid == 0) {
-                asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.count) : "memory");
-                const unsigned target = p.count0 + (x + 1) * (unsigned)p.ctas;
-                long long t0 = 0;
-                while (ok) {
-                    unsigned v;
-                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p.count) : "memory");
-                    if ((int)(v - target) >= 0) break;
-                    if (t0 == 0) t0 = grid_sync_timer();
-                    ok = !sync_give_up(p.err, t0, p.timeout_ns);
-                }
-            }
-            if (__syncthreads_or(ok ? 0 : 1)) return false;
+            // every CTA has stored its entries and read the last operand
+            if (!count_wait(p.count, p.count0 + (x + 1) * (unsigned)p.ctas, p.err, p.timeout_ns)) return false;
             const float4* src = reinterpret_cast<const float4*>(p.sop + (size_t)(x & 1) * ldw);
             for (int k = tid; k < (ldw >> 2); k += kThreads) reinterpret_cast<float4*>(sv)[k] = __ldcg(src + k);
             __syncthreads();
@@ -533,7 +479,7 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
                     red_max(s_red, RED_RP, (v - zi) * f);
                     red_max(s_red, RED_AX, v * f);
                     red_max(s_red, RED_Z, zi * f);
-                    if (is_grid(F)) put_word(p.wls + i, ls, tag);
+                    if (is_grid(F)) put_word(p.wls + i, __float_as_uint(ls), tag);
                     else if (F == FORM_ONE) svk[i] = ls;
                 }
                 if (F == FORM_CLUSTER)
@@ -571,7 +517,7 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
         __syncthreads();
         // every CTA's maxima
         if (is_grid(F)) {
-            if (tid < RED_WORDS) put_word(p.wred + RED_WORDS * cta + tid, __uint_as_float(s_red[tid]), tag);
+            if (tid < RED_WORDS) put_word(p.wred + RED_WORDS * cta + tid, s_red[tid], tag);
             if (!gather(p, p.wred, reds, RED_WORDS * p.ctas, tag)) return;
         } else if (F == FORM_CLUSTER) {
             for (int t = tid; t < 2 * p.ctas; t += kThreads) {

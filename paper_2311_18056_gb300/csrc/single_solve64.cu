@@ -19,16 +19,27 @@
 // shrinks as the solve converges, and each layer costs an FP32 row product
 // instead of an FP64 one (GB300's FP64 rate is ~1/60 of its FP32 rate).
 //
-// Work split: the R = n + m rows of Wt (FP64, R x R) are cut into contiguous
-// slices, one per CTA of 16 warps; each warp produces one row at a time (lanes over the
-// columns, shuffle reduction); the operand s lives in shared memory.  Rows
-// stream from L2 (the FP64 bank of n + m = 3000 is 72 MB).  A grid barrier
-// with a deadline separates layers.
+// Work split and exchange as in single_solve.cu: each CTA owns a slice of the rows
+// of x and of A x with their state in shared memory, a warp takes a row at a time,
+// and the operand's entries carry their own arrival (an FP64 entry is two tagged
+// words side by side, an increment one), or, above kTagMax words, the CTAs are
+// counted.  The rows of the layer that fit are cached in shared memory: the FP32
+// bank's for the increments, else the FP64 bank's; FP64 rows otherwise stream from
+// L2 (the FP64 bank of n + m = 3000 is 72 MB).  An FP64 entry goes out only where
+// the next layer, or a check, reads it.
+//
+// Bound: n + m = 513 by the exchange and the chain of FP64 operations behind a row's
+// sum (an SM issues one FP64 warp instruction in 16 clocks); n + m = 3000 by the FP64
+// pipe, 59 k FMAs per SM and layer at two a clock.  A solve of 100 layers: n = 342 (FP64)
+// 599 us with a grid barrier and the rows' state in global memory, 320 us so; n = 1110
+// (anchored) 817 and 340 us.
 #include "common.h"
 #include "grid_sync.h"
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
+#include <functional>
 
 namespace rq {
 namespace {
@@ -37,28 +48,36 @@ constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 // operand s in shared memory: n + m doubles at most
 constexpr int kMaxRows64 = 24576;
+// words of an exchange up to which they are tagged
+constexpr int kTagMax = 2048;
+constexpr int kState = 11;   // doubles of state per row
 
 enum { RED_RP = 0, RED_RD, RED_AX, RED_Z, RED_PX, RED_ATL, RED_WORDS = 8 };
-enum { OUT_STATUS = 0, OUT_ITERS, OUT_RHO, OUT_SWITCHES, OUT_ERR, OUT_WORDS = 8 };
+enum { DEC_STOP = 6, DEC_RHO = 7 };   // of the decision's words: 1 + the status to stop with, or 0; bank entry
+enum { OUT_STATUS = 0, OUT_ITERS, OUT_RHO, OUT_SWITCHES, OUT_LAST, OUT_COUNTED, OUT_WORDS = 8 };
 
 struct SP64 {
     int n, m, R, nr;
     const double* Wt[RQ_MAX_RHO];
     const float* Wt32[RQ_MAX_RHO];   // refined form: FP32 bank, rows of ldw floats (zero padded)
     int ldw, anchor_every;
-    double *c, *sref;                // refined form: anchor product and operand (R each)
-    float* d32;                      // refined form: (float)(s - s_ref) of the next layer (ldw, zero padded)
     const double* bias[RQ_MAX_RHO];
     double rho[RQ_MAX_RHO];
     const double *P, *A, *At, *q, *l, *u;
     const float* rs;              // per-row penalty scale (1 or eq_scale)
     const double *rsx, *rsz;      // scaled problems: residual factors 1/(c D), 1/E (else nullptr)
-    double *y, *z, *lam, *Ay, *s0, *s1, *Py, *Axf, *lstd;
+    const double *xin, *lin;      // warm start (or nullptr)
+    double *xo, *zo, *lo;         // results
+    // exchanges: the operand buffers [2] of 2 R words (tagged words, FP64 entries or FP32
+    // increments), lam_std, the maxima of three checks, the count of arrivals from count0 on
+    unsigned long long* wop;
+    double* ls;
     unsigned long long* red;
-    unsigned* bar;
-    int* out_i;
+    unsigned *count, count0;
+    unsigned tag0;                // exchange e is tagged tag0 + 1 + e
+    int *err, *out_i;
     double* out_f;
-    int rho_index0, check_interval, adaptive, max_iter, rows_per_cta, rows2_per_cta;
+    int rho_index0, check_interval, adaptive, max_iter, xr, ar, ctas, cached, share;
     double eps_abs, eps_rel, qnorm;
     long long timeout_ns;
 };
@@ -69,38 +88,36 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// Grid-wide barrier over all CTAs of the cooperative launch (grid_sync.h).
-__device__ __forceinline__ bool grid_barrier(const SP64& p, GridSyncState* s_ok) {
-    return grid_sync(p.bar, p.out_i + OUT_ERR, p.timeout_ns, s_ok);
-}
-
-// Dot product of a row (global, read-only) with a vector in shared memory;
-// the result is valid in every lane.  Eight independent loads per lane are in
-// flight per step: a row streams from L2, and with one CTA of 8 warps per SM
-// fewer loads in flight leave the FP64 pipe waiting on L2 latency.
-__device__ __forceinline__ double row_dot(const double* __restrict__ w, const double* __restrict__ s, int len,
-                                          int lane) {
+// Dot product of a row (in global or, GLOBAL false, in shared memory) with a vector in
+// shared memory; the result is valid in every lane.  Eight independent loads per lane are in
+// flight per step: a row streams from L2, and fewer leave the FP64 pipe waiting on it.
+template <bool GLOBAL>
+__device__ __forceinline__ double row_dot(const double* __restrict__ w, const double* __restrict__ s, int len, int lane) {
     double a[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     int k = lane;
     for (; k + 7 * 32 < len; k += 8 * 32) {
         double wv[8];
 #pragma unroll
-        for (int t = 0; t < 8; ++t) wv[t] = __ldg(w + k + 32 * t);
+        for (int t = 0; t < 8; ++t) wv[t] = GLOBAL ? __ldg(w + k + 32 * t) : w[k + 32 * t];
 #pragma unroll
         for (int t = 0; t < 8; ++t) a[t] = fma(wv[t], s[k + 32 * t], a[t]);
     }
-    for (; k < len; k += 32) a[0] = fma(__ldg(w + k), s[k], a[0]);   // at most 7 steps
+#pragma unroll
+    for (int t = 0; t < 7; ++t, k += 32)   // at most 7 steps
+        if (k < len) a[t] = fma(GLOBAL ? __ldg(w + k) : w[k], s[k], a[t]);
     return warp_sum(((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7])));
 }
 
 // FP32 row (ld floats, 16-byte aligned, zero padded) times an FP32 vector in
 // shared memory; the result is valid in every lane.
+template <bool GLOBAL>
 __device__ __forceinline__ float row_dot32(const float* __restrict__ w, const float* __restrict__ s, int ld, int lane) {
     const float4* w4 = reinterpret_cast<const float4*>(w);
     const float4* s4 = reinterpret_cast<const float4*>(s);
     float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+#pragma unroll 4
     for (int k = lane; k < (ld >> 2); k += 32) {
-        const float4 a = __ldg(w4 + k);
+        const float4 a = GLOBAL ? __ldg(w4 + k) : w4[k];
         const float4 b = s4[k];
         a0 = fmaf(a.x, b.x, a0);
         a1 = fmaf(a.y, b.y, a1);
@@ -113,11 +130,6 @@ __device__ __forceinline__ float row_dot32(const float* __restrict__ w, const fl
     return v;
 }
 
-// Vector written by other CTAs into shared memory, bypassing L1.
-__device__ __forceinline__ void load_shared_cg(double* dst, const double* src, int len) {
-    for (int k = threadIdx.x; k < len; k += blockDim.x) dst[k] = __ldcg(src + k);
-}
-
 __device__ __forceinline__ void red_max(unsigned long long* slot, int word, double v) {
     atomicMax(slot + word, (unsigned long long)__double_as_longlong(fabs(v)));
 }
@@ -126,233 +138,338 @@ __device__ __forceinline__ double red_get(const unsigned long long* slot, int wo
     return __longlong_as_double((long long)__ldcg(slot + word));
 }
 
-template <bool REFINED>
-__global__ void __launch_bounds__(kThreads, 1) single64_kernel(SP64 p) {
-    extern __shared__ __align__(16) double sv[];   // R doubles (refined layers: ldw floats of the increment)
-    __shared__ GridSyncState s_ok;
-    grid_sync_init(&s_ok);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n = p.n, m = p.m, R = p.R;
-    const int row0 = blockIdx.x * p.rows_per_cta;
-    const int row1 = min(row0 + p.rows_per_cta, R);
-    const int r2_0 = blockIdx.x * p.rows2_per_cta;
-    const int r2_1 = min(r2_0 + p.rows2_per_cta, n);
+// TAG: tagged words, else counted CTAs.
+template <bool REFINED, bool TAG>
+__global__ void __launch_bounds__(kThreads, 1) single64_kernel(const __grid_constant__ SP64 p) {
+    extern __shared__ __align__(16) double smem[];
+    __shared__ double s_dec[RED_WORDS];
+    __shared__ unsigned long long s_red[RED_WORDS];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
+    const int n = p.n, m = p.m, R = p.R, cta = blockIdx.x;
+    if (cta >= p.ctas) return;
+    const int x0 = cta * p.xr, nx = max(0, min(p.xr, n - x0));
+    const int a0 = cta * p.ar, na = max(0, min(p.ar, m - a0));
+    const int rows = nx + na, per = p.xr + p.ar, ncache = min(p.cached, rows);
+    // the operand (R doubles, or ldw floats of increments), lam_std, the rows' state, cached rows
+    double* sv = smem;
+    float* dv = reinterpret_cast<float*>(sv);
+    const int op = (max(R, (p.ldw + 1) / 2) + 1) & ~1;
+    double* svk = p.share ? sv : sv + op;
+    double* st = sv + op + (p.share ? 0 : (m + 1) & ~1);
+    double *st_bias = st, *st_rr = st + per, *st_z = st_rr + per, *st_lam = st_z + per, *st_rho = st_lam + per,
+           *st_l = st_rho + per, *st_u = st_l + per, *st_chk = st_u + per, *st_ls = st_chk + per, *st_c = st_ls + per,
+           *st_sref = st_c + per;
+    double* wc64 = st + kState * (size_t)per + ((kState * per) & 1);
+    float* wc32 = reinterpret_cast<float*>(wc64);
+    auto row_of = [&](int lr) { return lr < nx ? x0 + lr : n + a0 + (lr - nx); };
+    int ri = p.rho_index0, switches = 0;
+    unsigned e = 0, counted = 0, checks = 0;
+    // ---- exchange x: FP64 entries or FP32 increments ----
+    auto publish64 = [&](unsigned x, int r, double v) {
+        if (TAG) {
+            const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+            put_words2(p.wop + ((size_t)(x & 1) * R + r) * 2, (unsigned)b, (unsigned)(b >> 32), p.tag0 + 1 + x);
+        } else {
+            reinterpret_cast<double*>(p.wop)[(size_t)(x & 1) * R + r] = v;
+        }
+    };
+    auto publish32 = [&](unsigned x, int r, float v) {
+        if (TAG) put_word(p.wop + (size_t)(x & 1) * R * 2 + r, __float_as_uint(v), p.tag0 + 1 + x);
+        else reinterpret_cast<float*>(p.wop)[(size_t)(x & 1) * R * 4 + r] = v;
+    };
+    auto all_arrived = [&]() { return count_wait(p.count, p.count0 + ++counted * (unsigned)p.ctas, p.err, p.timeout_ns); };
+    auto receive64 = [&](unsigned x) -> bool {
+        if (TAG) {
+            __syncthreads();   // the operand's readers are done
+            return gather_words<kThreads>(p.wop + (size_t)(x & 1) * R * 2, 2 * R, p.tag0 + 1 + x, p.err, p.timeout_ns,
+                                          [&](int k, unsigned a, unsigned b, bool) {
+                                              sv[k >> 1] = __longlong_as_double((long long)(((unsigned long long)b << 32) | a));
+                                          });
+        }
+        if (!all_arrived()) return false;
+        for (int k = tid; k < R; k += kThreads) sv[k] = __ldcg(reinterpret_cast<const double*>(p.wop) + (size_t)(x & 1) * R + k);
+        __syncthreads();
+        return true;
+    };
+    auto receive32 = [&](unsigned x) -> bool {
+        if (TAG) {
+            __syncthreads();
+            for (int k = R + tid; k < p.ldw; k += kThreads) dv[k] = 0.f;
+            return gather_words<kThreads>(p.wop + (size_t)(x & 1) * R * 2, R, p.tag0 + 1 + x, p.err, p.timeout_ns,
+                                          [&](int k, unsigned a, unsigned b, bool two) {
+                                              dv[k] = __uint_as_float(a);
+                                              if (two) dv[k + 1] = __uint_as_float(b);
+                                          });
+        }
+        if (!all_arrived()) return false;
+        for (int k = tid; k < p.ldw; k += kThreads)
+            dv[k] = k < R ? __ldcg(reinterpret_cast<const float*>(p.wop) + (size_t)(x & 1) * R * 4 + k) : 0.f;
+        __syncthreads();
+        return true;
+    };
+    auto load_bank = [&]() {
+        if (REFINED) {
+            const int c4 = p.ldw >> 2;
+            for (int k = tid; k < ncache * c4; k += kThreads)
+                reinterpret_cast<float4*>(wc32)[k] =
+                    __ldg(reinterpret_cast<const float4*>(p.Wt32[ri] + (size_t)row_of(k / c4) * p.ldw) + k % c4);
+        } else {
+            for (int lr = warp; lr < ncache; lr += kWarps)
+                for (int k = lane; k < R; k += 32) wc64[(size_t)lr * R + k] = __ldg(p.Wt[ri] + (size_t)row_of(lr) * R + k);
+        }
+        for (int lr = tid; lr < rows; lr += kThreads) st_bias[lr] = __ldg(p.bias[ri] + row_of(lr));
+    };
 
-    int ri = p.rho_index0;
-    int switches = 0, checks = 0, cur = 0;
+    // ---------------- start state ----------------
+    if (p.xin)
+        for (int k = tid; k < n; k += kThreads) sv[k] = p.xin[k];
+    if (tid < RED_WORDS) s_red[tid] = 0ull;
+    for (int lr = nx + tid; lr < rows; lr += kThreads) {
+        const int i = a0 + lr - nx;
+        st_rho[lr] = p.rho[ri] * (double)__ldg(p.rs + i);
+        st_l[lr] = __ldg(p.l + i);
+        st_u[lr] = __ldg(p.u + i);
+        st_lam[lr] = p.lin ? p.lin[i] : 0.0;
+        st_z[lr] = 0.0;
+    }
+    load_bank();
+    __syncthreads();
+    if (p.xin) {
+        for (int lr = nx + warp; lr < rows; lr += kWarps) {
+            const double v = row_dot<true>(p.A + (size_t)(a0 + lr - nx) * n, sv, n, lane);
+            if (lane == 0) st_z[lr] = v;
+        }
+        __syncthreads();
+    }
+    for (int lr = tid; lr < rows; lr += kThreads) {
+        const int r = row_of(lr);
+        if (lr >= nx) st_rr[lr] = st_lam[lr] / st_rho[lr];   // A x - z = 0
+        publish64(0, r, lr < nx ? (p.xin ? p.xin[r] : 0.0) : 2.0 * st_rho[lr] * st_z[lr] - st_lam[lr]);
+    }
+    if (!receive64(0)) return;
+
     for (int it = 1; it <= p.max_iter; ++it) {
-        // ---------------- one layer: s[cur] -> s[cur^1] ----------------
-        const double* scur = cur ? p.s1 : p.s0;
-        double* snext = cur ? p.s0 : p.s1;
+        // ---------------- one layer ----------------
         // refined form: an FP64 anchor layer at the start of every check interval (so also
         // after every bank switch), FP32 increment layers in between
         const bool anchor = !REFINED || (it - 1) % p.anchor_every == 0;
-        float* dv = reinterpret_cast<float*>(sv);
-        if (anchor) {
-            load_shared_cg(sv, scur, R);
-        } else {
-            for (int k = threadIdx.x; k < p.ldw; k += blockDim.x)
-                dv[k] = __ldcg(p.d32 + k);   // written by the owners of the rows in the last layer
-        }
-        __syncthreads();
-        const double* Wg = p.Wt[ri];
-        const double* bias = p.bias[ri];
-        const double rho = p.rho[ri];
-        for (int r = row0 + warp; r < row1; r += kWarps) {
-            const double acc = anchor ? row_dot(Wg + (size_t)r * R, sv, R, lane)
-                                      : (double)row_dot32(p.Wt32[ri] + (size_t)r * p.ldw, dv, p.ldw, lane);
+        const bool last = it == p.max_iter;
+        // the next layer is an anchor, or a check reads x
+        const bool full = !REFINED || it % p.anchor_every == 0 || last;
+        for (int lr = warp; lr < rows; lr += kWarps) {
+            const int r = row_of(lr);
+            double t;
+            if (anchor) {
+                t = !REFINED && lr < ncache ? row_dot<false>(wc64 + (size_t)lr * R, sv, R, lane)
+                                            : row_dot<true>(p.Wt[ri] + (size_t)r * R, sv, R, lane);
+            } else {
+                t = (double)(lr < ncache ? row_dot32<false>(wc32 + (size_t)lr * p.ldw, dv, p.ldw, lane)
+                                         : row_dot32<true>(p.Wt32[ri] + (size_t)r * p.ldw, dv, p.ldw, lane));
+            }
             if (lane == 0) {
-                double t;
-                if (!REFINED) {
-                    t = acc + __ldg(bias + r);
-                } else if (anchor) {
-                    t = acc + __ldg(bias + r);
-                    p.c[r] = t;
-                    p.sref[r] = scur[r];
-                } else {
-                    t = p.c[r] + acc;
+                t += anchor ? st_bias[lr] : st_c[lr];
+                if (REFINED && anchor) {
+                    st_c[lr] = t;
+                    st_sref[lr] = sv[r];
                 }
-                if (r < n) {
-                    p.y[r] = t;
-                    snext[r] = t;
-                    if (REFINED) p.d32[r] = (float)(t - p.sref[r]);
+                double snew = t, z = t;
+                if (lr >= nx) {
+                    const double rr = st_rr[lr], lam = st_rho[lr] * rr;
+                    z = fmin(fmax(t + rr, st_l[lr]), st_u[lr]);
+                    snew = 2.0 * st_rho[lr] * z - lam;
+                    if (full) publish64(e + 1, r, snew);
+                    else publish32(e + 1, r, (float)(snew - st_sref[lr]));
+                    st_lam[lr] = lam;
+                    st_rr[lr] = t - z + rr;
+                } else if (full) {
+                    publish64(e + 1, r, snew);
                 } else {
-                    const int i = r - n;
-                    const double rho_i = rho * (double)__ldg(p.rs + i);
-                    const double rr = p.Ay[i] - p.z[i] + p.lam[i] / rho_i;
-                    const double zn = fmin(fmax(t + rr, __ldg(p.l + i)), __ldg(p.u + i));
-                    const double ln = rho_i * rr;
-                    p.Ay[i] = t;
-                    p.z[i] = zn;
-                    p.lam[i] = ln;
-                    snext[r] = 2.0 * rho_i * zn - ln;
-                    if (REFINED) p.d32[r] = (float)(snext[r] - p.sref[r]);
+                    publish32(e + 1, r, (float)(snew - st_sref[lr]));
                 }
+                st_z[lr] = z;
             }
         }
-        cur ^= 1;
-        if (!grid_barrier(p, &s_ok)) return;
+        ++e;
+        if (!(full ? receive64(e) : receive32(e))) return;
 
         const bool is_check = (p.check_interval > 0) && (it % p.check_interval == 0);
-        const bool last = (it == p.max_iter);
         if (!is_check && !last) continue;
 
         // ---------------- residuals (Eqs. primal, dual) ----------------
         unsigned long long* slot = p.red + (checks % 3) * RED_WORDS;
-        if (blockIdx.x == 0 && threadIdx.x < RED_WORDS) p.red[((checks + 1) % 3) * RED_WORDS + threadIdx.x] = 0ull;
+        if (cta == 0 && tid < RED_WORDS) p.red[((checks + 1) % 3) * RED_WORDS + tid] = 0ull;
         ++checks;
-        load_shared_cg(sv, p.y, n);
-        __syncthreads();
-        for (int r = row0 + warp; r < row1; r += kWarps) {
-            if (r < n) {
-                const double v = row_dot(p.P + (size_t)r * n, sv, n, lane);
-                if (lane == 0) {
-                    p.Py[r] = v;
-                    red_max(slot, RED_PX, p.rsx ? v * p.rsx[r] : v);
-                }
+        for (int lr = warp; lr < rows; lr += kWarps) {
+            const int i = a0 + lr - nx;
+            const double v = row_dot<true>(lr < nx ? p.P + (size_t)(x0 + lr) * n : p.A + (size_t)i * n, sv, n, lane);
+            if (lane != 0) continue;
+            st_chk[lr] = v;
+            if (lr < nx) {
+                red_max(s_red, RED_PX, p.rsx ? v * p.rsx[x0 + lr] : v);
             } else {
-                const int i = r - n;
-                const double v = row_dot(p.A + (size_t)i * n, sv, n, lane);
-                if (lane == 0) {
-                    const double zi = p.z[i];
-                    const double rho_i = p.rho[ri] * (double)__ldg(p.rs + i);
-                    const double f = p.rsz ? p.rsz[i] : 1.0;
-                    p.Axf[i] = v;
-                    p.lstd[i] = p.lam[i] + rho_i * (v - zi);
-                    red_max(slot, RED_RP, (v - zi) * f);
-                    red_max(slot, RED_AX, v * f);
-                    red_max(slot, RED_Z, zi * f);
-                }
+                const double zi = st_z[lr], f = p.rsz ? p.rsz[i] : 1.0, ls = st_lam[lr] + st_rho[lr] * (v - zi);
+                st_ls[lr] = ls;
+                p.ls[i] = ls;
+                red_max(s_red, RED_RP, (v - zi) * f);
+                red_max(s_red, RED_AX, v * f);
+                red_max(s_red, RED_Z, zi * f);
             }
         }
-        if (!grid_barrier(p, &s_ok)) return;
-        if (m > 0) load_shared_cg(sv, p.lstd, m);
+        if (!all_arrived()) return;
+        for (int k = tid; k < m; k += kThreads) svk[k] = __ldcg(p.ls + k);
         __syncthreads();
-        for (int j = r2_0 + warp; j < r2_1; j += kWarps) {
-            const double v = (m > 0) ? row_dot(p.At + (size_t)j * m, sv, m, lane) : 0.0;
+        for (int lr = warp; lr < nx; lr += kWarps) {
+            const int j = x0 + lr;
+            const double v = (m > 0) ? row_dot<true>(p.At + (size_t)j * m, svk, m, lane) : 0.0;
             if (lane == 0) {
                 const double f = p.rsx ? p.rsx[j] : 1.0;
-                red_max(slot, RED_RD, (__ldcg(p.Py + j) + __ldg(p.q + j) + v) * f);
-                red_max(slot, RED_ATL, v * f);
+                red_max(s_red, RED_RD, (st_chk[lr] + __ldg(p.q + j) + v) * f);
+                red_max(s_red, RED_ATL, v * f);
             }
         }
-        if (!grid_barrier(p, &s_ok)) return;
+        __syncthreads();
+        if (tid < RED_WORDS) {
+            atomicMax(slot + tid, s_red[tid]);
+            s_red[tid] = 0ull;
+        }
+        if (!all_arrived()) return;
 
-        // ---------------- decision (identical in every CTA) ----------------
-        const double rp = red_get(slot, RED_RP), rd = red_get(slot, RED_RD);
-        const double nAx = red_get(slot, RED_AX), nz = red_get(slot, RED_Z);
-        const double nPx = red_get(slot, RED_PX), nAtl = red_get(slot, RED_ATL);
-        const bool numerical = !(isfinite(rp) && isfinite(rd) && isfinite(nPx) && isfinite(nAtl));
-        const double eps_p = p.eps_abs + p.eps_rel * fmax(nAx, nz);
-        const double eps_d = p.eps_abs + p.eps_rel * fmax(fmax(nPx, nAtl), p.qnorm);
-        const bool converged = is_check && !numerical && rp <= eps_p && rd <= eps_d;
-        if (converged || numerical || last) {
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
-                p.out_i[OUT_STATUS] = numerical ? RELU_QP_NUMERICAL : (converged ? RELU_QP_SOLVED : RELU_QP_MAX_ITER);
+        // ---------------- decision (identical in every CTA; one warp's FP64) ----------------
+        if (warp == 0) {
+            const double rp = red_get(slot, RED_RP), rd = red_get(slot, RED_RD);
+            const double nAx = red_get(slot, RED_AX), nz = red_get(slot, RED_Z);
+            const double nPx = red_get(slot, RED_PX), nAtl = red_get(slot, RED_ATL);
+            const bool numerical = !(isfinite(rp) && isfinite(rd) && isfinite(nPx) && isfinite(nAtl));
+            const double eps_p = p.eps_abs + p.eps_rel * fmax(nAx, nz);
+            const double eps_d = p.eps_abs + p.eps_rel * fmax(fmax(nPx, nAtl), p.qnorm);
+            const bool converged = is_check && !numerical && rp <= eps_p && rd <= eps_d;
+            int nri = ri;
+            if (p.adaptive && is_check && !converged && !numerical) {
+                // Eq. rho_update (inf-norms, 1e-4 floors), nearest bank entry in log distance
+                const double num = rp * fmax(fmax(nPx, nAtl), fmax(p.qnorm, 1e-4));
+                const double den = rd * fmax(fmax(nAx, nz), 1e-4);
+                if (num > 0.0 && den > 0.0) nri = nearest_entry(p.rho, p.nr, ri, p.rho[ri] * p.rho[ri] * (num / den));
+            }
+            if (lane == 0) {
+                s_dec[RED_RP] = rp;
+                s_dec[RED_RD] = rd;
+                s_dec[DEC_STOP] = numerical ? 1 + RELU_QP_NUMERICAL : converged ? 1 + RELU_QP_SOLVED : last ? 1 + RELU_QP_MAX_ITER : 0;
+                s_dec[DEC_RHO] = nri;
+            }
+        }
+        __syncthreads();
+        const int stop = (int)s_dec[DEC_STOP], nri = (int)s_dec[DEC_RHO];
+        if (stop) {
+            for (int lr = tid; lr < rows; lr += kThreads) {
+                if (lr < nx) {
+                    p.xo[x0 + lr] = st_z[lr];
+                } else {
+                    p.zo[a0 + lr - nx] = st_z[lr];
+                    p.lo[a0 + lr - nx] = st_ls[lr];
+                }
+            }
+            if (cta == 0 && tid == 0) {
+                p.out_i[OUT_STATUS] = stop - 1;
                 p.out_i[OUT_ITERS] = it;
                 p.out_i[OUT_RHO] = ri;
                 p.out_i[OUT_SWITCHES] = switches;
-                p.out_f[0] = rp;
-                p.out_f[1] = rd;
+                p.out_i[OUT_COUNTED] = (int)counted;
+                p.out_i[OUT_LAST] = (int)e;
+                p.out_f[0] = s_dec[RED_RP];
+                p.out_f[1] = s_dec[RED_RD];
             }
             return;
         }
-        // the directly computed Ax replaces the carried one
-        for (int r = max(row0, n) + threadIdx.x; r < row1; r += blockDim.x) p.Ay[r - n] = p.Axf[r - n];
-        if (!p.adaptive || !is_check) continue;
-        // Eq. rho_update (inf-norms, 1e-4 floors), nearest bank entry in log distance
-        const double num = rp * fmax(fmax(nPx, nAtl), fmax(p.qnorm, 1e-4));
-        const double den = rd * fmax(fmax(nAx, nz), 1e-4);
-        int nri = ri;
-        if (num > 0.0 && den > 0.0) {
-            const double est = p.rho[ri] * sqrt(num / den);
-            if (isfinite(est) && est > 0.0) {
-                const double le = log(est);
-                double best = 1e300;
-                for (int k = 0; k < p.nr; ++k) {
-                    const double d = fabs(le - log(p.rho[k]));
-                    if (d < best) {
-                        best = d;
-                        nri = k;
-                    }
-                }
+        if (nri == ri) {
+            // the directly computed Ax replaces the carried one
+            for (int lr = nx + tid; lr < rows; lr += kThreads)
+                st_rr[lr] = st_chk[lr] - st_z[lr] + st_lam[lr] / st_rho[lr];
+            if (p.share) {
+                if (!receive64(e)) return;   // (lam_std was staged over the operand)
+            } else {
+                __syncthreads();
             }
+            continue;
         }
-        if (nri == ri) continue;
         // switch: rebase lam' so that the next layer is standard ADMM with the new rho
-        double* scur2 = cur ? p.s1 : p.s0;
-        for (int r = max(row0, n) + threadIdx.x; r < row1; r += blockDim.x) {
-            const int i = r - n;
-            const double rho_i = p.rho[nri] * (double)__ldg(p.rs + i);
-            const double zi = p.z[i];
-            const double lnew = p.lstd[i] - rho_i * (p.Axf[i] - zi);
-            p.lam[i] = lnew;
-            scur2[r] = 2.0 * rho_i * zi - lnew;
-        }
         ri = nri;
         ++switches;
-        if (!grid_barrier(p, &s_ok)) return;
-    }
-}
-
-// Start state: x given (or 0), z = A x, carried Ax = A x, lam' = lam (or 0),
-// s0 = [x; 2 rho z - lam'] for the starting bank entry.
-__global__ void init64_kernel(int n, int m, const double* __restrict__ A, const double* __restrict__ xin,
-                              const double* __restrict__ lin, const float* __restrict__ rs, double rho, double* y,
-                              double* z, double* lam, double* Ay, double* s0) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int r = warp; r < n + m; r += nw) {
-        if (r < n) {
-            if (lane == 0) {
-                const double v = xin ? xin[r] : 0.0;
-                y[r] = v;
-                s0[r] = v;
+        for (int lr = tid; lr < rows; lr += kThreads) {
+            const int r = row_of(lr);
+            double v = st_z[lr];
+            if (lr >= nx) {
+                const double rho_i = p.rho[ri] * (double)__ldg(p.rs + (r - n)), d = st_chk[lr] - v;
+                const double lnew = st_ls[lr] - rho_i * d;
+                st_lam[lr] = lnew;
+                st_rho[lr] = rho_i;
+                st_rr[lr] = d + lnew / rho_i;
+                v = 2.0 * rho_i * v - lnew;
             }
-        } else {
-            const int i = r - n;
-            double v = 0.0;
-            if (xin) {
-                for (int k = lane; k < n; k += 32) v = fma(A[(size_t)i * n + k], xin[k], v);
-                v = warp_sum(v);
-            }
-            if (lane == 0) {
-                const double li = lin ? lin[i] : 0.0;
-                const double rho_i = rho * (double)rs[i];
-                z[i] = v;
-                Ay[i] = v;
-                lam[i] = li;
-                s0[r] = 2.0 * rho_i * v - li;
-            }
+            publish64(e + 1, r, v);
         }
+        load_bank();
+        ++e;
+        if (!receive64(e)) return;
     }
 }
 
-// out[r] = sum_k M[r][k] x[k] (row-major, ld = cols), one warp per row.
-__global__ void matvec64_kernel(const double* __restrict__ M, int rows, int cols, const double* __restrict__ x,
-                                double* __restrict__ out) {
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int r = warp; r < rows; r += nw) {
-        double v = 0.0;
-        for (int k = lane; k < cols; k += 32) v = fma(M[(size_t)r * cols + k], x[k], v);
-        v = warp_sum(v);
-        if (lane == 0) out[r] = v;
-    }
+// b_r = Bop_r q for every bank entry (blockIdx.y), one warp per row.
+struct Bias64 {
+    const double* Bop[RQ_MAX_RHO];
+    double* bias[RQ_MAX_RHO];
+};
+
+__global__ void __launch_bounds__(256) bias64_kernel(Bias64 b, int rows, int n, const double* __restrict__ q) {
+    const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (r >= rows) return;
+    const double* w = b.Bop[blockIdx.y] + (size_t)r * n;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    int k = lane;
+    for (; k + 96 < n; k += 128)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) a[t] = fma(__ldg(w + k + 32 * t), __ldg(q + k + 32 * t), a[t]);
+    for (; k < n; k += 32) a[0] = fma(__ldg(w + k), __ldg(q + k), a[0]);
+    const double v = warp_sum((a[0] + a[1]) + (a[2] + a[3]));
+    if (lane == 0) b.bias[blockIdx.y][r] = v;
 }
 
-void fill_params(relu_qp_t h, SP64& p, int grid) {
+bool refined(relu_qp_t h) { return h->opts.single_precision == RELU_QP_PREC_FP64R; }
+// (an FP64 exchange is 2 R words; the refined form's common exchange R)
+bool tagged(relu_qp_t h) { return (refined(h) ? 1 : 2) * h->R <= kTagMax; }
+bool share_lam(relu_qp_t h) { return h->R + h->m > 20000; }
+
+const void* kernel_for(relu_qp_t h) {
+    if (refined(h)) return tagged(h) ? (const void*)single64_kernel<true, true> : (const void*)single64_kernel<true, false>;
+    return tagged(h) ? (const void*)single64_kernel<false, true> : (const void*)single64_kernel<false, false>;
+}
+
+// bytes of a cached row, and of everything else
+size_t row_bytes(relu_qp_t h) { return refined(h) ? sizeof(float) * h->ldw : sizeof(double) * h->R; }
+size_t smem64(relu_qp_t h, int grid, int cached) {
+    const size_t per = ceil_div(h->n, grid) + (h->m > 0 ? ceil_div(h->m, grid) : 0);
+    const size_t op = round_up(std::max(h->R, (h->ldw + 1) / 2), 2), lam = share_lam(h) ? 0 : round_up(h->m, 2);
+    return sizeof(double) * (op + lam + round_up(kState * per, 2)) + round_up(cached * row_bytes(h), 16);
+}
+
+int reset_words(relu_qp_t h) {
+    SingleWork64& w = h->sw64;
+    RQ_CUDA(h, cudaMemsetAsync(w.words, 0, sizeof(unsigned long long) * 4 * h->R, h->stream));
+    RQ_CUDA(h, cudaMemsetAsync(w.count, 0, sizeof(unsigned) * 4, h->stream));
+    w.tag = w.counted = 0;
+    return RELU_QP_OK;
+}
+
+int launch(relu_qp_t h, int grid, const double* xin, const double* lin, int rho_index, double eps_abs, double eps_rel,
+           int max_iter, int check_interval, int adaptive) {
+    SingleWork64& w = h->sw64;
+    if (w.tag > 0xC0000000u) RQ_TRY(reset_words(h));
+    SP64 p{};
     p.n = h->n;
     p.m = h->m;
     p.R = h->R;
     p.nr = h->nr;
     p.ldw = h->ldw;
     p.anchor_every = h->opts.check_interval > 0 ? h->opts.check_interval : 25;
-    p.c = h->sw64.c;
-    p.sref = h->sw64.sref;
-    p.d32 = h->sw64.d32;
     for (int r = 0; r < h->nr; ++r) {
         p.Wt32[r] = h->be[r].Wt;
         p.Wt[r] = h->be[r].Wt64;
@@ -363,58 +480,55 @@ void fill_params(relu_qp_t h, SP64& p, int grid) {
     p.q = h->q64; p.l = h->l64; p.u = h->u64; p.rs = h->rs32;
     p.rsx = h->sc64_rx;
     p.rsz = h->sc64_z;
-    SingleWork64& w = h->sw64;
-    p.y = w.y; p.z = w.z; p.lam = w.lam; p.Ay = w.Ay; p.s0 = w.s0; p.s1 = w.s1;
-    p.Py = w.Py; p.Axf = w.Axf; p.lstd = w.lstd;
-    p.red = w.red; p.bar = w.bar; p.out_i = w.out_i; p.out_f = w.out_f;
-    p.rows_per_cta = ceil_div(h->R, grid);
-    p.rows2_per_cta = ceil_div(h->n, grid);
-    p.timeout_ns = 2000000000LL;
-    p.qnorm = h->qnorm;
-}
-
-// the operand in shared memory: R doubles, or (refined layers) ldw floats of the increment
-size_t smem64(relu_qp_t h) {
-    return std::max(sizeof(double) * (size_t)h->R, sizeof(float) * (size_t)h->ldw);
-}
-
-bool refined(relu_qp_t h) { return h->opts.single_precision == RELU_QP_PREC_FP64R; }
-
-const void* kernel_for(relu_qp_t h) {
-    return refined(h) ? (const void*)single64_kernel<true> : (const void*)single64_kernel<false>;
-}
-
-int init_state(relu_qp_t h, const double* x, const double* lam, int rho_index) {
-    SingleWork64& w = h->sw64;
-    const int R = h->R;
-    // s1 and the padding of s0 start at zero
-    RQ_CUDA(h, cudaMemsetAsync(w.s1, 0, sizeof(double) * R, h->stream));
-    const int blocks = std::max(1, std::min(1024, ceil_div(R * 32, 256)));
-    init64_kernel<<<blocks, 256, 0, h->stream>>>(h->n, h->m, h->A64, x, lam, h->rs32, h->be[rho_index].rho, w.y, w.z,
-                                                 w.lam, w.Ay, w.s0);
-    RQ_CUDA(h, cudaGetLastError());
-    return RELU_QP_OK;
-}
-
-int launch(relu_qp_t h, int grid, int rho_index, double eps_abs, double eps_rel, int max_iter, int check_interval,
-           int adaptive) {
-    SP64 p{};
-    fill_params(h, p, grid);
+    p.xin = xin;
+    p.lin = lin;
+    p.xo = w.out;
+    p.zo = w.out + h->n;
+    p.lo = w.out + h->n + h->m;
+    p.wop = w.words;
+    p.ls = w.lstd;
+    p.red = w.red;
+    p.count = w.count;
+    p.err = reinterpret_cast<int*>(w.count + 2);
+    p.count0 = w.counted;
+    p.tag0 = w.tag;
+    p.out_i = w.out_i;
+    p.out_f = w.out_f;
     p.rho_index0 = rho_index;
     p.check_interval = check_interval;
     p.adaptive = adaptive;
     p.max_iter = max_iter;
     p.eps_abs = eps_abs;
     p.eps_rel = eps_rel;
-    SingleWork64& w = h->sw64;
+    p.qnorm = h->qnorm;
+    p.xr = ceil_div(h->n, grid);
+    p.ar = h->m > 0 ? ceil_div(h->m, grid) : 0;
+    p.ctas = std::max(ceil_div(h->n, p.xr), p.ar > 0 ? ceil_div(h->m, p.ar) : 0);
+    p.share = share_lam(h) ? 1 : 0;
+    p.timeout_ns = 2000000000LL;
+    // the rows of the bank that fit beside the rest
+    const size_t room = w.smem_max - smem64(h, grid, 0);
+    p.cached = (int)std::min<size_t>(p.xr + p.ar, room / row_bytes(h));
+    const size_t smem = smem64(h, grid, p.cached);
+    w.last_ctas = p.ctas;
+    w.out_i[OUT_LAST] = -1;   // the kernel's results go to host memory
     RQ_CUDA(h, cudaMemsetAsync(w.red, 0, sizeof(unsigned long long) * 3 * RED_WORDS, h->stream));
-    RQ_CUDA(h, cudaMemsetAsync(w.bar, 0, sizeof(unsigned) * 2, h->stream));
-    RQ_CUDA(h, cudaMemsetAsync(w.out_i, 0, sizeof(int) * OUT_WORDS, h->stream));
-    const size_t smem = smem64(h);
     RQ_CUDA(h, cudaFuncSetAttribute(kernel_for(h), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     void* args[] = {&p};
-    RQ_CUDA(h, cudaLaunchCooperativeKernel(kernel_for(h), dim3(grid), dim3(kThreads), args, smem,
-                                           h->stream));
+    RQ_CUDA(h, cudaLaunchCooperativeKernel(kernel_for(h), dim3(grid), dim3(kThreads), args, smem, h->stream));
+    return RELU_QP_OK;
+}
+
+// After the launch has been waited for: its error, or the next free exchange numbers.
+int finish(relu_qp_t h, const char* what) {
+    SingleWork64& w = h->sw64;
+    if (w.out_i[OUT_LAST] < 0) {
+        RQ_TRY(reset_words(h));
+        RQ_CUDA(h, cudaStreamSynchronize(h->stream));
+        return fail(h, RELU_QP_ERR_TIMEOUT, std::string("a wait passed its deadline ") + what);
+    }
+    w.tag += (unsigned)w.out_i[OUT_LAST] + 2u;
+    w.counted += (unsigned)w.out_i[OUT_COUNTED] * (unsigned)w.last_ctas;
     return RELU_QP_OK;
 }
 
@@ -428,18 +542,23 @@ int single64_alloc(relu_qp_t h, const double* P, const double* A) {
     RQ_TRY(alloc(h, &h->P64, (size_t)n * n));
     RQ_TRY(alloc(h, &h->A64, (size_t)mm * n));
     RQ_TRY(alloc(h, &h->At64, (size_t)n * mm));
-    RQ_TRY(alloc(h, &h->q64, (size_t)n));
-    RQ_TRY(alloc(h, &h->l64, (size_t)mm));
-    RQ_TRY(alloc(h, &h->u64, (size_t)mm));
+    RQ_TRY(alloc(h, &h->q64, (size_t)n + 2 * (size_t)m));   // q, l, u
+    h->l64 = h->q64 + n;
+    h->u64 = h->l64 + m;
     for (int r = 0; r < h->nr; ++r) RQ_TRY(alloc(h, &h->be[r].bias64, (size_t)R));
     SingleWork64& w = h->sw64;
-    for (double** v : {&w.y, &w.z, &w.lam, &w.Ay, &w.s0, &w.s1, &w.Py, &w.Axf, &w.lstd, &w.xin, &w.lin, &w.c, &w.sref})
-        RQ_TRY(alloc(h, v, (size_t)R));
-    RQ_TRY(alloc(h, &w.d32, (size_t)h->ldw));   // zero beyond R (set once here)
+    RQ_TRY(alloc(h, &w.words, 4 * (size_t)R));
+    RQ_TRY(alloc(h, &w.lstd, (size_t)mm));
+    RQ_TRY(alloc(h, &w.in, (size_t)R));
     RQ_TRY(alloc(h, &w.red, 3 * RED_WORDS));
-    RQ_TRY(alloc(h, &w.bar, 2));
-    RQ_TRY(alloc(h, &w.out_i, OUT_WORDS));
-    RQ_TRY(alloc(h, &w.out_f, 8));
+    RQ_TRY(alloc(h, &w.count, 4));
+    // pinned: staging of q, l, u, staging of a warm start, the results the kernel writes
+    const size_t doubles = 2 * ((size_t)n + 2 * m) + (size_t)R + 2 * RED_WORDS;
+    RQ_CUDA(h, cudaHostAlloc(reinterpret_cast<void**>(&w.pin), sizeof(double) * doubles, cudaHostAllocDefault));
+    w.pin_in = w.pin + n + 2 * (size_t)m;
+    w.out = w.pin_in + R;
+    w.out_f = w.out + n + 2 * (size_t)m;
+    w.out_i = reinterpret_cast<int*>(w.out_f + RED_WORDS);
     RQ_CUDA(h, cudaMemcpy(h->P64, P, sizeof(double) * n * n, cudaMemcpyHostToDevice));
     if (m > 0) {
         std::vector<double> At((size_t)n * m);
@@ -460,56 +579,56 @@ int single64_alloc(relu_qp_t h, const double* P, const double* A) {
     return RELU_QP_OK;
 }
 
-int single64_upload(relu_qp_t h, const double* q, const double* l, const double* u) {
-    const int n = h->n, m = h->m, R = h->R;
-    RQ_CUDA(h, cudaMemcpyAsync(h->q64, q, sizeof(double) * n, cudaMemcpyHostToDevice, h->stream));
-    if (m > 0) {
-        RQ_CUDA(h, cudaMemcpyAsync(h->l64, l, sizeof(double) * m, cudaMemcpyHostToDevice, h->stream));
-        RQ_CUDA(h, cudaMemcpyAsync(h->u64, u, sizeof(double) * m, cudaMemcpyHostToDevice, h->stream));
-    }
-    const int blocks = std::max(1, std::min(2048, ceil_div(R * 32, 256)));
+void single64_release(relu_qp_t h) {
+    if (h->sw64.pin) cudaFreeHost(h->sw64.pin);
+    h->sw64.pin = nullptr;
+}
+
+int single64_update(relu_qp_t h) {
+    RQ_CUDA(h, cudaMemcpyAsync(h->q64, h->sw64.pin, sizeof(double) * (h->n + 2 * (size_t)h->m), cudaMemcpyHostToDevice,
+                               h->stream));
+    Bias64 b{};
     for (int r = 0; r < h->nr; ++r) {
-        matvec64_kernel<<<blocks, 256, 0, h->stream>>>(h->be[r].Bop64, R, n, h->q64, h->be[r].bias64);
-        RQ_CUDA(h, cudaGetLastError());
+        b.Bop[r] = h->be[r].Bop64;
+        b.bias[r] = h->be[r].bias64;
     }
-    // the host arrays are the caller's temporaries: finish the copies before returning
-    RQ_CUDA(h, cudaStreamSynchronize(h->stream));
+    bias64_kernel<<<dim3(ceil_div(h->R, 8), h->nr), 256, 0, h->stream>>>(b, h->R, h->n, h->q64);
+    RQ_CUDA(h, cudaGetLastError());
     return RELU_QP_OK;
 }
 
-// CTA count of the cooperative launch: the fastest of the co-resident
-// candidates over 50 fixed-rho layers (no checks).
+// CTA count of the cooperative launch: the fastest of the co-resident candidates over 50
+// fixed-rho layers (no checks), the largest first, until one is 1.3x slower than the best.
 int single64_prepare(relu_qp_t h) {
-    int per_sm = 0;
-    const size_t smem = smem64(h);
-    RQ_CUDA(h, cudaFuncSetAttribute(kernel_for(h), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    RQ_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel_for(h), kThreads, smem));
-    if (per_sm < 1) return fail(h, RELU_QP_ERR_UNSUPPORTED, "FP64 solve kernel does not fit on an SM");
-    std::vector<int> cands;
-    for (int g = 1; g <= h->num_sms; g *= 2) cands.push_back(g);
-    cands.push_back(h->num_sms);
-    int best_g = 1;
+    SingleWork64& w = h->sw64;
+    cudaFuncAttributes fa{};
+    RQ_CUDA(h, cudaFuncGetAttributes(&fa, kernel_for(h)));
+    int v = 0;
+    RQ_CUDA(h, cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
+    w.smem_max = (size_t)v - fa.sharedSizeBytes - 256;
+    std::vector<int> cands{h->num_sms};
+    for (int g = 1; g < h->num_sms; g *= 2) cands.push_back(g);
+    std::sort(cands.begin(), cands.end(), std::greater<int>());
+    w.grid = 0;
     float best_t = 1e30f;
     for (int g : cands) {
-        if (g > h->R || g > per_sm * h->num_sms) continue;
-        RQ_TRY(init_state(h, nullptr, nullptr, 0));
-        RQ_TRY(launch(h, g, 0, 0.0, 0.0, 10, 0, 0));   // warm-up
-        RQ_TRY(init_state(h, nullptr, nullptr, 0));
-        RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
-        RQ_TRY(launch(h, g, 0, 0.0, 0.0, 50, 0, 0));
-        RQ_CUDA(h, cudaEventRecord(h->ev1, h->stream));
-        RQ_CUDA(h, cudaStreamSynchronize(h->stream));
-        int err = 0;
-        RQ_CUDA(h, cudaMemcpy(&err, h->sw64.out_i + OUT_ERR, sizeof(int), cudaMemcpyDeviceToHost));
-        if (err) return fail(h, RELU_QP_ERR_TIMEOUT, "grid barrier deadline passed while tuning the FP64 solve");
+        if (g > h->R || smem64(h, g, 0) > w.smem_max) continue;
         float ms = 0.f;
-        RQ_CUDA(h, cudaEventElapsedTime(&ms, h->ev0, h->ev1));
+        for (int layers : {10, 50}) {   // a warm-up, then the timed run
+            RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
+            RQ_TRY(launch(h, g, nullptr, nullptr, 0, 0.0, 0.0, layers, 0, 0));
+            RQ_CUDA(h, cudaEventRecord(h->ev1, h->stream));
+            RQ_CUDA(h, cudaStreamSynchronize(h->stream));
+            RQ_TRY(finish(h, "while tuning the FP64 solve"));
+            RQ_CUDA(h, cudaEventElapsedTime(&ms, h->ev0, h->ev1));
+        }
+        if (ms > 1.3f * best_t) break;
         if (ms < best_t) {
             best_t = ms;
-            best_g = g;
+            w.grid = g;
         }
     }
-    h->sw64.grid = best_g;
+    if (w.grid == 0) return fail(h, RELU_QP_ERR_UNSUPPORTED, "FP64 solve kernel does not fit on an SM");
     return RELU_QP_OK;
 }
 
@@ -517,41 +636,32 @@ int single64_solve(relu_qp_t h, const double* x_warm, const double* lam_warm, in
                    double eps_rel, int max_iter, double* x_out, double* z_out, double* lam_out,
                    relu_qp_info* info) {
     SingleWork64& w = h->sw64;
-    const int n = h->n, m = h->m;
-    const double* xin = nullptr;
-    const double* lin = nullptr;
+    const size_t n = h->n, m = h->m;
+    const bool lam = x_warm && lam_warm && m > 0;
     if (x_warm) {
-        RQ_CUDA(h, cudaMemcpyAsync(w.xin, x_warm, sizeof(double) * n, cudaMemcpyHostToDevice, h->stream));
-        xin = w.xin;
-        if (lam_warm && m > 0) {
-            RQ_CUDA(h, cudaMemcpyAsync(w.lin, lam_warm, sizeof(double) * m, cudaMemcpyHostToDevice, h->stream));
-            lin = w.lin;
-        }
+        std::memcpy(w.pin_in, x_warm, sizeof(double) * n);
+        if (lam) std::memcpy(w.pin_in + n, lam_warm, sizeof(double) * m);
+        RQ_CUDA(h, cudaMemcpyAsync(w.in, w.pin_in, sizeof(double) * (n + (lam ? m : 0)), cudaMemcpyHostToDevice, h->stream));
     }
-    RQ_TRY(init_state(h, xin, lin, rho_index));
     RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
-    RQ_TRY(launch(h, w.grid, rho_index, eps_abs, eps_rel, max_iter, h->opts.check_interval, h->opts.adaptive_rho));
-    h->launches += 2;
+    RQ_TRY(launch(h, w.grid, x_warm ? w.in : nullptr, lam ? w.in + n : nullptr, rho_index, eps_abs, eps_rel, max_iter,
+                  h->opts.check_interval, h->opts.adaptive_rho));
+    h->launches += 1;
     RQ_CUDA(h, cudaEventRecord(h->ev1, h->stream));
-    int oi[OUT_WORDS];
-    double of[2];
-    RQ_CUDA(h, cudaMemcpyAsync(oi, w.out_i, sizeof(oi), cudaMemcpyDeviceToHost, h->stream));
-    RQ_CUDA(h, cudaMemcpyAsync(of, w.out_f, sizeof(of), cudaMemcpyDeviceToHost, h->stream));
-    RQ_CUDA(h, cudaMemcpyAsync(x_out, w.y, sizeof(double) * n, cudaMemcpyDeviceToHost, h->stream));
-    if (z_out && m > 0) RQ_CUDA(h, cudaMemcpyAsync(z_out, w.z, sizeof(double) * m, cudaMemcpyDeviceToHost, h->stream));
-    if (lam_out && m > 0)
-        RQ_CUDA(h, cudaMemcpyAsync(lam_out, w.lstd, sizeof(double) * m, cudaMemcpyDeviceToHost, h->stream));
     RQ_CUDA(h, cudaStreamSynchronize(h->stream));
-    if (oi[OUT_ERR]) return fail(h, RELU_QP_ERR_TIMEOUT, "grid barrier deadline passed in the FP64 solve");
+    RQ_TRY(finish(h, "in the FP64 solve"));
+    std::memcpy(x_out, w.out, sizeof(double) * n);
+    if (z_out && m > 0) std::memcpy(z_out, w.out + n, sizeof(double) * m);
+    if (lam_out && m > 0) std::memcpy(lam_out, w.out + n + m, sizeof(double) * m);
     if (info) {
         float ms = 0.f;
         cudaEventElapsedTime(&ms, h->ev0, h->ev1);
-        info->status = oi[OUT_STATUS];
-        info->iters = oi[OUT_ITERS];
-        info->rho_index = oi[OUT_RHO];
-        info->rho_switches = oi[OUT_SWITCHES];
-        info->r_prim = of[0];
-        info->r_dual = of[1];
+        info->status = w.out_i[OUT_STATUS];
+        info->iters = w.out_i[OUT_ITERS];
+        info->rho_index = w.out_i[OUT_RHO];
+        info->rho_switches = w.out_i[OUT_SWITCHES];
+        info->r_prim = w.out_f[0];
+        info->r_dual = w.out_f[1];
         info->solve_ms = ms;
     }
     return RELU_QP_OK;

@@ -195,3 +195,36 @@ def test_fp64_anchored_with_scaling(rq):
     assert res["r_prim"] <= EPS * (1 + 1e-6) and res["r_dual"] <= EPS * (1 + 1e-6)
     assert abs(out["iters"] - orc.iters) <= 25
     assert np.max(np.abs(out["x"] - orc.x)) <= 1e-5
+
+
+@pytest.mark.parametrize("n,m,eq", [(1, 0, 0), (3, 2, 1), (20, 0, 0), (33, 7, 2), (200, 310, 9), (700, 900, 20), (1100, 1000, 30)])
+def test_fp64_forms_on_ragged_sizes(rq, n, m, eq):
+    """Both FP64 forms where rows do not divide over the CTAs, without constraint rows, and on
+    both sides of the tagged exchanges' limits (2048 words: n + m = 1024 in FP64, 2048 anchored):
+    fixed layers against the oracle's iterates, and warm-started solves with checks every layer."""
+    rng = np.random.default_rng([4, n, m])
+    M = rng.standard_normal((n, n))
+    P = M @ M.T / n + 0.5 * np.eye(n)
+    A = rng.standard_normal((m, n)) / np.sqrt(n)
+    q = 2.0 * rng.standard_normal(n)
+    l, u = -rng.uniform(0.1, 1.0, m), rng.uniform(0.1, 1.0, m)
+    l[:eq] = u[:eq]
+    bank = (0.1, 1.0, 10.0)
+    ref = O.layer_iterates(P, q, A, l, u, 1e-6, bank[0], 30)[-1] if n + m < 1200 else None
+    for prec, tol in ((rq.PREC_FP64, 1e-11), (rq.PREC_FP64R, 1e-6)):
+        s = rq.ReluQP(P, A if m else None, l, u, q=q, sigma=1e-6, rho_bank=bank, check_interval=0, single_precision=prec)
+        o = s.solve(eps_abs=0.0, max_iter=30)
+        if ref is not None:
+            got = np.concatenate([o["x"], o["z"]])
+            assert np.max(np.abs(got - ref[:n + m])) <= tol * np.max(np.abs(ref[:n + m])), prec
+        s.set_opts(check_interval=25)
+        cold = s.solve(eps_abs=1e-6)
+        s.set_opts(check_interval=1)
+        warm = s.solve(x_warm=cold["x"], lam_warm=cold["lam"], rho_index=cold["rho_index"], eps_abs=1e-6)
+        s.close()
+        for r in (cold, warm):
+            assert r["status"] == rq.SOLVED
+            assert np.max(np.abs(P @ r["x"] + q + A.T @ r["lam"])) <= 1.01e-6
+            if m:
+                assert np.max(np.abs(A @ r["x"] - r["z"])) <= 1.01e-6
+        assert warm["iters"] <= 25 and np.max(np.abs(warm["x"] - cold["x"])) <= 1e-4
