@@ -23,11 +23,8 @@
 //   F_j = (sum_{a = 0}^{N-1-j} V_a Abar^a) Abar^j,  V_a = T_a^T Q Abar - U_a^T R K.
 //
 // K: the Riccati iteration X <- Q + A^T X (A - B K(X)), K(X) = (R + B^T X B)^{-1} B^T X A,
-// run until max|X+ - X| <= 1e-13 max(1, max|X+|).  Where Q >= 0 and R > 0 its iterates are
-// first doubled (structure-preserving doubling, Chu, Fan, Lin and Wang 2004): H_k is the
-// iterate after 2^k steps, so that 128 steps take 7 doublings; one plain step from the
-// result, corrected by one Newton step, then has to meet the same test.  Everything else, and a doubling that does not
-// get there, takes the plain iteration from X = Q, with its results and errors.
+// run until max|X+ - X| <= 1e-13 max(1, max|X+|), 16 steps between the host's looks.  Up to
+// kOneMaxX states the 16 steps are one launch of one cluster (riccati_kernel).
 #include "common.h"
 
 #include <algorithm>
@@ -122,104 +119,166 @@ __global__ void prefix_kernel(const double* __restrict__ Y, const double* __rest
     }
 }
 
-// Winv = (I + W)^{-1} (n x n, n <= kGaussMax) in one CTA: in-place Gauss-Jordan
-// elimination with row pivoting in shared memory.  A thread keeps its column (j = lane +
-// 32 c) while it walks down the rows, so an element costs two shared reads, an FMA and a
-// store; rows are exchanged by name (piv) and moved once at the end.  Bound by the FP64
-// pipe of one SM (n^3 FMAs at two a clock, 52 us at n = 60) and three barriers a step.
-// (226 us a call at n = 60; 279 with a division per element for its row and column.)  A singular matrix
-// leaves infinities or NaN, which the caller's convergence test sees.
-constexpr int kGaussMax = 160;
-constexpr int kGaussThreads = 512;
+// `steps` steps of the Riccati iteration (X in X[0], then X[1], ..) by one cluster of 16
+// CTAs, or (steps = 0) K of X[0] alone.  The matrices stay in L2; a thread forms one entry
+// of a product, with a hardware cluster barrier between products.  R + B^T X B is inverted
+// by every CTA for itself (Gauss-Jordan, one barrier a step, the next pivot's reciprocal
+// taken by the thread that has it); a pivot <= 0 sets *flag and counts as 1, as in the
+// blocked Cholesky.  Bound by the FP64 pipes of 16 SMs (0.7 M FMAs a step at nx = 60,
+// nu = 20: 11 us), the inverse's 20 dependent steps and eight barriers: 51 us a step with a
+// product's entries dealt out CTA by CTA.  A launch per product took 75 us.
+constexpr int kOneMaxX = 96, kOneMaxU = 48, kOneCtas = 16, kOneThreads = 256;
 
-__global__ void __launch_bounds__(kGaussThreads) gauss_inverse_kernel(const double* __restrict__ W, int n,
-                                                                      double* __restrict__ Winv) {
-    extern __shared__ double gsm[];
-    __shared__ double col[kGaussMax], row[kGaussMax];
-    __shared__ int piv[kGaussMax], used[kGaussMax];   // step k's row; whether a row has been one
-    __shared__ double s_inv;
-    const int ld = n | 1, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int kW = kGaussThreads / 32;
-    for (int i = warp; i < n; i += kW)
-        for (int j = lane; j < n; j += 32) gsm[i * ld + j] = W[(size_t)i * n + j] + (i == j ? 1.0 : 0.0);
-    for (int i = tid; i < n; i += kGaussThreads) used[i] = 0;
-    __syncthreads();
-    for (int k = 0; k < n; ++k) {
-        if (warp == 0) {
-            // the largest element of column k among the rows not used yet (the first of equals)
-            double best = -1.0;
-            int at = n;
-            for (int i = lane; i < n; i += 32) {
-                const double v = used[i] ? -1.0 : fabs(gsm[i * ld + k]);
-                if (v > best) {
-                    best = v;
-                    at = i;
-                }
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                const double v = __shfl_xor_sync(0xffffffffu, best, o);
-                const int a = __shfl_xor_sync(0xffffffffu, at, o);
-                if (v > best || (v == best && a < at)) {
-                    best = v;
-                    at = a;
-                }
-            }
-            if (at >= n) {   // only NaN left: any unused row
-                at = 0;
-                while (at < n - 1 && used[at]) ++at;
-            }
-            if (lane == 0) {
-                piv[k] = at;
-                used[at] = 1;
-                s_inv = 1.0 / gsm[at * ld + k];
-            }
-        }
-        __syncthreads();
-        const int p = piv[k];
-        const double inv = s_inv;
-        // minus column k, and row p times the inverse pivot
-        if (tid < kGaussThreads / 2) {
-            for (int i = tid; i < n; i += kGaussThreads / 2) col[i] = -gsm[i * ld + k];
-        } else {
-            for (int j = tid - kGaussThreads / 2; j < n; j += kGaussThreads / 2) row[j] = j == k ? inv : gsm[p * ld + j] * inv;
-        }
-        __syncthreads();
-        for (int j = lane; j < n; j += 32) {
-            const double r = row[j];
-            for (int i = warp; i < n; i += kW) {
-                double* w = gsm + i * ld + j;
-                *w = i == p ? r : j == k ? col[i] * inv : fma(col[i], r, *w);
-            }
-        }
-        __syncthreads();
-    }
-    // step k worked on row piv[k] and column k: element (piv[i], j) is the inverse's (i, piv[j])
-    for (int i = warp; i < n; i += kW)
-        for (int j = lane; j < n; j += 32) Winv[(size_t)i * n + piv[j]] = gsm[piv[i] * ld + j];
+struct OneArgs {
+    int nx, nu, steps;
+    const double *A, *B, *Q, *R;
+    double *X[2], *BtX, *G, *K0, *K, *T, *XA;
+    unsigned long long* red;
+    int* flag;
+};
+
+__device__ __forceinline__ void cluster_barrier_hw() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// X <- (X + X^T) / 2 (n x n, rows of ld) and, with red, the convergence measures of a
-// Riccati step: red[0] = max |X_new - X_old|, red[1] = max |X_new| (bits of non-negative doubles).
-__global__ void sym_diff_kernel(double* __restrict__ Xn, const double* __restrict__ X, int n, int ld,
+// sum_k a(k) b(k), loads past the L1 (other CTAs write these matrices), in k order
+template <class FA, class FB>
+__device__ __forceinline__ double dot_k(int n, FA a, FB b) {
+    double acc = 0.0;
+    int k = 0;
+    constexpr int U = 12;   // loads in flight: an L2 trip is some 700 clocks
+    for (; k + U <= n; k += U) {
+        double u[U], v[U];
+#pragma unroll
+        for (int t = 0; t < U; ++t) {
+            u[t] = a(k + t);
+            v[t] = b(k + t);
+        }
+#pragma unroll
+        for (int t = 0; t < U; ++t) acc = fma(u[t], v[t], acc);
+    }
+    for (; k < n; ++k) acc = fma(a(k), b(k), acc);
+    return acc;
+}
+
+__global__ void __launch_bounds__(kOneThreads) riccati_kernel(const OneArgs g) {
+    __shared__ double s_g[2][kOneMaxU][kOneMaxU + 1];
+    __shared__ double s_inv[2];
+    // (a product's entries go to the CTAs warp by warp, so that a small one uses every SM)
+    const int nx = g.nx, nu = g.nu, tid = threadIdx.x, gt = ((tid >> 5) * kOneCtas + blockIdx.x) * 32 + (tid & 31);
+    constexpr int NT = kOneCtas * kOneThreads;
+    for (int s = 0; s < (g.steps > 0 ? g.steps : 1); ++s) {
+        const double* X = g.X[s & 1];
+        double* Xn = g.X[(s & 1) ^ 1];
+        // B^T X
+        for (int o = gt; o < nu * nx; o += NT) {
+            const int i = o / nx, j = o % nx;
+            g.BtX[o] = dot_k(nx, [&](int k) { return __ldg(g.B + (size_t)k * nu + i); },
+                             [&](int k) { return __ldcg(X + (size_t)k * nx + j); });
+        }
+        cluster_barrier_hw();
+        // B^T X A and R + B^T X B
+        for (int o = gt; o < nu * (nx + nu); o += NT) {
+            const int i = o / (nx + nu), j = o % (nx + nu);
+            const double v = dot_k(nx, [&](int k) { return __ldcg(g.BtX + (size_t)i * nx + k); },
+                                   [&](int k) { return j < nx ? __ldg(g.A + (size_t)k * nx + j) : __ldg(g.B + (size_t)k * nu + j - nx); });
+            if (j < nx) g.K0[(size_t)i * nx + j] = v;
+            else g.G[(size_t)i * nu + j - nx] = __ldg(g.R + (size_t)i * nu + j - nx) + v;
+        }
+        cluster_barrier_hw();
+        // the inverse of its lower triangle's symmetric matrix, in every CTA
+        auto pivot = [&](double d) {
+            if (!(d > 0.0)) {
+                if (blockIdx.x == 0) atomicExch(g.flag, 1);
+                d = 1.0;
+            }
+            return 1.0 / d;
+        };
+        for (int o = tid; o < nu * nu; o += kOneThreads) {
+            const int i = o / nu, j = o % nu;
+            const double v = __ldcg(g.G + (i >= j ? (size_t)i * nu + j : (size_t)j * nu + i));
+            s_g[0][i][j] = v;
+            if (o == 0) s_inv[0] = pivot(v);
+        }
+        __syncthreads();
+        for (int k = 0; k < nu; ++k) {
+            const double(*a)[kOneMaxU + 1] = s_g[k & 1];
+            double(*b)[kOneMaxU + 1] = s_g[(k & 1) ^ 1];
+            const double inv = s_inv[k & 1];
+            for (int o = tid; o < nu * nu; o += kOneThreads) {
+                const int i = o / nu, j = o % nu;
+                double v;
+                if (i == k) v = j == k ? inv : a[k][j] * inv;
+                else if (j == k) v = -a[i][k] * inv;
+                else v = fma(-a[i][k] * inv, a[k][j], a[i][j]);
+                b[i][j] = v;
+                if (i == k + 1 && j == k + 1) s_inv[(k & 1) ^ 1] = pivot(v);
+            }
+            __syncthreads();
+        }
+        const double(*gi)[kOneMaxU + 1] = s_g[nu & 1];
+        for (int o = gt; o < nu * nx; o += NT) {
+            const int i = o / nx, j = o % nx;
+            g.K[o] = dot_k(nu, [&](int k) { return gi[i][k]; }, [&](int k) { return __ldcg(g.K0 + (size_t)k * nx + j); });
+        }
+        if (g.steps == 0) break;
+        cluster_barrier_hw();
+        // A - B K, X (A - B K), Q + A^T X (A - B K)
+        for (int o = gt; o < nx * nx; o += NT) {
+            const int i = o / nx, j = o % nx;
+            g.T[o] = __ldg(g.A + o) - dot_k(nu, [&](int k) { return __ldg(g.B + (size_t)i * nu + k); },
+                                            [&](int k) { return __ldcg(g.K + (size_t)k * nx + j); });
+        }
+        cluster_barrier_hw();
+        for (int o = gt; o < nx * nx; o += NT) {
+            const int i = o / nx, j = o % nx;
+            g.XA[o] = dot_k(nx, [&](int k) { return __ldcg(X + (size_t)i * nx + k); },
+                            [&](int k) { return __ldcg(g.T + (size_t)k * nx + j); });
+        }
+        cluster_barrier_hw();
+        for (int o = gt; o < nx * nx; o += NT) {
+            const int i = o / nx, j = o % nx;
+            g.T[o] = __ldg(g.Q + o) + dot_k(nx, [&](int k) { return __ldg(g.A + (size_t)k * nx + i); },
+                                            [&](int k) { return __ldcg(g.XA + (size_t)k * nx + j); });
+        }
+        cluster_barrier_hw();
+        // symmetrised, and its change (as sym_diff_kernel)
+        unsigned long long d = 0, mx = 0;
+        for (int o = gt; o < nx * nx; o += NT) {
+            const int i = o / nx, j = o % nx;
+            const double v = 0.5 * (i <= j ? __ldcg(g.T + o) + __ldcg(g.T + (size_t)j * nx + i)
+                                           : __ldcg(g.T + (size_t)j * nx + i) + __ldcg(g.T + o));
+            Xn[o] = v;
+            d = max(d, (unsigned long long)__double_as_longlong(fabs(v - __ldcg(X + o))));
+            mx = max(mx, (unsigned long long)__double_as_longlong(fabs(v)));
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            d = max(d, __shfl_xor_sync(0xffffffffu, d, o));
+            mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        }
+        if ((tid & 31) == 0) {
+            atomicMax(g.red + 2 * s, d);
+            atomicMax(g.red + 2 * s + 1, mx);
+        }
+        cluster_barrier_hw();
+    }
+    cluster_barrier_hw();
+}
+
+// X <- (X + X^T) / 2 (n x n) and the convergence measures of the Riccati step:
+// red[0] = max |X_new - X_old|, red[1] = max |X_new| (bits of non-negative doubles).
+__global__ void sym_diff_kernel(double* __restrict__ Xn, const double* __restrict__ X, int n,
                                 unsigned long long* red) {
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n * n; e += gridDim.x * blockDim.x) {
         const int i = e / n, j = e % n;
         if (j < i) continue;
-        const double v = 0.5 * (Xn[(size_t)i * ld + j] + Xn[(size_t)j * ld + i]);
-        Xn[(size_t)i * ld + j] = v;
-        Xn[(size_t)j * ld + i] = v;
-        if (!red) continue;
-        const double d = fmax(fabs(v - X[(size_t)i * ld + j]), fabs(v - X[(size_t)j * ld + i]));
+        const double v = 0.5 * (Xn[(size_t)i * n + j] + Xn[(size_t)j * n + i]);
+        Xn[(size_t)i * n + j] = v;
+        Xn[(size_t)j * n + i] = v;
+        const double d = fmax(fabs(v - X[(size_t)i * n + j]), fabs(v - X[(size_t)j * n + i]));
         atomicMax(red, (unsigned long long)__double_as_longlong(d));
         atomicMax(red + 1, (unsigned long long)__double_as_longlong(fabs(v)));
     }
-}
-
-// out = a X + b Y
-__global__ void combine_kernel(double a, const double* __restrict__ X, double b, const double* __restrict__ Y, size_t count,
-                               double* __restrict__ out) {
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < count; e += (size_t)gridDim.x * blockDim.x)
-        out[e] = a * X[e] + b * Y[e];
 }
 
 struct Ctx {
@@ -243,7 +302,6 @@ struct Riccati {
     int nx, nu;
     const double *A, *B, *Q, *R;
     double *X, *Xn, *BtX, *G, *K0, *S, *XA;
-    double *W, *Wi, *AG, *AG2, *Z, *HZ;     // doubling (nx <= kGaussMax)
     unsigned long long* red;                // (max|X+ - X|, max|X+|) of up to kRiccatiCheckEvery steps
     int* flag;
 };
@@ -271,7 +329,7 @@ int riccati_step(Ctx& c, Riccati& r, double* K, int slot) {
     RQ_TRY(dgemm(h, false, false, nx, nx, nx, 1.0, r.X, nx, r.Xn, nx, 0.0, r.XA, nx));          // X (A - B K)
     RQ_CUDA(h, cudaMemcpyAsync(r.Xn, r.Q, sizeof(double) * nx * nx, cudaMemcpyDeviceToDevice, h->stream));
     RQ_TRY(dgemm(h, true, false, nx, nx, nx, 1.0, r.A, nx, r.XA, nx, 1.0, r.Xn, nx));           // Q + A^T X (A - B K)
-    sym_diff_kernel<<<grid_for((size_t)nx * nx), 256, 0, h->stream>>>(r.Xn, r.X, nx, nx, r.red + 2 * slot);
+    sym_diff_kernel<<<grid_for((size_t)nx * nx), 256, 0, h->stream>>>(r.Xn, r.X, nx, r.red + 2 * slot);
     RQ_CUDA(h, cudaGetLastError());
     std::swap(r.X, r.Xn);
     return RELU_QP_OK;
@@ -302,148 +360,41 @@ int clear_changes(Ctx& c, const Riccati& r) {
     return RELU_QP_OK;
 }
 
-// The iterate after 2^k steps for k = 1, 2, .. until it no longer changes; *ok = 0 when
-// it does not settle within the plain iteration's 2^17 > kRiccatiMaxIter steps.  A_k and
-// G_k sit side by side (AG, nx x 2 nx): with Z = (I + G_k H_k)^{-1} [A_k G_k],
-//   A+ = A_k Z_A,  G+ = G_k + (A_k Z_G) A_k^T,  H+ = H_k + A_k^T H_k Z_A;
-// A_0 = A, G_0 = B R^{-1} B^T, H_0 = Q.
-int riccati_doubling(Ctx& c, Riccati& r, bool* ok, int* doublings) {
+// riccati_kernel: `steps` steps from r.X, or (0) K(r.X); RELU_QP_ERR_UNSUPPORTED when the
+// cluster cannot be launched here.
+int riccati_cluster(Ctx& c, Riccati& r, int steps, double* K) {
     relu_qp_t h = &c.h;
-    const int nx = r.nx, nu = r.nu, w = 2 * nx;
-    const size_t uu = (size_t)nu * nu, row = sizeof(double) * nx;
-    *ok = false;
-    RQ_TRY(clear_changes(c, r));
+    if (r.nx > kOneMaxX || r.nu > kOneMaxU) return RELU_QP_ERR_UNSUPPORTED;
+    OneArgs g{r.nx, r.nu, steps, r.A, r.B, r.Q, r.R, {r.X, r.Xn}, r.BtX, r.G, r.K0, K, r.S, r.XA, r.red, r.flag};
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(kOneCtas);
+    cfg.blockDim = dim3(kOneThreads);
+    cfg.stream = h->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kOneCtas;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(riccati_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaLaunchKernelEx(&cfg, riccati_kernel, g) != cudaSuccess) {
+        cudaGetLastError();
+        return RELU_QP_ERR_UNSUPPORTED;
+    }
+    if (steps & 1) std::swap(r.X, r.Xn);
+    return RELU_QP_OK;
+}
+
+int lqr_gain(Ctx& c, Riccati& r, double* K) {
+    relu_qp_t h = &c.h;
+    bool converged = false, one = true;
     RQ_CUDA(h, cudaMemsetAsync(r.flag, 0, sizeof(int), h->stream));
-    RQ_CUDA(h, cudaMemcpyAsync(r.X, r.Q, sizeof(double) * nx * nx, cudaMemcpyDeviceToDevice, h->stream));
-    RQ_CUDA(h, cudaMemcpy2DAsync(r.AG, 2 * row, r.A, row, row, nx, cudaMemcpyDeviceToDevice, h->stream));
-    RQ_CUDA(h, cudaMemcpyAsync(r.G, r.R, sizeof(double) * uu, cudaMemcpyDeviceToDevice, h->stream));
-    RQ_TRY(spd_inverse(h, 1, nu, r.G, r.S, r.S + uu, (long long)uu, r.S + 2 * uu, nu, (long long)uu, r.flag));
-    RQ_TRY(dgemm(h, false, true, nu, nx, nu, 1.0, r.S + 2 * uu, nu, r.B, nu, 0.0, r.BtX, nx));   // R^{-1} B^T
-    RQ_TRY(dgemm(h, false, false, nx, nx, nu, 1.0, r.B, nu, r.BtX, nx, 0.0, r.AG + nx, w));
-    const size_t smem = sizeof(double) * nx * (nx | 1);
-    RQ_CUDA(h, cudaFuncSetAttribute(gauss_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    constexpr int kMost = 17, kUnread = 5;   // (the first doublings are not waited for)
-    static_assert(kMost <= 2 * kRiccatiCheckEvery, "one pair of words per doubling");
-    for (int k = 0; k < kMost; ++k) {
-        const int slot = k % kRiccatiCheckEvery;
-        if (k == kRiccatiCheckEvery) RQ_TRY(clear_changes(c, r));
-        RQ_TRY(dgemm(h, false, false, nx, nx, nx, 1.0, r.AG + nx, w, r.X, nx, 0.0, r.W, nx));
-        gauss_inverse_kernel<<<1, kGaussThreads, smem, h->stream>>>(r.W, nx, r.Wi);
-        RQ_CUDA(h, cudaGetLastError());
-        RQ_TRY(dgemm(h, false, false, nx, w, nx, 1.0, r.Wi, nx, r.AG, w, 0.0, r.Z, w));
-        RQ_TRY(dgemm(h, false, false, nx, w, nx, 1.0, r.AG, w, r.Z, w, 0.0, r.AG2, w));         // [A+, A_k Z_G]
-        RQ_TRY(dgemm(h, false, false, nx, nx, nx, 1.0, r.X, nx, r.Z, w, 0.0, r.HZ, nx));
-        RQ_CUDA(h, cudaMemcpyAsync(r.Xn, r.X, sizeof(double) * nx * nx, cudaMemcpyDeviceToDevice, h->stream));
-        RQ_TRY(dgemm(h, true, false, nx, nx, nx, 1.0, r.AG, w, r.HZ, nx, 1.0, r.Xn, nx));
-        // G+ over G_k, then beside A+
-        RQ_TRY(dgemm(h, false, true, nx, nx, nx, 1.0, r.AG2 + nx, w, r.AG, w, 1.0, r.AG + nx, w));
-        RQ_CUDA(h, cudaMemcpy2DAsync(r.AG2 + nx, 2 * row, r.AG + nx, 2 * row, row, nx, cudaMemcpyDeviceToDevice, h->stream));
-        sym_diff_kernel<<<grid_for((size_t)nx * nx), 256, 0, h->stream>>>(r.AG2 + nx, r.AG2 + nx, nx, w, nullptr);
-        sym_diff_kernel<<<grid_for((size_t)nx * nx), 256, 0, h->stream>>>(r.Xn, r.X, nx, nx, r.red + 2 * slot);
-        RQ_CUDA(h, cudaGetLastError());
-        std::swap(r.X, r.Xn);
-        std::swap(r.AG, r.AG2);
-        if (k + 1 < kUnread) continue;
-        Change ch[kRiccatiCheckEvery];
-        int fl = 0;
-        RQ_TRY(read_changes(c, r, slot + 1, ch, &fl));
-        if (fl || !ch[slot].finite()) return RELU_QP_OK;
-        if (ch[slot].met()) {
-            *ok = true;
-            *doublings = k + 1;
-            return RELU_QP_OK;
-        }
-    }
-    return RELU_QP_OK;
-}
-
-// One Newton step on X = F(X) from a converged X: X + D with D = F(X) - X + P^T D P,
-// P = A - B K(X), the sum over P's powers doubled.  The doubling's own rounding (the gain
-// off by 1e-13, as much as the plain iteration's stop test leaves) falls to 1e-15, which
-// the gradient map F needs: at the optimal gain its terms cancel to 1e-4 of their size.
-int riccati_newton(Ctx& c, Riccati& r, int doublings, double* K) {
-    relu_qp_t h = &c.h;
-    const int nx = r.nx, nu = r.nu, g = grid_for((size_t)nx * nx);
-    const size_t xx = (size_t)nx * nx;
-    RQ_TRY(riccati_step(c, r, K, 0));        // r.X = F(X), r.Xn = X
-    double *D = r.W, *T = r.HZ, *P = r.Z, *P2 = r.Z + xx;
-    combine_kernel<<<g, 256, 0, h->stream>>>(1.0, r.X, -1.0, r.Xn, xx, D);
-    RQ_CUDA(h, cudaGetLastError());
-    RQ_CUDA(h, cudaMemcpyAsync(P, r.A, sizeof(double) * xx, cudaMemcpyDeviceToDevice, h->stream));
-    RQ_TRY(dgemm(h, false, false, nx, nx, nu, -1.0, r.B, nu, K, nx, 1.0, P, nx));
-    for (int k = 0; k < doublings; ++k) {
-        RQ_TRY(dgemm(h, false, false, nx, nx, nx, 1.0, D, nx, P, nx, 0.0, T, nx));
-        RQ_TRY(dgemm(h, true, false, nx, nx, nx, 1.0, P, nx, T, nx, 1.0, D, nx));
-        if (k + 1 == doublings) break;
-        RQ_TRY(dgemm(h, false, false, nx, nx, nx, 1.0, P, nx, P, nx, 0.0, P2, nx));
-        std::swap(P, P2);
-    }
-    sym_diff_kernel<<<g, 256, 0, h->stream>>>(D, D, nx, nx, nullptr);
-    combine_kernel<<<g, 256, 0, h->stream>>>(1.0, r.Xn, 1.0, D, xx, r.X);
-    RQ_CUDA(h, cudaGetLastError());
-    return RELU_QP_OK;
-}
-
-bool symmetric(const double* M, int n) {
-    for (int i = 0; i < n; ++i)
-        for (int j = 0; j < i; ++j)
-            if (M[(size_t)i * n + j] != M[(size_t)j * n + i]) return false;
-    return true;
-}
-
-// Symmetric and positive definite (a Cholesky factorisation exists).
-bool positive_definite(const double* M, int n) {
-    if (!symmetric(M, n)) return false;
-    std::vector<double> a(M, M + (size_t)n * n);
-    for (int k = 0; k < n; ++k) {
-        double d = a[(size_t)k * n + k];
-        for (int t = 0; t < k; ++t) d -= a[(size_t)k * n + t] * a[(size_t)k * n + t];
-        if (!(d > 0.0)) return false;
-        d = std::sqrt(d);
-        a[(size_t)k * n + k] = d;
-        for (int i = k + 1; i < n; ++i) {
-            double v = a[(size_t)i * n + k];
-            for (int t = 0; t < k; ++t) v -= a[(size_t)i * n + t] * a[(size_t)k * n + t];
-            a[(size_t)i * n + k] = v / d;
-        }
-    }
-    return true;
-}
-
-// Symmetric positive semidefinite as far as that is plain: diagonal with no negative
-// entry, or positive definite.
-bool semidefinite(const double* M, int n) {
-    bool diagonal = true;
-    for (int i = 0; i < n && diagonal; ++i)
-        for (int j = 0; j < n && diagonal; ++j)
-            diagonal = i == j ? M[(size_t)i * n + j] >= 0.0 : M[(size_t)i * n + j] == 0.0;
-    return diagonal || positive_definite(M, n);
-}
-
-int lqr_gain(Ctx& c, Riccati& r, bool doubling, double* K) {
-    relu_qp_t h = &c.h;
-    const int nx = r.nx;
-    bool converged = false;
-    if (doubling) {
-        int doublings = 0;
-        RQ_TRY(riccati_doubling(c, r, &converged, &doublings));
-        if (converged) {   // one plain step has to meet the plain iteration's own test
-            Change ch;
-            int fl = 0;
-            RQ_TRY(riccati_newton(c, r, doublings, K));
-            RQ_TRY(clear_changes(c, r));
-            RQ_TRY(riccati_step(c, r, K, 0));
-            RQ_TRY(read_changes(c, r, 1, &ch, &fl));
-            converged = !fl && ch.met();
-        }
-    }
-    if (!converged) {
-        RQ_CUDA(h, cudaMemsetAsync(r.flag, 0, sizeof(int), h->stream));
-        RQ_CUDA(h, cudaMemcpyAsync(r.X, r.Q, sizeof(double) * nx * nx, cudaMemcpyDeviceToDevice, h->stream));
-    }
+    RQ_CUDA(h, cudaMemcpyAsync(r.X, r.Q, sizeof(double) * r.nx * r.nx, cudaMemcpyDeviceToDevice, h->stream));
     for (int it = 0; it < kRiccatiMaxIter && !converged; it += kRiccatiCheckEvery) {
         RQ_TRY(clear_changes(c, r));
-        for (int s = 0; s < kRiccatiCheckEvery; ++s) RQ_TRY(riccati_step(c, r, K, s));
+        one = one && riccati_cluster(c, r, kRiccatiCheckEvery, K) == RELU_QP_OK;
+        for (int s = 0; s < kRiccatiCheckEvery && !one; ++s) RQ_TRY(riccati_step(c, r, K, s));
         Change ch[kRiccatiCheckEvery];
         int fl = 0;
         RQ_TRY(read_changes(c, r, kRiccatiCheckEvery, ch, &fl));
@@ -458,7 +409,7 @@ int lqr_gain(Ctx& c, Riccati& r, bool doubling, double* K) {
     }
     if (!converged)
         return fail(h, RELU_QP_ERR_INVALID, "condense: the Riccati iteration did not converge");
-    return gain(c, r, K);
+    return one && riccati_cluster(c, r, 0, K) == RELU_QP_OK ? RELU_QP_OK : gain(c, r, K);
 }
 
 int condense(Ctx& c, int nx, int nu, int N, const double* hA, const double* hB, const double* hQ, const double* hR,
@@ -468,7 +419,6 @@ int condense(Ctx& c, int nx, int nu, int N, const double* hA, const double* hB, 
     const int n = N * nu, nc = nx + nu, rows = n + (state ? N * nx : 0);
     const size_t xx = (size_t)nx * nx, xu = (size_t)nx * nu, uu = (size_t)nu * nu, nn = (size_t)n * n;
     const bool lqr = !hK && precondition, ownQN = hQN && std::memcmp(hQN, hQ, sizeof(double) * xx) != 0;
-    const bool doubling = lqr && nx <= kGaussMax && nu <= kGaussMax && positive_definite(hR, nu) && semidefinite(hQ, nx);
     // one allocation: inputs (as on the host), the iteration's buffers, the products
     double *in, *Z, *W, *TU, *HTU, *HTN, *G, *GN, *P, *F, *Acon, *E, *HM, *V, *VN, *Y, *YN, *S;
     Riccati r{};
@@ -488,18 +438,10 @@ int condense(Ctx& c, int nx, int nu, int N, const double* hA, const double* hB, 
             get(r.BtX, xu);
             get(r.K0, xu);
             get(r.G, uu);
-            get(r.S, 3 * uu);
+            get(r.S, std::max(3 * uu, xx));   // spd_inverse's scratch, or the cluster's X (A - B K)
             get(words, 2 * kRiccatiCheckEvery + 1);
             r.red = reinterpret_cast<unsigned long long*>(words);
             r.flag = reinterpret_cast<int*>(words ? words + 2 * kRiccatiCheckEvery : nullptr);
-            if (doubling) {
-                get(r.W, xx);
-                get(r.Wi, xx);
-                get(r.HZ, xx);
-                get(r.AG, 2 * xx);
-                get(r.AG2, 2 * xx);
-                get(r.Z, 2 * xx);
-            }
         }
         get(Z, (size_t)N * nx * nc);
         get(W, (size_t)N * nu * nc);
@@ -536,7 +478,7 @@ int condense(Ctx& c, int nx, int nu, int N, const double* hA, const double* hB, 
         r.B = B;
         r.Q = Q;
         r.R = R;
-        RQ_TRY(lqr_gain(c, r, doubling, K));
+        RQ_TRY(lqr_gain(c, r, K));
     }
     // Z_0 = [A - B K | B], doubled; W = -K Z
     const size_t zb = (size_t)nx * nc, wb = (size_t)nu * nc;

@@ -114,10 +114,11 @@ def test_condense_smallest_shapes(rq):
                 assert close(g[k], o[k], 1e-9), (nx, N, k)
 
 
-@pytest.mark.parametrize("nx,nu,N", [(15, 17, 3), (33, 5, 17), (65, 31, 2), (160, 3, 4), (161, 3, 4)])
-def test_condense_at_tile_and_doubling_edges(rq, nx, nu, N):
+@pytest.mark.parametrize("nx,nu,N", [(15, 17, 3), (33, 5, 17), (65, 31, 2), (96, 48, 3), (97, 3, 4), (40, 49, 2)])
+def test_condense_at_tile_and_cluster_edges(rq, nx, nu, N):
     """Sizes around the product tiles, ragged doublings of the powers, and both sides of the
-    largest plant whose Riccati iterates are doubled (160 states); full weight matrices."""
+    largest plant whose Riccati iteration one cluster runs (96 states, 48 controls); full weight
+    matrices."""
     A, B, _, _ = plant(nx * 100 + nu, nx, nu)
     rng = np.random.default_rng(nx)
     M = rng.standard_normal((nx, nx)) / np.sqrt(nx)
@@ -129,10 +130,9 @@ def test_condense_at_tile_and_doubling_edges(rq, nx, nu, N):
         assert close(g[k], o[k], 1e-9), k
 
 
-def test_condense_weights_outside_the_doubling(rq):
-    """Weights that the doubling does not take: R semidefinite (B'XB makes the step's matrix
-    definite), and an indefinite Q, go through the plain iteration as before; R + B'XB that is not
-    positive definite is still refused."""
+def test_condense_semidefinite_and_indefinite_weights(rq):
+    """R semidefinite (B'XB makes the step's matrix definite) is taken; R + B'XB that is not
+    positive definite is refused."""
     A, B, Q, _ = plant(21, 6, 2)
     R = np.zeros((2, 2))
     g = rq.condense_mpc(A, B, Q, R, 5, umin=-np.ones(2), umax=np.ones(2))
