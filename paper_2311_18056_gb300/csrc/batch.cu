@@ -142,14 +142,17 @@ __global__ void __launch_bounds__(256) map_kernel(int M, int K, const float* __r
 // long sequential FP32 sum would lose ~sqrt(K) units in the last place of its
 // largest partial sum (measured: dual residuals off by 1e-3 on the humanoid
 // workload).  The arithmetic of an output does not depend on TS or TR.
-// k tiles stream through a STAGES-deep cp.async pipeline into shared memory
-// laid out [slot or row][k] with a padded stride, so that the copies run
-// ahead of the arithmetic by STAGES - 1 steps.
+// k tiles of KB columns stream through a STAGES-deep cp.async pipeline into shared
+// memory laid out [slot or row][k] with a padded stride, so that the copies run
+// ahead of the arithmetic by STAGES - 1 tiles.  Small tiles take more columns at a time:
+// a 32 x 32 tile's 16 columns are 30 clocks of FMAs per scheduler, less than the barrier
+// and the copies' bookkeeping around them (15.2 us a layer at n + m = 420 with KB = 16).
 template <int TS, int TR>
 struct F32Tile {
     static constexpr int SA = TS / 16, RA = TR / 16;
-    static constexpr int LDS = 20;           // padded k stride in floats (80 bytes, 16-byte aligned)
-    static constexpr int STAGES = 4;
+    static constexpr int KB = TS * TR <= 64 * 64 ? 64 : 32;   // (64 divides every range of k)
+    static constexpr int LDS = KB + 4;       // padded k stride in floats (16-byte aligned, rows 4 banks apart)
+    static constexpr int STAGES = TS * TR <= 64 * 64 ? 3 : 4;
     static constexpr int XS = TS * LDS, WS = TR * LDS;
     static constexpr int BYTES = STAGES * (XS + WS) * 4;
 };
@@ -175,63 +178,76 @@ __device__ __forceinline__ void fp32_tile(const float* __restrict__ X, const flo
     for (int a = 0; a < T::SA; ++a)
 #pragma unroll
         for (int b = 0; b < T::RA; ++b) acc[a][b] = 0.f;
-    // one k tile: TS rows of X and TR rows of W, 4 chunks of 16 bytes each
-    auto load = [&](int stage, int k0) {
-        for (int e = threadIdx.x; e < 4 * (TS + TR); e += 256) {
-            const int c = e & 3;
-            if (e < 4 * TS) {
-                const int sl = e >> 2;
-                cp_async16(Xs + stage * T::XS + sl * T::LDS + 4 * c, X + (size_t)(slot0 + sl) * ld + k0 + 4 * c, true);
-            } else {
-                const int rw = (e - 4 * TS) >> 2;
-                const bool ok = row0 + rw < nrows;
-                cp_async16(Ws + stage * T::WS + rw * T::LDS + 4 * c,
-                           ok ? W + (size_t)(row0 + rw) * ld + k0 + 4 * c : W, ok);
-            }
+    // one k tile of X (TS rows) or of W (TR rows), KB / 4 chunks of 16 bytes a row
+    constexpr int C = T::KB / 4;
+    auto load_x = [&](int stage, int k0) {
+        for (int e = threadIdx.x; e < C * TS; e += 256) {
+            const int c = e % C, sl = e / C;
+            cp_async16(Xs + stage * T::XS + sl * T::LDS + 4 * c, X + (size_t)(slot0 + sl) * ld + k0 + 4 * c, true);
         }
     };
+    auto load_w = [&](int stage, int k0) {
+        for (int e = threadIdx.x; e < C * TR; e += 256) {
+            const int c = e % C, rw = e / C;
+            const bool ok = row0 + rw < nrows;
+            cp_async16(Ws + stage * T::WS + rw * T::LDS + 4 * c, ok ? W + (size_t)(row0 + rw) * ld + k0 + 4 * c : W, ok);
+        }
+    };
+    // the weights of the first stages do not depend on the previous kernel of the stream
+#pragma unroll
+    for (int s = 0; s < T::STAGES - 1; ++s)
+        if (kbeg + T::KB * s < kend) load_w(s, kbeg + T::KB * s);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 #pragma unroll
     for (int s = 0; s < T::STAGES - 1; ++s) {
-        if (kbeg + 16 * s < kend) load(s, kbeg + 16 * s);
-        cp_async_commit();
+        if (kbeg + T::KB * s < kend) load_x(s, kbeg + T::KB * s);
+        cp_async_commit();   // (the first group also holds the weights above)
     }
     int it = 0;
-    for (int k0 = kbeg; k0 < kend; k0 += 16, ++it) {
+    for (int k0 = kbeg; k0 < kend; k0 += T::KB, ++it) {
         cp_async_wait<T::STAGES - 2>();
         __syncthreads();
-        const int kn = k0 + 16 * (T::STAGES - 1);
-        if (kn < kend) load((it + T::STAGES - 1) % T::STAGES, kn);
+        const int kn = k0 + T::KB * (T::STAGES - 1);
+        if (kn < kend) {
+            load_w((it + T::STAGES - 1) % T::STAGES, kn);
+            load_x((it + T::STAGES - 1) % T::STAGES, kn);
+        }
         cp_async_commit();
         const float* xs = Xs + (it % T::STAGES) * T::XS;
         const float* ws = Ws + (it % T::STAGES) * T::WS;
-        float part[T::SA][T::RA];
 #pragma unroll
-        for (int a = 0; a < T::SA; ++a)
-#pragma unroll
-            for (int b = 0; b < T::RA; ++b) part[a][b] = 0.f;
-#pragma unroll
-        for (int kk = 0; kk < 16; kk += 4) {
-            float4 xa[T::SA], wb[T::RA];
-#pragma unroll
-            for (int a = 0; a < T::SA; ++a) xa[a] = *reinterpret_cast<const float4*>(xs + (ty + 16 * a) * T::LDS + kk);
-#pragma unroll
-            for (int b = 0; b < T::RA; ++b) wb[b] = *reinterpret_cast<const float4*>(ws + (tx + 16 * b) * T::LDS + kk);
+        for (int k1 = 0; k1 < T::KB; k1 += 16) {
+            float part[T::SA][T::RA];
 #pragma unroll
             for (int a = 0; a < T::SA; ++a)
 #pragma unroll
-                for (int b = 0; b < T::RA; ++b) {
-                    part[a][b] = fmaf(xa[a].x, wb[b].x, part[a][b]);
-                    part[a][b] = fmaf(xa[a].y, wb[b].y, part[a][b]);
-                    part[a][b] = fmaf(xa[a].z, wb[b].z, part[a][b]);
-                    part[a][b] = fmaf(xa[a].w, wb[b].w, part[a][b]);
-                }
+                for (int b = 0; b < T::RA; ++b) part[a][b] = 0.f;
+#pragma unroll
+            for (int kk = k1; kk < k1 + 16; kk += 4) {
+                float4 xa[T::SA], wb[T::RA];
+#pragma unroll
+                for (int a = 0; a < T::SA; ++a) xa[a] = *reinterpret_cast<const float4*>(xs + (ty + 16 * a) * T::LDS + kk);
+#pragma unroll
+                for (int b = 0; b < T::RA; ++b) wb[b] = *reinterpret_cast<const float4*>(ws + (tx + 16 * b) * T::LDS + kk);
+#pragma unroll
+                for (int a = 0; a < T::SA; ++a)
+#pragma unroll
+                    for (int b = 0; b < T::RA; ++b) {
+                        part[a][b] = fmaf(xa[a].x, wb[b].x, part[a][b]);
+                        part[a][b] = fmaf(xa[a].y, wb[b].y, part[a][b]);
+                        part[a][b] = fmaf(xa[a].z, wb[b].z, part[a][b]);
+                        part[a][b] = fmaf(xa[a].w, wb[b].w, part[a][b]);
+                    }
+            }
+#pragma unroll
+            for (int a = 0; a < T::SA; ++a)
+#pragma unroll
+                for (int b = 0; b < T::RA; ++b) acc[a][b] += part[a][b];
         }
-#pragma unroll
-        for (int a = 0; a < T::SA; ++a)
-#pragma unroll
-            for (int b = 0; b < T::RA; ++b) acc[a][b] += part[a][b];
     }
     cp_async_wait<0>();
+    // the next kernel may set up and load its weights while this one's epilogue runs
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Slot range of a CTA: TS-slot sub-tiles of the 128-slot tiles; a sub-tile
@@ -247,7 +263,7 @@ __device__ __forceinline__ bool fp32_slots(const BatchParams& p, int& tile, int&
 
 // One layer for every active slot tile (FP32 backend).
 template <int TS, int TR>
-__global__ void __launch_bounds__(256) batch_layer_fp32_kernel(BatchParams p, W32Ptrs wp) {
+__global__ void __launch_bounds__(256) batch_layer_fp32_kernel(BatchParams p, const __grid_constant__ W32Ptrs wp) {
     int tile, slot0;
     if (!fp32_slots<TS>(p, tile, slot0)) return;
     const int ri = p.tile_rho[tile];
@@ -321,38 +337,76 @@ __global__ void __launch_bounds__(256) batch_check_fp32_kernel(BatchParams p, co
     }
 }
 
-// Launch helpers: the full-width tile (128 slots x 64 rows) while more than
-// two slot tiles are active, else 32 x 32 sub-tiles, which skip the empty
-// slots of the last tile of a bank group and give the convergence tail more
-// CTAs.
-template <int TS, int TR>
-int launch_layer32(relu_qp_t h, const BatchParams& q, const W32Ptrs& wp, int tiles_max) {
-    auto k = batch_layer_fp32_kernel<TS, TR>;
-    RQ_CUDA(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, F32Tile<TS, TR>::BYTES));
-    k<<<dim3(ceil_div(h->R, TR), tiles_max * (kSlotTile / TS)), 256, F32Tile<TS, TR>::BYTES, h->stream>>>(q, wp);
-    RQ_CUDA(h, cudaGetLastError());
+// Tile of a launch over `rows` rows and `active` QPs (nr bank groups, each with a part of a
+// tile left over).  A tile's time is its FMAs, shared by the CTAs of an SM, but at least some
+// 250 clocks per 16 columns of k (loads, barriers), so small problems want more, smaller
+// tiles: n + m = 420, 333 QPs in 21 CTAs of 128 x 64 took 66 us a layer, in 154 of 32 x 32 15.
+struct Tile32 {
+    int ts, tr;
+};
+
+Tile32 tile32(relu_qp_t h, int rows, int active) {
+    Tile32 best{32, 32};
+    double best_t = 1e300;
+    for (const Tile32 c : {Tile32{128, 64}, Tile32{64, 64}, Tile32{64, 32}, Tile32{32, 32}}) {
+        const double ctas = (double)ceil_div(rows, c.tr) * (ceil_div(active, c.ts) + (active > c.ts ? 0.5 * (h->nr - 1) : 0.0));
+        const double per_sm = std::ceil(ctas / h->num_sms);
+        // FMAs of 16 columns at 60 % of 128 a clock (the smallest tile: of its shared memory reads)
+        const double fma = c.ts * c.tr * 16 / (c.ts * c.tr > 1024 ? 77.0 : 50.0);
+        const double t = std::max(per_sm * fma, 250.0);
+        if (t < best_t) {
+            best_t = t;
+            best = c;
+        }
+    }
+    return best;
+}
+
+template <class K, class... Args>
+int launch32(relu_qp_t h, K k, dim3 grid, int smem, bool pdl, Args... args) {
+    RQ_CUDA(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = h->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    RQ_CUDA(h, cudaLaunchKernelEx(&cfg, k, args...));
     return RELU_QP_OK;
 }
 
-int layer32(relu_qp_t h, const BatchParams& q, const W32Ptrs& wp, int tiles_max, int active) {
-    if (ceil_div(active, kSlotTile) <= 2) return launch_layer32<32, 32>(h, q, wp, tiles_max);
-    return launch_layer32<128, 64>(h, q, wp, tiles_max);
+template <int TS, int TR>
+int launch_layer32(relu_qp_t h, const BatchParams& q, const W32Ptrs& wp, int tiles_max, bool pdl) {
+    return launch32(h, batch_layer_fp32_kernel<TS, TR>, dim3(ceil_div(h->R, TR), tiles_max * (kSlotTile / TS)),
+                    F32Tile<TS, TR>::BYTES, pdl, q, wp);
+}
+
+// pdl: the previous kernel of the stream is the previous layer (programmatic dependent launch)
+int layer32(relu_qp_t h, const BatchParams& q, const W32Ptrs& wp, int tiles_max, int active, bool pdl) {
+    const Tile32 t = tile32(h, h->R, active);
+    if (t.ts == 128) return launch_layer32<128, 64>(h, q, wp, tiles_max, pdl);
+    if (t.tr == 64) return launch_layer32<64, 64>(h, q, wp, tiles_max, pdl);
+    if (t.ts == 64) return launch_layer32<64, 32>(h, q, wp, tiles_max, pdl);
+    return launch_layer32<32, 32>(h, q, wp, tiles_max, pdl);
 }
 
 template <int TS, int TR>
 int launch_check32(relu_qp_t h, const BatchParams& q, const float* Wc, int tiles_max, int phase) {
-    auto k = batch_check_fp32_kernel<TS, TR>;
-    RQ_CUDA(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, F32Tile<TS, TR>::BYTES));
     const int rows = phase == 1 ? h->n + h->m : h->n;
-    k<<<dim3(ceil_div(rows, TR), tiles_max * (kSlotTile / TS)), 256, F32Tile<TS, TR>::BYTES, h->stream>>>(q, Wc,
-                                                                                                         phase);
-    RQ_CUDA(h, cudaGetLastError());
-    return RELU_QP_OK;
+    return launch32(h, batch_check_fp32_kernel<TS, TR>, dim3(ceil_div(rows, TR), tiles_max * (kSlotTile / TS)),
+                    F32Tile<TS, TR>::BYTES, false, q, Wc, phase);
 }
 
 int check32(relu_qp_t h, const BatchParams& q, const float* Wc, int tiles_max, int active, int phase) {
-    if (ceil_div(active, kSlotTile) <= 2) return launch_check32<32, 32>(h, q, Wc, tiles_max, phase);
-    return launch_check32<128, 64>(h, q, Wc, tiles_max, phase);
+    const Tile32 t = tile32(h, phase == 1 ? h->n + h->m : h->n, active);
+    if (t.ts == 128) return launch_check32<128, 64>(h, q, Wc, tiles_max, phase);
+    if (t.tr == 64) return launch_check32<64, 64>(h, q, Wc, tiles_max, phase);
+    if (t.ts == 64) return launch_check32<64, 32>(h, q, Wc, tiles_max, phase);
+    return launch_check32<32, 32>(h, q, Wc, tiles_max, phase);
 }
 
 // Stop test and penalty rule per QP (one 128-thread block per QP: thread 0
@@ -1102,7 +1156,7 @@ int run_layers(relu_qp_t h, const BatchParams& p, int len, bool check, int activ
             q.CK32 = w.CK32;
             const bool timed32 = h->prof_on && prof_used + 2 <= h->prof_ev.size();
             if (timed32) RQ_CUDA(h, cudaEventRecord(h->prof_ev[prof_used], h->stream));
-            RQ_TRY(layer32(h, q, wp, tiles_max, active));
+            RQ_TRY(layer32(h, q, wp, tiles_max, active, j > j_begin && !timed32));
             ++h->launches;
             ++h->layer_launches;
             h->layer_flops += 2.0 * (double)R * (double)R * (double)active;   // one FP32 product per QP
