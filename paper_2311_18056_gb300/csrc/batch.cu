@@ -144,15 +144,15 @@ __global__ void __launch_bounds__(256) map_kernel(int M, int K, const float* __r
 // workload).  The arithmetic of an output does not depend on TS or TR.
 // k tiles of KB columns stream through a STAGES-deep cp.async pipeline into shared
 // memory laid out [slot or row][k] with a padded stride, so that the copies run
-// ahead of the arithmetic by STAGES - 1 tiles.  Small tiles take more columns at a time:
-// a 32 x 32 tile's 16 columns are 30 clocks of FMAs per scheduler, less than the barrier
-// and the copies' bookkeeping around them (15.2 us a layer at n + m = 420 with KB = 16).
+// ahead of the arithmetic by STAGES - 1 tiles.  (A 32 x 32 tile's 16 columns are 32 clocks of
+// FMAs per scheduler, less than the barrier and the copies' bookkeeping around them: with
+// KB = 16 a layer at n + m = 420 took 15.2 us, now 9.)
 template <int TS, int TR>
 struct F32Tile {
     static constexpr int SA = TS / 16, RA = TR / 16;
-    static constexpr int KB = TS * TR <= 64 * 64 ? 64 : 32;   // (64 divides every range of k)
+    static constexpr int KB = 64;            // (divides every range of k)
     static constexpr int LDS = KB + 4;       // padded k stride in floats (16-byte aligned, rows 4 banks apart)
-    static constexpr int STAGES = TS * TR <= 64 * 64 ? 3 : 4;
+    static constexpr int STAGES = 3;
     static constexpr int XS = TS * LDS, WS = TR * LDS;
     static constexpr int BYTES = STAGES * (XS + WS) * 4;
 };
@@ -165,10 +165,11 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-template <int TS, int TR>
+// `prep` runs once the results of the previous kernel can be read, the first copies in flight.
+template <int TS, int TR, class F>
 __device__ __forceinline__ void fp32_tile(const float* __restrict__ X, const float* __restrict__ W, int ld,
                                           int kbeg, int kend, int nrows, int slot0, int row0,
-                                          float (&acc)[TS / 16][TR / 16]) {
+                                          float (&acc)[TS / 16][TR / 16], F prep) {
     using T = F32Tile<TS, TR>;
     extern __shared__ __align__(16) float fsm[];
     float* Xs = fsm;
@@ -203,6 +204,7 @@ __device__ __forceinline__ void fp32_tile(const float* __restrict__ X, const flo
         if (kbeg + T::KB * s < kend) load_x(s, kbeg + T::KB * s);
         cp_async_commit();   // (the first group also holds the weights above)
     }
+    prep();
     int it = 0;
     for (int k0 = kbeg; k0 < kend; k0 += T::KB, ++it) {
         cp_async_wait<T::STAGES - 2>();
@@ -258,28 +260,50 @@ __device__ __forceinline__ bool fp32_slots(const BatchParams& p, int& tile, int&
     tile = (blockIdx.y * TS) / kSlotTile;
     slot0 = blockIdx.y * TS;
     if (tile >= p.counters[CNT_TILES]) return false;
-    return TS == kSlotTile || p.perm[slot0] >= 0;
+    return p.perm[slot0] >= 0;
 }
 
-// One layer for every active slot tile (FP32 backend).
+// One layer for every active slot tile (FP32 backend).  What the element-wise part reads is
+// loaded for all elements of a thread before any of them is written: the compiler cannot move
+// a load above a store that might alias it, and one round trip to L2 per element (some 0.5 us)
+// took longer than the product.  Up to 8 elements it is loaded under the product (at most 56
+// registers), beyond that a row of the tile at a time after it.
 template <int TS, int TR>
 __global__ void __launch_bounds__(256) batch_layer_fp32_kernel(BatchParams p, const __grid_constant__ W32Ptrs wp) {
+    constexpr int SA = TS / 16, RA = TR / 16;
+    constexpr bool EARLY = SA * RA <= 8;
     int tile, slot0;
     if (!fp32_slots<TS>(p, tile, slot0)) return;
     const int ri = p.tile_rho[tile];
     const int row0 = blockIdx.x * TR;
-    float acc[TS / 16][TR / 16];
-    fp32_tile<TS, TR>(p.Sin, wp.w[ri], p.ldk, 0, p.ldk, p.R, slot0, row0, acc);
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    int qp[SA];
 #pragma unroll
-    for (int a = 0; a < TS / 16; ++a) {
-        const int slot = slot0 + ty + 16 * a;
-        const int qp = p.perm[slot];
-        if (qp < 0) continue;
+    for (int a = 0; a < SA; ++a) qp[a] = p.perm[slot0 + ty + 16 * a];
+    LayerIn in[EARLY ? SA : 1][RA];
+    auto load = [&](int a, LayerIn (&v)[RA]) {
+        if (qp[a] < 0) return;
 #pragma unroll
-        for (int b = 0; b < TR / 16; ++b) {
+        for (int b = 0; b < RA; ++b) {
             const int r = row0 + tx + 16 * b;
-            if (r < p.R) layer_elem(p, slot, qp, ri, r, acc[a][b]);
+            if (r < p.R) layer_load(p, qp[a], ri, r, v[b]);
+        }
+    };
+    float acc[SA][RA];
+    fp32_tile<TS, TR>(p.Sin, wp.w[ri], p.ldk, 0, p.ldk, p.R, slot0, row0, acc, [&] {
+        if constexpr (EARLY) {
+#pragma unroll
+            for (int a = 0; a < SA; ++a) load(a, in[a]);
+        }
+    });
+#pragma unroll
+    for (int a = 0; a < SA; ++a) {
+        if (!EARLY) load(a, in[0]);
+        if (qp[a] < 0) continue;
+#pragma unroll
+        for (int b = 0; b < RA; ++b) {
+            const int r = row0 + tx + 16 * b;
+            if (r < p.R) layer_apply(p, slot0 + ty + 16 * a, qp[a], ri, r, acc[a][b], in[EARLY ? a : 0][b]);
         }
     }
 }
@@ -302,9 +326,9 @@ __global__ void __launch_bounds__(256) batch_check_fp32_kernel(BatchParams p, co
     const int rows = phase == 1 ? p.n + p.m : p.n;
     float acc[TS / 16][TR / 16];
     if (phase == 1)
-        fp32_tile<TS, TR>(p.CK32, Wc, p.ldkc, 0, p.n64, rows, slot0, row0, acc);
+        fp32_tile<TS, TR>(p.CK32, Wc, p.ldkc, 0, p.n64, rows, slot0, row0, acc, [] {});
     else
-        fp32_tile<TS, TR>(p.CK32, Wc, p.ldkc, p.n64, p.ldkc, rows, slot0, row0, acc);
+        fp32_tile<TS, TR>(p.CK32, Wc, p.ldkc, p.n64, p.ldkc, rows, slot0, row0, acc, [] {});
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 #pragma unroll
     for (int a = 0; a < TS / 16; ++a) {
@@ -339,8 +363,10 @@ __global__ void __launch_bounds__(256) batch_check_fp32_kernel(BatchParams p, co
 
 // Tile of a launch over `rows` rows and `active` QPs (nr bank groups, each with a part of a
 // tile left over).  A tile's time is its FMAs, shared by the CTAs of an SM, but at least some
-// 250 clocks per 16 columns of k (loads, barriers), so small problems want more, smaller
-// tiles: n + m = 420, 333 QPs in 21 CTAs of 128 x 64 took 66 us a layer, in 154 of 32 x 32 15.
+// 250 clocks per 16 columns of k (loads, barriers), so small problems want more, smaller tiles.
+// Whole solves, ms, with one tile throughout (32 x 32, 64 x 32, 64 x 64, 128 x 64):
+// n + m = 420, 333 QPs: 5.4, 6.2, 9.7, 13.8; n + m = 1600, 300 QPs: 32.6, 30.7, 38.2, 55.5;
+// 1000 QPs: 75, 67, 63, 78 (128 x 64 was the best nowhere and is gone).
 struct Tile32 {
     int ts, tr;
 };
@@ -348,11 +374,11 @@ struct Tile32 {
 Tile32 tile32(relu_qp_t h, int rows, int active) {
     Tile32 best{32, 32};
     double best_t = 1e300;
-    for (const Tile32 c : {Tile32{128, 64}, Tile32{64, 64}, Tile32{64, 32}, Tile32{32, 32}}) {
+    for (const Tile32 c : {Tile32{64, 64}, Tile32{64, 32}, Tile32{32, 32}}) {
         const double ctas = (double)ceil_div(rows, c.tr) * (ceil_div(active, c.ts) + (active > c.ts ? 0.5 * (h->nr - 1) : 0.0));
         const double per_sm = std::ceil(ctas / h->num_sms);
         // FMAs of 16 columns at 60 % of 128 a clock (the smallest tile: of its shared memory reads)
-        const double fma = c.ts * c.tr * 16 / (c.ts * c.tr > 1024 ? 77.0 : 50.0);
+        const double fma = c.ts * c.tr * 16 / (c.ts * c.tr > 1024 ? 77.0 : 56.0);
         const double t = std::max(per_sm * fma, 250.0);
         if (t < best_t) {
             best_t = t;
@@ -388,7 +414,6 @@ int launch_layer32(relu_qp_t h, const BatchParams& q, const W32Ptrs& wp, int til
 // pdl: the previous kernel of the stream is the previous layer (programmatic dependent launch)
 int layer32(relu_qp_t h, const BatchParams& q, const W32Ptrs& wp, int tiles_max, int active, bool pdl) {
     const Tile32 t = tile32(h, h->R, active);
-    if (t.ts == 128) return launch_layer32<128, 64>(h, q, wp, tiles_max, pdl);
     if (t.tr == 64) return launch_layer32<64, 64>(h, q, wp, tiles_max, pdl);
     if (t.ts == 64) return launch_layer32<64, 32>(h, q, wp, tiles_max, pdl);
     return launch_layer32<32, 32>(h, q, wp, tiles_max, pdl);
@@ -403,7 +428,6 @@ int launch_check32(relu_qp_t h, const BatchParams& q, const float* Wc, int tiles
 
 int check32(relu_qp_t h, const BatchParams& q, const float* Wc, int tiles_max, int active, int phase) {
     const Tile32 t = tile32(h, phase == 1 ? h->n + h->m : h->n, active);
-    if (t.ts == 128) return launch_check32<128, 64>(h, q, Wc, tiles_max, phase);
     if (t.tr == 64) return launch_check32<64, 64>(h, q, Wc, tiles_max, phase);
     if (t.ts == 64) return launch_check32<64, 32>(h, q, Wc, tiles_max, phase);
     return launch_check32<32, 32>(h, q, Wc, tiles_max, phase);

@@ -123,27 +123,51 @@ __device__ __forceinline__ float ax_row_carry(float ay, float zi, float li, floa
     return ay - zi + li / rho_i;
 }
 
-// One row of an FP32 layer (FP32 backend; the split form's is chunk4_apply).
-__device__ __forceinline__ void layer_elem(const BatchParams& p, int slot, int qp, int ri, int r, float acc) {
+// One row of an FP32 layer (FP32 backend; the split form's is chunk4_apply), in two halves:
+// what it reads, none of which depends on the product, and the update.
+struct LayerIn {
+    float b, ay, z, lam, lo, up, rs;
+};
+
+__device__ __forceinline__ void layer_load(const BatchParams& p, int qp, int ri, int r, LayerIn& in) {
+    in.b = p.BIAS[((size_t)ri * p.cap + qp) * p.ldR + r + (r >= p.n ? p.bsh : 0)];
+    if (r < p.n) return;
+    const int i = r - p.n;
+    const size_t o = (size_t)qp * p.ldm + i;
+    in.ay = p.AY[o];
+    in.z = p.Z[o];
+    in.lam = p.LAM[o];
+    in.lo = p.L[o];
+    in.up = p.U[o];
+    in.rs = p.rs[i];
+}
+
+__device__ __forceinline__ void layer_apply(const BatchParams& p, int slot, int qp, int ri, int r, float acc,
+                                            const LayerIn& in) {
     const unsigned f = p.flags;
-    const float t = acc + p.BIAS[((size_t)ri * p.cap + qp) * p.ldR + r + (r >= p.n ? p.bsh : 0)];
+    const float t = acc + in.b;
     float s_new;
     if (r < p.n) {
         p.Y[(size_t)qp * p.ldn + r] = t;
         s_new = t;
         if (f & EPI_CHECK) put_check(p, slot, r, t);
     } else {
-        const int i = r - p.n;
-        const size_t o = (size_t)qp * p.ldm + i;
-        const float rho_i = p.rho[ri] * p.rs[i];
-        const float rr = ax_row_carry(p.AY[o], p.Z[o], p.LAM[o], rho_i);
+        const size_t o = (size_t)qp * p.ldm + (r - p.n);
+        const float rho_i = p.rho[ri] * in.rs;
+        const float rr = ax_row_carry(in.ay, in.z, in.lam, rho_i);
         float zn, ln;
-        ax_row_update(t, rr, p.L[o], p.U[o], rho_i, zn, ln, s_new);
+        ax_row_update(t, rr, in.lo, in.up, rho_i, zn, ln, s_new);
         p.AY[o] = t;
         p.Z[o] = zn;
         p.LAM[o] = ln;
     }
     if (!(f & EPI_LAST)) p.Sout[(size_t)slot * p.ldk + r] = s_new;
+}
+
+__device__ __forceinline__ void layer_elem(const BatchParams& p, int slot, int qp, int ri, int r, float acc) {
+    LayerIn in{};
+    layer_load(p, qp, ri, r, in);
+    layer_apply(p, slot, qp, ri, r, acc, in);
 }
 
 __device__ __forceinline__ void ld4(const float* __restrict__ src, float (&v)[4]) {
