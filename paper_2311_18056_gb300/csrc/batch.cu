@@ -809,8 +809,8 @@ int batch_alloc(relu_qp_t h) {
         RQ_TRY(dev_alloc(h, &w.CK, sizeof(uint16_t) * 3 * (size_t)w.slots * w.ldkc + 1024));
         RQ_TRY(dev_alloc(h, &w.WB, sizeof(uint16_t) * (size_t)nr * 3 * w.Rpad * w.ldk + 1024));
         RQ_TRY(dev_alloc(h, &w.WCB, sizeof(uint16_t) * 3 * (size_t)w.npad * w.ldkc + 1024));
-        RQ_TRY(alloc(h, &w.chunk_sync, 2 * (size_t)w.slots / kSlotTile));   // layer counters, done counters
-        RQ_CUDA(h, cudaMemset(w.chunk_sync, 0, sizeof(unsigned) * 2 * (w.slots / kSlotTile)));
+        RQ_TRY(alloc(h, &w.chunk_sync, tc_sync_words(h)));   // layer counters, done counters
+        RQ_CUDA(h, cudaMemset(w.chunk_sync, 0, sizeof(unsigned) * tc_sync_words(h)));
     } else {
         RQ_TRY(alloc(h, &w.S32, 2 * (size_t)w.slots * w.ldk));
         RQ_TRY(alloc(h, &w.CK32, (size_t)w.slots * w.ldkc));
@@ -886,10 +886,10 @@ int tc_tune(relu_qp_t h) {
             int layers = 0;
             bool chunked = false;
             if (w.chunk_sync) {
-                RQ_CUDA(h, cudaMemsetAsync(w.chunk_sync, 0, sizeof(unsigned) * 2 * tiles, h->stream));
+                RQ_CUDA(h, cudaMemsetAsync(w.chunk_sync, 0, sizeof(unsigned) * tc_sync_words(h), h->stream));
                 const int rc = tc_chunk(h, p, 2, 0u, t);    // warm-up (and eligibility)
                 if (rc == RELU_QP_OK) {
-                    RQ_CUDA(h, cudaMemsetAsync(w.chunk_sync, 0, sizeof(unsigned) * 2 * tiles, h->stream));
+                    RQ_CUDA(h, cudaMemsetAsync(w.chunk_sync, 0, sizeof(unsigned) * tc_sync_words(h), h->stream));
                     RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
                     RQ_TRY(tc_chunk(h, p, 8, 0u, t));
                     RQ_CUDA(h, cudaEventRecord(h->ev1, h->stream));
@@ -927,10 +927,10 @@ int tc_tune(relu_qp_t h) {
         for (int u = t; u <= tiles; ++u) table[u] = best_c;   // until the next measured count
         if (t == 1 && tc_small_eligible(h, per_tile, 1)) {
             // the resident-weight kernel for one tile of few QPs against the best tiled one
-            RQ_CUDA(h, cudaMemsetAsync(w.chunk_sync, 0, sizeof(unsigned) * 2 * tiles, h->stream));
+            RQ_CUDA(h, cudaMemsetAsync(w.chunk_sync, 0, sizeof(unsigned) * tc_sync_words(h), h->stream));
             int rc = tc_small(h, p, 2, 0u, per_tile, 1);
             if (rc == RELU_QP_OK) {
-                RQ_CUDA(h, cudaMemsetAsync(w.chunk_sync, 0, sizeof(unsigned) * 2 * tiles, h->stream));
+                RQ_CUDA(h, cudaMemsetAsync(w.chunk_sync, 0, sizeof(unsigned) * tc_sync_words(h), h->stream));
                 RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
                 RQ_TRY(tc_small(h, p, 8, 0u, per_tile, 1));
                 RQ_CUDA(h, cudaEventRecord(h->ev1, h->stream));
@@ -1121,7 +1121,7 @@ int run_layers(relu_qp_t h, const BatchParams& p, int len, bool check, int activ
     const bool timed = h->prof_on && bf16 && len > 1 && prof_used + 2 <= h->prof_ev.size();
     // layer counters of the persistent chunk kernel start at zero
     if (bf16 && w.chunk_sync && len > 1 && j_end > 1)
-        RQ_CUDA(h, cudaMemsetAsync(w.chunk_sync, 0, sizeof(unsigned) * 2 * tiles_max, h->stream));
+        RQ_CUDA(h, cudaMemsetAsync(w.chunk_sync, 0, sizeof(unsigned) * tc_sync_words(h), h->stream));
     for (int j = j_begin; j < std::min(len, j_end); ++j) {
         BatchParams q = layer_params(h, p);
         q.flags = 0;

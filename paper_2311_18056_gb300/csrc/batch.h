@@ -189,12 +189,19 @@ __device__ __forceinline__ void st4(float* __restrict__ dst, const float (&v)[4]
 // the loads of all its 4-row pieces before the first apply, so one memory
 // round trip covers 16 rows of 8 QPs; 4 lanes per QP make each warp-wide
 // 128-bit access cover 8 QPs' contiguous 64-byte row segments.
+// Where a layer of a chunk writes, and its flags: beside the launch's parameters, which a kernel
+// that runs several layers would otherwise copy into local memory to change them (0.5 KB a
+// thread, more than the L1 that the staged operands leave).
+struct LayerOut {
+    unsigned flags;
+    __nv_bfloat16 *Dhi, *Dlo;                // BF16 split operand out
+};
+
 struct Chunk4 {
     float t[4], sref[4], ay[4], zz[4], lm[4], lo[4], up[4];
 };
 
-__device__ __forceinline__ void chunk4_load(const BatchParams& p, int qp, int ri, int r0, Chunk4& c) {
-    const unsigned f = p.flags;
+__device__ __forceinline__ void chunk4_load(const BatchParams& p, unsigned f, int qp, int ri, int r0, Chunk4& c) {
     const size_t oR = (size_t)qp * p.ldR + r0;
     const bool refine_only = (f & EPI_REFINE) && !(f & EPI_REBASE);
     ld4(refine_only ? p.C + oR : p.BIAS + (size_t)ri * p.cap * p.ldR + oR, c.t);
@@ -212,9 +219,9 @@ __device__ __forceinline__ void chunk4_load(const BatchParams& p, int qp, int ri
 }
 
 // rs = p.rs[r0 - n .. r0 - n + 3] for Ax rows (unused for x rows)
-__device__ __forceinline__ void chunk4_apply(const BatchParams& p, int slot, int qp, int ri, int r0,
-                                             const float (&acc)[4], Chunk4& c, const float (&rs)[4]) {
-    const unsigned f = p.flags;
+__device__ __forceinline__ void chunk4_apply(const BatchParams& p, const LayerOut& e, int slot, int qp, int ri,
+                                             int r0, const float (&acc)[4], Chunk4& c, const float (&rs)[4]) {
+    const unsigned f = e.flags;
     const size_t oR = (size_t)qp * p.ldR + r0;
     // x, Ax, z and lam' are written only at a chunk's last layer (its other layers, the
     // accurate first one included, keep chunk-local data: c, s_ref, r and the operand)
@@ -267,8 +274,8 @@ __device__ __forceinline__ void chunk4_apply(const BatchParams& p, int slot, int
             vh.y = (uint32_t)__bfloat16_as_ushort(hi[2]) | ((uint32_t)__bfloat16_as_ushort(hi[3]) << 16);
             vl.x = (uint32_t)__bfloat16_as_ushort(lo[0]) | ((uint32_t)__bfloat16_as_ushort(lo[1]) << 16);
             vl.y = (uint32_t)__bfloat16_as_ushort(lo[2]) | ((uint32_t)__bfloat16_as_ushort(lo[3]) << 16);
-            *reinterpret_cast<uint2*>(p.Dhi + so) = vh;
-            *reinterpret_cast<uint2*>(p.Dlo + so) = vl;
+            *reinterpret_cast<uint2*>(e.Dhi + so) = vh;
+            *reinterpret_cast<uint2*>(e.Dlo + so) = vl;
         } else {
             st4(p.Sout + so, s_new);
         }
@@ -281,7 +288,7 @@ struct Chunk4R {
     float t[4], sref[4], rr[4], lo[4], up[4];
 };
 
-__device__ __forceinline__ void chunk4_load(const BatchParams& p, int qp, int ri, int r0, Chunk4R& c) {
+__device__ __forceinline__ void chunk4_load(const BatchParams& p, unsigned, int qp, int ri, int r0, Chunk4R& c) {
     const size_t oR = (size_t)qp * p.ldR + r0;
     ld4(p.C + oR, c.t);
     ld4(p.SREF + oR, c.sref);
@@ -293,35 +300,40 @@ __device__ __forceinline__ void chunk4_load(const BatchParams& p, int qp, int ri
     }
 }
 
-__device__ __forceinline__ void chunk4_apply(const BatchParams& p, int slot, int qp, int ri, int r0,
-                                             const float (&acc)[4], Chunk4R& c, const float (&rs)[4]) {
-    const unsigned f = p.flags;
+// CARRY: the caller keeps c for the next layer, so r stays there instead of in RR.
+template <bool CARRY = false>
+__device__ __forceinline__ void chunk4_apply(const BatchParams& p, const LayerOut& e, int slot, int qp, int ri,
+                                             int r0, const float (&acc)[4], Chunk4R& c, const float (&rs)[4]) {
+    const unsigned f = e.flags;
     const bool last = (f & EPI_LAST) != 0;
-    float s_new[4];
+    float t[4], s_new[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) t[k] = c.t[k] + acc[k];
     if (r0 < p.n) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            c.t[k] += acc[k];
-            s_new[k] = c.t[k];
-        }
-        if (last) st4(p.Y + (size_t)qp * p.ldn + r0, c.t);
+        for (int k = 0; k < 4; ++k) s_new[k] = t[k];
+        if (last) st4(p.Y + (size_t)qp * p.ldn + r0, t);
         if (f & EPI_CHECK)
-            for (int k = 0; k < 4; ++k) put_check(p, slot, r0 + k, c.t[k]);
+            for (int k = 0; k < 4; ++k) put_check(p, slot, r0 + k, t[k]);
     } else {
         const size_t o = (size_t)qp * p.ldm + (r0 - p.n);
         float zn[4], ln[4], rn[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            c.t[k] += acc[k];
             const float rho_i = p.rho[ri] * rs[k];
-            zn[k] = fminf(fmaxf(c.t[k] + c.rr[k], c.lo[k]), c.up[k]);
+            zn[k] = fminf(fmaxf(t[k] + c.rr[k], c.lo[k]), c.up[k]);
             ln[k] = lam_layer(rho_i, c.rr[k]);
-            rn[k] = c.t[k] - zn[k] + c.rr[k];
+            rn[k] = t[k] - zn[k] + c.rr[k];
             s_new[k] = next_operand(rho_i, zn[k], ln[k]);
         }
-        st4(p.RR + o, rn);
+        if (CARRY) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) c.rr[k] = rn[k];
+        } else {
+            st4(p.RR + o, rn);
+        }
         if (last) {
-            st4(p.AY + o, c.t);
+            st4(p.AY + o, t);
             st4(p.Z + o, zn);
             st4(p.LAM + o, ln);
         }
@@ -336,8 +348,8 @@ __device__ __forceinline__ void chunk4_apply(const BatchParams& p, int slot, int
         vh.y = (uint32_t)__bfloat16_as_ushort(hi[2]) | ((uint32_t)__bfloat16_as_ushort(hi[3]) << 16);
         vl.x = (uint32_t)__bfloat16_as_ushort(lo[0]) | ((uint32_t)__bfloat16_as_ushort(lo[1]) << 16);
         vl.y = (uint32_t)__bfloat16_as_ushort(lo[2]) | ((uint32_t)__bfloat16_as_ushort(lo[3]) << 16);
-        *reinterpret_cast<uint2*>(p.Dhi + so) = vh;
-        *reinterpret_cast<uint2*>(p.Dlo + so) = vl;
+        *reinterpret_cast<uint2*>(e.Dhi + so) = vh;
+        *reinterpret_cast<uint2*>(e.Dlo + so) = vl;
     }
 }
 
@@ -523,6 +535,7 @@ bool tc_chunk_fits(relu_qp_t h, LayerCfg c, int active_tiles);   // whether tc_c
 // RELU_QP_ERR_UNSUPPORTED: not possible here (more tiles or QPs, too large a
 // problem for one wave, or a refused launch, which disables it for the handle).
 bool tc_small_eligible(relu_qp_t h, int active, int active_tiles);
+size_t tc_sync_words(relu_qp_t h);   // words of BatchWork::chunk_sync
 int tc_small(relu_qp_t h, const BatchParams& p, int nl, unsigned last_flags, int active, int active_tiles);
 void tc_small_set(relu_qp_t h, bool use);   // use it where eligible (set by the tuner)
 bool tc_small_chosen(relu_qp_t h);

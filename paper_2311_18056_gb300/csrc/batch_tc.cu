@@ -200,6 +200,26 @@ __device__ __forceinline__ void tmem_ld16x2(uint32_t ta, uint32_t tb, float (&v)
     }
 }
 
+// a[i] + b[i] of 32 columns of each accumulator, behind one wait
+__device__ __forceinline__ void tmem_sum32(uint32_t ta, uint32_t tb, float (&v)[32]) {
+    uint32_t r[32], s[32];
+#define RQ_LD32(x, addr)                                                                                          \
+    asm volatile(                                                                                                 \
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"          \
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"                                \
+        : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]), "=r"(x[7]),         \
+          "=r"(x[8]), "=r"(x[9]), "=r"(x[10]), "=r"(x[11]), "=r"(x[12]), "=r"(x[13]), "=r"(x[14]), "=r"(x[15]),   \
+          "=r"(x[16]), "=r"(x[17]), "=r"(x[18]), "=r"(x[19]), "=r"(x[20]), "=r"(x[21]), "=r"(x[22]), "=r"(x[23]), \
+          "=r"(x[24]), "=r"(x[25]), "=r"(x[26]), "=r"(x[27]), "=r"(x[28]), "=r"(x[29]), "=r"(x[30]), "=r"(x[31])  \
+        : "r"(addr))
+    RQ_LD32(r, ta);
+    RQ_LD32(s, tb);
+#undef RQ_LD32
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]) + __uint_as_float(s[i]);
+}
+
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     uint32_t r[16];
     asm volatile(
@@ -234,6 +254,14 @@ __device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
 
 __device__ __forceinline__ void st_cluster4(uint32_t addr, float a, float b, float c, float d) {
     asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d)
+                 : "memory");
+}
+
+// The same, its 16 bytes counted on the receiver's mbarrier when they are there (nothing for
+// the sender to release or wait for).
+__device__ __forceinline__ void st_async4(uint32_t addr, uint32_t bar, float a, float b, float c, float d) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr),
+                 "f"(a), "f"(b), "f"(c), "f"(d), "r"(bar)
                  : "memory");
 }
 
@@ -536,7 +564,7 @@ __device__ __forceinline__ int recv_off(int slot, int col) {
 // element-wise part of the mode to this warp's columns.  Returns false after a
 // deadline (the error is recorded).
 template <int MODE, int BN, int KS>
-__device__ __forceinline__ bool tile_epilogue(const BatchParams& p, const TcArgs& g, int warp, int lane, int rank,
+__device__ __forceinline__ bool tile_epilogue(const BatchParams& p, const LayerOut& e, const TcArgs& g, int warp, int lane, int rank,
                                               int slot0, int row0, int ri, uint32_t tmem, float* xpose, float* recv,
                                               uint32_t bar_acc, uint32_t par_acc, uint32_t bar_recv,
                                               uint32_t par_recv, int* s_fail, float* drain = nullptr, int nkb = 0,
@@ -586,7 +614,7 @@ __device__ __forceinline__ bool tile_epilogue(const BatchParams& p, const TcArgs
     float rs[4] = {1.f, 1.f, 1.f, 1.f}, rs_next[4] = {1.f, 1.f, 1.f, 1.f};
     // inputs of one 4-row piece of the 16-column chunk at c0 (pass = QP group)
     auto load_pass = [&](int c0, int pass) {
-        if (qq[pass] >= 0) chunk4_load(p, qq[pass], ri, row0 + c0 + cg, in[pass]);
+        if (qq[pass] >= 0) chunk4_load(p, e.flags, qq[pass], ri, row0 + c0 + cg, in[pass]);
     };
     auto load_rs = [&](int c0, float (&dst)[4]) {
         const int r0 = row0 + c0 + cg;
@@ -813,7 +841,7 @@ __device__ __forceinline__ bool tile_epilogue(const BatchParams& p, const TcArgs
                     float a4[4];
 #pragma unroll
                     for (int t = 0; t < 4; ++t) a4[t] = base[sl * stride + off + cg + t];
-                    chunk4_apply(p, slot0 + q * 32 + sl, qq[pass], ri, r0 + cg, a4, in[pass], rs);
+                    chunk4_apply(p, e, slot0 + q * 32 + sl, qq[pass], ri, r0 + cg, a4, in[pass], rs);
                 }
                 if (next) load_pass(cn, pass);
             }
@@ -982,7 +1010,8 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
         // the previous kernel's writes (the carried r, the state) are read and the
         // operand it read is overwritten: wait for it
         griddep_wait();
-        tile_epilogue<MODE, BN, KS>(p, g, warp, lane, rank, slot0, row0, ri, tmem, xpose, recv,
+        const LayerOut e{p.flags, p.Dhi, p.Dlo};
+        tile_epilogue<MODE, BN, KS>(p, e, g, warp, lane, rank, slot0, row0, ri, tmem, xpose, recv,
                                     smem_u32(&bars[2 * STAGES]), 0, smem_u32(&bars[2 * STAGES + 1]), 0, &s_fail,
                                     drain, kb_count, smem_u32(&bars[2 * STAGES + 2]), smem_u32(&bars[2 * STAGES + 4]));
     }
@@ -1163,11 +1192,9 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
         griddep_wait();
         constexpr int kEpiThreads = 32 * 4 * HALVES;
         for (int j = 1; j <= c.nl; ++j) {
-            BatchParams q = p;
-            q.flags = EPI_REFINE | (j == c.nl ? c.last_flags : 0u);
-            q.Dhi = c.OP + (size_t)(2 * (j & 1)) * c.opart;
-            q.Dlo = q.Dhi + c.opart;
-            tile_epilogue<MODE_LAYER_REFINED, BN, KS>(q, g, warp, lane, rank, slot0, row0, ri, tmem, xpose, recv,
+            __nv_bfloat16* const dhi = c.OP + (size_t)(2 * (j & 1)) * c.opart;
+            const LayerOut e{EPI_REFINE | (j == c.nl ? c.last_flags : 0u), dhi, dhi + c.opart};
+            tile_epilogue<MODE_LAYER_REFINED, BN, KS>(p, e, g, warp, lane, rank, slot0, row0, ri, tmem, xpose, recv,
                                                       smem_u32(&bars[2 * STAGES]), (uint32_t)((j - 1) & 1),
                                                       smem_u32(&bars[2 * STAGES + 1]), (uint32_t)((j - 1) & 1),
                                                       &s_fail);
@@ -1233,17 +1260,30 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
 // w1 and w2 of 128 rows x 256 k are 128 KB); every CTA sends its partial sums
 // of rows 16 r .. 16 r + 15 to rank r through distributed shared memory, and
 // rank r adds the 8 partials in rank order and applies the element-wise layer
-// (chunk4_apply) to its 16 rows x NS slots.  Layers are ordered by the tile's
-// counter as in tc_chunk_kernel (release after the epilogue, acquire before
-// the next operand load); every wait has a deadline.
+// (chunk4_apply) to its 16 rows x NS slots.
 // Warps: 0 TMA, 1 MMA (one lane), 2-5 epilogue (warp w reads TMEM lanes of
 // quadrant w % 4).
+//
+// A layer is a chain of latencies (its MMAs are 0.5 us), so each link is kept short:
+// - a counter per row block (8 CTAs), 128 bytes apart; a CTA waits for the 2 or 3 blocks that
+//   write its k range, and for its own (below), not for the whole grid;
+// - the partial sums are st.async, counted in bytes on the receiver's mbarrier: no
+//   release by the sender, no arrival;
+// - c, s_ref, l, u and the carried r stay in the registers of the thread that
+//   finalises them, so that only the next operand is stored before the release.
+// Waiting for its own row block orders a CTA's reuse of its operand buffer, its MMAs and the
+// receive buffers of its cluster.  A CTA finalises layer j + 1 only with the partials of all
+// ranks, whose k ranges together cover every row block, so its stores into operand pair
+// (j + 1) & 1 come after every CTA's reads of that pair for layer j.  Every wait has a deadline.
+// n + m = 1600, a layer with 33 to 64 slots: 8.7 us with one counter, loads and stores of the
+// state in every layer and a release per sender, 7.4 now; up to 32 slots 7.5, now 6.1.
 // ---------------------------------------------------------------------------
 constexpr int kSmallKS = 8;                          // K split over a cluster of 8 CTAs
 constexpr int kSmallRows = 128;                      // rows of Wt per CTA (the MMA M dimension)
 constexpr int kSmallMaxKb = 4;                       // k-blocks per CTA at most
 constexpr int kSmallOwn = kSmallRows / kSmallKS;     // rows each CTA finalises
 constexpr int kSmallThreads = 192;
+constexpr int kSmallSyncStride = 32;                 // words between the row blocks' counters
 
 template <int NS>
 struct SmallSmem {
@@ -1283,6 +1323,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
     const int kb_begin = rank * g.num_kb / kSmallKS;
     const int kb_count = (rank + 1) * g.num_kb / kSmallKS - kb_begin;
     const unsigned nct = gridDim.x;
+    const uint32_t recv_bytes = (uint32_t)(kSmallKS * kSmallOwn * 4 * c.ncols);
 
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -1301,8 +1342,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
         mbar_init(smem_u32(&bars[1]), 1);
         mbar_init(smem_u32(&bars[2]), 1);
         mbar_init(smem_u32(&bars[3]), 4);             // one arrival per epilogue warp
-        mbar_init(smem_u32(&bars[4]), kSmallKS);      // one arrival per sender CTA
+        mbar_init(smem_u32(&bars[4]), 1);             // armed with the bytes of a layer
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        mbar_expect_tx(smem_u32(&bars[4]), recv_bytes);
         s_fail = 0;
     }
     if (warp == 1) {
@@ -1319,30 +1361,36 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
 
     if (warp == 0) {
         // ------------------------- TMA producer -------------------------
+        const uint32_t wfull = smem_u32(&bars[0]), opfull = smem_u32(&bars[1]);
         if (lane == 0) {
             prefetch_map(&tmA32);
             prefetch_map(&tmW);
             // the weight slice, once: parts w1, w2 of rows row0 .. row0 + 127, this CTA's k-blocks
-            const uint32_t wfull = smem_u32(&bars[0]);
             mbar_expect_tx(wfull, (uint32_t)(2 * kb_count * L::kWPart));
             for (int b = 0; b < kb_count; ++b)
                 for (int part = 0; part < 2; ++part)
                     tma_load_2d(smem_u32(sW + (part * kSmallMaxKb + b) * L::kWPart), &tmW,
                                 (kb_begin + b) * kBK, g.b_row[part] + ri * g.b_rho_stride + row0, wfull);
-            const uint32_t opfull = smem_u32(&bars[1]);
-            int loads = 0;
-            for (int j = 1; j <= c.nl; ++j) {
-                if (*(volatile int*)&s_fail) break;
-                if (j > 1) {
-                    // every CTA of the tile is done with layer j - 1 (which also means this
-                    // CTA's MMAs of layer j - 1 have read the operand buffer)
-                    if (!wait_counter_geq(c.sync + tile, (unsigned)(j - 1) * nct, kWaitNs)) {
-                        wait_failed(g.err, WS_PROD_SYNC);
-                        s_fail = 1;
-                        break;
-                    }
-                    asm volatile("fence.proxy.async.global;" ::: "memory");
-                }
+        }
+        // lane l watches a row block of this CTA's k range, the last of them its own
+        const int blk0 = kb_begin * kBK / kSmallRows;
+        const int blk1 = min((kb_begin + kb_count) * kBK - 1, g.rows - 1) / kSmallRows;
+        const int nwatch = blk1 - blk0 + 2;
+        const unsigned* watch =
+            c.sync + kSmallSyncStride * (lane < nwatch - 1 ? blk0 + lane : (int)blockIdx.x / kSmallKS);
+        int loads = 0;
+        for (int j = 1; j <= c.nl; ++j) {
+            bool ok = *(volatile int*)&s_fail == 0;
+            if (ok && j > 1 && lane < nwatch &&
+                !wait_counter_geq(watch, (unsigned)((j - 1) * kSmallKS), kWaitNs)) {
+                wait_failed(g.err, WS_PROD_SYNC);
+                s_fail = 1;
+                ok = false;
+            }
+            __syncwarp();      // what the lanes have acquired is ordered before lane 0's copies
+            if (!__all_sync(0xffffffffu, ok)) break;
+            if (lane == 0) {
+                if (j > 1) asm volatile("fence.proxy.async.global;" ::: "memory");
                 const int a0 = 2 * ((j - 1) & 1) * c.slots + slot0;
                 mbar_expect_tx(opfull, (uint32_t)(2 * kb_count * ((c.ncols + 31) / 32) * 4096));
                 for (int b = 0; b < kb_count; ++b)
@@ -1350,12 +1398,15 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
                         for (int gr = 0; gr < (c.ncols + 31) / 32; ++gr)
                             tma_load_2d(smem_u32(sOp + (part * kSmallMaxKb + b) * L::kOpPart + gr * 4096), &tmA32,
                                         (kb_begin + b) * kBK, a0 + part * c.slots + 32 * gr, opfull);
-                ++loads;
             }
-            // the copies in flight land before the CTA may exit (bounded waits)
+            ++loads;
+        }
+        // the copies in flight land before the CTA may exit (bounded waits)
+        if (lane == 0) {
             if (loads > 0) mbar_wait(opfull, (uint32_t)((loads - 1) & 1));
             mbar_wait(wfull, 0);
         }
+        __syncwarp();
     } else if (warp == 1) {
         // ------------------------- MMA issuer -------------------------
         if (lane == 0) {
@@ -1407,89 +1458,89 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
         // ------------------------- epilogue (warps 2-5) -------------------------
         const int q = warp & 3;                       // TMEM lane quadrant: rows 32 q .. 32 q + 31
         const int et = (warp - 2) * 32 + lane;        // 0 .. 127
-        // the element this thread finalises: slot es, rows fr0 .. fr0 + 7 of the block
+        // this thread finalises slot es, rows fr .. fr + 3 and fr + 8 .. fr + 11 of the CTA's 16
+        // (the two threads of a slot then read the received sums from different banks)
         const int es = et >> 1;
-        const int fr = rank * kSmallOwn + (et & 1) * 8;          // row within the 128-row block
-        const int fr0 = row0 + fr;
+        const int fr = (et & 1) * 4;
+        const int fr0 = row0 + rank * kSmallOwn + fr;
         const bool mine = es < c.ncols;
         const int eqp = mine ? p.perm[slot0 + es] : -1;
         // sender side: lane = row 32 q + lane of the block; rows 16 o .. 16 o + 15 go to rank o
         const int srow = q * 32 + lane;
         const int owner = srow / kSmallOwn;
-        const uint32_t recv_remote = mapa(smem_u32(recv), (uint32_t)owner);
-        for (int j = 1; j <= c.nl; ++j) {
-            BatchParams pj = p;
-            pj.flags = EPI_REFINE | (j == c.nl ? c.last_flags : 0u);
-            pj.Dhi = c.OP + (size_t)(2 * (j & 1)) * c.opart;
-            pj.Dlo = pj.Dhi + c.opart;
-            // this thread's inputs load while the MMAs run
-            Chunk4R in[2];
-            if (eqp >= 0) {
+        const uint32_t recv_bar = mapa(smem_u32(&bars[4]), (uint32_t)owner);
+        // partial sums of row srow go to the owner's receive slot `rank` at row srow % 16
+        const uint32_t dst = mapa(smem_u32(recv), (uint32_t)owner) + 4u * (uint32_t)(rank * kSmallOwn * NS);
+        const int rw = srow % kSmallOwn;
+        // the inputs of the whole chunk
+        Chunk4R in[2];
+        float rs4[2][4];
 #pragma unroll
-                for (int h2 = 0; h2 < 2; ++h2)
-                    if (fr0 + 4 * h2 < g.rows) chunk4_load(pj, eqp, ri, fr0 + 4 * h2, in[h2]);
+        for (int h2 = 0; h2 < 2; ++h2) {
+            const int r0 = fr0 + 8 * h2;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) rs4[h2][i] = 1.f;
+            if (eqp >= 0 && r0 < g.rows) {
+                chunk4_load(p, 0u, eqp, ri, r0, in[h2]);
+                if (r0 >= p.n) ld4(p.rs + (r0 - p.n), rs4[h2]);
             }
+        }
+        for (int j = 1; j <= c.nl; ++j) {
+            __nv_bfloat16* const dhi = c.OP + (size_t)(2 * (j & 1)) * c.opart;
+            const LayerOut e{EPI_REFINE | (j == c.nl ? c.last_flags : 0u), dhi, dhi + c.opart};
             // the accumulators of layer j
-            bool ready = true;
-            if (lane == 0) ready = mbar_wait_sleep(smem_u32(&bars[2]), (uint32_t)((j - 1) & 1), 128);
-            ready = __shfl_sync(0xffffffffu, ready, 0);
-            if (ready) ready = mbar_wait(smem_u32(&bars[2]), (uint32_t)((j - 1) & 1));
-            ready = __all_sync(0xffffffffu, ready);
+            bool ready = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars[2]), (uint32_t)((j - 1) & 1)));
             if (ready) {
                 fence_after();
                 const uint32_t tl = tmem + ((uint32_t)(q * 32) << 16);
-                // partial sums of this CTA's k range for row srow, all NS slots -> rank owner,
-                // into its receive slot `rank` at row srow % 16
-                const uint32_t dst = recv_remote + 4u * (uint32_t)(rank * kSmallOwn * NS);
-                const int rw = srow % kSmallOwn;
-                for (int c0 = 0; c0 < c.ncols; c0 += 16) {
+                int c0 = 0;
+                if constexpr (NS >= 32) {
+                    for (; c0 + 32 <= c.ncols; c0 += 32) {
+                        float v[32];
+                        tmem_sum32(tl + c0, tl + NS + c0, v);
+#pragma unroll
+                        for (int t = 0; t < 32; t += 4)
+                            st_async4(dst + 4u * (uint32_t)small_off<NS>(rw, c0 + t), recv_bar, v[t], v[t + 1], v[t + 2],
+                                      v[t + 3]);
+                    }
+                }
+                if (c0 < c.ncols) {
                     float v[16], w[16];
                     tmem_ld16x2(tl + c0, tl + NS + c0, v, w);
 #pragma unroll
                     for (int t = 0; t < 16; t += 4)
-                        st_cluster4(dst + 4u * (uint32_t)small_off<NS>(rw, c0 + t), v[t] + w[t], v[t + 1] + w[t + 1],
-                                    v[t + 2] + w[t + 2], v[t + 3] + w[t + 3]);
+                        st_async4(dst + 4u * (uint32_t)small_off<NS>(rw, c0 + t), recv_bar, v[t] + w[t],
+                                  v[t + 1] + w[t + 1], v[t + 2] + w[t + 2], v[t + 3] + w[t + 3]);
                 }
             }
             fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&bars[3]));          // this warp's TMEM reads are done
-            // lanes 0 and 16 announce their half-warp's rows to the two owners
-            if ((lane & 15) == 0) mbar_arrive_cluster(mapa(smem_u32(&bars[4]), (uint32_t)owner));
-            bool got = ready;
-            if (got) {
-                if (lane == 0) got = mbar_wait_cluster(smem_u32(&bars[4]), (uint32_t)((j - 1) & 1), 64);
-                got = __shfl_sync(0xffffffffu, got, 0);
-                if (got) got = mbar_wait_cluster(smem_u32(&bars[4]), (uint32_t)((j - 1) & 1), 0);
-                got = __all_sync(0xffffffffu, got);
-            }
+            const bool got =
+                __all_sync(0xffffffffu, ready && mbar_wait_cluster(smem_u32(&bars[4]), (uint32_t)((j - 1) & 1), 0));
             if (!ready || !got) {
                 if (lane == 0) {
                     wait_failed(g.err, ready ? WS_EPI_RECV : WS_EPI_ACC);
                     s_fail = 1;
                 }
             } else if (eqp >= 0) {
-                // the 8 partials of rows fr .. fr + 7, slot es, added in rank order
-                float acc[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    float tsum = 0.f;
-#pragma unroll
-                    for (int k = 0; k < kSmallKS; ++k) {
-                        const float v = recv[k * kSmallOwn * NS + small_off<NS>((fr - rank * kSmallOwn) + i, es)];
-                        tsum = k == 0 ? v : tsum + v;
-                    }
-                    acc[i] = tsum;
-                }
+                // the 8 partials of each row, added in rank order
 #pragma unroll
                 for (int h2 = 0; h2 < 2; ++h2) {
-                    const int r0 = fr0 + 4 * h2;
-                    if (r0 < g.rows) {
-                        float rs4[4] = {1.f, 1.f, 1.f, 1.f};
-                        if (r0 >= p.n) ld4(p.rs + (r0 - p.n), rs4);
-                        const float a4[4] = {acc[4 * h2], acc[4 * h2 + 1], acc[4 * h2 + 2], acc[4 * h2 + 3]};
-                        chunk4_apply(pj, slot0 + es, eqp, ri, r0, a4, in[h2], rs4);
+                    const int r0 = fr0 + 8 * h2;
+                    if (r0 >= g.rows) break;
+                    float a4[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        float tsum = 0.f;
+#pragma unroll
+                        for (int k = 0; k < kSmallKS; ++k) {
+                            const float v = recv[k * kSmallOwn * NS + small_off<NS>(fr + 8 * h2 + i, es)];
+                            tsum = k == 0 ? v : tsum + v;
+                        }
+                        a4[i] = tsum;
                     }
+                    chunk4_apply<true>(p, e, slot0 + es, eqp, ri, r0, a4, in[h2], rs4[h2]);
                 }
             }
             // release this CTA's part of layer j (operand and state stores) before the
@@ -1507,13 +1558,16 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
             if (any) break;
             if (warp == 2 && lane == 0) {
                 if (j < c.nl) {
-                    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(c.sync + tile) : "memory");
+                    // the next layer's partial sums may come (their senders wait for this counter)
+                    mbar_expect_tx(smem_u32(&bars[4]), recv_bytes);
+                    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(
+                                     c.sync + kSmallSyncStride * (blockIdx.x / kSmallKS))
+                                 : "memory");
                 } else {
                     __threadfence();
-                    const unsigned done = atomicAdd(c.sync + c.done_off + tile, 1u) + 1u;
+                    const unsigned done = atomicAdd(c.sync + c.done_off, 1u) + 1u;
                     if (done == nct) {
-                        atomicExch(c.sync + tile, 0u);
-                        atomicExch(c.sync + c.done_off + tile, 0u);
+                        for (int b = 0; b * kSmallSyncStride <= c.done_off; ++b) atomicExch(c.sync + kSmallSyncStride * b, 0u);
                     }
                 }
             }
@@ -1942,6 +1996,13 @@ int small_clusters_fit(relu_qp_t h) {
     return n;
 }
 
+// Words of the counters: per slot tile the tiled chunk kernel's layer and done counts, then the
+// resident-weight kernel's, 128 bytes apart: a row block each and its done count.
+static int small_sync_off(const BatchWork& w) { return ceil_div(2 * (w.slots / kSlotTile), kSmallSyncStride) * kSmallSyncStride; }
+size_t tc_sync_words(relu_qp_t h) {
+    return (size_t)small_sync_off(h->bw) + (size_t)kSmallSyncStride * (ceil_div(h->bw.RP, kSmallRows) + 1);
+}
+
 bool tc_small_eligible(relu_qp_t h, int active, int active_tiles) {
     const BatchWork& w = h->bw;
     TcState* st = static_cast<TcState*>(w.tc);
@@ -1972,8 +2033,8 @@ int tc_small(relu_qp_t h, const BatchParams& p, int nl, unsigned last_flags, int
     c.OP = static_cast<__nv_bfloat16*>(w.OPND);
     c.opart = (size_t)w.slots * w.ldk;
     c.slots = w.slots;
-    c.sync = w.chunk_sync;
-    c.done_off = w.slots / kSlotTile;
+    c.sync = w.chunk_sync + small_sync_off(w);
+    c.done_off = kSmallSyncStride * ceil_div(w.RP, kSmallRows);
     c.ncols = std::max(16, (active + 15) / 16 * 16);   // the MMA's N covers the active slots
     const int rc = active <= 32 ? launch_small<32>(h, st->opnd_map[1], st->wb_map[4], p, g, c)
                                 : launch_small<64>(h, st->opnd_map[1], st->wb_map[4], p, g, c);
