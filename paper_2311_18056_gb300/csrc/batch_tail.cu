@@ -27,7 +27,14 @@
 // residual products of the checks, spread over all warps of the grid, use a
 // warp per row: lane l computes the steps l, l + 32, ... and lane j adds QP j's
 // partials in step order.
-// Every barrier wait has a deadline after which the kernel records
+// Between two layers of a chunk the operand goes from CTA to CTA in one of two ways,
+// chosen per chunk from its live QPs.  Tagged words: an entry is one 64-bit word, value and
+// layer number together, that the readers poll themselves, so neither a barrier nor a second
+// trip for the data stands between layers.  Plain entries and a grid barrier, where so many
+// polled words would crowd the L2.  Two word buffers suffice: a CTA publishes the operand of
+// layer e + 1 (over e - 1's) once it has all of e's, which every CTA with rows sends after it
+// has all of e - 1's; a CTA without rows reads none, and every chunk ends in a barrier.
+// Every wait has a deadline after which the kernel records
 // RELU_QP_ERR_TIMEOUT and returns.
 #include "batch.h"
 #include "grid_sync.h"
@@ -47,6 +54,10 @@ struct TailArgs {
     const float* W[RQ_MAX_RHO];  // FP32 Wt of every bank entry, rows of ldk floats
     const float* Wc;            // FP32 check matrix [[P, A^T], [A, 0]], rows of ldkc floats
     float* S;                   // operand double buffer [2][kTailMax][ldk]
+    unsigned long long* words;  // the same as tagged words [2][word_stride], compact slot by slot
+    size_t word_stride;
+    unsigned tag0;              // the operand of layer `it` (counted from it0) is tagged tag0 + 1 + it
+    int word_max;               // words up to which a chunk takes them (0: never)
     float* CKB;                 // check operand [kTailMax][ldkc]
     unsigned* red;              // [3][kTailMax][RW_WORDS] reduction words, rotated per check
     unsigned* bar;              // grid barrier: arrival count of the launch (+ pad word)
@@ -65,6 +76,12 @@ struct TailArgs {
 __device__ __forceinline__ bool tail_barrier(const TailArgs& a, GridSyncState* s_ok) {
     return grid_sync(a.bar, a.err, a.timeout_ns, s_ok);
 }
+
+// Words up to which the live QPs' operands go as tagged words: what a gather keeps in flight in
+// one round (four pairs a thread).  Whole tails, us, with barriers only / 3072 / 5000 / 8000 words:
+// 8 QPs of n + m = 420 830 / 768 / 806 / 807, of 720 967 / 947 / 962 / 1037, of 1600 2375 / 2240 /
+// 2241 / 2326; one QP of 1600 579 / 413 / 414 / 413.
+constexpr int kTailWordMax = 8 * kTailThreads;
 
 constexpr int kStep = 16;       // k per partial (the tiled kernels' step)
 constexpr int kStepPad = 20;    // floats per staged step (bank spread of 16-byte reads)
@@ -422,12 +439,28 @@ __global__ void __launch_bounds__(kTailThreads, 1) batch_tail_kernel(TailArgs a)
                 rrho = p.rho[o_ri] * p.rs[o_r - p.n];
             }
         }
+        const bool tagged = nl * p.R <= a.word_max;
         for (int jl = 0; jl < len; ++jl) {
             const float* Sc = a.S + (size_t)cur * kTailMax * p.ldk;
             float* Sout = a.S + (size_t)(cur ^ 1) * kTailMax * p.ldk;
             const bool last = jl == len - 1;
-            stage_list(tsm, ops, Sc, p.ldk, p.ldk, L);
-            __syncthreads();
+            const unsigned tag = a.tag0 + 1u + (unsigned)(it - a.it0 + jl);   // of the operand this layer reads
+            if (jl == 0 || !tagged) {
+                stage_list(tsm, ops, Sc, p.ldk, p.ldk, L);     // (the padding's zeros too)
+                __syncthreads();
+            } else if (nr > 0) {
+                // over the last layer's operand, which every warp has read (barriers below)
+                auto put = [&](int k, float v) {
+                    const int j = nl == 1 ? 0 : k / p.R, r = k - j * p.R;
+                    tsm[(size_t)j * ops + (r >> 4) * kStepPad + (r & 15)] = v;
+                };
+                if (!gather_words<kTailThreads>(a.words + (tag & 1u) * a.word_stride, nl * p.R, tag, a.err, a.timeout_ns,
+                                                [&](int k, unsigned v, unsigned w, bool two) {
+                                                    put(k, __uint_as_float(v));
+                                                    if (two) put(k + 1, __uint_as_float(w));
+                                                }))
+                    return;
+            }
             for (int rl0 = 0; rl0 < nr; rl0 += a.pr) {
                 const int rl1 = min(nr, rl0 + a.pr), npr = rl1 - rl0;
                 if (rl0 > 0) __syncthreads();   // the previous pass's sums have read pbuf
@@ -479,11 +512,17 @@ __global__ void __launch_bounds__(kTailThreads, 1) batch_tail_kernel(TailArgs a)
                             p.LAM[oo] = ln;
                         }
                     }
-                    if (!last) Sout[(size_t)j * p.ldk + r] = s_new;
+                    if (!last) {
+                        if (tagged)
+                            put_word(a.words + ((tag + 1u) & 1u) * a.word_stride + (size_t)ok * p.R + r,
+                                     __float_as_uint(s_new), tag + 1u);
+                        else
+                            Sout[(size_t)j * p.ldk + r] = s_new;
+                    }
                 }
             }
             cur ^= 1;
-            if (!tail_barrier(a, &s_ok)) return;
+            if ((last || !tagged) && !tail_barrier(a, &s_ok)) return;
         }
         it += len;
         if (check) {
@@ -641,6 +680,10 @@ int batch_tail_alloc(relu_qp_t h) {
     RQ_TRY(alloc(h, &w.TRED, 3 * (size_t)kTailMax * RW_WORDS));
     RQ_TRY(alloc(h, &w.TBAR, 4));
     RQ_TRY(alloc(h, &w.TLIST, kTailMax));
+    w.tail_word_stride = round_up((size_t)kTailMax * h->R, 2);
+    RQ_TRY(alloc(h, &w.TWORDS, 2 * w.tail_word_stride));
+    RQ_CUDA(h, cudaMemset(w.TWORDS, 0, sizeof(unsigned long long) * 2 * w.tail_word_stride));
+    w.tail_tag = 0;
     int smem_max = 0;
     RQ_CUDA(h, cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
     w.tail_grid = 0;
@@ -704,6 +747,16 @@ int batch_tail(relu_qp_t h, const BatchParams& p, const DecideArgs& d, int nq, i
     a.wcache = w.tail_cache;
     a.regs = w.tail_pr >= w.tail_rpc && w.tail_rpc * kTailMax <= kTailThreads ? 1 : 0;
     a.timeout_ns = 2000000000LL;
+    a.words = w.TWORDS;
+    a.word_stride = w.tail_word_stride;
+    // the layer numbers start above every tag an earlier launch left in the words
+    if (w.tail_tag > 0x40000000u) {
+        RQ_CUDA(h, cudaMemsetAsync(w.TWORDS, 0, sizeof(unsigned long long) * 2 * w.tail_word_stride, h->stream));
+        w.tail_tag = 0;
+    }
+    a.tag0 = w.tail_tag;
+    w.tail_tag += (unsigned)(max_iter - it0) + 2u;
+    a.word_max = a.regs ? kTailWordMax : 0;
     void* args[] = {&a};
     RQ_CUDA(h, cudaLaunchCooperativeKernel((const void*)batch_tail_kernel, dim3(w.tail_grid), dim3(kTailThreads), args,
                                            w.tail_smem, h->stream));

@@ -124,6 +124,9 @@ struct BatchWork {
     float *TS = nullptr, *TCK = nullptr;
     unsigned *TRED = nullptr, *TBAR = nullptr;
     int* TLIST = nullptr;
+    unsigned long long* TWORDS = nullptr;  // its operands as tagged words, two buffers
+    size_t tail_word_stride = 0;
+    unsigned tail_tag = 0;                 // tags used so far
     int tail_grid = 0;                     // CTAs of its cooperative launch (0: unavailable)
     int tail_rpc = 0, tail_cache = 0;      // rows per CTA; 1 = those rows of Wt cached in shared memory
     int tail_pr = 0;                       // rows of the layer product per pass of the tail kernel

@@ -387,3 +387,29 @@ def test_padded_row_layout(rq, n, m):
                 assert rel(got, v[:n + m]) <= TOL_ITER[1], b
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("n,m,B", [(3, 0, 1), (5, 2, 8), (17, 20, 3), (33, 1, 2), (210, 77, 7), (400, 401, 1)])
+def test_tail_exchange_on_ragged_sizes(rq, n, m, B):
+    """The tail's operands as tagged words: an odd number of them, one CTA, CTAs without rows, one
+    to eight QPs, over several chunks, a cut-off last chunk and a second solve (other tags).  FP32:
+    the bits of the tiled kernels."""
+    rng = np.random.default_rng([5, n, m])
+    M = rng.standard_normal((n, n))
+    P = M @ M.T / n + 0.5 * np.eye(n)
+    A = rng.standard_normal((m, n)) / np.sqrt(n)
+    Q = 2.0 * rng.standard_normal((9, n))
+    L = -rng.uniform(0.1, 1.0, (9, m))
+    U = rng.uniform(0.1, 1.0, (9, m))
+    outs = []
+    for nb in (B, 9):
+        s = rq.ReluQP(P, A if m else None, L[0], U[0], q=Q[0], sigma=SIGMA, rho_bank=BANK, check_interval=7,
+                      adaptive_rho=False, rho0=BANK[0], max_batch=nb, precision=0)
+        for _ in range(2):
+            s.update_batch(Q[:nb], L[:nb], U[:nb])
+            outs.append(s.solve_batch(eps_abs=1e-12, eps_rel=0.0, max_iter=60))
+        s.close()
+    for out in outs:
+        assert np.all(out["iters"][:B] == 60)
+        for k in ("x", "z", "lam"):
+            assert np.array_equal(out[k][:B], outs[2][k][:B]), k
