@@ -1162,7 +1162,8 @@ int run_layers(relu_qp_t h, const BatchParams& p, int len, bool check, int activ
             // operand set read by this layer: 4..6 = s (3-way), else pair ((j-1)&1)
             if (timed && j == 1) RQ_CUDA(h, cudaEventRecord(h->prof_ev[prof_used], h->stream));
             RQ_TRY(tc_layer(h, q, j == 0 ? -1 : ((j - 1) & 1), tiles_max,
-                            tiles_now > 0 ? tiles_now : ceil_div(active, kSlotTile) + h->nr - 1, j > 0));
+                            tiles_now > 0 ? tiles_now : w.tiles_hint > 0 ? w.tiles_hint : ceil_div(active, kSlotTile) + h->nr - 1,
+                            j > 0));
             ++h->launches;
             if (j > 0) {
                 ++h->layer_launches;
@@ -1204,7 +1205,8 @@ int run_check(relu_qp_t h, const BatchParams& p, int active, int tiles_now) {
     if (w.prec == RELU_QP_PREC_BF16X3) {
         q.CK = static_cast<__nv_bfloat16*>(w.CK);
         const int active_tiles =
-            tiles_now > 0 ? tiles_now : std::min(tiles_max, ceil_div(active, kSlotTile) + h->nr - 1);
+            tiles_now > 0 ? tiles_now
+                          : w.tiles_hint > 0 ? w.tiles_hint : std::min(tiles_max, ceil_div(active, kSlotTile) + h->nr - 1);
         RQ_TRY(tc_check(h, q, 1, tiles_max, active_tiles));
         RQ_TRY(tc_check(h, q, 2, tiles_max, active_tiles));
     } else {
@@ -1762,6 +1764,11 @@ int server_create(relu_qp_server_t* out, relu_qp_t const* families, int nf, cons
         h->stream = f.stream;
         // families share the GPU: no persistent (one-wave, co-resident) chunk kernels
         if (h->bw.tc) tc_disable_chunk(h);
+        // The launches take the configuration tuned for the tiles that the family's slots fill.  (Any
+        // number of tiles runs under any configuration.  One tile per bank entry more, the bound on
+        // them, is mostly three times the truth; the number at hand would let a request's rounding
+        // depend on what shares the batch.)
+        h->bw.tiles_hint = ceil_div(f.cap, kSlotTile);
         const size_t cap = f.cap, cl = f.clients > 0 ? f.clients : 1;
         RQ_TRY(sdev(s, f, &f.d.idx, cap));
         RQ_TRY(sdev(s, f, &f.d.cl, cap));
@@ -1889,7 +1896,10 @@ int server_poll(relu_qp_server_t s, int max_results, relu_qp_result* results, fl
 void server_destroy(relu_qp_server_t s) {
     for (auto& f : s->fam) {
         if (f.stream) cudaStreamSynchronize(f.stream);
-        if (f.h) f.h->stream = f.saved_stream;
+        if (f.h) {
+            f.h->stream = f.saved_stream;
+            f.h->bw.tiles_hint = 0;
+        }
         for (void* p : f.dev_allocs) cudaFree(p);
         for (void* p : f.host_allocs) cudaFreeHost(p);
         if (f.ev) cudaEventDestroy(f.ev);

@@ -1039,8 +1039,8 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
 // That also orders the reuse of TMEM and of the receive buffers (a partner
 // sends layer j's partial sums only after all of layer j - 1 is done).  The
 // CTAs of a tile must be co-resident: the host launches it only when the grid
-// is at most one CTA per SM and nothing else of the handle runs beside it;
-// every wait has a deadline.
+// is at most one CTA per SM and nothing else of the handle runs beside it, or
+// with the CTAs of a tile as one cluster; every wait has a deadline.
 // ---------------------------------------------------------------------------
 struct ChunkArgs {
     int nl;                    // refined layers of the chunk (1 .. nl)
@@ -1626,6 +1626,7 @@ struct TcState {
     LayerCfg cfg{1, 128};                // refined layer: K split and width when no table is set
     std::vector<LayerCfg> cfg_by_tiles;  // [t] = the tuned configuration for t active slot tiles
     bool chunk_ok = true;                // persistent chunk kernel usable (cleared after a refused launch)
+    bool cluster_ok = true;              // the same with one cluster per slot tile
     bool small_ok = true;                // resident-weight chunk kernel usable (cleared after a refused launch)
     bool small_use = false;              // the tuner found it faster for one slot tile of few QPs
     int small_clusters = -1;             // clusters of it that fit co-resident (-1: not asked yet)
@@ -1695,7 +1696,7 @@ int launch_tc(relu_qp_t h, const CUtensorMap* a, const CUtensorMap& b, const Bat
 
 template <int BN, int KS>
 int launch_chunk(relu_qp_t h, const CUtensorMap* a, const CUtensorMap& b, const BatchParams& p, const TcArgs& g,
-                 const ChunkArgs& c, int tiles_y) {
+                 const ChunkArgs& c, int tiles_y, int cluster) {
     constexpr int S = stages_for<MODE_LAYER_REFINED, BN, KS>();
     using L = TcSmem<2, 2, BN, S, KS>;
     auto kern = tc_chunk_kernel<BN, S, KS>;
@@ -1707,9 +1708,10 @@ int launch_chunk(relu_qp_t h, const CUtensorMap* a, const CUtensorMap& b, const 
     cfg.stream = h->stream;
     cudaLaunchAttribute attr[1];
     int na = 0;
-    if (KS > 1) {
+    if (cluster > 8) RQ_CUDA(h, cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    if (cluster > 1) {
         attr[na].id = cudaLaunchAttributeClusterDimension;
-        attr[na].val.clusterDim.x = KS;
+        attr[na].val.clusterDim.x = cluster;
         attr[na].val.clusterDim.y = 1;
         attr[na].val.clusterDim.z = 1;
         ++na;
@@ -1718,13 +1720,18 @@ int launch_chunk(relu_qp_t h, const CUtensorMap* a, const CUtensorMap& b, const 
     // order after the previous launch and the host's reset) before any CTA starts
     cfg.attrs = attr;
     cfg.numAttrs = na;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a[0], a[1], b, p, g, c);
+    int fit = 1;
+    cudaError_t e = cluster > KS ? cudaOccupancyMaxActiveClusters(&fit, kern, &cfg) : cudaSuccess;
+    if (e == cudaSuccess) e = fit < 1 ? cudaErrorLaunchOutOfResources : cudaLaunchKernelEx(&cfg, kern, a[0], a[1], b, p, g, c);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return RELU_QP_ERR_UNSUPPORTED;     // the caller falls back to one launch per layer
     }
     return RELU_QP_OK;
 }
+
+// CTAs of a slot tile that may form one cluster (the non-portable limit).
+constexpr int kTileCluster = 16;
 
 // (K split, width) pairs the persistent chunk kernel is built for
 bool chunk_has(int ks, int bn) {
@@ -1734,25 +1741,25 @@ bool chunk_has(int ks, int bn) {
 }
 
 int dispatch_chunk(relu_qp_t h, int bn, int ks, const CUtensorMap* wmaps, const BatchParams& p, const TcArgs& g,
-                   const CUtensorMap* a, const ChunkArgs& c, int tiles_y) {
+                   const CUtensorMap* a, const ChunkArgs& c, int tiles_y, int cluster) {
     if (ks == 4) {
         switch (bn) {
-            case 64: return launch_chunk<64, 4>(h, a, wmaps[2], p, g, c, tiles_y);
-            case 128: return launch_chunk<128, 4>(h, a, wmaps[4], p, g, c, tiles_y);
+            case 64: return launch_chunk<64, 4>(h, a, wmaps[2], p, g, c, tiles_y, cluster);
+            case 128: return launch_chunk<128, 4>(h, a, wmaps[4], p, g, c, tiles_y, cluster);
         }
     } else if (ks == 2) {
         switch (bn) {
-            case 64: return launch_chunk<64, 2>(h, a, wmaps[2], p, g, c, tiles_y);
-            case 128: return launch_chunk<128, 2>(h, a, wmaps[4], p, g, c, tiles_y);
-            case 192: return launch_chunk<192, 2>(h, a, wmaps[6], p, g, c, tiles_y);
+            case 64: return launch_chunk<64, 2>(h, a, wmaps[2], p, g, c, tiles_y, cluster);
+            case 128: return launch_chunk<128, 2>(h, a, wmaps[4], p, g, c, tiles_y, cluster);
+            case 192: return launch_chunk<192, 2>(h, a, wmaps[6], p, g, c, tiles_y, cluster);
         }
     } else {
         switch (bn) {
-            case 16: return launch_chunk<16, 1>(h, a, wmaps[0], p, g, c, tiles_y);
-            case 32: return launch_chunk<32, 1>(h, a, wmaps[1], p, g, c, tiles_y);
-            case 64: return launch_chunk<64, 1>(h, a, wmaps[2], p, g, c, tiles_y);
-            case 96: return launch_chunk<96, 1>(h, a, wmaps[3], p, g, c, tiles_y);
-            case 128: return launch_chunk<128, 1>(h, a, wmaps[4], p, g, c, tiles_y);
+            case 16: return launch_chunk<16, 1>(h, a, wmaps[0], p, g, c, tiles_y, cluster);
+            case 32: return launch_chunk<32, 1>(h, a, wmaps[1], p, g, c, tiles_y, cluster);
+            case 64: return launch_chunk<64, 1>(h, a, wmaps[2], p, g, c, tiles_y, cluster);
+            case 96: return launch_chunk<96, 1>(h, a, wmaps[3], p, g, c, tiles_y, cluster);
+            case 128: return launch_chunk<128, 1>(h, a, wmaps[4], p, g, c, tiles_y, cluster);
         }
     }
     return RELU_QP_ERR_UNSUPPORTED;
@@ -1940,11 +1947,27 @@ bool tc_chunk_fits(relu_qp_t h, LayerCfg c, int active_tiles) {
 int tc_chunk(relu_qp_t h, const BatchParams& p, int nl, unsigned last_flags, int active_tiles) {
     BatchWork& w = h->bw;
     TcState* st = static_cast<TcState*>(w.tc);
-    if (!st->chunk_ok || nl < 1 || active_tiles < 1) return RELU_QP_ERR_UNSUPPORTED;
-    const LayerCfg lc = cfg_for(st, active_tiles);
+    const bool own = active_tiles < 1;      // a cluster per tile
+    if (!(own ? st->cluster_ok : st->chunk_ok) || nl < 1) return RELU_QP_ERR_UNSUPPORTED;
+    LayerCfg lc{1, 16};
+    int tiles_y, cluster;
+    if (own) {
+        // The active tiles are not known and other kernels may run beside this one (served): the
+        // CTAs of a tile as one cluster, which the hardware places all together or not at all.
+        // Only tiles of 16 rows, n + m <= 256: 240 requests of one family, cluster / a launch per
+        // layer, us: n + m = 160 3779 / 3855, 240 3568 / 3603, but in tiles of 32 rows 350 5855 /
+        // 5747, 480 5471 / 5357.  Beside a family of n + m = 1600 a layer at 160 takes 4.7 us
+        // instead of 12: its CTAs no longer queue for an SM in every layer.
+        cluster = ceil_div(w.RP, lc.bn);
+        if (cluster > kTileCluster || !w.chunk_sync) return RELU_QP_ERR_UNSUPPORTED;
+        tiles_y = w.slots / kSlotTile;
+    } else {
+        lc = cfg_for(st, active_tiles);
+        if (!tc_chunk_fits(h, lc, active_tiles)) return RELU_QP_ERR_UNSUPPORTED;
+        cluster = lc.ks;
+        tiles_y = std::min(active_tiles, w.slots / kSlotTile);
+    }
     const int bn = lc.bn;
-    if (!tc_chunk_fits(h, lc, active_tiles)) return RELU_QP_ERR_UNSUPPORTED;
-    const int tiles_y = std::min(active_tiles, w.slots / kSlotTile);
     TcArgs g{};
     g.num_kb = w.ldk / kBK;
     g.rows = w.RP;
@@ -1959,8 +1982,8 @@ int tc_chunk(relu_qp_t h, const BatchParams& p, int nl, unsigned last_flags, int
     c.slots = w.slots;
     c.sync = w.chunk_sync;
     c.done_off = w.slots / kSlotTile;
-    const int rc = dispatch_chunk(h, bn, lc.ks, st->wb_map, p, g, st->opnd_map, c, tiles_y);
-    if (rc == RELU_QP_ERR_UNSUPPORTED) st->chunk_ok = false;   // launch refused: not again for this handle
+    const int rc = dispatch_chunk(h, bn, lc.ks, st->wb_map, p, g, st->opnd_map, c, tiles_y, cluster);
+    if (rc == RELU_QP_ERR_UNSUPPORTED) (own ? st->cluster_ok : st->chunk_ok) = false;   // refused: not again for this handle
     return rc;
 }
 

@@ -171,3 +171,27 @@ def test_budget_holds_requests_back_then_admits(rq, families):
         assert r["iters"] == alone[0]["iters"]
         assert np.max(np.abs(r["x"] - alone[0]["x"])) <= 1e-6 * (1 + np.max(np.abs(r["x"])))
 
+
+
+@pytest.mark.parametrize("nx,nu,N", [(6, 2, 4), (6, 2, 9), (9, 3, 25), (12, 4, 32), (12, 4, 33)])
+def test_small_family_beside_a_large_one(rq, families, nx, nu, N):
+    """Families of 2 to 16 row blocks of 16 (a cluster per slot tile) and one of 17 (a launch per layer), sharing
+    the GPU with a larger one: every request as the batched solve answers it."""
+    pq = mpc.mpc_problem(nx, nu, N, 1.0, 900 + N)
+    h = rq.ReluQP(pq.P, pq.A, pq.l0, pq.u0, sigma=SIGMA, rho_bank=BANK, max_batch=150, precision=1)
+    h.set_parametric(pq.F, pq.E, pq.l0, pq.u0)
+    rng = np.random.default_rng(N)
+    X = (0.5 * rng.standard_normal((200, nx))).astype(np.float32)
+    srv = rq.Server([h, families[1][3]], eps_abs=1e-3)
+    for tag, x0 in enumerate(X):
+        srv.submit(0, x0, tag=tag)
+        if tag % 5 == 0:
+            srv.submit(1, (families[1][2] * rng.standard_normal(families[1][1].nx)).astype(np.float32), tag=1000 + tag)
+    res = {r["tag"]: r for r in run_all(srv)}
+    srv.close()
+    assert len(res) == 240 and all(r["status"] == rq.SOLVED for r in res.values())
+    for tag in range(0, 200, 9):
+        q, l, u = pq.instance(X[tag].astype(np.float64))
+        orc = O.solve(pq.P, q, pq.A, l, u, sigma=SIGMA, rho_bank=BANK, eps_abs=1e-3, max_iter=4000)
+        assert np.max(np.abs(res[tag]["x"] - orc.x)) <= 1e-3, tag
+    h.close()
