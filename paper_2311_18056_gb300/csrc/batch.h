@@ -57,6 +57,12 @@ struct BatchParams {
     unsigned flags;
 };
 
+// Programmatic dependent launch: let the next kernel of the stream start its
+// set-up, and wait until the previous kernel's results are visible (a no-op
+// for a kernel launched without the programmatic-serialisation attribute).
+__device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // max that keeps a NaN (fmaxf would drop it)
 __device__ __forceinline__ float nmax(float a, float b) { return (b > a || b != b) ? b : a; }
 

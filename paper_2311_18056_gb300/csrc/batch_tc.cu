@@ -133,12 +133,6 @@ __device__ __forceinline__ bool mbar_wait_sleep(uint32_t bar, uint32_t parity, u
     }
 }
 
-// Programmatic dependent launch: let the next kernel of the stream start its
-// set-up, and wait until the previous kernel's results are visible (a no-op
-// for a kernel launched without the programmatic-serialisation attribute).
-__device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 __device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
@@ -902,6 +896,8 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
     static_assert(PER % 16 == 0, "the epilogue works on 16-column pieces");
     using L = TcSmem<NA, NB, BN, STAGES, KS>;
 
+    // the first layer of a chunk follows the regroup, which writes the counters, perm and tile_rho
+    if (MODE == MODE_LAYER_ACCURATE) griddep_wait();
     const int tile = blockIdx.y;
     if (tile >= p.counters[CNT_TILES]) return;     // uniform over the CTA (and the cluster)
     // the partial-sum exchange addresses KS CTAs of a cluster: refuse any other launch shape
@@ -1358,6 +1354,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
     fence_after();
     cluster_sync();        // every partner's barriers are initialised before anything is sent
     const uint32_t tmem = *tmem_holder;
+    griddep_launch();
 
     if (warp == 0) {
         // ------------------------- TMA producer -------------------------
@@ -1372,6 +1369,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
                     tma_load_2d(smem_u32(sW + (part * kSmallMaxKb + b) * L::kWPart), &tmW,
                                 (kb_begin + b) * kBK, g.b_row[part] + ri * g.b_rho_stride + row0, wfull);
         }
+        griddep_wait();
         // lane l watches a row block of this CTA's k range, the last of them its own
         const int blk0 = kb_begin * kBK / kSmallRows;
         const int blk1 = min((kb_begin + kb_count) * kBK - 1, g.rows - 1) / kSmallRows;
@@ -1456,6 +1454,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
         __syncwarp();
     } else {
         // ------------------------- epilogue (warps 2-5) -------------------------
+        griddep_wait();
         const int q = warp & 3;                       // TMEM lane quadrant: rows 32 q .. 32 q + 31
         const int et = (warp - 2) * 32 + lane;        // 0 .. 127
         // this thread finalises slot es, rows fr .. fr + 3 and fr + 8 .. fr + 11 of the CTA's 16
@@ -1706,7 +1705,7 @@ int launch_chunk(relu_qp_t h, const CUtensorMap* a, const CUtensorMap& b, const 
     cfg.blockDim = dim3(kThreadsTC);
     cfg.dynamicSmemBytes = L::kBytes;
     cfg.stream = h->stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     int na = 0;
     if (cluster > 8) RQ_CUDA(h, cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     if (cluster > 1) {
@@ -1716,8 +1715,11 @@ int launch_chunk(relu_qp_t h, const CUtensorMap* a, const CUtensorMap& b, const 
         attr[na].val.clusterDim.z = 1;
         ++na;
     }
-    // no programmatic dependent launch: the layer counters must be at zero (stream
-    // order after the previous launch and the host's reset) before any CTA starts
+    // (the layer counters are at zero: the previous launch that used them put them back, and
+    // kernels that waited for its end lie between)
+    attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[na].val.programmaticStreamSerializationAllowed = 1;
+    ++na;
     cfg.attrs = attr;
     cfg.numAttrs = na;
     int fit = 1;
@@ -1776,13 +1778,15 @@ int launch_small(relu_qp_t h, const CUtensorMap& a32, const CUtensorMap& w128, c
     cfg.blockDim = dim3(kSmallThreads);
     cfg.dynamicSmemBytes = L::kBytes;
     cfg.stream = h->stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = kSmallKS;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a32, w128, p, g, c);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -1839,10 +1843,10 @@ int dispatch_3part(relu_qp_t h, int active_tiles, const CUtensorMap& b64, const 
     const long long w96 = (long long)ceil_div(g.rows, 96) * active_tiles;
     // few active tiles: the k-blocks of every tile split over a cluster of 4 or 2 CTAs
     // (at least 2 k-blocks each) while the CTAs still fit one wave
-    if (4 * w64 <= h->num_sms && g.num_kb >= 8) return launch_tc<MODE, 64, 4>(h, a, b64, p, g, tiles, false);
-    if (2 * w64 <= h->num_sms && g.num_kb >= 4) return launch_tc<MODE, 64, 2>(h, a, b64, p, g, tiles, false);
-    if (w64 > h->num_sms && w96 <= h->num_sms) return launch_tc<MODE, 96, 1>(h, a, b96, p, g, tiles, false);
-    return launch_tc<MODE, 64, 1>(h, a, b64, p, g, tiles, false);
+    if (4 * w64 <= h->num_sms && g.num_kb >= 8) return launch_tc<MODE, 64, 4>(h, a, b64, p, g, tiles, true);
+    if (2 * w64 <= h->num_sms && g.num_kb >= 4) return launch_tc<MODE, 64, 2>(h, a, b64, p, g, tiles, true);
+    if (w64 > h->num_sms && w96 <= h->num_sms) return launch_tc<MODE, 96, 1>(h, a, b96, p, g, tiles, true);
+    return launch_tc<MODE, 64, 1>(h, a, b64, p, g, tiles, true);
 }
 
 }  // namespace
