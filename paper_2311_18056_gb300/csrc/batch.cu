@@ -15,6 +15,7 @@
 // that stores c = Wt s_ref + b, and the other layers apply the 2-way split
 // only to the increment: t = c + Wt (s - s_ref).
 #include "batch.h"
+#include "grid_sync.h"
 
 #include <algorithm>
 #include <chrono>
@@ -303,7 +304,7 @@ __global__ void __launch_bounds__(256) batch_layer_fp32_kernel(BatchParams p, co
 #pragma unroll
         for (int b = 0; b < RA; ++b) {
             const int r = row0 + tx + 16 * b;
-            if (r < p.R) layer_apply(p, slot0 + ty + 16 * a, qp[a], ri, r, acc[a][b], in[EARLY ? a : 0][b]);
+            if (r < p.R) layer_apply(p, p.flags, slot0 + ty + 16 * a, qp[a], ri, r, acc[a][b], in[EARLY ? a : 0][b]);
         }
     }
 }
@@ -357,6 +358,153 @@ __global__ void __launch_bounds__(256) batch_check_fp32_kernel(BatchParams p, co
         } else {
             red_slot(p.RED, qp, RW_RD, r0);
             red_slot(p.RED, qp, RW_ATL, r1);
+        }
+    }
+}
+
+// All `nl` layers of a chunk (FP32 backend, n + m <= 512), TS slots per cluster of up to 8 CTAs
+// with 64 rows each.  A launch per layer is bound by what lies between two products: the launch,
+// the weights and the operand from L2 again, the state in and out.  Here a CTA keeps its rows of
+// Wt and the slots' operand in shared memory and its elements' state in registers, and a layer
+// is the product, one cluster barrier - every CTA has read the operand - under the element-wise
+// part, and the new operand sent by st.async into every CTA's copy, counted in bytes on its
+// mbarrier.  The arithmetic of an output is fp32_tile's and layer_apply's.
+// What bounds it is the product's shared memory reads: a 16-byte read of 32 rows is four passes
+// whoever else reads them, so a warp takes 64 rows and 4 slots (12 passes to 32 FMA
+// instructions; with 32 rows and 4 slots in 16 lanes each, 18).  The exchange takes 1.1 us.
+// A layer at n + m = 420: 7.9 us (16 slots a cluster) and 12.3 (32), with a launch per layer 12 to
+// 18; solves, ms, one launch per layer / per chunk: n + m = 420, 40 QPs 3.42 / 2.94, 333 QPs 5.13 /
+// 4.22, 1000 QPs 8.06 / 7.41; 500, 200 QPs 5.46 / 4.02; 80, 600 QPs 1.91 / 1.75.
+constexpr int kChunk32Rows = 64;
+constexpr int kChunk32MaxK = 512;      // 8 CTAs, the portable cluster
+
+template <int TS>
+constexpr int chunk32_bytes(int ld) { return (kChunk32Rows + TS) * (ld + 4) * (int)sizeof(float); }
+
+template <int TS>
+__global__ void __launch_bounds__(8 * TS, 1) batch_chunk_fp32_kernel(BatchParams p, const __grid_constant__ W32Ptrs wp,
+                                                               int nl, unsigned last_flags, int* err,
+                                                               long long timeout_ns) {
+    constexpr int THREADS = 8 * TS, NW = TS / 4, SA = 4, RA = kChunk32Rows / 32;   // a warp: 4 slots, 64 rows
+    extern __shared__ __align__(16) float fsm[];
+    __shared__ __align__(8) unsigned long long s_bar;
+    int tile, slot0;
+    if (!fp32_slots<TS>(p, tile, slot0)) return;       // uniform over the cluster
+    const int ri = p.tile_rho[tile], ld = p.ldk, lds = ld + 4, c4 = ld / 4;
+    const int row0 = blockIdx.x * kChunk32Rows, ctas = gridDim.x;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // slots ty + NW a, rows tx + 32 b
+    float* Ws = fsm;                                   // [64][lds] (rows 4 banks apart)
+    float* Xs = fsm + kChunk32Rows * lds;              // [TS][lds]
+    const uint32_t bar = cl_smem(&s_bar);
+    const uint32_t bytes = (uint32_t)(TS * ld * 4);    // a layer's operand: every CTA sends TS x 64
+    if (threadIdx.x == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        cl_expect(bar, bytes);
+    }
+    const float* W = wp.w[ri];
+    for (int e = threadIdx.x; e < kChunk32Rows * c4; e += THREADS) {
+        const int rw = e / c4, c = e - rw * c4;
+        const bool ok = row0 + rw < p.R;
+        cp_async16(Ws + rw * lds + 4 * c, ok ? W + (size_t)(row0 + rw) * ld + 4 * c : W, ok);
+    }
+    griddep_wait();
+    griddep_launch();
+    for (int e = threadIdx.x; e < TS * c4; e += THREADS) {
+        const int sl = e / c4, c = e - sl * c4;
+        cp_async16(Xs + sl * lds + 4 * c, p.Sin + (size_t)(slot0 + sl) * ld + 4 * c, true);
+    }
+    cp_async_commit();
+    int qp[SA];
+    LayerIn in[SA][RA];
+#pragma unroll
+    for (int a = 0; a < SA; ++a) {
+        qp[a] = p.perm[slot0 + ty + NW * a];
+#pragma unroll
+        for (int b = 0; b < RA; ++b)
+            if (const int r = row0 + tx + 32 * b; qp[a] >= 0 && r < p.R) layer_load(p, qp[a], ri, r, in[a][b]);
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+    cl_sync_hw();                                      // every CTA's mbarrier is armed
+    bool failed = false;                               // then only the barriers are kept
+    for (int j = 0; j < nl; ++j) {
+        const bool last = j == nl - 1;
+        if (j > 0) {
+            if (!failed && !cl_wait(bar, (uint32_t)((j - 1) & 1), err, timeout_ns)) failed = true;
+            if (threadIdx.x == 0 && !failed && !last) cl_expect(bar, bytes);
+        }
+        float acc[SA][RA];
+#pragma unroll
+        for (int a = 0; a < SA; ++a)
+#pragma unroll
+            for (int b = 0; b < RA; ++b) acc[a][b] = 0.f;
+        for (int k0 = 0; k0 < ld; k0 += 16) {
+            float part[SA][RA];
+#pragma unroll
+            for (int a = 0; a < SA; ++a)
+#pragma unroll
+                for (int b = 0; b < RA; ++b) part[a][b] = 0.f;
+#pragma unroll
+            for (int kk = k0; kk < k0 + 16; kk += 4) {
+                float4 xa[SA], wb[RA];
+#pragma unroll
+                for (int a = 0; a < SA; ++a) xa[a] = *reinterpret_cast<const float4*>(Xs + (ty + NW * a) * lds + kk);
+#pragma unroll
+                for (int b = 0; b < RA; ++b) wb[b] = *reinterpret_cast<const float4*>(Ws + (tx + 32 * b) * lds + kk);
+#pragma unroll
+                for (int a = 0; a < SA; ++a)
+#pragma unroll
+                    for (int b = 0; b < RA; ++b) {
+                        part[a][b] = fmaf(xa[a].x, wb[b].x, part[a][b]);
+                        part[a][b] = fmaf(xa[a].y, wb[b].y, part[a][b]);
+                        part[a][b] = fmaf(xa[a].z, wb[b].z, part[a][b]);
+                        part[a][b] = fmaf(xa[a].w, wb[b].w, part[a][b]);
+                    }
+            }
+#pragma unroll
+            for (int a = 0; a < SA; ++a)
+#pragma unroll
+                for (int b = 0; b < RA; ++b) acc[a][b] += part[a][b];
+        }
+        if (last) {
+            if (failed) break;
+#pragma unroll
+            for (int a = 0; a < SA; ++a)
+#pragma unroll
+                for (int b = 0; b < RA; ++b)
+                    if (const int r = row0 + tx + 32 * b; qp[a] >= 0 && r < p.R)
+                        layer_apply(p, last_flags, slot0 + ty + NW * a, qp[a], ri, r, acc[a][b], in[a][b]);
+            break;
+        }
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        float sn[SA][RA];
+#pragma unroll
+        for (int a = 0; a < SA; ++a)
+#pragma unroll
+            for (int b = 0; b < RA; ++b) {
+                const int r = row0 + tx + 32 * b;
+                sn[a][b] = qp[a] >= 0 && r < p.R ? layer_carry(p, ri, r, acc[a][b], in[a][b]) : 0.f;
+            }
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        __syncwarp();
+        // four lanes hold rows 4 q .. 4 q + 3 of two slots, for either b: transposed, a lane has
+        // four consecutive rows to send at once
+        const int jl = tx & 3;
+#pragma unroll
+        for (int a = 0; a < SA; a += 2) {
+            float o[4];
+#pragma unroll
+            for (int st = 0; st < 4; ++st) {
+                const int c = jl ^ st;
+                const float v = c == 0 ? sn[a][0] : c == 1 ? sn[a][1] : c == 2 ? sn[a + 1][0] : sn[a + 1][1];
+                const float g = __shfl_xor_sync(0xffffffffu, v, st);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (i == c) o[i] = g;
+            }
+            const uint32_t dst = cl_smem(Xs + (ty + NW * (a + (jl >> 1))) * lds + row0 + 32 * (jl & 1) + (tx & 28));
+            for (int q = 0; q < ctas; ++q) cl_send4(dst, bar, q, o[0], o[1], o[2], o[3]);
         }
     }
 }
@@ -436,6 +584,54 @@ int check32(relu_qp_t h, const BatchParams& q, const float* Wc, int tiles_max, i
     if (t.tr == 64) return launch_check32<64, 64>(h, q, Wc, tiles_max, phase);
     if (t.ts == 64) return launch_check32<64, 32>(h, q, Wc, tiles_max, phase);
     return launch_check32<32, 32>(h, q, Wc, tiles_max, phase);
+}
+
+template <int TS>
+int launch_chunk32(relu_qp_t h, const BatchParams& q, const W32Ptrs& wp, int tiles_max, int nl, unsigned last_flags) {
+    BatchWork& w = h->bw;
+    auto k = batch_chunk_fp32_kernel<TS>;
+    const int smem = chunk32_bytes<TS>(w.ldk), ctas = w.ldk / kChunk32Rows;
+    RQ_CUDA(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ctas, tiles_max * (kSlotTile / TS));
+    cfg.blockDim = dim3(8 * TS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = h->stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = ctas;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    int& fit = w.chunk32_fit[TS == 32];
+    if (fit < 0) {
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&fit, k, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            fit = 0;
+        }
+        cfg.numAttrs = 2;
+    }
+    if (nl <= 0) return RELU_QP_OK;        // (nl = 0: only w.chunk32_fit)
+    RQ_CUDA(h, cudaLaunchKernelEx(&cfg, k, q, wp, nl, last_flags, w.counters + CNT_ERR, 2000000000LL));
+    return RELU_QP_OK;
+}
+
+// The chunk's layers in one launch, or RELU_QP_ERR_UNSUPPORTED where a launch per layer is better:
+// the clusters of all slots must fit the GPU at once, preferably of 16 slots.  (In two waves the
+// tiles that fill every SM win: n + m = 420, 600 QPs 6.23 ms against 5.17, 1000 QPs 7.63 against 7.47.)
+int chunk32(relu_qp_t h, const BatchParams& q, const W32Ptrs& wp, int tiles_max, int active, int nl, unsigned last_flags) {
+    BatchWork& w = h->bw;
+    if (w.ldk > kChunk32MaxK) return RELU_QP_ERR_UNSUPPORTED;
+    auto fits = [&](int ts, int fit) { return ceil_div(active, ts) + (active > ts ? h->nr - 1 : 0) <= fit; };
+    if (w.chunk32_fit[0] < 0) RQ_TRY(launch_chunk32<16>(h, q, wp, tiles_max, 0, 0u));
+    if (fits(16, w.chunk32_fit[0])) return launch_chunk32<16>(h, q, wp, tiles_max, nl, last_flags);
+    if (w.chunk32_fit[1] < 0) RQ_TRY(launch_chunk32<32>(h, q, wp, tiles_max, 0, 0u));
+    if (fits(32, w.chunk32_fit[1])) return launch_chunk32<32>(h, q, wp, tiles_max, nl, last_flags);
+    return RELU_QP_ERR_UNSUPPORTED;
 }
 
 // Stop test and penalty rule per QP (one 128-thread block per QP: thread 0
@@ -813,6 +1009,7 @@ int batch_alloc(relu_qp_t h) {
     RQ_TRY(alloc(h, &w.perm, (size_t)w.slots));
     RQ_TRY(alloc(h, &w.tile_rho, (size_t)w.slots / kSlotTile));
     RQ_TRY(alloc(h, &w.counters, CNT_WORDS));
+    RQ_CUDA(h, cudaMemset(w.counters, 0, sizeof(int) * CNT_WORDS));
     if (bf16) {
         RQ_TRY(alloc(h, &w.C, cap * w.ldR));
         RQ_TRY(alloc(h, &w.SREF, cap * w.ldR));
@@ -1149,6 +1346,27 @@ int run_layers(relu_qp_t h, const BatchParams& p, int len, bool check, int activ
     // profiling: one event pair around the refined layers of the chunk (events
     // between them would break the programmatic overlap of consecutive layers)
     const bool timed = h->prof_on && bf16 && len > 1 && prof_used + 2 <= h->prof_ev.size();
+    if (!bf16 && j_begin == 0 && j_end >= len) {
+        BatchParams q = layer_params(h, p);
+        q.flags = 0;
+        q.Sin = w.S32;
+        q.CK32 = w.CK32;
+        const bool timed32 = h->prof_on && prof_used + 2 <= h->prof_ev.size();
+        if (timed32) RQ_CUDA(h, cudaEventRecord(h->prof_ev[prof_used], h->stream));
+        const int rc = chunk32(h, q, wp, tiles_max, active, len, EPI_LAST | (check ? EPI_CHECK : 0u));
+        if (rc != RELU_QP_ERR_UNSUPPORTED) {
+            RQ_TRY(rc);
+            ++h->launches;
+            h->layer_launches += len;
+            h->layer_flops += len * 2.0 * (double)R * (double)R * (double)active;
+            if (timed32) {
+                RQ_CUDA(h, cudaEventRecord(h->prof_ev[prof_used + 1], h->stream));
+                h->prof_span_launches.push_back(len);
+                prof_used += 2;
+            }
+            return RELU_QP_OK;
+        }
+    }
     for (int j = j_begin; j < std::min(len, j_end); ++j) {
         BatchParams q = layer_params(h, p);
         q.flags = 0;
@@ -1283,7 +1501,7 @@ int batch_solve(relu_qp_t h, int B, const float* Xw, const float* Lw, const int*
         RQ_TRY(scale_rows(h, w.LSTD, B, m, w.ldm, h->sc_li));
     }
     RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
-    if (bf16) RQ_CUDA(h, cudaMemsetAsync(w.counters + CNT_ERR, 0, 2 * sizeof(int), h->stream));
+    RQ_CUDA(h, cudaMemsetAsync(w.counters + CNT_ERR, 0, 2 * sizeof(int), h->stream));
     RQ_TRY(zero_chunk_sync(h));
     batch_init_kernel<<<w.cap, kInitThreads, 0, h->stream>>>(p, B, Xw != nullptr, Lw != nullptr && m > 0,
                                                                         rw_dev, rho0, w.status, w.rho_idx, w.iters,
@@ -1364,12 +1582,16 @@ int batch_solve(relu_qp_t h, int B, const float* Xw, const float* Lw, const int*
             RQ_TRY(fill_slots(h, p, true));
         }
     }
+    if (!bf16)
+        RQ_CUDA(h, cudaMemcpyAsync(w.cnt_host, w.counters, sizeof(int) * CNT_WORDS, cudaMemcpyDeviceToHost, h->stream));
     RQ_CUDA(h, cudaEventRecord(h->ev1, h->stream));
     RQ_CUDA(h, cudaStreamSynchronize(h->stream));
     if (bf16) {
         const int e = tc_error(h);
         if (e == RELU_QP_ERR_TIMEOUT) return fail(h, e, "a tensor-core kernel wait passed its deadline");
         if (e) return fail(h, RELU_QP_ERR_CUDA, "a tensor-core kernel found a launch shape it cannot run");
+    } else if (w.cnt_host[CNT_ERR]) {
+        return fail(h, RELU_QP_ERR_TIMEOUT, "a wait of the FP32 chunk kernel passed its deadline");
     }
     if (tail_used && batch_tail_error(h))
         return fail(h, RELU_QP_ERR_TIMEOUT, "a grid barrier of the convergence-tail kernel passed its deadline");

@@ -148,9 +148,8 @@ __device__ __forceinline__ void layer_load(const BatchParams& p, int qp, int ri,
     in.rs = p.rs[i];
 }
 
-__device__ __forceinline__ void layer_apply(const BatchParams& p, int slot, int qp, int ri, int r, float acc,
-                                            const LayerIn& in) {
-    const unsigned f = p.flags;
+__device__ __forceinline__ void layer_apply(const BatchParams& p, unsigned f, int slot, int qp, int ri, int r,
+                                            float acc, const LayerIn& in) {
     const float t = acc + in.b;
     float s_new;
     if (r < p.n) {
@@ -170,10 +169,22 @@ __device__ __forceinline__ void layer_apply(const BatchParams& p, int slot, int 
     if (!(f & EPI_LAST)) p.Sout[(size_t)slot * p.ldk + r] = s_new;
 }
 
+// The same update with the state kept in `in`: the operand entry of the next layer.
+__device__ __forceinline__ float layer_carry(const BatchParams& p, int ri, int r, float acc, LayerIn& in) {
+    const float t = acc + in.b;
+    if (r < p.n) return t;
+    const float rho_i = p.rho[ri] * in.rs;
+    const float rr = ax_row_carry(in.ay, in.z, in.lam, rho_i);
+    float s_new;
+    ax_row_update(t, rr, in.lo, in.up, rho_i, in.z, in.lam, s_new);
+    in.ay = t;
+    return s_new;
+}
+
 __device__ __forceinline__ void layer_elem(const BatchParams& p, int slot, int qp, int ri, int r, float acc) {
     LayerIn in{};
     layer_load(p, qp, ri, r, in);
-    layer_apply(p, slot, qp, ri, r, acc, in);
+    layer_apply(p, p.flags, slot, qp, ri, r, acc, in);
 }
 
 __device__ __forceinline__ void ld4(const float* __restrict__ src, float (&v)[4]) {

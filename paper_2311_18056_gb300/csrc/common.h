@@ -98,6 +98,7 @@ struct BatchWork {
     // rows of the layer: x in [0, nP), A x in [nP, RP).  FP32 form: nP = n, RP = n + m.  BF16
     // form: both parts padded with zero rows to multiples of 16, the epilogues' piece
     int nP = 0, RP = 0;
+    int chunk32_fit[2] = {-1, -1};  // FP32 chunk kernel, 16 and 32 slots: clusters the GPU holds (-1: not asked yet)
     int tiles_hint = 0;  // served: slot tiles the launches are configured for (0: not served)
     int ldn = 0, ldm = 0, ldR = 0, ldk = 0, n64 = 0, m64 = 0, ldkc = 0, Rpad = 0, npad = 0;
     // check matrix [[P, A^T], [A, 0]]: (n + m) rows (padded to npad), ldkc = n64 + m64 columns

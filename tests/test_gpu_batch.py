@@ -413,3 +413,31 @@ def test_tail_exchange_on_ragged_sizes(rq, n, m, B):
         assert np.all(out["iters"][:B] == 60)
         for k in ("x", "z", "lam"):
             assert np.array_equal(out[k][:B], outs[2][k][:B]), k
+
+
+@pytest.mark.parametrize("n,m", [(3, 0), (33, 31), (64, 64), (70, 59), (250, 262), (500, 12), (257, 256)])
+def test_fp32_chunk_kernel_on_ragged_sizes(rq, n, m):
+    """FP32 chunks in one launch per chunk (up to n + m = 512, one to eight CTAs a cluster, 16 or 32 slots) and in
+    one per layer (more QPs than fit at once, n + m = 513): the same bits in a batch of 20, 300 and 700, over whole
+    and cut-off chunks."""
+    rng = np.random.default_rng([7, n, m])
+    M = rng.standard_normal((n, n))
+    P = M @ M.T / n + 0.5 * np.eye(n)
+    A = rng.standard_normal((m, n)) / np.sqrt(n)
+    Q = 2.0 * rng.standard_normal((700, n))
+    L = -rng.uniform(0.1, 1.0, (700, m))
+    U = rng.uniform(0.1, 1.0, (700, m))
+    outs = []
+    for nb in (20, 300, 700):
+        s = rq.ReluQP(P, A if m else None, L[0], U[0], q=Q[0], sigma=SIGMA, rho_bank=BANK, check_interval=7,
+                      adaptive_rho=False, rho0=BANK[0], max_batch=nb, precision=0)
+        s.update_batch(Q[:nb], L[:nb], U[:nb])
+        outs.append(s.solve_batch(eps_abs=1e-12, eps_rel=0.0, max_iter=17))
+        s.close()
+    for out in outs[1:]:
+        for k in ("x", "z", "lam"):
+            assert np.array_equal(out[k][:20], outs[0][k]), k
+    for b in (0, 19):
+        v = O.layer_iterates(P, Q[b], A, L[b], U[b], SIGMA, BANK[0], 17)[-1]
+        got = np.concatenate([outs[0]["x"][b], outs[0]["z"][b]]).astype(np.float64)
+        assert rel(got, v[:n + m]) <= TOL_ITER[0], b
