@@ -170,7 +170,7 @@ int relu_qp_update(relu_qp_t h, const double* q, const double* l, const double* 
  *   x_out             n FP64 (required); z_out, lam_out m FP64 (may be NULL).
  *                     lam_out is the standard ADMM multiplier lam' + rho (Ax - z).
  *   info              may be NULL
- * The whole loop runs in one cooperative kernel on the device (FP32, or FP64
+ * The whole loop runs in one kernel on the device (FP32, or FP64
  * when opts.single_precision = RELU_QP_PREC_FP64); the host waits only for
  * its end.  Errors: INVALID, CUDA, TIMEOUT.
  */
