@@ -333,7 +333,7 @@ __device__ __forceinline__ void tail_fill(const TailArgs& a, float* S, const int
 __global__ void __launch_bounds__(kTailThreads, 1) batch_tail_kernel(TailArgs a) {
     extern __shared__ __align__(16) float tsm[];
     __shared__ GridSyncState s_ok;
-    __shared__ int s_live[kTailMax], s_ri[kTailMax], s_act[kTailMax], s_nri[kTailMax], s_any;
+    __shared__ int s_live[kTailMax], s_ri[kTailMax], s_act[kTailMax], s_nri[kTailMax], s_any, s_switched;
     grid_sync_init(&s_ok);
     __shared__ unsigned s_red[kTailMax][RW_WORDS];
     // the launch's parameters are read in place: per-layer values (the operand the layer
@@ -485,7 +485,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) batch_tail_kernel(TailArgs a)
                     if (!a.regs) {
                         BatchParams q = p;
                         q.Sout = Sout;
-                        q.flags = last ? (EPI_LAST | (check ? EPI_CHECK : 0u)) : 0u;
+                        q.flags = last ? (last_chunk ? EPI_LAST : 0u) | (check ? EPI_CHECK : 0u) : 0u;
                         layer_elem(q, j, a.qlist[j], s_ri[j], r, acc);
                         continue;
                     }
@@ -512,8 +512,8 @@ __global__ void __launch_bounds__(kTailThreads, 1) batch_tail_kernel(TailArgs a)
                             p.LAM[oo] = ln;
                         }
                     }
-                    if (!last) {
-                        if (tagged)
+                    if (!last || !last_chunk) {
+                        if (tagged && !last)
                             put_word(a.words + ((tag + 1u) & 1u) * a.word_stride + (size_t)ok * p.R + r,
                                      __float_as_uint(s_new), tag + 1u);
                         else
@@ -606,13 +606,14 @@ __global__ void __launch_bounds__(kTailThreads, 1) batch_tail_kernel(TailArgs a)
             }
             __syncthreads();
             if (threadIdx.x == 0) {
-                int any = 0;
+                int any = 0, sw = 0;
                 for (int j = 0; j < nq; ++j) {
                     if (s_act[j] == 1) s_live[j] = 0;
-                    if (s_act[j] == 2) s_ri[j] = s_nri[j];
+                    if (s_act[j] == 2) s_ri[j] = s_nri[j], sw = 1;
                     any |= s_live[j];
                 }
                 s_any = any;
+                s_switched = sw;
             }
             __syncthreads();
             // outputs of finished QPs; lam' rebase of switched ones
@@ -632,13 +633,18 @@ __global__ void __launch_bounds__(kTailThreads, 1) batch_tail_kernel(TailArgs a)
                     p.LAM[oo] = lam_standard(p.LSTD[oo], -rho_i, p.AY[oo] - p.Z[oo]);
                 }
             }
-            if (!s_any) return;
-            if (!tail_barrier(a, &s_ok)) return;
+            if (!s_any || last_chunk) return;
+            // The next chunk's first operand is the one this chunk's last layer has written.  Only a
+            // switch of penalty changes lam' and with it the operand (every CTA knows: they all decide
+            // alike); a fill and two barriers after every check took 2 us (tail of one QP, n + m = 1600:
+            // 413 -> 406 us; of an FP32 batch of 333, n = 210: 846 -> 823).
+            if (s_switched) {
+                if (!tail_barrier(a, &s_ok)) return;
+                tail_fill(a, a.S + (size_t)cur * kTailMax * p.ldk, s_live, s_ri);
+                if (!tail_barrier(a, &s_ok)) return;
+            }
         }
         if (last_chunk) return;
-        // operand of the next chunk's first layer from the state
-        tail_fill(a, a.S + (size_t)cur * kTailMax * p.ldk, s_live, s_ri);
-        if (!tail_barrier(a, &s_ok)) return;
     }
 }
 
