@@ -240,6 +240,8 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
     // the check's product, lam_std
     float *st_rr = st_bias + per, *st_z = st_rr + per, *st_lam = st_z + per, *st_rho = st_lam + per,
           *st_l = st_rho + per, *st_u = st_l + per, *st_chk = st_u + per, *st_ls = st_chk + per;
+    // (from the rounded lam' in every layer, as the batched FP32 path forms it: with t - z + r instead
+    // a multiplier that is zero keeps other rounding noise)
     auto carry = [&](float ax, float z, float lam, float rho_i) { return ax - z + lam / rho_i; };
     // barriers (cluster form): operand buffers 0 and 1, lam_std, maxima
     const uint32_t bar0 = cl_smem(mbar);
@@ -314,7 +316,11 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
         // z = A x
         const float* x = is_grid(F) ? sv : sv + ldw;
         for (int lr = nx + warp; lr < rows; lr += kWarps) {
-            const float v = row_dot(p.A + (size_t)(a0 + lr - nx) * p.ldp, x, p.ldp, lane);
+            const float* a = p.A + (size_t)(a0 + lr - nx) * p.ldp;
+            float v = 0.f;
+#pragma unroll 4
+            for (int k = lane; k < n; k += 32) v = fmaf(__ldg(a + k), x[k], v);
+            v = warp_sum(v);
             if (lane == 0) st_z[lr] = v;
         }
         __syncthreads();
@@ -391,17 +397,17 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
             const bool ax = work && lr >= nx;
             const float bias = work ? st_bias[lr] : 0.f, rho_i = ax ? st_rho[lr] : 0.f, lo = ax ? st_l[lr] : 0.f,
                         up = ax ? st_u[lr] : 0.f, rho2 = 2.0f * rho_i;
-            float rr = ax ? st_rr[lr] : 0.f, z = 0.f, lam = 0.f;
+            float rr = ax ? st_rr[lr] : 0.f, t = 0.f, z = 0.f, lam = 0.f;
             for (int k = 0; k < len; ++k) {
                 if (work && !failed) {
-                    z = product(G, cur()) + bias;
+                    if (ax && k > 0) rr = carry(t, z, lam, rho_i);   // (beside the product, not after it)
+                    t = product(G, cur()) + bias;
+                    z = t;
                     float snew = z;
                     if (ax) {
-                        const float t = z;
                         z = fminf(fmaxf(t + rr, lo), up);
                         lam = __fmul_rn(rho_i, rr);
                         snew = fmaf(rho2, z, -lam);
-                        rr = t - z + rr;
                     }
                     hand_on(G, lr, valid, one, snew);
                 }
@@ -428,14 +434,13 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
                         z = fminf(fmaxf(t + rr, st_l[lr]), st_u[lr]);
                         lam = __fmul_rn(st_rho[lr], rr);
                         snew = fmaf(2.0f * st_rho[lr], z, -lam);
-                        rr = t - z + rr;
                     }
                     hand_on(G, lr, valid, one, snew);
                     if (one) {
                         st_z[lr] = z;
                         if (ax) {
                             st_lam[lr] = lam;
-                            st_rr[lr] = rr;
+                            st_rr[lr] = carry(t, z, lam, st_rho[lr]);
                         }
                     }
                     __syncwarp();
@@ -661,22 +666,17 @@ __global__ void __launch_bounds__(256) bias_kernel(BiasPtrs b, int rows, int n, 
     const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (r >= rows) return;
     const float* w = b.Bop[blockIdx.y] + (size_t)r * n;
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-    if ((n & 3) == 0) {
-        const float4 *w4 = reinterpret_cast<const float4*>(w), *q4 = reinterpret_cast<const float4*>(q);
-#pragma unroll 4
-        for (int k = lane; k < (n >> 2); k += 32) {
-            const float4 x = __ldg(w4 + k), y = __ldg(q4 + k);
-            a0 = fmaf(x.x, y.x, a0);
-            a1 = fmaf(x.y, y.y, a1);
-            a2 = fmaf(x.z, y.z, a2);
-            a3 = fmaf(x.w, y.w, a3);
-        }
-    } else {
-#pragma unroll 4
-        for (int k = lane; k < n; k += 32) a0 = fmaf(__ldg(w + k), __ldg(q + k), a0);
+    float v = 0.f;
+    int k = lane;
+    for (; k + 7 * 32 < n; k += 8 * 32) {      // eight loads in flight, the products in order
+        float x[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) x[t] = __ldg(w + k + 32 * t);
+#pragma unroll
+        for (int t = 0; t < 8; ++t) v = fmaf(x[t], __ldg(q + k + 32 * t), v);
     }
-    const float v = warp_sum((a0 + a1) + (a2 + a3));
+    for (; k < n; k += 32) v = fmaf(__ldg(w + k), __ldg(q + k), v);
+    v = warp_sum(v);
     if (lane == 0) b.bias[blockIdx.y][r] = v;
 }
 
