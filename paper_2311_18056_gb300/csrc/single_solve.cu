@@ -35,7 +35,7 @@
 // registers while every warp has one group of rows; a check's FP64 decision is one warp's.
 //
 // Measured, us per layer at n = m = 20 / 160 / 320 / 640 / 800 / 1600 (200 fixed layers,
-// best shape): 0.44 / 0.77 / 1.19 / 1.80 / 2.54 / 4.26; with a barrier between layers and
+// best shape): 0.55 / 0.90 / 1.22 / 2.04 / 2.47 / 4.34; with a barrier between layers and
 // the operand loaded after it 1.61 / 1.98 / 2.23 / 2.72 / 2.92 / 4.75.  The last is bound
 // by reading the rows (41 MB a layer from shared memory and L2), the others by the
 // exchange: 0.25 (one CTA), 0.6 (cluster), 1.2 (words), 2.2 (count).
