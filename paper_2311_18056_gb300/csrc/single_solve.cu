@@ -266,6 +266,12 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
     auto wait_bar = [&](uint32_t bar, uint32_t parity) {
         if (!failed && !cl_wait(bar, parity, p.err, p.timeout_ns)) failed = true;
     };
+    // (count form) exchange x, all of it stored, into shared memory
+    auto load_operand = [&](unsigned x) {
+        const float4* src = reinterpret_cast<const float4*>(p.sop + (size_t)(x & 1) * ldw);
+        for (int k = tid; k < (ldw >> 2); k += kThreads) reinterpret_cast<float4*>(sv)[k] = __ldcg(src + k);
+        __syncthreads();
+    };
     auto receive = [&](unsigned x) -> bool {
         if (F == FORM_GRID) {
             __syncthreads();   // the buffer's readers are done
@@ -274,9 +280,7 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
         if (F == FORM_COUNT) {
             // every CTA has stored its entries and read the last operand
             if (!count_wait(p.count, p.count0 + (x + 1) * (unsigned)p.ctas, p.err, p.timeout_ns)) return false;
-            const float4* src = reinterpret_cast<const float4*>(p.sop + (size_t)(x & 1) * ldw);
-            for (int k = tid; k < (ldw >> 2); k += kThreads) reinterpret_cast<float4*>(sv)[k] = __ldcg(src + k);
-            __syncthreads();
+            load_operand(x);
             return true;
         }
         if (F == FORM_ONE) {
@@ -595,11 +599,11 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
         if (nri == ri) {
             // the directly computed Ax replaces the carried one
             for (int lr = nx + tid; lr < rows; lr += kThreads) st_rr[lr] = carry(st_chk[lr], st_z[lr], st_lam[lr], st_rho[lr]);
-            if (is_grid(F) && p.share) {
-                if (!receive(e)) return;
-            } else {
-                __syncthreads();   // the state above is read by the rows' warps
-            }
+            // lam_std was staged over the operand: read that again.  Without another arrival: the
+            // exchange is complete, and its buffer is stored to again (e + 2) only after every CTA
+            // has arrived at e + 1, which it does after this.
+            if (F == FORM_COUNT && p.share) load_operand(e);
+            else __syncthreads();   // the state above is read by the rows' warps
             continue;
         }
         // switch: rebase lam' so that the next layer is standard ADMM with the new rho, and

@@ -332,3 +332,28 @@ def test_operand_larger_than_both_staged_vectors(rq):
     assert np.max(np.abs(A @ o["x"] - o["z"])) <= 1e-3 * RES_SLACK
     assert np.max(np.abs(P @ o["x"] + q + A.T @ o["lam"])) <= 1e-3 * RES_SLACK
     assert np.all(o["z"] >= l - 1e-6) and np.all(o["z"] <= u + 1e-6)
+
+
+def test_operand_read_again_after_checks_stays_in_step(rq):
+    """n + m above 32768 with a check every 5 layers and no switch of penalty: the operand is read again after
+    every check without a second arrival in the count that orders the layers.  Entries of another layer would
+    change the bits from solve to solve and from grid to grid, and miss the oracle's iterates."""
+    n, m, layers = 100, 32720, 50
+    rng = np.random.default_rng(8)
+    M = rng.standard_normal((n, n))
+    P = M @ M.T / n + 0.5 * np.eye(n)
+    A = rng.standard_normal((m, n)) / np.sqrt(n)
+    q = 2.0 * rng.standard_normal(n)
+    l, u = -np.ones(m), np.ones(m)
+    s = rq.ReluQP(P, A, l, u, q=q, sigma=SIGMA, rho_bank=(0.1,), rho0=0.1, adaptive_rho=False, check_interval=5)
+    outs = []
+    for ctas in (152, 64):
+        s.set_single_config(ctas)
+        outs += [s.solve(eps_abs=0.0, max_iter=layers) for _ in range(2)]
+    s.close()
+    x, z, _ = O.admm_iterates(P, q, A, l, u, SIGMA, 0.1, layers)[-1]
+    for o in outs:
+        assert o["iters"] == layers and o["rho_switches"] == 0
+        for k in ("x", "z", "lam"):
+            assert np.array_equal(o[k], outs[0][k]), k
+        assert rel(np.concatenate([o["x"], o["z"]]), np.concatenate([x, z])) <= 1e-5
