@@ -471,7 +471,9 @@ int relu_qp_single_set_config(relu_qp_t h, int ctas, int cluster);
  *   arrival count (passes; the control case); kind 2: an mbarrier wait that
  *   nothing completes; kind 3: a layer-counter wait that nothing increments;
  *   kind 4: a cluster of 2 CTAs whose exchange (the one the single-QP solve
- *   uses in its cluster form) expects one word more than is sent;
+ *   uses in its cluster form) expects one word more than is sent, with half of
+ *   each warp's lanes on a wait that has completed (status INVALID if a lane
+ *   went on without its warp);
  *   kind 5: the same exchange with the right count, three rounds (passes).  timeout_ns in [1e3, 1e9].  *status receives the
  *   kernel's error word (RELU_QP_ERR_TIMEOUT, or 0 when the wait completed),
  *   *ms (may be NULL) the device time of the launch.  Returns INVALID, OOM,

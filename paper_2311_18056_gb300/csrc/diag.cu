@@ -33,29 +33,39 @@ __global__ void diag_grid_kernel(unsigned* bar, int* err, unsigned expected, lon
 
 // One cluster of CTAs that hand each other one word `rounds` times; each CTA's
 // mbarrier expects `extra` words more than are sent (extra = 1: every CTA waits
-// until the deadline).  Every CTA then reaches the final hardware cluster
-// barrier (no CTA exits while a partner may still write its shared memory).
+// until the deadline).  Whole warps wait.  With extra words half of every warp's
+// lanes wait on a barrier that has completed instead: the warp's verdict must be
+// the other half's, and a lane that went on alone leaves RELU_QP_ERR_INVALID.
+// Every CTA then reaches the final hardware cluster barrier (no CTA exits while
+// a partner may still write its shared memory).
 __global__ void diag_cluster_kernel(int* err, int ctas, int extra, int rounds, long long timeout_ns) {
     // two barriers, as in the solve: a word of round k + 2 (round k's barrier) leaves only
     // once its sender has round k + 1, which every CTA sends after it has all of round k
-    __shared__ __align__(8) unsigned long long s_bar[2];
+    __shared__ __align__(8) unsigned long long s_bar[3];   // [2]: complete from the start
     __shared__ float s_words[2][16];
     const uint32_t bytes = 4u * (uint32_t)(ctas + extra);
     if (threadIdx.x == 0) {
-        for (int b = 0; b < 2; ++b) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(cl_smem(&s_bar[b])) : "memory");
+        for (int b = 0; b < 3; ++b) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(cl_smem(&s_bar[b])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         for (int b = 0; b < 2; ++b) cl_expect(cl_smem(&s_bar[b]), bytes);
+        cl_expect(cl_smem(&s_bar[2]), 0u);
     }
     cl_sync_hw();
-    if (threadIdx.x == 0)
-        for (int k = 0; k < rounds; ++k) {
-            const uint32_t bar = cl_smem(&s_bar[k & 1]);
+    const bool apart = extra > 0 && (threadIdx.x & 16);
+    bool alone = false;
+    for (int k = 0; k < rounds; ++k) {
+        const uint32_t bar = cl_smem(&s_bar[k & 1]);
+        if (threadIdx.x == 0)
             for (int q = 0; q < ctas; ++q) cl_send1(cl_smem(&s_words[k & 1][blockIdx.x]), bar, q, (float)k);
-            if (!cl_wait(bar, (k >> 1) & 1, err, timeout_ns)) break;
-            cl_expect(bar, bytes);
-        }
+        __syncwarp();
+        const bool ok = cl_wait_warp(apart ? cl_smem(&s_bar[2]) : bar, apart ? 0 : (k >> 1) & 1, err, timeout_ns);
+        alone = extra > 0 && ok;
+        if (__syncthreads_or(ok ? 0 : 1)) break;
+        if (threadIdx.x == 0) cl_expect(bar, bytes);
+    }
     __syncthreads();
     cl_sync_hw();
+    if (alone) atomicExch(err, RELU_QP_ERR_INVALID);
 }
 
 // Host policy of barrier_arrive_wait: C++ atomics on the same words.

@@ -245,6 +245,12 @@ __device__ __forceinline__ bool cl_wait(uint32_t bar, uint32_t parity, int* err,
     }
     return true;
 }
+// The same by a whole warp, with one verdict for it: lanes poll apart, so that the word of an
+// error elsewhere can reach some before the phase completes and find the others done, and a
+// warp that went on in part would wait for ever in its next shuffle or barrier.
+__device__ __forceinline__ bool cl_wait_warp(uint32_t bar, uint32_t parity, int* err, long long timeout_ns) {
+    return __all_sync(0xffffffffu, cl_wait(bar, parity, err, timeout_ns)) != 0;
+}
 // hardware barrier of every thread of the cluster (no deadline: only where every CTA is
 // known to arrive, at the start and at the end of a kernel)
 __device__ __forceinline__ void cl_sync_hw() {

@@ -262,9 +262,10 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
             for (int q = 0; q < p.ctas; ++q) cl_send1(sv_a + 4u * ((x & 1) * ldw + r), bar0 + 8 * (x & 1), q, v);
         }
     };
-    // all of exchange x (cluster form: a warp's own wait, by the warps that compute rows)
+    // all of exchange x (cluster form: a warp's own wait, by the warps that compute rows; whole
+    // warps call it, and `failed` is the same in every lane)
     auto wait_bar = [&](uint32_t bar, uint32_t parity) {
-        if (!failed && !cl_wait(bar, parity, p.err, p.timeout_ns)) failed = true;
+        if (!failed && !cl_wait_warp(bar, parity, p.err, p.timeout_ns)) failed = true;
     };
     // (count form) exchange x, all of it stored, into shared memory
     auto load_operand = [&](unsigned x) {

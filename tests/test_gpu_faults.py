@@ -64,6 +64,15 @@ def test_device_wait_gives_up_at_its_deadline(rq, kind, what):
     assert np.max(np.abs(out["x"] - ref.x)) <= 1e-3
 
 
+def test_cluster_wait_has_one_verdict_per_warp(rq):
+    """Half of each warp's lanes wait on a barrier that has completed, the others on a word that never comes: every
+    lane gives up with its warp (kind 4 answers INVALID for a lane that went on), at more than one deadline."""
+    for ns in (50_000, 200_000, 1_000_000):
+        rc, status, ms = device_wait(rq, 4, ns)
+        assert (rc, status) == (0, TIMEOUT), ns
+        assert ms < 100.0
+
+
 @pytest.mark.parametrize("kind", [1, 5], ids=["grid barrier", "cluster barrier"])
 def test_barrier_with_every_arrival_passes(rq, kind):
     rc, status, ms = device_wait(rq, kind, 1_000_000)
