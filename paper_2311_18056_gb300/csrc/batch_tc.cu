@@ -25,6 +25,7 @@
 // mbarrier wait has a deadline; on expiry the kernel records an error, waits
 // (bounded) for its own copies and MMAs, frees TMEM and returns.
 #include "batch.h"
+#include "grid_sync.h"
 
 #include <cuda.h>
 
@@ -1575,6 +1576,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
     fence_before();
     __syncthreads();
     cluster_sync();        // no CTA leaves while a partner may still write into its shared memory
+    if (s_fail) cl_settle();
     if (warp == 1) {
         fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TCOLS) : "memory");

@@ -36,8 +36,7 @@ __global__ void diag_grid_kernel(unsigned* bar, int* err, unsigned expected, lon
 // until the deadline).  Whole warps wait.  With extra words half of every warp's
 // lanes wait on a barrier that has completed instead: the warp's verdict must be
 // the other half's, and a lane that went on alone leaves RELU_QP_ERR_INVALID.
-// Every CTA then reaches the final hardware cluster barrier (no CTA exits while
-// a partner may still write its shared memory).
+// Every CTA then reaches the closing cluster barrier.
 __global__ void diag_cluster_kernel(int* err, int ctas, int extra, int rounds, long long timeout_ns) {
     // two barriers, as in the solve: a word of round k + 2 (round k's barrier) leaves only
     // once its sender has round k + 1, which every CTA sends after it has all of round k
@@ -63,8 +62,7 @@ __global__ void diag_cluster_kernel(int* err, int ctas, int extra, int rounds, l
         if (__syncthreads_or(ok ? 0 : 1)) break;
         if (threadIdx.x == 0) cl_expect(bar, bytes);
     }
-    __syncthreads();
-    cl_sync_hw();
+    cl_close(extra > 0);
     if (alone) atomicExch(err, RELU_QP_ERR_INVALID);
 }
 

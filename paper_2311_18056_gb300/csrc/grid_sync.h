@@ -256,6 +256,25 @@ __device__ __forceinline__ bool cl_wait_warp(uint32_t bar, uint32_t parity, int*
 __device__ __forceinline__ void cl_sync_hw() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// What partners sent before a closing cluster barrier lands some us later at most.  A CTA that has
+// waited for every byte sent to it can leave after the barrier; one whose wait gave up stays this
+// long before its shared memory goes to another.
+__device__ __forceinline__ void cl_settle() {
+    for (const long long t0 = grid_sync_timer(); grid_sync_timer() - t0 < 50000;) {}
+}
+// The end of a kernel whose CTAs write into each other's shared memory: reached by every thread
+// of the cluster, so that no CTA leaves while a partner may still send to it.  A thread arrives
+// once it sends no more, and waits last (`failed`: a wait of this thread gave up).
+__device__ __forceinline__ void cl_close_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cl_close_wait(bool failed) {
+    const int gave_up = __syncthreads_or(failed ? 1 : 0);
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    if (gave_up) cl_settle();
+}
+__device__ __forceinline__ void cl_close(bool failed) {
+    cl_close_arrive();
+    cl_close_wait(failed);
+}
 #endif
 
 }  // namespace rq

@@ -217,9 +217,9 @@ __device__ __forceinline__ void red_max(unsigned* slot, int word, float v) {
     atomicMax(slot + word, __float_as_uint(fabsf(v)));
 }
 
-// The solve.
+// The solve; false if a wait gave up.
 template <int F>
-__device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned long long* mbar, unsigned* s_red,
+__device__ __forceinline__ bool solve_body(const SP& p, float* smem, unsigned long long* mbar, unsigned* s_red,
                                            unsigned* s_dec) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
     const int n = p.n, m = p.m, R = p.R, ldw = p.ldw, cta = blockIdx.x;
@@ -342,7 +342,7 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
         failed = __syncthreads_or(failed ? 1 : 0) != 0;
         if (tid == 0 && !failed) cl_expect(bar0, 4u * R);
     } else if (!receive(0)) {
-        return;
+        return false;
     }
 
     // Groups: the rows that are not in shared memory first (their loads take longest), one to
@@ -417,7 +417,7 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
                     hand_on(G, lr, valid, one, snew);
                 }
                 ++e;
-                if (!receive(e)) return;
+                if (!receive(e)) return false;
             }
             if (one) {
                 st_z[lr] = z;
@@ -451,7 +451,7 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
                     __syncwarp();
                 }
                 ++e;
-                if (!receive(e)) return;
+                if (!receive(e)) return false;
             }
         }
         it += len;
@@ -460,7 +460,7 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
 
         // ---------------- residuals (Eqs. primal, dual) ----------------
         // (a warp of the cluster form that gave up leaves here, with its CTA)
-        if (__syncthreads_or(failed ? 1 : 0)) return;
+        if (__syncthreads_or(failed ? 1 : 0)) return false;
         const float* svc = cur();
         const unsigned tag = p.tag0 + 1 + e;
         constexpr int kC = 2, kPer = 32 / kC;   // rows of a warp (in global memory: P, A, A^T)
@@ -501,12 +501,12 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
                 __syncthreads();
                 for (int k = m + tid; k < p.ldt; k += kThreads) svk[k] = 0.f;
             }
-            if (m > 0 && !gather(p, p.wls, svk, m, tag)) return;
+            if (m > 0 && !gather(p, p.wls, svk, m, tag)) return false;
         } else if (F == FORM_ONE) {
             __syncthreads();
         } else if (m > 0) {
             wait_bar(bar0 + 16, checks & 1);
-            if (__syncthreads_or(failed ? 1 : 0)) return;
+            if (__syncthreads_or(failed ? 1 : 0)) return false;
             if (tid == 0) cl_expect(bar0 + 16, 4u * m);
         }
         for (int lr0 = warp * kC; lr0 < nx; lr0 += kWarps * kC) {
@@ -528,14 +528,14 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
         // every CTA's maxima
         if (is_grid(F)) {
             if (tid < RED_WORDS) put_word(p.wred + RED_WORDS * cta + tid, s_red[tid], tag);
-            if (!gather(p, p.wred, reds, RED_WORDS * p.ctas, tag)) return;
+            if (!gather(p, p.wred, reds, RED_WORDS * p.ctas, tag)) return false;
         } else if (F == FORM_CLUSTER) {
             for (int t = tid; t < 2 * p.ctas; t += kThreads) {
                 const float* v = reinterpret_cast<const float*>(s_red) + 4 * (t & 1);
                 cl_send4(reds_a + 4u * (uint32_t)(RED_WORDS * cta + 4 * (t & 1)), bar0 + 24, t >> 1, v[0], v[1], v[2], v[3]);
             }
             wait_bar(bar0 + 24, checks & 1);
-            if (__syncthreads_or(failed ? 1 : 0)) return;
+            if (__syncthreads_or(failed ? 1 : 0)) return false;
             if (tid == 0) cl_expect(bar0 + 24, 4u * RED_WORDS * p.ctas);
         } else {
             if (tid < RED_WORDS) reinterpret_cast<unsigned*>(reds)[tid] = s_red[tid];
@@ -594,7 +594,7 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
                 p.out_f[0] = __uint_as_float(s_dec[RED_RP]);
                 p.out_f[1] = __uint_as_float(s_dec[RED_RD]);
             }
-            return;
+            return true;
         }
         const int nri = (int)s_dec[DEC_RHO];
         if (nri == ri) {
@@ -630,7 +630,7 @@ __device__ __forceinline__ void solve_body(const SP& p, float* smem, unsigned lo
         load_w_cache(p, wcache, ri, x0, nx, a0, ncache);
         __syncthreads();
         ++e;
-        if (!receive(e)) return;
+        if (!receive(e)) return false;
     }
 }
 
@@ -652,13 +652,8 @@ __global__ void __launch_bounds__(kThreads, 1) single_solve_kernel(const __grid_
         }
         cl_sync_hw();   // every CTA's barriers stand before anything is sent
     }
-    if ((int)blockIdx.x < p.ctas) solve_body<F>(p, smem, s_bar, s_red, s_dec);
-    if (F == FORM_CLUSTER) {
-        // no CTA leaves while a partner may still write its shared memory (every
-        // wait before this point has a deadline, so every CTA gets here)
-        __syncthreads();
-        cl_sync_hw();
-    }
+    const bool done = (int)blockIdx.x >= p.ctas || solve_body<F>(p, smem, s_bar, s_red, s_dec);
+    if (F == FORM_CLUSTER) cl_close(!done);   // (every wait before has a deadline, so every CTA gets here)
 }
 
 // b_r = Bop_r q for every bank entry (blockIdx.y), one warp per row.
