@@ -87,7 +87,7 @@ struct SP {
     double eps_abs, eps_rel, qnorm;
     int xr, ar, ctas;         // rows of x and of A x per CTA, CTAs with rows
     int gs, gu, cached_rows;  // rows of a warp's group, of a group outside shared memory
-    int share;                // grid form of a problem too large for both: lam_std staged over the operand
+    int share;                // count form, where both do not fit: lam_std staged over the operand
     long long timeout_ns;
 };
 
@@ -234,7 +234,7 @@ __device__ __forceinline__ bool solve_body(const SP& p, float* smem, unsigned lo
     float* sv = smem + (size_t)p.cached_rows * ldw;        // operand: two buffers (grids: one)
     float* svk = sv + (size_t)(is_grid(F) ? 1 : 2) * ldw;  // lam_std (ldt floats)
     float* reds = svk + (p.share ? 0 : p.ldt);             // every CTA's maxima [ctas][8]
-    if (is_grid(F) && p.share) svk = sv;                   // (read again after the check)
+    if (F == FORM_COUNT && p.share) svk = sv;              // (read again after the check)
     float* st_bias = reds + RED_WORDS * p.ctas;
     // per row: bias, r = (Ax) - z + lam'/rho of the next layer, z (x of a row of x), lam', rho, l, u,
     // the check's product, lam_std
@@ -497,7 +497,7 @@ __device__ __forceinline__ bool solve_body(const SP& p, float* smem, unsigned lo
             }
         }
         if (is_grid(F)) {
-            if (p.share) {
+            if (F == FORM_COUNT && p.share) {
                 __syncthreads();
                 for (int k = m + tid; k < p.ldt; k += kThreads) svk[k] = 0.f;
             }
@@ -702,8 +702,12 @@ Form form_of(relu_qp_t h, int ctas, int cluster) {
     return cluster > 1 ? FORM_CLUSTER : ctas == 1 ? FORM_ONE : h->R <= kTagMax ? FORM_GRID : FORM_COUNT;
 }
 
-// lam_std has no room of its own beside an operand of more than 32768 entries (128 KB)
-bool share_lam(relu_qp_t h, int ctas, int cluster) { return is_grid(form_of(h, ctas, cluster)) && h->ldw > 32768; }
+// lam_std is staged over the operand where the two together pass 208 KB: of a CTA's 227 KB the
+// maxima and the state of its rows take up to 15 KB on 152 CTAs (n + m = 40000).
+constexpr size_t kStageMax = 53248;
+bool share_lam(relu_qp_t h, int ctas, int cluster) {
+    return form_of(h, ctas, cluster) == FORM_COUNT && h->ldw + round_up(h->m, 4) > kStageMax;
+}
 
 // gs: rows of a warp's group (the cluster form: 4, one 16-byte store)
 void fill_params(relu_qp_t h, SP& p, int ctas, int cluster, int gs, int cached) {

@@ -357,3 +357,31 @@ def test_operand_read_again_after_checks_stays_in_step(rq):
         for k in ("x", "z", "lam"):
             assert np.array_equal(o[k], outs[0][k]), k
         assert rel(np.concatenate([o["x"], o["z"]]), np.concatenate([x, z])) <= 1e-5
+
+
+@pytest.mark.parametrize("n,m", [(100, 26500), (100, 26700), (100, 28300), (1, 32703), (2700, 28000)])
+def test_every_split_of_a_large_problem_is_taken(rq, n, m):
+    """Operand and lam_std beside each other in shared memory (n + 2 m up to about 53000) and one over the other
+    beyond it, whatever n + m is: every size below the limit of n + m sets up, and layers with checks match the
+    oracle's."""
+    layers = 15
+    rng = np.random.default_rng(9)
+    P = np.diag(rng.uniform(0.5, 1.5, n))
+    A = np.zeros((m, n))
+    A[np.arange(m), rng.integers(0, n, m)] = rng.uniform(0.5, 1.5, m)
+    q = 2.0 * rng.standard_normal(n)
+    l, u = -rng.uniform(0.1, 1.0, m), rng.uniform(0.1, 1.0, m)
+    s = rq.ReluQP(P, A, l, u, q=q, sigma=SIGMA, rho_bank=(0.1,), rho0=0.1, adaptive_rho=False, check_interval=5)
+    o = s.solve(eps_abs=0.0, max_iter=layers)
+    s.close()
+    assert o["iters"] == layers
+    # one entry a row of A and P diagonal: the oracle's step, element by element
+    col, a = A.argmax(1), A.max(1)
+    D = 1.0 / (np.diag(P) + SIGMA + 0.1 * np.bincount(col, a * a, n))
+    x, z, lam = np.zeros(n), np.zeros(m), np.zeros(m)
+    for _ in range(layers):
+        x = D * (SIGMA * x - q + np.bincount(col, a * (0.1 * z - lam), n))
+        ax = a * x[col]
+        z = np.clip(ax + lam / 0.1, l, u)
+        lam = lam + 0.1 * (ax - z)
+    assert rel(np.concatenate([o["x"], o["z"]]), np.concatenate([x, z])) <= 1e-5
