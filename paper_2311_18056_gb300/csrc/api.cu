@@ -270,6 +270,16 @@ int dev_alloc(relu_qp_t h, void** p, size_t bytes) {
     return RELU_QP_OK;
 }
 
+int allow_shared(relu_qp_t h, const void* k, int* room) {
+    int optin = 0;
+    cudaFuncAttributes fa{};
+    RQ_CUDA(h, cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
+    RQ_CUDA(h, cudaFuncGetAttributes(&fa, k));
+    *room = optin - (int)fa.sharedSizeBytes;
+    RQ_CUDA(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, *room));
+    return RELU_QP_OK;
+}
+
 }  // namespace rq
 
 extern "C" {

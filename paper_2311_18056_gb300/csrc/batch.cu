@@ -597,7 +597,6 @@ int launch_chunk32(relu_qp_t h, const BatchParams& q, const W32Ptrs& wp, int til
     BatchWork& w = h->bw;
     auto k = batch_chunk_fp32_kernel<TS>;
     const int smem = chunk32_bytes<TS>(w.ldk), ctas = w.ldk / kChunk32Rows;
-    RQ_CUDA(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(ctas, tiles_max * (kSlotTile / TS));
     cfg.blockDim = dim3(8 * TS);
@@ -614,6 +613,8 @@ int launch_chunk32(relu_qp_t h, const BatchParams& q, const W32Ptrs& wp, int til
     cfg.numAttrs = 2;
     int& fit = w.chunk32_fit[TS == 32];
     if (fit < 0) {
+        int room = 0;
+        RQ_TRY(allow_shared(h, (const void*)k, &room));
         cfg.numAttrs = 1;
         if (cudaOccupancyMaxActiveClusters(&fit, k, &cfg) != cudaSuccess) {
             cudaGetLastError();

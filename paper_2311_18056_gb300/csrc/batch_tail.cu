@@ -691,7 +691,7 @@ int batch_tail_alloc(relu_qp_t h) {
     RQ_CUDA(h, cudaMemset(w.TWORDS, 0, sizeof(unsigned long long) * 2 * w.tail_word_stride));
     w.tail_tag = 0;
     int smem_max = 0;
-    RQ_CUDA(h, cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
+    RQ_TRY(allow_shared(h, (const void*)batch_tail_kernel, &smem_max));
     w.tail_grid = 0;
     // one CTA per SM and (while the SMs suffice) one row of the layer per warp; the CTA's
     // rows of Wt cached in shared memory when they fit (every CTA co-resident: grid
@@ -701,9 +701,7 @@ int batch_tail_alloc(relu_qp_t h) {
     for (int cache = 1; cache >= 0; --cache) {
         for (int pr = rpc;; pr = std::max(kRG, pr / 2)) {
             const size_t smem = tail_smem(h, pr, cache ? rpc : 0);
-            if (smem + 1024 <= (size_t)smem_max) {
-                RQ_CUDA(h, cudaFuncSetAttribute(batch_tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)smem));
+            if (smem <= (size_t)smem_max) {
                 int per_sm = 0;
                 RQ_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_tail_kernel, kTailThreads,
                                                                          smem));

@@ -198,6 +198,11 @@ int alloc(relu_qp_t h, T** p, size_t count) {
     return dev_alloc(h, reinterpret_cast<void**>(p), count * sizeof(T) + 16);
 }
 
+// Lets kernel k use all the dynamic shared memory that a block of h's device can have beside the
+// kernel's own (*room).  The limit belongs to the kernel, not to a launch: were it a handle's own
+// size, another handle's set-up, or a launch from another thread, would put it below this one's.
+int allow_shared(relu_qp_t h, const void* k, int* room);
+
 // FP64 building blocks of the offline stage (setup_fp64.cu), on h->stream:
 // C = alpha op(A) op(B) + beta C (row-major); D (ldd) <- K^{-1} for nb symmetric positive
 // definite n x n matrices s doubles apart (lower triangles read, Km overwritten; Lm and Li:

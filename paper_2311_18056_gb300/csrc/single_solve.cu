@@ -756,16 +756,13 @@ const void* kernel_of(relu_qp_t h, int ctas, int cluster) {
 }
 
 // Rows of Wt a CTA can cache: what the opt-in shared memory holds beside the rest; -1 when
-// not even the rest fits.
+// not even the rest fits.  (Also readies the shape's kernel for its launches.)
 int cached_rows_for(relu_qp_t h, int ctas, int cluster) {
-    int v = 0;
-    cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-    cudaFuncAttributes fa{};
-    if (cudaFuncGetAttributes(&fa, kernel_of(h, ctas, cluster)) == cudaSuccess) v -= (int)fa.sharedSizeBytes;
-    cudaGetLastError();
+    int room = 0;
+    if (allow_shared(h, kernel_of(h, ctas, cluster), &room) != RELU_QP_OK) return -1;
     int xr, ar, used;
     slices(h, ctas, cluster > 1, &xr, &ar, &used);
-    const long left = (long)v - 256 - (long)smem_bytes(h, 0, ctas, cluster);
+    const long left = (long)room - 256 - (long)smem_bytes(h, 0, ctas, cluster);
     if (left < 0) return -1;
     return (int)std::min<long>(xr + ar, left / (long)((size_t)h->ldw * sizeof(float)));
 }
@@ -790,8 +787,6 @@ cudaLaunchConfig_t cluster_config(relu_qp_t h, int ctas, size_t smem, cudaLaunch
 int launch_kernel(relu_qp_t h, SP& p, int ctas, int cluster) {
     const size_t smem = smem_bytes(h, p.cached_rows, ctas, cluster);
     const void* k = kernel_of(h, ctas, cluster);
-    RQ_CUDA(h, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (cluster > 8) RQ_CUDA(h, cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     void* args[] = {&p};
     if (cluster > 1) {
         cudaLaunchAttribute at[1];
@@ -805,20 +800,19 @@ int launch_kernel(relu_qp_t h, SP& p, int ctas, int cluster) {
     return RELU_QP_OK;
 }
 
-// Whether the shape can be resident.  (Each launch sets the kernel's shared-memory limit to
-// its own size; the queries need it at least this large.)
+// Whether the shape can be resident.
 bool fits(relu_qp_t h, int ctas, int cluster, int cached) {
     if (cached < 0) return false;
     const size_t smem = smem_bytes(h, cached, ctas, cluster);
     const void* k = kernel_of(h, ctas, cluster);
-    bool ok = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
+    bool ok;
     int n = 0;
-    if (ok && cluster > 1) {
+    if (cluster > 1) {
         ok = cluster <= 8 || cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
         cudaLaunchAttribute at[1];
         const cudaLaunchConfig_t cfg = cluster_config(h, ctas, smem, at);
         ok = ok && cudaOccupancyMaxActiveClusters(&n, k, &cfg) == cudaSuccess && n >= 1;
-    } else if (ok) {
+    } else {
         ok = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, kThreads, smem) == cudaSuccess && n >= 1 &&
              ctas <= n * h->num_sms;
     }

@@ -513,7 +513,6 @@ int launch(relu_qp_t h, int grid, const double* xin, const double* lin, int rho_
     w.last_ctas = p.ctas;
     w.out_i[OUT_LAST] = -1;   // the kernel's results go to host memory
     RQ_CUDA(h, cudaMemsetAsync(w.red, 0, sizeof(unsigned long long) * 3 * RED_WORDS, h->stream));
-    RQ_CUDA(h, cudaFuncSetAttribute(kernel_for(h), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     void* args[] = {&p};
     RQ_CUDA(h, cudaLaunchCooperativeKernel(kernel_for(h), dim3(grid), dim3(kThreads), args, smem, h->stream));
     return RELU_QP_OK;
@@ -601,11 +600,9 @@ int single64_update(relu_qp_t h) {
 // fixed-rho layers (no checks), the largest first, until one is 1.3x slower than the best.
 int single64_prepare(relu_qp_t h) {
     SingleWork64& w = h->sw64;
-    cudaFuncAttributes fa{};
-    RQ_CUDA(h, cudaFuncGetAttributes(&fa, kernel_for(h)));
-    int v = 0;
-    RQ_CUDA(h, cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
-    w.smem_max = (size_t)v - fa.sharedSizeBytes - 256;
+    int room = 0;
+    RQ_TRY(allow_shared(h, kernel_for(h), &room));
+    w.smem_max = (size_t)room - 256;
     std::vector<int> cands{h->num_sms};
     for (int g = 1; g < h->num_sms; g *= 2) cands.push_back(g);
     std::sort(cands.begin(), cands.end(), std::greater<int>());

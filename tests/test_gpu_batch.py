@@ -441,3 +441,55 @@ def test_fp32_chunk_kernel_on_ragged_sizes(rq, n, m):
         v = O.layer_iterates(P, Q[b], A, L[b], U[b], SIGMA, BANK[0], 17)[-1]
         got = np.concatenate([outs[0]["x"][b], outs[0]["z"][b]]).astype(np.float64)
         assert rel(got, v[:n + m]) <= TOL_ITER[0], b
+
+
+def _box_problem(rq, n, B, prec, seed=0):
+    rng = np.random.default_rng([13, n, seed])
+    M = rng.standard_normal((n, n))
+    P = M @ M.T / n + 0.5 * np.eye(n)
+    A = rng.standard_normal((n, n)) / np.sqrt(n)
+    Q = 2.0 * rng.standard_normal((B, n))
+    one = np.ones((B, n))
+    return rq.ReluQP(P, A, -one[0], one[0], sigma=SIGMA, rho_bank=BANK, max_batch=B, precision=prec), Q, one
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_handles_of_two_sizes_side_by_side(rq, prec):
+    """A handle set up after another one leaves the first one's launches alone (batch tail, FP32 chunk kernel, both
+    single solves take shared memory by the handle's size), from one thread and from two."""
+    import threading
+    a, Qa, ua = _box_problem(rq, 230, 6, prec)
+
+    def run(s, Q, u):
+        s.update_batch(Q, -u, u)
+        out = s.solve_batch(eps_abs=1e-3)
+        s.update(Q[0].astype(np.float64), -u[0], u[0])
+        return out, s.solve(eps_abs=1e-3)
+
+    ref = run(a, Qa, ua)
+    assert np.all(ref[0]["status"] == rq.SOLVED)
+    b, Qb, ub = _box_problem(rq, 20, 6, prec)
+    refb = run(b, Qb, ub)
+    faults = []
+
+    def again(s, Q, u, want, times):
+        try:
+            for _ in range(times):
+                for o, r in zip(run(s, Q, u), want):
+                    assert all(np.array_equal(o[k], r[k]) for k in ("x", "z", "lam"))
+        except Exception as e:   # noqa: BLE001
+            faults.append(repr(e))
+
+    again(a, Qa, ua, ref, 1)
+    threads = [threading.Thread(target=again, args=x) for x in ((a, Qa, ua, ref, 40), (b, Qb, ub, refb, 40))]
+    for t in threads:
+        t.start()
+    for k in range(3):
+        c, Qc, uc = _box_problem(rq, 31, 6, prec, k)
+        run(c, Qc, uc)
+        c.close()
+    for t in threads:
+        t.join()
+    a.close()
+    b.close()
+    assert not faults, faults
