@@ -44,6 +44,7 @@
 // in the error word; the other waits see it and leave too.
 #include "common.h"
 #include "grid_sync.h"
+#include "shape_search.h"
 
 #include <algorithm>
 #include <cmath>
@@ -934,51 +935,49 @@ int default_gs(relu_qp_t h, int ctas, int cluster) {
 int single_prepare(relu_qp_t h) {
     SingleWork& w = h->sw;
     w.grid = 0;
-    float best_t = 1e30f;
-    auto time = [&](int g, int cl, int cached, int gs, float* out) -> int {
-        float ms = 0.f;
-        for (int layers : {10, 50}) {   // a warm-up, then the timed run
-            RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
-            RQ_TRY(launch(h, g, cl, cached, gs, nullptr, nullptr, 0, 0.0, 0.0, layers, 0, 0));
-            RQ_CUDA(h, cudaEventRecord(h->ev1, h->stream));
-            RQ_CUDA(h, cudaStreamSynchronize(h->stream));
-            RQ_TRY(finish(h, "while tuning the solve"));
-            RQ_CUDA(h, cudaEventElapsedTime(&ms, h->ev0, h->ev1));
-        }
-        if (ms < best_t) {
-            best_t = ms;
-            w.grid = g;
-            w.cluster = cl;
-            w.cached_rows = cached;
-            w.gs = gs;
-        }
-        *out = ms;
+    float best = 1e30f;
+    auto time = [&](int g, int cl, int cached, int gs, int layers, float* ms) -> int {
+        RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
+        RQ_TRY(launch(h, g, cl, cached, gs, nullptr, nullptr, 0, 0.0, 0.0, layers, 0, 0));
+        RQ_CUDA(h, cudaEventRecord(h->ev1, h->stream));
+        RQ_CUDA(h, cudaStreamSynchronize(h->stream));
+        RQ_TRY(finish(h, "while tuning the solve"));
+        RQ_CUDA(h, cudaEventElapsedTime(ms, h->ev0, h->ev1));
         return RELU_QP_OK;
     };
-    // Grids, then clusters, the largest first.  The time falls, if at all, to one minimum and
-    // then rises with the rows per CTA, so a family ends at the first shape 1.3x slower than its
-    // best (a small grid or cluster of a large problem takes 100 times the best: 25 ms of the
+    // Grids, then clusters, the largest first: beyond its minimum the time rises with the rows
+    // per CTA (a small grid or cluster of a large problem takes 100 times the best: 25 ms of the
     // setup at n = m = 800).
     std::vector<int> grids{h->num_sms}, clusters{16, 8, 4, 2};
     for (int g = 1; g <= 4 * h->num_sms; g *= 2) grids.push_back(g);
     std::sort(grids.begin(), grids.end(), std::greater<int>());
     for (const bool cl : {false, true}) {
-        float family = 1e30f;
-        for (int c : cl ? clusters : grids) {
-            const int cached = c <= h->R ? cached_rows_for(h, c, cl ? c : 0) : -1;
-            if (!fits(h, c, cl ? c : 0, cached)) continue;
-            float ms = 0.f;
-            RQ_TRY(time(c, cl ? c : 0, cached, default_gs(h, c, cl ? c : 0), &ms));
-            if (ms > 1.3f * family || ms > 3.0f * best_t) break;
-            family = std::min(family, ms);
-        }
+        const std::vector<int>& ctas = cl ? clusters : grids;
+        int cached = -1, chosen = -1;
+        RQ_TRY(search_family((int)ctas.size(), [&](int k, bool warm, float* ms) -> int {
+            const int c = ctas[k], cluster = cl ? c : 0;
+            if (warm) {
+                cached = c <= h->R ? cached_rows_for(h, c, cluster) : -1;
+                *ms = -1.f;
+                if (!fits(h, c, cluster, cached)) return RELU_QP_OK;
+            }
+            return time(c, cluster, cached, default_gs(h, c, cluster), warm ? 10 : 50, ms);
+        }, &best, &chosen));
+        if (chosen < 0) continue;
+        w.grid = ctas[chosen];
+        w.cluster = cl ? w.grid : 0;
+        w.cached_rows = cached_rows_for(h, w.grid, w.cluster);
+        w.gs = default_gs(h, w.grid, w.cluster);
     }
     if (w.grid == 0) return fail(h, RELU_QP_ERR_UNSUPPORTED, "the single-QP solve does not fit on an SM");
-    if (w.cluster <= 1) {
-        const int g = w.grid, cached = w.cached_rows, gs0 = w.gs;
-        float ms;
-        for (int gs : {1, 2, 4})
-            if (gs != gs0) RQ_TRY(time(g, 0, cached, gs, &ms));
+    const int gs0 = w.gs;
+    for (int gs : {1, 2, 4}) {
+        float ms = 0.f;
+        if (w.cluster > 1 || gs == gs0) continue;
+        for (int layers : {10, 50}) RQ_TRY(time(w.grid, 0, w.cached_rows, gs, layers, &ms));
+        if (ms >= best) continue;
+        best = ms;
+        w.gs = gs;
     }
     return RELU_QP_OK;
 }

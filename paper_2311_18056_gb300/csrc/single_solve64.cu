@@ -35,6 +35,7 @@
 // (anchored) 817 and 340 us.
 #include "common.h"
 #include "grid_sync.h"
+#include "shape_search.h"
 
 #include <algorithm>
 #include <cmath>
@@ -597,7 +598,7 @@ int single64_update(relu_qp_t h) {
 }
 
 // CTA count of the cooperative launch: the fastest of the co-resident candidates over 50
-// fixed-rho layers (no checks), the largest first, until one is 1.3x slower than the best.
+// fixed-rho layers (no checks), the largest first.
 int single64_prepare(relu_qp_t h) {
     SingleWork64& w = h->sw64;
     int room = 0;
@@ -606,26 +607,22 @@ int single64_prepare(relu_qp_t h) {
     std::vector<int> cands{h->num_sms};
     for (int g = 1; g < h->num_sms; g *= 2) cands.push_back(g);
     std::sort(cands.begin(), cands.end(), std::greater<int>());
-    w.grid = 0;
-    float best_t = 1e30f;
-    for (int g : cands) {
-        if (g > h->R || smem64(h, g, 0) > w.smem_max) continue;
-        float ms = 0.f;
-        for (int layers : {10, 50}) {   // a warm-up, then the timed run
-            RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
-            RQ_TRY(launch(h, g, nullptr, nullptr, 0, 0.0, 0.0, layers, 0, 0));
-            RQ_CUDA(h, cudaEventRecord(h->ev1, h->stream));
-            RQ_CUDA(h, cudaStreamSynchronize(h->stream));
-            RQ_TRY(finish(h, "while tuning the FP64 solve"));
-            RQ_CUDA(h, cudaEventElapsedTime(&ms, h->ev0, h->ev1));
-        }
-        if (ms > 1.3f * best_t) break;
-        if (ms < best_t) {
-            best_t = ms;
-            w.grid = g;
-        }
-    }
-    if (w.grid == 0) return fail(h, RELU_QP_ERR_UNSUPPORTED, "FP64 solve kernel does not fit on an SM");
+    float best = 1e30f;
+    int chosen = -1;
+    RQ_TRY(search_family((int)cands.size(), [&](int k, bool warm, float* ms) -> int {
+        const int g = cands[k];
+        *ms = -1.f;
+        if (g > h->R || smem64(h, g, 0) > w.smem_max) return RELU_QP_OK;
+        RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
+        RQ_TRY(launch(h, g, nullptr, nullptr, 0, 0.0, 0.0, warm ? 10 : 50, 0, 0));
+        RQ_CUDA(h, cudaEventRecord(h->ev1, h->stream));
+        RQ_CUDA(h, cudaStreamSynchronize(h->stream));
+        RQ_TRY(finish(h, "while tuning the FP64 solve"));
+        RQ_CUDA(h, cudaEventElapsedTime(ms, h->ev0, h->ev1));
+        return RELU_QP_OK;
+    }, &best, &chosen));
+    if (chosen < 0) return fail(h, RELU_QP_ERR_UNSUPPORTED, "FP64 solve kernel does not fit on an SM");
+    w.grid = cands[chosen];
     return RELU_QP_OK;
 }
 
