@@ -16,6 +16,7 @@
 // only to the increment: t = c + Wt (s - s_ref).
 #include "batch.h"
 #include "grid_sync.h"
+#include "tile32.h"
 
 #include <algorithm>
 #include <chrono>
@@ -515,33 +516,6 @@ __global__ void __launch_bounds__(8 * TS, 1) batch_chunk_fp32_kernel(BatchParams
     cl_close_wait(failed);
 }
 
-// Tile of a launch over `rows` rows and `active` QPs (nr bank groups, each with a part of a
-// tile left over).  A tile's time is its FMAs, shared by the CTAs of an SM, but at least some
-// 250 clocks per 16 columns of k (loads, barriers), so small problems want more, smaller tiles.
-// Whole solves, ms, with one tile throughout (32 x 32, 64 x 32, 64 x 64, 128 x 64):
-// n + m = 420, 333 QPs: 5.4, 6.2, 9.7, 13.8; n + m = 1600, 300 QPs: 32.6, 30.7, 38.2, 55.5;
-// 1000 QPs: 75, 67, 63, 78 (128 x 64 was the best nowhere and is gone).
-struct Tile32 {
-    int ts, tr;
-};
-
-Tile32 tile32(relu_qp_t h, int rows, int active) {
-    Tile32 best{32, 32};
-    double best_t = 1e300;
-    for (const Tile32 c : {Tile32{64, 64}, Tile32{64, 32}, Tile32{32, 32}}) {
-        const double ctas = (double)ceil_div(rows, c.tr) * (ceil_div(active, c.ts) + (active > c.ts ? 0.5 * (h->nr - 1) : 0.0));
-        const double per_sm = std::ceil(ctas / h->num_sms);
-        // FMAs of 16 columns at 60 % of 128 a clock (the smallest tile: of its shared memory reads)
-        const double fma = c.ts * c.tr * 16 / (c.ts * c.tr > 1024 ? 77.0 : 56.0);
-        const double t = std::max(per_sm * fma, 250.0);
-        if (t < best_t) {
-            best_t = t;
-            best = c;
-        }
-    }
-    return best;
-}
-
 // pdl: the kernel may start before the previous one of the stream has ended (its griddep_wait)
 template <class K, class... Args>
 int launch_pdl(relu_qp_t h, K k, dim3 grid, int threads, int smem, bool pdl, Args... args) {
@@ -572,7 +546,7 @@ int launch_layer32(relu_qp_t h, const BatchParams& q, const W32Ptrs& wp, int til
 }
 
 int layer32(relu_qp_t h, const BatchParams& q, const W32Ptrs& wp, int tiles_max, int active, bool pdl) {
-    const Tile32 t = tile32(h, h->R, active);
+    const Tile32 t = tile32(h->R, active, h->nr, h->num_sms);
     if (t.tr == 64) return launch_layer32<64, 64>(h, q, wp, tiles_max, pdl);
     if (t.ts == 64) return launch_layer32<64, 32>(h, q, wp, tiles_max, pdl);
     return launch_layer32<32, 32>(h, q, wp, tiles_max, pdl);
@@ -586,7 +560,7 @@ int launch_check32(relu_qp_t h, const BatchParams& q, const float* Wc, int tiles
 }
 
 int check32(relu_qp_t h, const BatchParams& q, const float* Wc, int tiles_max, int active, int phase) {
-    const Tile32 t = tile32(h, phase == 1 ? h->n + h->m : h->n, active);
+    const Tile32 t = tile32(phase == 1 ? h->n + h->m : h->n, active, h->nr, h->num_sms);
     if (t.tr == 64) return launch_check32<64, 64>(h, q, Wc, tiles_max, phase);
     if (t.ts == 64) return launch_check32<64, 32>(h, q, Wc, tiles_max, phase);
     return launch_check32<32, 32>(h, q, Wc, tiles_max, phase);
