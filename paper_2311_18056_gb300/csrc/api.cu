@@ -26,12 +26,6 @@ bool bounds_ok(const double* l, const double* u, int m) {
     return true;
 }
 
-std::vector<float> to_f32(const double* p, size_t n) {
-    std::vector<float> v(n);
-    for (size_t i = 0; i < n; ++i) v[i] = (float)p[i];
-    return v;
-}
-
 // Algorithm 1 "Scale problem" (Sec. III-D "Preconditioning"): a modified Ruiz
 // equilibration of the KKT matrix K = [[P, A^T], [A, 0]] in FP64.  Each iteration
 // divides column j of K (and row j, K being symmetric) by the square root of its

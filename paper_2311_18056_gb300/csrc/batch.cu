@@ -1457,7 +1457,7 @@ int nearest_rho(relu_qp_t h, double rho) {
 int batch_solve(relu_qp_t h, int B, const float* Xw, const float* Lw, const int* rw, double eps_abs,
                 double eps_rel, int max_iter, float* Xo, float* Zo, float* Lo, relu_qp_info* infos) {
     BatchWork& w = h->bw;
-    const int n = h->n, m = h->m, R = h->R;
+    const int n = h->n, m = h->m;
     const bool bf16 = w.prec == RELU_QP_PREC_BF16X3;
     BatchParams p = base_params(h);
     const int tiles_max = w.slots / kSlotTile;

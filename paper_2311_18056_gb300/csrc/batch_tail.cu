@@ -421,7 +421,8 @@ __global__ void __launch_bounds__(kTailThreads, 1) batch_tail_kernel(TailArgs a)
         // a.regs: thread o owns output (row row_beg + o % nr, compact slot o / nr); its state
         // (bias of the QP's bank entry, and for rows of A x the carried A x, z, lam', l, u,
         // rho_i) stays in registers for the chunk: loaded here, written back at the chunk's
-        // last layer (the checks, the decision and the next chunk's fill read it from memory)
+        // last layer (the check, the decision, the next chunk's loads here and, after a switch of
+        // penalty, the fill read it from memory)
         const int ok = nr > 0 ? (int)threadIdx.x / nr : kTailMax, orl = nr > 0 ? (int)threadIdx.x % nr : 0;
         const bool own = a.regs && ok < nl;
         const int oj = own ? L.j[ok] : 0;

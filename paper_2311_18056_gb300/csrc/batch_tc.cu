@@ -215,18 +215,6 @@ __device__ __forceinline__ void tmem_sum32(uint32_t ta, uint32_t tb, float (&v)[
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]) + __uint_as_float(s[i]);
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 // --- thread-block cluster (K-split pair) helpers ---
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
@@ -1032,7 +1020,8 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
 // one to the tile's counter, and a producer requests the operand of layer j
 // only once the counter shows every CTA of the tile done with layer j - 1.  The
 // counters start at zero and the tile's last CTA puts them back to zero at the
-// end (launches are in stream order, without programmatic overlap).
+// end: the launch may overlap the kernel before it, but that one is never a chunk
+// of the same counters (launch_chunk).
 // That also orders the reuse of TMEM and of the receive buffers (a partner
 // sends layer j's partial sums only after all of layer j - 1 is done).  The
 // CTAs of a tile must be co-resident: the host launches it only when the grid

@@ -36,9 +36,9 @@
 //
 // Measured, us per layer at n = m = 20 / 160 / 320 / 640 / 800 / 1600 (200 fixed layers,
 // best shape): 0.55 / 0.90 / 1.22 / 2.04 / 2.47 / 4.34; with a barrier between layers and
-// the operand loaded after it 1.61 / 1.98 / 2.23 / 2.72 / 2.92 / 4.75.  The last is bound
-// by reading the rows (41 MB a layer from shared memory and L2), the others by the
-// exchange: 0.25 (one CTA), 0.6 (cluster), 1.2 (words), 2.2 (count).
+// the operand loaded after it 1.61 / 1.98 / 2.23 / 2.72 / 2.92 / 4.75.  They are bound by the
+// exchange: 0.25 (one CTA), 0.6 (cluster), 1.2 (words), 2.2 (count); the last by that and by
+// reading the rows, about half each (a CTA's 22 rows, 16 from shared memory and 6 from L2).
 //
 // Every wait has a deadline after which the kernel records RELU_QP_ERR_TIMEOUT
 // in the error word; the other waits see it and leave too.
@@ -61,7 +61,7 @@ constexpr int kWarps = kThreads / 32;
 
 enum { RED_RP = 0, RED_RD, RED_AX, RED_Z, RED_PX, RED_ATL, RED_WORDS = 8 };
 enum { DEC_STOP = 6, DEC_RHO = 7 };   // of the decision's words: 1 + the status to stop with, or 0; bank entry
-enum { OUT_STATUS = 0, OUT_ITERS, OUT_RHO, OUT_SWITCHES, OUT_ERR, OUT_LAST, OUT_WORDS = 8 };
+enum { OUT_STATUS = 0, OUT_ITERS, OUT_RHO, OUT_SWITCHES, OUT_LAST, OUT_WORDS = 8 };
 // FORM_GRID and FORM_COUNT are cooperative grids: tagged words, or plain operand buffers and a
 // count of the CTAs that have written theirs.
 enum Form { FORM_GRID = 0, FORM_CLUSTER = 1, FORM_ONE = 2, FORM_COUNT = 3 };
@@ -98,32 +98,13 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
-// Dot product of a padded row with a padded vector in shared memory; the
-// result is valid in every lane.  Rows and vectors are 16-byte aligned and
-// zero padded to a multiple of 4 floats.
-__device__ __forceinline__ float row_dot(const float* __restrict__ w, const float* __restrict__ s,
-                                         int ld, int lane) {
-    const float4* w4 = reinterpret_cast<const float4*>(w);
-    const float4* s4 = reinterpret_cast<const float4*>(s);
-    const int n4 = ld >> 2;
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-    for (int k = lane; k < n4; k += 32) {
-        const float4 a = w4[k];
-        const float4 b = s4[k];
-        a0 = fmaf(a.x, b.x, a0);
-        a1 = fmaf(a.y, b.y, a1);
-        a2 = fmaf(a.z, b.z, a2);
-        a3 = fmaf(a.w, b.w, a3);
-    }
-    return warp_sum((a0 + a1) + (a2 + a3));
-}
-
 constexpr int kRows = 4;   // rows of a warp whose dot products run together (a group)
 
 // Dot products of NR (1, 2 or 4) padded rows (w[j], in shared or global memory) with one
-// padded vector in shared memory, in one pass over k: every row keeps the four accumulators
-// and the summation tree of row_dot, so each result has row_dot's bits, while the rows' loads
-// overlap.  The sums are scattered as they are formed (a lane keeps half of its rows at each
+// padded vector in shared memory, in one pass over k, so that the rows' loads overlap.  Rows and
+// vector are 16-byte aligned and zero padded to a multiple of 4 floats.  Every row keeps four
+// accumulators and one summation tree of its own, whatever NR is, so that a row's bits do not
+// depend on its group.  The sums are scattered as they are formed (a lane keeps half of its rows at each
 // of the first steps: 6 shuffles for 4 rows where one reduction per row takes 20, and a
 // CTA's shuffles go one warp a clock): lane l returns row l / (32 / NR).
 template <int NR, bool LDG>

@@ -281,6 +281,9 @@ __global__ void __launch_bounds__(kThreads, 1) single64_kernel(const __grid_cons
                     if (full) publish64(e + 1, r, snew);
                     else publish32(e + 1, r, (float)(snew - st_sref[lr]));
                     st_lam[lr] = lam;
+                    // (t - z + lam / rho, as the FP32 solve has it, would put an FP64 division
+                    // into every layer: n = 342 450 us against 415, n = 1110 anchored 480 against
+                    // 425, and the same error against more digits, 2.0e-10 and 3.8e-10)
                     st_rr[lr] = t - z + rr;
                 } else if (full) {
                     publish64(e + 1, r, snew);
