@@ -428,17 +428,16 @@ __global__ void __launch_bounds__(8 * TS, 1) batch_chunk_fp32_kernel(BatchParams
     cp_async_wait<0>();
     __syncthreads();
     cl_sync_hw();                                      // every CTA's mbarrier is armed
-    // a warp whose wait gave up keeps only the barriers: it sends nothing, so that its partners'
-    // waits find the error word and not their bytes, and nobody goes on sending to a CTA that
-    // no longer counts what arrives
+    // a thread whose wait gave up goes through the layers (its warp's shuffles and the barriers name
+    // it) but sends nothing, so that its partners' waits find the error word and not their bytes,
+    // and nobody goes on sending to a CTA that no longer counts what arrives
     bool failed = false;
     for (int j = 0; j < nl; ++j) {
         const bool last = j == nl - 1;
         if (j > 0) {
-            if (!failed && !cl_wait_warp(bar, (uint32_t)((j - 1) & 1), err, timeout_ns)) failed = true;
+            if (!failed && !cl_wait(bar, (uint32_t)((j - 1) & 1), err, timeout_ns)) failed = true;
             if (threadIdx.x == 0 && !failed && !last) cl_expect(bar, bytes);
         }
-        if (last) cl_close_arrive();                   // (the last operand was sent a layer ago)
         float acc[SA][RA];
 #pragma unroll
         for (int a = 0; a < SA; ++a)
@@ -493,7 +492,6 @@ __global__ void __launch_bounds__(8 * TS, 1) batch_chunk_fp32_kernel(BatchParams
             }
         asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
         __syncwarp();
-        if (failed) continue;
         // four lanes hold rows 4 q .. 4 q + 3 of two slots, for either b: transposed, a lane has
         // four consecutive rows to send at once
         const int jl = tx & 3;
@@ -510,10 +508,10 @@ __global__ void __launch_bounds__(8 * TS, 1) batch_chunk_fp32_kernel(BatchParams
                     if (i == c) o[i] = g;
             }
             const uint32_t dst = cl_smem(Xs + (ty + NW * (a + (jl >> 1))) * lds + row0 + 32 * (jl & 1) + (tx & 28));
-            for (int q = 0; q < ctas; ++q) cl_send4(dst, bar, q, o[0], o[1], o[2], o[3]);
+            for (int q = 0; q < (failed ? 0 : ctas); ++q) cl_send4(dst, bar, q, o[0], o[1], o[2], o[3]);
         }
     }
-    cl_close_wait(failed);
+    cl_close(failed);
 }
 
 // pdl: the kernel may start before the previous one of the stream has ended (its griddep_wait)

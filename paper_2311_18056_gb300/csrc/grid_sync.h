@@ -263,17 +263,13 @@ __device__ __forceinline__ void cl_settle() {
     for (const long long t0 = grid_sync_timer(); grid_sync_timer() - t0 < 50000;) {}
 }
 // The end of a kernel whose CTAs write into each other's shared memory: reached by every thread
-// of the cluster, so that no CTA leaves while a partner may still send to it.  A thread arrives
-// once it sends no more, and waits last (`failed`: a wait of this thread gave up).
-__device__ __forceinline__ void cl_close_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-__device__ __forceinline__ void cl_close_wait(bool failed) {
-    const int gave_up = __syncthreads_or(failed ? 1 : 0);
-    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-    if (gave_up) cl_settle();
-}
+// of the cluster, so that no CTA leaves while a partner may still send to it (a lifetime, no
+// order of memory).  `failed`: a wait of this thread gave up; one thread that stays keeps the
+// CTA's shared memory.
 __device__ __forceinline__ void cl_close(bool failed) {
-    cl_close_arrive();
-    cl_close_wait(failed);
+    __syncthreads();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (failed) cl_settle();
 }
 #endif
 

@@ -10,7 +10,7 @@ import re
 
 CSRC = os.path.join(os.path.dirname(os.path.abspath(__file__)), "..", "paper_2311_18056_gb300", "csrc")
 SEND = re.compile(r"\b(cl_send1|cl_send4|st_async4|st_cluster4|tile_epilogue<|solve_body<)")
-CLOSE = re.compile(r"\b(cl_close|cl_close_wait|cluster_sync)\(")
+CLOSE = re.compile(r"\b(cl_close|cluster_sync)\(")
 
 
 def kernels():
