@@ -61,7 +61,7 @@ constexpr int kWarps = kThreads / 32;
 
 enum { RED_RP = 0, RED_RD, RED_AX, RED_Z, RED_PX, RED_ATL, RED_WORDS = 8 };
 enum { DEC_STOP = 6, DEC_RHO = 7 };   // of the decision's words: 1 + the status to stop with, or 0; bank entry
-enum { OUT_STATUS = 0, OUT_ITERS, OUT_RHO, OUT_SWITCHES, OUT_LAST, OUT_WORDS = 8 };
+enum { OUT_STATUS = 0, OUT_ITERS, OUT_RHO, OUT_SWITCHES, OUT_LAST, OUT_GAVE_UP, OUT_WORDS = 8 };
 // FORM_GRID and FORM_COUNT are cooperative grids: tagged words, or plain operand buffers and a
 // count of the CTAs that have written theirs.
 enum Form { FORM_GRID = 0, FORM_CLUSTER = 1, FORM_ONE = 2, FORM_COUNT = 3 };
@@ -635,6 +635,8 @@ __global__ void __launch_bounds__(kThreads, 1) single_solve_kernel(const __grid_
         cl_sync_hw();   // every CTA's barriers stand before anything is sent
     }
     const bool done = (int)blockIdx.x >= p.ctas || solve_body<F>(p, smem, s_bar, s_red, s_dec);
+    // (the CTA that reports the results may have had all it waits for when another had not)
+    if (!done && threadIdx.x == 0) p.out_i[OUT_GAVE_UP] = 1;
     if (F == FORM_CLUSTER) cl_close(!done);   // (every wait before has a deadline, so every CTA gets here)
 }
 
@@ -852,13 +854,14 @@ int launch(relu_qp_t h, int ctas, int cluster, int cached, int gs, const float* 
     p.out_i = w.out_i;
     p.out_f = w.out_f;
     w.out_i[OUT_LAST] = -1;    // the kernel's results go to host memory
+    w.out_i[OUT_GAVE_UP] = 0;
     return launch_kernel(h, p, ctas, cluster);
 }
 
 // After the launch has been waited for: its error, or the next free exchange number.
 int finish(relu_qp_t h, const char* what) {
     SingleWork& w = h->sw;
-    if (w.out_i[OUT_LAST] < 0) {
+    if (w.out_i[OUT_LAST] < 0 || w.out_i[OUT_GAVE_UP]) {
         RQ_TRY(reset_words(h));
         RQ_CUDA(h, cudaStreamSynchronize(h->stream));
         return fail(h, RELU_QP_ERR_TIMEOUT, std::string("a wait passed its deadline ") + what);
@@ -1143,12 +1146,14 @@ int single_solve_noalloc(relu_qp_t h, const float* x_warm, const float* lam_warm
     p.out_i = w.out_i;
     p.out_f = w.out_f;
     w.out_i[OUT_LAST] = -1;
+    w.out_i[OUT_GAVE_UP] = 0;
     RQ_CUDA(h, cudaMemsetAsync(base, 0, sizeof(float) * (2 * words + 4), h->stream));
     RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
     RQ_TRY(launch_kernel(h, p, w.grid, w.cluster));
     RQ_CUDA(h, cudaEventRecord(h->ev1, h->stream));
     RQ_CUDA(h, cudaStreamSynchronize(h->stream));
-    if (w.out_i[OUT_LAST] < 0) return fail(h, RELU_QP_ERR_TIMEOUT, "a wait passed its deadline in relu_qp_solve_noalloc");
+    if (w.out_i[OUT_LAST] < 0 || w.out_i[OUT_GAVE_UP])
+        return fail(h, RELU_QP_ERR_TIMEOUT, "a wait passed its deadline in relu_qp_solve_noalloc");
     fill_info(h, info);
     return RELU_QP_OK;
 }

@@ -55,7 +55,7 @@ constexpr int kState = 11;   // doubles of state per row
 
 enum { RED_RP = 0, RED_RD, RED_AX, RED_Z, RED_PX, RED_ATL, RED_WORDS = 8 };
 enum { DEC_STOP = 6, DEC_RHO = 7 };   // of the decision's words: 1 + the status to stop with, or 0; bank entry
-enum { OUT_STATUS = 0, OUT_ITERS, OUT_RHO, OUT_SWITCHES, OUT_LAST, OUT_COUNTED, OUT_WORDS = 8 };
+enum { OUT_STATUS = 0, OUT_ITERS, OUT_RHO, OUT_SWITCHES, OUT_LAST, OUT_COUNTED, OUT_GAVE_UP, OUT_WORDS = 8 };
 
 struct SP64 {
     int n, m, R, nr;
@@ -139,15 +139,11 @@ __device__ __forceinline__ double red_get(const unsigned long long* slot, int wo
     return __longlong_as_double((long long)__ldcg(slot + word));
 }
 
-// TAG: tagged words, else counted CTAs.
+// TAG: tagged words, else counted CTAs.  False if a wait gave up.
 template <bool REFINED, bool TAG>
-__global__ void __launch_bounds__(kThreads, 1) single64_kernel(const __grid_constant__ SP64 p) {
-    extern __shared__ __align__(16) double smem[];
-    __shared__ double s_dec[RED_WORDS];
-    __shared__ unsigned long long s_red[RED_WORDS];
+__device__ __forceinline__ bool solve64_body(const SP64& p, double* smem, double* s_dec, unsigned long long* s_red) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
     const int n = p.n, m = p.m, R = p.R, cta = blockIdx.x;
-    if (cta >= p.ctas) return;
     const int x0 = cta * p.xr, nx = max(0, min(p.xr, n - x0));
     const int a0 = cta * p.ar, na = max(0, min(p.ar, m - a0));
     const int rows = nx + na, per = p.xr + p.ar, ncache = min(p.cached, rows);
@@ -247,7 +243,7 @@ __global__ void __launch_bounds__(kThreads, 1) single64_kernel(const __grid_cons
         if (lr >= nx) st_rr[lr] = st_lam[lr] / st_rho[lr];   // A x - z = 0
         publish64(0, r, lr < nx ? (p.xin ? p.xin[r] : 0.0) : 2.0 * st_rho[lr] * st_z[lr] - st_lam[lr]);
     }
-    if (!receive64(0)) return;
+    if (!receive64(0)) return false;
 
     for (int it = 1; it <= p.max_iter; ++it) {
         // ---------------- one layer ----------------
@@ -294,7 +290,7 @@ __global__ void __launch_bounds__(kThreads, 1) single64_kernel(const __grid_cons
             }
         }
         ++e;
-        if (!(full ? receive64(e) : receive32(e))) return;
+        if (!(full ? receive64(e) : receive32(e))) return false;
 
         const bool is_check = (p.check_interval > 0) && (it % p.check_interval == 0);
         if (!is_check && !last) continue;
@@ -319,7 +315,7 @@ __global__ void __launch_bounds__(kThreads, 1) single64_kernel(const __grid_cons
                 red_max(s_red, RED_Z, zi * f);
             }
         }
-        if (!all_arrived()) return;
+        if (!all_arrived()) return false;
         for (int k = tid; k < m; k += kThreads) svk[k] = __ldcg(p.ls + k);
         __syncthreads();
         for (int lr = warp; lr < nx; lr += kWarps) {
@@ -336,7 +332,7 @@ __global__ void __launch_bounds__(kThreads, 1) single64_kernel(const __grid_cons
             atomicMax(slot + tid, s_red[tid]);
             s_red[tid] = 0ull;
         }
-        if (!all_arrived()) return;
+        if (!all_arrived()) return false;
 
         // ---------------- decision (identical in every CTA; one warp's FP64) ----------------
         if (warp == 0) {
@@ -382,14 +378,14 @@ __global__ void __launch_bounds__(kThreads, 1) single64_kernel(const __grid_cons
                 p.out_f[0] = s_dec[RED_RP];
                 p.out_f[1] = s_dec[RED_RD];
             }
-            return;
+            return true;
         }
         if (nri == ri) {
             // the directly computed Ax replaces the carried one
             for (int lr = nx + tid; lr < rows; lr += kThreads)
                 st_rr[lr] = st_chk[lr] - st_z[lr] + st_lam[lr] / st_rho[lr];
             if (p.share) {
-                if (!receive64(e)) return;   // (lam_std was staged over the operand)
+                if (!receive64(e)) return false;   // (lam_std was staged over the operand)
             } else {
                 __syncthreads();
             }
@@ -413,8 +409,19 @@ __global__ void __launch_bounds__(kThreads, 1) single64_kernel(const __grid_cons
         }
         load_bank();
         ++e;
-        if (!receive64(e)) return;
+        if (!receive64(e)) return false;
     }
+    return true;
+}
+
+template <bool REFINED, bool TAG>
+__global__ void __launch_bounds__(kThreads, 1) single64_kernel(const __grid_constant__ SP64 p) {
+    extern __shared__ __align__(16) double smem[];
+    __shared__ double s_dec[RED_WORDS];
+    __shared__ unsigned long long s_red[RED_WORDS];
+    if ((int)blockIdx.x >= p.ctas) return;
+    // (the CTA that reports the results may have had all it waits for when another had not)
+    if (!solve64_body<REFINED, TAG>(p, smem, s_dec, s_red) && threadIdx.x == 0) p.out_i[OUT_GAVE_UP] = 1;
 }
 
 // b_r = Bop_r q for every bank entry (blockIdx.y), one warp per row.
@@ -516,6 +523,7 @@ int launch(relu_qp_t h, int grid, const double* xin, const double* lin, int rho_
     const size_t smem = smem64(h, grid, p.cached);
     w.last_ctas = p.ctas;
     w.out_i[OUT_LAST] = -1;   // the kernel's results go to host memory
+    w.out_i[OUT_GAVE_UP] = 0;
     RQ_CUDA(h, cudaMemsetAsync(w.red, 0, sizeof(unsigned long long) * 3 * RED_WORDS, h->stream));
     void* args[] = {&p};
     RQ_CUDA(h, cudaLaunchCooperativeKernel(kernel_for(h), dim3(grid), dim3(kThreads), args, smem, h->stream));
@@ -525,7 +533,7 @@ int launch(relu_qp_t h, int grid, const double* xin, const double* lin, int rho_
 // After the launch has been waited for: its error, or the next free exchange numbers.
 int finish(relu_qp_t h, const char* what) {
     SingleWork64& w = h->sw64;
-    if (w.out_i[OUT_LAST] < 0) {
+    if (w.out_i[OUT_LAST] < 0 || w.out_i[OUT_GAVE_UP]) {
         RQ_TRY(reset_words(h));
         RQ_CUDA(h, cudaStreamSynchronize(h->stream));
         return fail(h, RELU_QP_ERR_TIMEOUT, std::string("a wait passed its deadline ") + what);
