@@ -145,3 +145,29 @@ def test_condense_semidefinite_and_indefinite_weights(rq):
     with pytest.raises(rq.ReluQPError) as e:
         rq.condense_mpc(A, B, -Q, 1e-3 * np.eye(2), 5, umin=-np.ones(2), umax=np.ones(2))
     assert e.value.kind in ("NOT_PD", "INVALID")
+
+
+def test_condense_long_horizon_of_an_unstable_plant_keeps_its_digits(rq):
+    """Spectral radius 1.2, no preconditioning, N = 60: powers up to 6e4 whose rounding must grow as that of a
+    product formed step by step does (about sqrt(N) units of 64 bits, some 2e-15), not as N."""
+    nx, nu, N = 4, 1, 60
+    rng = np.random.default_rng([nx, nu, N])
+    A = np.eye(nx) + 0.3 * rng.standard_normal((nx, nx))
+    A *= 1.2 / np.max(np.abs(np.linalg.eigvals(A)))
+    B, Q, R, QN = rng.standard_normal((nx, nu)), np.eye(nx), 0.1 * np.eye(nu), 3.0 * np.eye(nx)
+    g = rq.condense_mpc(A, B, Q, R, N, QN=QN, umin=-np.ones(nu), umax=np.ones(nu), xmin=-np.ones(nx),
+                        lqr_precondition=False)
+    ld = np.longdouble
+    S, M, Sx, Mx = np.zeros((nx, N * nu), ld), np.eye(nx, dtype=ld), [], []
+    for k in range(N):
+        S = A.astype(ld) @ S
+        S[:, k * nu:(k + 1) * nu] += B
+        M = A.astype(ld) @ M
+        Sx.append(S.copy())
+        Mx.append(M.copy())
+    H = [QN.astype(ld) if k == N - 1 else Q.astype(ld) for k in range(N)]
+    P = ld(0.1) * np.eye(N * nu, dtype=ld) + sum(s.T @ h @ s for s, h in zip(Sx, H))
+    F = sum(s.T @ h @ m for s, h, m in zip(Sx, H, Mx))
+    n = N * nu
+    for got, want in ((g["P"], P), (g["F"], F), (g["A"][n:], np.vstack(Sx)), (g["E"][n:], np.vstack(Mx))):
+        assert np.max(np.abs(got - want)) <= 4e-15 * np.max(np.abs(want))
