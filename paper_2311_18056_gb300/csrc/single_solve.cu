@@ -919,10 +919,9 @@ int default_gs(relu_qp_t h, int ctas, int cluster) {
 int single_prepare(relu_qp_t h) {
     SingleWork& w = h->sw;
     w.grid = 0;
-    float best = 1e30f;
-    auto time = [&](int g, int cl, int cached, int gs, int layers, float* ms) -> int {
+    auto time = [&](int g, int cl, int cached, int gs, bool warm, float* ms) -> int {
         RQ_CUDA(h, cudaEventRecord(h->ev0, h->stream));
-        RQ_TRY(launch(h, g, cl, cached, gs, nullptr, nullptr, 0, 0.0, 0.0, layers, 0, 0));
+        RQ_TRY(launch(h, g, cl, cached, gs, nullptr, nullptr, 0, 0.0, 0.0, warm ? 10 : 50, 0, 0));
         RQ_CUDA(h, cudaEventRecord(h->ev1, h->stream));
         RQ_CUDA(h, cudaStreamSynchronize(h->stream));
         RQ_TRY(finish(h, "while tuning the solve"));
@@ -932,35 +931,63 @@ int single_prepare(relu_qp_t h) {
     // Grids, then clusters, the largest first: beyond its minimum the time rises with the rows
     // per CTA (a small grid or cluster of a large problem takes 100 times the best: 25 ms of the
     // setup at n = m = 800).
-    std::vector<int> grids{h->num_sms}, clusters{16, 8, 4, 2};
-    for (int g = 1; g <= 4 * h->num_sms; g *= 2) grids.push_back(g);
-    std::sort(grids.begin(), grids.end(), std::greater<int>());
-    for (const bool cl : {false, true}) {
-        const std::vector<int>& ctas = cl ? clusters : grids;
-        int cached = -1, chosen = -1;
-        RQ_TRY(search_family((int)ctas.size(), [&](int k, bool warm, float* ms) -> int {
-            const int c = ctas[k], cluster = cl ? c : 0;
-            if (warm) {
-                cached = c <= h->R ? cached_rows_for(h, c, cluster) : -1;
-                *ms = -1.f;
-                if (!fits(h, c, cluster, cached)) return RELU_QP_OK;
+    struct Shape {
+        int ctas, cluster, cached;
+    };
+    std::vector<Shape> shapes{{h->num_sms, 0, -1}};
+    for (int g = 1; g <= 4 * h->num_sms; g *= 2) shapes.push_back({g, 0, -1});
+    std::sort(shapes.begin(), shapes.end(), [](const Shape& a, const Shape& b) { return a.ctas > b.ctas; });
+    const int grids = (int)shapes.size();
+    for (int c : {16, 8, 4, 2}) shapes.push_back({c, c, -1});
+    auto possible = [&](Shape& s) {
+        s.cached = s.ctas <= h->R ? cached_rows_for(h, s.ctas, s.cluster) : -1;
+        return fits(h, s.ctas, s.cluster, s.cached);
+    };
+    auto use = [&](const Shape& s) {
+        w.grid = s.ctas;
+        w.cluster = s.cluster;
+        w.cached_rows = s.cached;
+        w.gs = default_gs(h, s.ctas, s.cluster);
+    };
+    if (h->opts.single_precision != RELU_QP_PREC_FP32) {
+        // a handle of FP64 solves never launches this one: any shape that fits
+        for (Shape& s : shapes)
+            if (possible(s)) {
+                use(s);
+                return RELU_QP_OK;
             }
-            return time(c, cluster, cached, default_gs(h, c, cluster), warm ? 10 : 50, ms);
-        }, &best, &chosen));
-        if (chosen < 0) continue;
-        w.grid = ctas[chosen];
-        w.cluster = cl ? w.grid : 0;
-        w.cached_rows = cached_rows_for(h, w.grid, w.cluster);
-        w.gs = default_gs(h, w.grid, w.cluster);
+        return fail(h, RELU_QP_ERR_UNSUPPORTED, "the single-QP solve does not fit on an SM");
     }
-    if (w.grid == 0) return fail(h, RELU_QP_ERR_UNSUPPORTED, "the single-QP solve does not fit on an SM");
+    auto shape_time = [&](int k, bool warm, float* ms) -> int {
+        Shape& s = shapes[k];
+        *ms = -1.f;
+        if (warm && !possible(s)) return RELU_QP_OK;
+        return time(s.ctas, s.cluster, s.cached, default_gs(h, s.ctas, s.cluster), warm, ms);
+    };
+    float best = 1e30f;
+    int chosen = -1;
+    std::vector<ShapeTime> timed, clusters;
+    RQ_TRY(search_family(grids, shape_time, &best, timed));
+    RQ_TRY(search_family((int)shapes.size() - grids,
+                         [&](int k, bool warm, float* ms) { return shape_time(grids + k, warm, ms); }, &best, clusters));
+    for (const ShapeTime& t : clusters) timed.push_back({grids + t.k, t.ms});
+    RQ_TRY(pick_shape(timed, shape_time, &chosen));
+    if (chosen < 0) return fail(h, RELU_QP_ERR_UNSUPPORTED, "the single-QP solve does not fit on an SM");
+    const Shape s = shapes[chosen];
+    use(s);
+    if (w.cluster > 1) return RELU_QP_OK;
+    // (groups of other sizes are within some 5 %: one run each)
+    float least = 1e30f;
+    for (const ShapeTime& t : timed)
+        if (t.k == chosen) least = t.ms;
     const int gs0 = w.gs;
     for (int gs : {1, 2, 4}) {
         float ms = 0.f;
-        if (w.cluster > 1 || gs == gs0) continue;
-        for (int layers : {10, 50}) RQ_TRY(time(w.grid, 0, w.cached_rows, gs, layers, &ms));
-        if (ms >= best) continue;
-        best = ms;
+        if (gs == gs0) continue;
+        RQ_TRY(time(s.ctas, 0, s.cached, gs, true, &ms));
+        RQ_TRY(time(s.ctas, 0, s.cached, gs, false, &ms));
+        if (ms >= least) continue;
+        least = ms;
         w.gs = gs;
     }
     return RELU_QP_OK;

@@ -620,7 +620,8 @@ int single64_prepare(relu_qp_t h) {
     std::sort(cands.begin(), cands.end(), std::greater<int>());
     float best = 1e30f;
     int chosen = -1;
-    RQ_TRY(search_family((int)cands.size(), [&](int k, bool warm, float* ms) -> int {
+    std::vector<ShapeTime> timed;
+    auto time = [&](int k, bool warm, float* ms) -> int {
         const int g = cands[k];
         *ms = -1.f;
         if (g > h->R || smem64(h, g, 0) > w.smem_max) return RELU_QP_OK;
@@ -631,7 +632,9 @@ int single64_prepare(relu_qp_t h) {
         RQ_TRY(finish(h, "while tuning the FP64 solve"));
         RQ_CUDA(h, cudaEventElapsedTime(ms, h->ev0, h->ev1));
         return RELU_QP_OK;
-    }, &best, &chosen));
+    };
+    RQ_TRY(search_family((int)cands.size(), time, &best, timed));
+    RQ_TRY(pick_shape(timed, time, &chosen));
     if (chosen < 0) return fail(h, RELU_QP_ERR_UNSUPPORTED, "FP64 solve kernel does not fit on an SM");
     w.grid = cands[chosen];
     return RELU_QP_OK;
